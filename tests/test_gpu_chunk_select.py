@@ -90,3 +90,14 @@ def test_rejections():
         binding.pulsar_chunk_select(ids, 100, 32, 8, 1, 0, "bm25")
     with pytest.raises(binding.PulsarError):                  # unknown score
         binding.pulsar_chunk_select(ids, 100, 2048, 16, 8, 16, 7)
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("chunk", [1, 31, 32, 33, 100, 1024])
+def test_chunk_lengths_around_a_warp(chunk, mode):
+    """The scores are formed 32 positions at a time: chunks at the edges of that, with a short last one, few
+    distinct tokens (long runs of repeats) and ids outside the vocabulary left out of the sums."""
+    rng = np.random.default_rng(chunk)
+    block = 2 * chunk + max(1, chunk // 2)
+    ids = rng.integers(0, max(3, chunk // 2), size=3 * block + chunk).astype(np.uint32)
+    run_and_compare(ids, 2000, block, chunk, 2, min(5, block), mode)
