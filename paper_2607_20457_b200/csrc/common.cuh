@@ -390,6 +390,17 @@ __device__ __forceinline__ float2 ex2_poly2(float2 x) {
     r.y = __int_as_float(__float_as_int(q.y) + (__float_as_int(t.y) << 23));
     return r;
 }
+// 32 bytes in one store where the address allows it (wide), in two otherwise.
+__device__ __forceinline__ void store_32b(void* dst, const uint32_t (&v)[8], bool wide) {
+    if (wide) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                     "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                     : "memory");
+    } else {
+        static_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        static_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
+}
 // Two floats -> packed bf16x2 (lo = a, hi = b), round to nearest even.
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
     uint32_t r;

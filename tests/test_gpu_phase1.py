@@ -182,3 +182,23 @@ def test_logits_that_jump_far_above_the_running_maximum(d):
     K = Kf.bfloat16()
     pidx, plen = W.first_k_prefix(w)
     print(run_phase1(w, Q, K, V, pidx, plen, what=f"jumping logits d={d}"))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_outputs_at_a_16_byte_aligned_base(d):
+    """Rows leave in 32-byte stores where the base allows it and in 16-byte ones otherwise: the same bits."""
+    w = W.shrink(W.CONFIGS["tiny"], L=600, block_size=200, d=d)
+    Q, K, V = (t.to(DEV) for t in W.qkv(w))
+    pidx, plen = (torch.from_numpy(x).to(DEV) for x in W.first_k_prefix(w))
+    O, LSE, _, _ = binding.pulsar_phase1_attn(Q, K, V, w.block_size, pidx, plen)
+    odd = torch.empty(Q.numel() + 8, dtype=torch.bfloat16, device=DEV)[8:].view(Q.shape)
+    assert odd.data_ptr() % 32 == 16
+    binding.pulsar_phase1_attn(Q, K, V, w.block_size, pidx, plen, out=odd)
+    assert torch.equal(odd, O)
+    Qq = W.phase2_query(w, nq=40).to(DEV)
+    _, _, pO, pL = binding.pulsar_phase2_attn(Qq, K, V, 1, w.L, n_splits=3, want_partials=True)
+    podd = torch.empty(pO.numel() + 4, device=DEV)[4:].view(pO.shape)
+    assert podd.data_ptr() % 32 == 16
+    pL2 = torch.empty_like(pL)
+    binding.pulsar_phase2_attn(Qq, K, V, 1, w.L, n_splits=3, partials=(podd, pL2))
+    assert torch.equal(podd, pO) and torch.equal(pL2, pL)
