@@ -1,12 +1,15 @@
-"""Builds the CUDA library in-tree: ``paper_2607_20457_b200/libpulsar.so`` (sm_100a only)."""
+"""Builds in-tree: the CUDA library ``libpulsar.so`` (sm_100a only) and ``_native.so``, the native half of the binding."""
 from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpulsar.so")
+NATIVE = os.path.join(HERE, "_native.so")
+NATIVE_SOURCE = os.path.join(CSRC, "binding.cpp")
 SOURCES = ["api.cu", "select.cu", "merge.cu", "attn.cu", "rope.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(os.path.dirname(HERE), "include", "pulsar.h")]
 NVCC_FLAGS = [
@@ -20,16 +23,35 @@ def _nvcc() -> str:
     return cand if os.path.exists(cand) else "nvcc"
 
 
+def _stale(target: str, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS
-    return any(os.path.getmtime(d) > t for d in deps)
+    return _stale(LIB, [os.path.join(CSRC, s) for s in SOURCES] + HEADERS)
+
+
+def build_native(force: bool = False) -> str:
+    """Compile the binding's extension module against the torch that is installed.  Returns its path."""
+    if not force and not _stale(NATIVE, [NATIVE_SOURCE, HEADERS[1]]):
+        return NATIVE
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    tmp = NATIVE + f".tmp{os.getpid()}"
+    subprocess.check_call([
+        "g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+        f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+        "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
+        "-I" + sysconfig.get_path("include"), "-I" + os.path.join(cuda, "include"), NATIVE_SOURCE, "-o", tmp,
+        "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+    os.replace(tmp, NATIVE)
+    return NATIVE
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu for sm_100a and link the shared library.  Returns its path."""
+    """Compile every .cu for sm_100a and link the shared library, and the binding's module.  Returns the library's path."""
+    build_native(force)
     if not force and not needs_build():
         return LIB
     objs = []
