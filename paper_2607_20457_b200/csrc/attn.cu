@@ -57,8 +57,6 @@ struct AttnArgs {
     int n_ctx_parts;       // phase 2: parts of the context KV; part n_ctx_parts (if any) is the generation shard
     int gen_len;           // phase 2: rows of the generation shard that precede the new tokens
     int gen_total;         // phase 2: gen_len + new tokens (0 = no generation shard)
-    int loader_waits;      // the launch before this one wrote rows the loader reads (the appended shard rows) and this
-                           // launch was allowed to start beside it: the loader waits for it first
     int quad;              // phase 2, at most 32 query rows per KV head: the rows are replicated into the four
                            // lane quarters of the tile and each softmax warp takes one quarter of the keys
     int single;            // phase 2, one query tile per KV head (at most 128 rows): the tile's logits alternate
@@ -83,15 +81,19 @@ struct AttnArgs {
 
 // ---------------------------------------------------------------------------------------------
 // Gather of the prefix rows: Kp[j] = K[prefix_idx[j]], Vp[j] = V[prefix_idx[j]] for j < total.
-// One CTA per prefix row; also checks that the row lies before the first block that uses it.
+// One CTA per prefix row; also checks that the row lies before the first block that uses it.  CTA 0 clears the
+// attention launch's work counter (a memset between the two launches would cost a launch of its own).
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128)
 gather_prefix_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, const int32_t* __restrict__ prefix_idx,
                      const int32_t* __restrict__ prefix_len, int n_blocks, int block_size, int64_t L,
-                     int row_vecs, uint4* __restrict__ Kp, uint4* __restrict__ Vp, int32_t* status) {
+                     int row_vecs, uint4* __restrict__ Kp, uint4* __restrict__ Vp, int32_t* counter, int32_t* status) {
     const int j = blockIdx.x;
     __shared__ int s_src;
+    grid_dependency_wait();                 // the prefix list may come from the launch before this one
+    grid_launch_dependents();
     if (threadIdx.x == 0) {
+        if (j == 0) *counter = 0;
         int64_t limit = -1;                 // stays -1 when no block uses entry j (the list may be shorter than its buffer)
         for (int i = 0; i < n_blocks; ++i)
             if (prefix_len[i] > j) { limit = static_cast<int64_t>(i) * block_size; break; }
@@ -125,11 +127,11 @@ gather_prefix_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, c
 }
 
 // KV(q) of the new tokens appended to the generation shard: one launch for both tensors.  The
-// attention launch that follows may start beside it; its loader waits for this grid before it
-// reads the shard.
+// attention launch that follows is placed beside it and waits for this grid before it reads anything.
 __global__ void __launch_bounds__(256)
 append_kv_kernel(const uint4* __restrict__ Knew, const uint4* __restrict__ Vnew, uint4* __restrict__ Kdst,
                  uint4* __restrict__ Vdst, int vecs) {
+    grid_dependency_wait();
     grid_launch_dependents();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < vecs) {
@@ -491,9 +493,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::kAbort);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // The launch that follows (the merge of this launch's partials, if any) may be scheduled as
-    // SMs become free; it waits for this grid to finish before it reads anything.
-    grid_launch_dependents();
 
     if (tid == 0) {
         *abort_flag = 0;
@@ -527,6 +526,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         tmem_alloc(tmem_ptr, 512);
         tmem_relinquish();
     }
+    // The CTAs of this launch may have been placed while the launch before it was still running; everything above
+    // (barriers, tensor maps, TMEM) overlaps its end, nothing below may.
+    grid_dependency_wait();
+    // The launch that follows (the merge of this launch's partials, or another call's) may be placed as
+    // SMs become free; it waits for this grid to finish before it reads anything.
+    grid_launch_dependents();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -551,7 +556,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             uint32_t q_use0 = 0, q_use1 = 0;
             bool ok = true;
             volatile int* item_q = reinterpret_cast<volatile int*>(smem + SL::kItemQ);
-            if (a.loader_waits) grid_dependency_wait();
             for (uint32_t seq = 0; ok; ++seq) {
                 // Reconverge once per iteration: every barrier is waited on at most once per
                 // iteration, so a lane that is still polling can never be more than one phase behind
@@ -1154,14 +1158,12 @@ bool make_map_2d(CUtensorMap* m, const void* base, int64_t rows, int64_t width) 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// overlap_prior: launch with programmatic stream serialization, i.e. the kernel may start while the
-// launch before it on the stream is still running (that launch must be this library's append
-// kernel, which releases its dependent at once); the loader then waits for it before its first
-// load (AttnArgs::loader_waits).
+// Launched with programmatic stream serialization: the CTAs may be placed while the launch before it on the stream
+// drains, and wait for that launch before they touch global memory.
 template <int D>
 int32_t launch_attn(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMap& v, const CUtensorMap& kp,
                     const CUtensorMap& vp, AttnArgs a, cudaStream_t stream,
-                    const VarlenTable* table = nullptr, bool overlap_prior = false) {
+                    const VarlenTable* table = nullptr) {
     constexpr int smem = SmemLayout<D>::kDynBytes;
     // The opt-in to more than 48 KB of dynamic shared memory is a per-device function attribute;
     // setting it on every launch keeps multi-device processes correct and costs well under a microsecond.
@@ -1181,7 +1183,7 @@ int32_t launch_attn(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMa
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = overlap_prior ? 1 : 0;
+    cfg.numAttrs = 1;
     PULSAR_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, q, k, v, kp, vp, a, table ? *table : kNoTable));
     PULSAR_CUDA_OK(cudaGetLastError());
     count_launch();
@@ -1232,9 +1234,12 @@ int32_t choose_splits(int32_t nq, int64_t L, int32_t Hq, int32_t Hkv, int32_t d)
     const double ctas = sm_count(), t_tile_us = 2.0, t_item_us = 6.0, hbm_bytes_per_us = 6.0e6;
     double best_t = 0;
     int64_t best = 1;
-    for (int64_t j = 1; j <= kv_tiles && j <= 1024; ++j) {
-        const int64_t tiles_per_part = (kv_tiles + j - 1) / j;
-        if ((kv_tiles + tiles_per_part - 1) / tiles_per_part != j) continue;      // some part would be empty
+    // Only the j without an empty part, ceil(tiles / ceil(tiles / j)) == j, are worth a look: at most twice the square
+    // root of the tiles.  After j comes the part count of the next smaller part size.  (Walking all j took 6.5 us of
+    // every call at 1024 tiles.)
+    for (int64_t j = 1, tiles_per_part; j <= kv_tiles && j <= 1024;
+         j = tiles_per_part > 1 ? (kv_tiles + tiles_per_part - 2) / (tiles_per_part - 1) : kv_tiles + 1) {
+        tiles_per_part = (kv_tiles + j - 1) / j;
         const double rounds = static_cast<double>((items * j + static_cast<int64_t>(ctas) - 1) / static_cast<int64_t>(ctas));
         const double partial = j > 1 ? 2.0 * j * nq * Hq * (d + 1) * 4.0 / hbm_bytes_per_us : 0.0;
         const double t = rounds * (static_cast<double>(tiles_per_part) * t_tile_us + t_item_us) + partial;
@@ -1306,15 +1311,14 @@ extern "C" int32_t pulsar_phase1_attn(const uint16_t* Q, const uint16_t* K, cons
         return PULSAR_ERR_CUDA;
 
     if (prefix_total > 0) {
-        gather_prefix_kernel<<<prefix_total, 128, 0, stream>>>(
-            reinterpret_cast<const uint4*>(K), reinterpret_cast<const uint4*>(V), prefix_idx, prefix_len, p.n_blocks,
-            block_size, L, Hkv * d * 2 / 16, reinterpret_cast<uint4*>(Kp), reinterpret_cast<uint4*>(Vp),
-            device_status);
-        PULSAR_CUDA_OK(cudaGetLastError());
+        PULSAR_CUDA_OK(launch_kernel(gather_prefix_kernel, dim3(prefix_total), dim3(128), 0, stream, true,
+                                     reinterpret_cast<const uint4*>(K), reinterpret_cast<const uint4*>(V), prefix_idx,
+                                     prefix_len, p.n_blocks, block_size, L, Hkv * d * 2 / 16, reinterpret_cast<uint4*>(Kp),
+                                     reinterpret_cast<uint4*>(Vp), counter, device_status));
         count_launch();
+    } else {
+        PULSAR_CUDA_OK(cudaMemsetAsync(counter, 0, sizeof(int32_t), stream));
     }
-
-    PULSAR_CUDA_OK(cudaMemsetAsync(counter, 0, sizeof(int32_t), stream));
 
     AttnArgs a{};
     a.mode = kModePhase1;
@@ -1626,11 +1630,10 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     // append KV(q) to the generation shard (Algorithm 1 line 15), then attend
     {
         const int vecs = static_cast<int>(n_new * row_bytes / 16);
-        append_kv_kernel<<<(vecs + 255) / 256, 256, 0, stream>>>(
-            reinterpret_cast<const uint4*>(Knew), reinterpret_cast<const uint4*>(Vnew),
-            reinterpret_cast<uint4*>(reinterpret_cast<char*>(Kgen) + gen_len * row_bytes),
-            reinterpret_cast<uint4*>(reinterpret_cast<char*>(Vgen) + gen_len * row_bytes), vecs);
-        PULSAR_CUDA_OK(cudaGetLastError());
+        PULSAR_CUDA_OK(launch_kernel(append_kv_kernel, dim3((vecs + 255) / 256), dim3(256), 0, stream, true,
+                                     reinterpret_cast<const uint4*>(Knew), reinterpret_cast<const uint4*>(Vnew),
+                                     reinterpret_cast<uint4*>(reinterpret_cast<char*>(Kgen) + gen_len * row_bytes),
+                                     reinterpret_cast<uint4*>(reinterpret_cast<char*>(Vgen) + gen_len * row_bytes), vecs));
         count_launch();
     }
 
@@ -1660,9 +1663,8 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     a.single = row_tiles == 1 ? 1 : 0;               // includes every decode shape (quad)
     a.pairs = (row_tiles + 1) / 2;
     a.n_items = a.pairs * Hkv * n_parts;
-    a.loader_waits = 1;                                // the shard rows are written by the append launch
-    rc = d == 128 ? launch_attn<128>(tmQ, tmK, tmV, tmKg, tmVg, a, stream, nullptr, true)
-                  : launch_attn<64>(tmQ, tmK, tmV, tmKg, tmVg, a, stream, nullptr, true);
+    rc = d == 128 ? launch_attn<128>(tmQ, tmK, tmV, tmKg, tmVg, a, stream)
+                  : launch_attn<64>(tmQ, tmK, tmV, tmKg, tmVg, a, stream);
     if (rc != PULSAR_OK) return rc;
     return launch_lse_merge(pO, pL, n_parts * copies, static_cast<int64_t>(n_new) * Hq, d, O, LSE, stream, true);
 }

@@ -32,9 +32,10 @@ __global__ void __launch_bounds__(kPresenceThreads)
 presence_kernel(const uint32_t* __restrict__ ids, int64_t L, int block_size, int vocab_size, int words,
                 uint32_t* __restrict__ bitmaps, int32_t* status) {
     extern __shared__ uint32_t bits[];
-    grid_launch_dependents();          // the next launch of the chain may be placed; it waits for this grid itself
     const int b = blockIdx.x;
     for (int w = threadIdx.x; w < words; w += blockDim.x) bits[w] = 0u;
+    grid_dependency_wait();            // the token ids, and the workspace, may be in use by the launch before this one
+    grid_launch_dependents();          // the next launch of the chain may be placed; it waits for this grid itself
     __syncthreads();
     const uint32_t* blk = ids + static_cast<size_t>(b) * block_size;
     const int len = static_cast<int>(min(static_cast<int64_t>(block_size), L - static_cast<int64_t>(b) * block_size));
@@ -206,6 +207,7 @@ topk_kernel(const uint16_t* __restrict__ level_all, int n_blocks, int64_t L, int
 
     for (int i = threadIdx.x; i < n_blocks + 3; i += blockDim.x) hist[i] = 0;
     grid_dependency_wait();                  // the chunk levels are complete
+    grid_launch_dependents();
     __syncthreads();
     for (int c = threadIdx.x; c < C; c += blockDim.x) {
         const int lv = level_all[static_cast<size_t>(b) * C + c];
@@ -379,6 +381,7 @@ topk_score_kernel(const double* __restrict__ score_all, int n_blocks, int64_t L,
     const int64_t lo = static_cast<int64_t>(b) * block_size;
     const int Cb = static_cast<int>((min(static_cast<int64_t>(block_size), L - lo) + chunk - 1) / chunk);
     grid_dependency_wait();                                // the scores are complete
+    grid_launch_dependents();
     for (int c = threadIdx.x; c < C; c += blockDim.x) sc[c] = score_all[static_cast<size_t>(b) * C + c];
     __syncthreads();
     int taken_before = 0;
@@ -493,9 +496,8 @@ extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, in
         PULSAR_CUDA_OK(cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             static_cast<int>(p.topk_smem)));
 
-    presence_kernel<<<p.n_blocks, kPresenceThreads, p.presence_smem, stream>>>(
-        token_ids, L, block_size, vocab_size, p.words, bitmaps, device_status);
-    PULSAR_CUDA_OK(cudaGetLastError());
+    PULSAR_CUDA_OK(launch_kernel(presence_kernel, dim3(p.n_blocks), dim3(kPresenceThreads), p.presence_smem, stream, true,
+                                 token_ids, L, block_size, vocab_size, p.words, bitmaps, device_status));
     count_launch();
     // The three launches that follow are programmatic dependents of the one before them: they are placed
     // while it runs and wait for it on the device, which takes the launch gaps out of the chain.
@@ -585,9 +587,8 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
     if (b.presence_smem > 48 * 1024)
         PULSAR_CUDA_OK(cudaFuncSetAttribute(presence_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             static_cast<int>(b.presence_smem)));
-    presence_kernel<<<b.n_blocks, kPresenceThreads, b.presence_smem, stream>>>(token_ids, L, block_size, vocab_size,
-                                                                               b.words, bitmaps, device_status);
-    PULSAR_CUDA_OK(cudaGetLastError());
+    PULSAR_CUDA_OK(launch_kernel(presence_kernel, dim3(b.n_blocks), dim3(kPresenceThreads), b.presence_smem, stream, true,
+                                 token_ids, L, block_size, vocab_size, b.words, bitmaps, device_status));
     count_launch();
     // Programmatic dependents of the launch before them, as in pulsar_maxidf_select.
     PULSAR_CUDA_OK(launch_kernel(df_idf_kernel, dim3((vocab_size + 255) / 256), dim3(256), 0, stream, true, bitmaps,
