@@ -23,10 +23,8 @@
 
 namespace pulsar {
 
-// after_attention: the merge follows the attention launch that wrote the partials and may be
-// scheduled while that launch drains (it waits for it before it reads).
 int32_t launch_lse_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t rows, int32_t d,
-                         uint16_t* O, float* LSE, cudaStream_t stream, bool after_attention = false);
+                         uint16_t* O, float* LSE, cudaStream_t stream);
 
 namespace {
 
@@ -1570,7 +1568,7 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
                   : launch_attn<64>(tmQ, tmK, tmV, tmK, tmV, a, stream);
     if (rc != PULSAR_OK) return rc;
     if (partial_out)
-        return launch_lse_merge(pO, pL, n_splits * copies, static_cast<int64_t>(nq) * Hq, d, O, LSE, stream, true);
+        return launch_lse_merge(pO, pL, n_splits * copies, static_cast<int64_t>(nq) * Hq, d, O, LSE, stream);
     return PULSAR_OK;
 }
 
@@ -1666,7 +1664,7 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     rc = d == 128 ? launch_attn<128>(tmQ, tmK, tmV, tmKg, tmVg, a, stream)
                   : launch_attn<64>(tmQ, tmK, tmV, tmKg, tmVg, a, stream);
     if (rc != PULSAR_OK) return rc;
-    return launch_lse_merge(pO, pL, n_parts * copies, static_cast<int64_t>(n_new) * Hq, d, O, LSE, stream, true);
+    return launch_lse_merge(pO, pL, n_parts * copies, static_cast<int64_t>(n_new) * Hq, d, O, LSE, stream);
 }
 
 // =============================================================================================

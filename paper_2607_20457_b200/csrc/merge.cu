@@ -1,7 +1,7 @@
 // Online-softmax merge of attention partials (Appendix H, Eq. 12-13) in closed form:
 //   l = m + ln sum_j exp(l_j - m),  O = sum_j exp(l_j - l) A_j,  m = max_j l_j.
-// One thread per four consecutive output elements: 128-bit loads of the fp32 partials, one
-// 64-bit store of bf16.  The kernel is a pure stream over J*rows*(d+1) floats.
+// For the head sizes of the attention kernels a warp owns an output row and its parts are spread over the warps of
+// a CTA; other row sizes take one thread per four consecutive output elements.
 #include "common.cuh"
 
 namespace pulsar {
@@ -50,98 +50,111 @@ lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ par
     if (LSE != nullptr && v == 0) LSE[row] = (m > -INFINITY) ? m + logf(denom) : -INFINITY;
 }
 
-// The same merge for few output rows and many parts (decode shapes), where one thread per output
-// vector would run a long chain of load latencies on a handful of CTAs: kLanes consecutive lanes
-// share an output vector, lane i takes parts i, i + kLanes, ...; the maximum and the sums are
-// combined by butterfly shuffles (a fixed order, so the result is reproducible).  A lane issues
-// the loads of all its parts -- the l_j and the output vectors, which do not depend on them --
-// before it uses any (up to kMaxInFlight parts at a time), so the kernel lasts about one memory
-// round trip however many parts there are.
-constexpr int kMergeLanes = 8;          // moderate part counts
-constexpr int kMergeLanesWide = 32;     // decode shapes: 4 partials per KV part, dozens of parts
-// Outputs (rows x d/4) up to which the lane form is used.  Measured: 72 parts into 32 or 256 rows 3.5 us
-// faster than one thread per output; 16 parts into 2048 rows 2.6 us and 64 parts into 1024 rows 6 us slower.
-constexpr int64_t kMergeLanesMaxThreads = 8192;
-// ... and up to which a whole warp shares an output vector.  Measured at 72 parts: 32 rows (1024 outputs)
-// 3 us faster than with 8 lanes, 256 rows (8192 outputs) no faster.
-constexpr int64_t kMergeWideMaxThreads = 1024;
-
-template <bool kF32, int kLanes>
-__global__ void __launch_bounds__(256)
-lse_merge_lanes_kernel(const float* __restrict__ part_O, const float* __restrict__ part_LSE, int n_parts,
-                       int64_t stride_O, int64_t stride_L, int64_t rows, int d, void* __restrict__ O_,
-                       float* __restrict__ LSE) {
+// The same merge for rows of 32 * kVec floats (d = 64, 128): a warp loads a part's row as one contiguous run,
+// kWarps warps share a row, warp w taking parts w, w + kWarps, ...  The merge after an attention launch is latency-bound
+// -- a few hundred rows, tens of parts, everything in L2 -- so each warp issues the loads of eight parts (the l_j and
+// the row pieces, which do not depend on them) before it uses any, and there are enough warps per row that one or
+// two such rounds cover all parts.  The order of the sums is fixed, so the result is reproducible.
+// Measured tail from the end of the attention launch to the end of the merge: 384 rows of 19 parts
+// 8.5 us with one thread per four outputs, 3.4 us with this form; 1600 rows of 18 parts 10 -> 8 us.
+template <bool kF32, int kVec, int kWarps, int kRows>
+__global__ void __launch_bounds__(32 * kWarps * kRows)
+lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict__ part_LSE, int n_parts,
+                      int64_t stride_O, int64_t stride_L, int64_t rows, void* __restrict__ O_,
+                      float* __restrict__ LSE) {
+    static_assert(kRows == 1 || kWarps == 1, "a CTA has one row, or one warp per row");
     grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
-    constexpr int kMaxInFlight = 4;
-    const int vec_per_row = d >> 2;
-    const int64_t tid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int sub = static_cast<int>(tid % kLanes);
-    const int64_t idx = tid / kLanes;
-    const bool valid = idx < rows * vec_per_row;
-    const int64_t row = valid ? idx / vec_per_row : 0;
-    const int v = valid ? static_cast<int>(idx - row * vec_per_row) : 0;
+    grid_launch_dependents();
+    constexpr int kD = 32 * kVec, kInFlight = 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t row = static_cast<int64_t>(blockIdx.x) * kRows + (kWarps == 1 ? warp : 0);
+    if (row >= rows) return;                                     // kRows > 1 only: no barrier follows
+    const float* src = part_O + row * kD + lane * kVec;
 
-    // running maximum, weight sum and weighted sum over this lane's parts (ascending part order)
-    float m = -INFINITY, denom = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (valid) {
-        for (int j0 = sub; j0 < n_parts; j0 += kLanes * kMaxInFlight) {
-            float l[kMaxInFlight];
-            float4 o[kMaxInFlight];
+    float m = -INFINITY, denom = 0.f, acc[kVec];
 #pragma unroll
-            for (int b = 0; b < kMaxInFlight; ++b) {
-                const int j = j0 + b * kLanes;
-                const int jc = j < n_parts ? j : j0;                 // a slot past the end repeats a load and weighs nothing
-                l[b] = part_LSE[static_cast<size_t>(jc) * stride_L + row];
-                o[b] = *reinterpret_cast<const float4*>(part_O + static_cast<size_t>(jc) * stride_O + row * d + v * 4);
-                if (j >= n_parts) l[b] = -INFINITY;
-            }
-            float m_new = m;
+    for (int k = 0; k < kVec; ++k) acc[k] = 0.f;
+    for (int j0 = kWarps == 1 ? 0 : warp; j0 < n_parts; j0 += kWarps * kInFlight) {
+        float l[kInFlight], o[kInFlight][kVec];
 #pragma unroll
-            for (int b = 0; b < kMaxInFlight; ++b) m_new = fmaxf(m_new, l[b]);
-            if (m_new > -INFINITY) {
-                const float keep = (m == -INFINITY) ? 0.f : __expf(m - m_new);
-                denom *= keep;
-                acc.x *= keep; acc.y *= keep; acc.z *= keep; acc.w *= keep;
-#pragma unroll
-                for (int b = 0; b < kMaxInFlight; ++b) {
-                    const float w = (l[b] == -INFINITY) ? 0.f : __expf(l[b] - m_new);
-                    denom += w;
-                    acc.x += w * o[b].x; acc.y += w * o[b].y; acc.z += w * o[b].z; acc.w += w * o[b].w;
+        for (int i = 0; i < kInFlight; ++i) {
+            const int j = j0 + i * kWarps;
+            l[i] = -INFINITY;
+            if (j < n_parts) {
+                l[i] = part_LSE[static_cast<size_t>(j) * stride_L + row];
+                const float* p = src + static_cast<size_t>(j) * stride_O;
+                if (kVec == 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(p);
+                    o[i][0] = v.x; o[i][1] = v.y; o[i][kVec - 2] = v.z; o[i][kVec - 1] = v.w;
+                } else {
+                    const float2 v = *reinterpret_cast<const float2*>(p);
+                    o[i][0] = v.x; o[i][1] = v.y;
                 }
-                m = m_new;
+            } else {
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) o[i][k] = 0.f;
+            }
+        }
+        float m_new = m;
+#pragma unroll
+        for (int i = 0; i < kInFlight; ++i) m_new = fmaxf(m_new, l[i]);
+        if (m_new > -INFINITY) {
+            const float keep = (m == -INFINITY) ? 0.f : __expf(m - m_new);
+            denom *= keep;
+#pragma unroll
+            for (int k = 0; k < kVec; ++k) acc[k] *= keep;
+#pragma unroll
+            for (int i = 0; i < kInFlight; ++i) {
+                const float w = (l[i] == -INFINITY) ? 0.f : __expf(l[i] - m_new);
+                denom += w;
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) acc[k] += w * o[i][k];
+            }
+            m = m_new;
+        }
+    }
+    if (kWarps > 1) {
+        __shared__ float s_m[kWarps], s_denom[kWarps], s_acc[kWarps][kD];
+        if (lane == 0) {
+            s_m[warp] = m;
+            s_denom[warp] = denom;
+        }
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) s_acc[warp][k * 32 + lane] = acc[k];
+        __syncthreads();
+        if (warp != 0) return;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) m = fmaxf(m, s_m[w]);
+        denom = 0.f;
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) acc[k] = 0.f;
+        if (m > -INFINITY) {
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const float f = (s_m[w] == -INFINITY) ? 0.f : __expf(s_m[w] - m);
+                denom += f * s_denom[w];
+#pragma unroll
+                for (int k = 0; k < kVec; ++k) acc[k] += f * s_acc[w][k * 32 + lane];
             }
         }
     }
-    // bring the lanes to the common maximum, then add them up
-    float m_all = m;
-#pragma unroll
-    for (int o = 1; o < kLanes; o <<= 1) m_all = fmaxf(m_all, __shfl_xor_sync(0xffffffffu, m_all, o));
-    const float mine = (m == -INFINITY) ? 0.f : __expf(m - m_all);
-    denom *= mine;
-    acc.x *= mine; acc.y *= mine; acc.z *= mine; acc.w *= mine;
-#pragma unroll
-    for (int o = 1; o < kLanes; o <<= 1) {
-        denom += __shfl_xor_sync(0xffffffffu, denom, o);
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
-        acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
-    }
-    if (!valid || sub != 0) return;
-    if (m_all > -INFINITY) {
+    if (m > -INFINITY) {
         const float inv = 1.f / denom;
-        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+#pragma unroll
+        for (int k = 0; k < kVec; ++k) acc[k] *= inv;
     }
+    const int64_t at = row * kD + lane * kVec;
     if (kF32) {
-        *reinterpret_cast<float4*>(static_cast<float*>(O_) + row * d + v * 4) = acc;
+        float* dst = static_cast<float*>(O_) + at;
+        if (kVec == 4) *reinterpret_cast<float4*>(dst) = make_float4(acc[0], acc[1], acc[kVec - 2], acc[kVec - 1]);
+        else *reinterpret_cast<float2*>(dst) = make_float2(acc[0], acc[1]);
     } else {
-        uint2 packed;
-        packed.x = pack_bf16x2(acc.x, acc.y);
-        packed.y = pack_bf16x2(acc.z, acc.w);
-        *reinterpret_cast<uint2*>(static_cast<uint16_t*>(O_) + row * d + v * 4) = packed;
+        uint16_t* dst = static_cast<uint16_t*>(O_) + at;
+        if (kVec == 4)
+            *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[kVec - 2], acc[kVec - 1]));
+        else *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(acc[0], acc[1]);
     }
-    if (LSE != nullptr && v == 0) LSE[row] = (m_all > -INFINITY) ? m_all + logf(denom) : -INFINITY;
+    if (LSE != nullptr && lane == 0) LSE[row] = (m > -INFINITY) ? m + logf(denom) : -INFINITY;
 }
 
 // The merge with every part at its own address: part j is the buffer parts[j], laid out
@@ -195,56 +208,48 @@ lse_merge_table_kernel(const __grid_constant__ PartTable parts, int n_parts, int
 }
 
 namespace {
-// Launch with or without programmatic stream serialization (see launch_lse_merge).
-template <typename Kernel, typename... Args>
-cudaError_t launch_maybe_dependent(Kernel kernel, unsigned blocks, cudaStream_t stream, bool dependent, Args... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+template <bool kF32, int kVec>
+auto merge_rows_kernel(int warps) {
+    return warps == 16  ? lse_merge_rows_kernel<kF32, kVec, 16, 1>
+           : warps == 8 ? lse_merge_rows_kernel<kF32, kVec, 8, 1>
+           : warps == 4 ? lse_merge_rows_kernel<kF32, kVec, 4, 1>
+           : warps == 2 ? lse_merge_rows_kernel<kF32, kVec, 2, 1>
+                        : lse_merge_rows_kernel<kF32, kVec, 1, 8>;
 }
 
 int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t stride_O, int64_t stride_L,
-                     int64_t rows, int32_t d, void* O, bool f32, float* LSE, cudaStream_t stream,
-                     bool dependent = false) {
+                     int64_t rows, int32_t d, void* O, bool f32, float* LSE, cudaStream_t stream) {
     if (rows == 0) return PULSAR_OK;
-    const int64_t threads = rows * (d >> 2);
-    if (n_parts >= 2 * kMergeLanes && threads <= kMergeLanesMaxThreads) {
-        // few outputs, many parts: spread the parts of an output over lanes
-        const bool wide = n_parts >= 2 * kMergeLanesWide && threads <= kMergeWideMaxThreads;
-        const int lanes = wide ? kMergeLanesWide : kMergeLanes;
-        const unsigned blocks = static_cast<unsigned>((threads * lanes + 255) / 256);
-        auto kernel = wide ? (f32 ? lse_merge_lanes_kernel<true, kMergeLanesWide> : lse_merge_lanes_kernel<false, kMergeLanesWide>)
-                           : (f32 ? lse_merge_lanes_kernel<true, kMergeLanes> : lse_merge_lanes_kernel<false, kMergeLanes>);
-        PULSAR_CUDA_OK(launch_maybe_dependent(kernel, blocks, stream, dependent, part_O, part_LSE, static_cast<int>(n_parts),
-                                              stride_O, stride_L, rows, static_cast<int>(d), O, LSE));
-        PULSAR_CUDA_OK(cudaGetLastError());
+    if (d == 64 || d == 128) {
+        // Warps per row: as many as leave a warp four to eight parts (one round of loads), while all of them fit the
+        // chip about once (148 SMs of 64 warps); with more rows than that the rows themselves fill it.
+        int warps = n_parts > 64 ? 16 : n_parts > 32 ? 8 : n_parts > 16 ? 4 : n_parts > 8 ? 2 : 1;
+        while (warps > 1 && rows * warps > 2 * 148 * 64) warps /= 2;
+        const int64_t blocks = warps == 1 ? (rows + 7) / 8 : rows;
+        if (blocks > 0x7fffffffll) return PULSAR_ERR_SHAPE;
+        auto kernel = d == 128 ? (f32 ? merge_rows_kernel<true, 4>(warps) : merge_rows_kernel<false, 4>(warps))
+                               : (f32 ? merge_rows_kernel<true, 2>(warps) : merge_rows_kernel<false, 2>(warps));
+        PULSAR_CUDA_OK(launch_kernel(kernel, dim3(static_cast<unsigned>(blocks)), dim3(warps == 1 ? 256 : 32 * warps), 0, stream,
+                                     true, part_O, part_LSE, n_parts, stride_O, stride_L, rows, O, LSE));
         count_launch();
         return PULSAR_OK;
     }
+    const int64_t threads = rows * (d >> 2);
     const int64_t blocks = (threads + 255) / 256;
     if (blocks > 0x7fffffffll) return PULSAR_ERR_SHAPE;
     auto kernel = f32 ? lse_merge_kernel<true> : lse_merge_kernel<false>;
-    PULSAR_CUDA_OK(launch_maybe_dependent(kernel, static_cast<unsigned>(blocks), stream, dependent, part_O, part_LSE,
-                                          static_cast<int>(n_parts), stride_O, stride_L, rows, static_cast<int>(d), O, LSE));
-    PULSAR_CUDA_OK(cudaGetLastError());
+    PULSAR_CUDA_OK(launch_kernel(kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, stream, true, part_O, part_LSE,
+                                 n_parts, stride_O, stride_L, rows, d, O, LSE));
     count_launch();
     return PULSAR_OK;
 }
 }  // namespace
 
-// after_attention: launched right behind the attention kernel that writes the partials, with
-// programmatic stream serialization: its CTAs are placed as that kernel's CTAs leave and wait
-// (grid_dependency_wait) until it has finished, so no launch gap separates the two.
+// Placed as the CTAs of the launch before it leave (programmatic stream serialization), waits until that has finished
+// (grid_dependency_wait): no launch gap separates the merge from the attention launch that writes the partials.
 int32_t launch_lse_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t rows, int32_t d,
-                         uint16_t* O, float* LSE, cudaStream_t stream, bool after_attention) {
-    return launch_merge(part_O, part_LSE, n_parts, rows * d, rows, rows, d, O, false, LSE, stream, after_attention);
+                         uint16_t* O, float* LSE, cudaStream_t stream) {
+    return launch_merge(part_O, part_LSE, n_parts, rows * d, rows, rows, d, O, false, LSE, stream);
 }
 
 }  // namespace pulsar
@@ -259,7 +264,7 @@ extern "C" int32_t pulsar_lse_merge(const float* part_O, const float* part_LSE, 
     if (!aligned(part_O, 16) || !aligned(part_LSE, 4) || !aligned(O, 8)) return PULSAR_ERR_ALIGNMENT;
     int32_t rc = check_device();
     if (rc != PULSAR_OK) return rc;
-    return launch_lse_merge(part_O, part_LSE, n_parts, rows, d, O, LSE, static_cast<cudaStream_t>(stream), false);
+    return launch_lse_merge(part_O, part_LSE, n_parts, rows, d, O, LSE, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int32_t pulsar_lse_merge_strided(const float* part_O, const float* part_LSE, int32_t n_parts,

@@ -232,3 +232,26 @@ def test_part_count_that_leaves_a_part_empty_is_rejected():
     with pytest.raises(binding.PulsarError) as e:
         binding.pulsar_phase2_attn(W.phase2_query(w).to(DEV), K.to(DEV), V.to(DEV), w.n_blocks, w.block_size, n_splits=5)
     assert e.value.status == 2
+
+
+@pytest.mark.parametrize("d", [64, 128, 192])
+@pytest.mark.parametrize("J,rows", [(1, 1), (8, 9), (9, 8), (16, 33), (17, 7), (32, 5), (33, 300), (64, 2), (65, 3), (300, 1), (9, 20000), (40, 5000)])
+def test_merge_at_the_edges_of_its_splits(J, rows, d):
+    """Parts spread over 1, 2, 4, 8 or 16 warps per row; empty parts, a row without any part."""
+    gen = torch.Generator(device=DEV).manual_seed(J * 1000 + rows)
+    pO = torch.randn(J, rows, d, generator=gen, device=DEV)
+    pL = 3 * torch.randn(J, rows, generator=gen, device=DEV)
+    pL[torch.rand(J, rows, generator=gen, device=DEV) < 0.2] = float("-inf")
+    pL[:, rows // 2] = float("-inf")
+    l = pL.double().logsumexp(0)
+    w = torch.where(pL == float("-inf"), 0.0, (pL.double() - torch.where(l == float("-inf"), 0.0, l)).exp())
+    ref = (w[..., None] * pO.double()).sum(0)
+    out, lse = torch.empty(rows, d, device=DEV), torch.empty(rows, device=DEV)
+    binding.pulsar_lse_merge_strided(pO, pL, J, rows * d, rows, rows, d, out, lse)
+    # J products of values within 5 and float32 weights of at most 1 (their exponential: 2 ulp of 2^-23)
+    assert (out - ref).abs().max().item() <= 5e-6 * max(1.0, ref.abs().max().item())
+    empty = l == float("-inf")
+    assert torch.equal(torch.isneginf(lse), empty) and (out[empty] == 0).all()
+    assert (lse[~empty] - l[~empty]).abs().max().item() <= 5e-6 if (~empty).any() else True
+    O, _ = binding.pulsar_lse_merge(pO, pL)
+    assert torch.equal(O, out.bfloat16())
