@@ -52,9 +52,13 @@ struct AttnArgs {
     const int32_t* prefix_len;
     int split_len;         // phase 2: keys per KV part (the last part may be shorter)
     int kv_len;            // phase 2: context keys in total
-    int n_ctx_parts;       // phase 2: parts of the context KV; part n_ctx_parts (if any) is the generation shard
+    int gen_part;          // phase 2: the part that has the generation shard in front of its context keys (if any)
     int gen_len;           // phase 2: rows of the generation shard that precede the new tokens
     int gen_total;         // phase 2: gen_len + new tokens (0 = no generation shard)
+    const uint4* Knew;     // phase 2, one query tile per KV head: KV(q) of the new tokens, appended to the generation shard by
+    const uint4* Vnew;     // the CTA that reads the head's part of it (null: appended by a launch of its own)
+    uint4* Kgen;
+    uint4* Vgen;
     int quad;              // phase 2, at most 32 query rows per KV head: the rows are replicated into the four
                            // lane quarters of the tile and each softmax warp takes one quarter of the keys
     int single;            // phase 2, one query tile per KV head (at most 128 rows): the tile's logits alternate
@@ -124,8 +128,8 @@ gather_prefix_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, c
     }
 }
 
-// KV(q) of the new tokens appended to the generation shard: one launch for both tensors.  The
-// attention launch that follows is placed beside it and waits for this grid before it reads anything.
+// KV(q) of the new tokens appended to the generation shard: one launch for both tensors, for calls with more than
+// one query tile per KV head (with one, the attention kernel appends: append_head).
 __global__ void __launch_bounds__(256)
 append_kv_kernel(const uint4* __restrict__ Knew, const uint4* __restrict__ Vnew, uint4* __restrict__ Kdst,
                  uint4* __restrict__ Vdst, int vecs) {
@@ -394,27 +398,36 @@ __device__ __forceinline__ void decode_item(const AttnArgs& a, const VarlenTable
         it.has1 = (it.token0_b < a.n_tokens) ? 1 : 0;
         it.row0_a = it.row0_b = 0;
         it.bad_length = 0;
-        int n;
-        if (a.gen_total > 0 && it.part == a.n_ctx_parts) {
-            // the generation shard: read through the second pair of tensor maps, causal by token
-            it.pref_len = a.gen_total;
-            it.n_pref_tiles = (a.gen_total + kTileN - 1) / kTileN;
-            it.main_row0 = 0;
-            it.main_len = 0;
-            it.gen_base = a.gen_len;
-            n = it.n_pref_tiles;
-        } else {
-            it.pref_len = 0;
-            it.n_pref_tiles = 0;
-            it.main_row0 = it.part * a.split_len;
-            it.main_len = min(a.split_len, a.kv_len - it.main_row0);
-            it.gen_base = -1;
-            n = (it.main_len + kTileN - 1) / kTileN;
-        }
+        // the generation shard: read through the second pair of tensor maps, causal by token
+        const bool shard = a.gen_total > 0 && it.part == a.gen_part;
+        it.pref_len = shard ? a.gen_total : 0;
+        it.n_pref_tiles = (it.pref_len + kTileN - 1) / kTileN;
+        it.gen_base = shard ? a.gen_len : -1;
+        it.main_row0 = it.part * a.split_len;
+        it.main_len = max(0, min(a.split_len, a.kv_len - it.main_row0));
+        const int n = it.n_pref_tiles + (it.main_len + kTileN - 1) / kTileN;
         it.n_tiles_a = n;
         it.n_tiles_b = it.has1 ? n : 0;
     }
     it.n_load = max(it.n_tiles_a, it.n_tiles_b);
+}
+
+// KV(q) of the new tokens of one KV head appended to the generation shard by the warp that is about to load the
+// head's shard rows through TMA: written with plain stores, made visible to the async proxy, then loaded.  No other CTA
+// of the launch touches the head's rows.  (As a launch of its own the append cost 2.8 us on the host and 2-3 us on the
+// device of every decoding step.)
+__device__ __forceinline__ void append_head(const AttnArgs& a, int kvh, int d, int lane) {
+    const int vecs = d / 8;                                   // 16-byte vectors of a head's row
+    const int n = (a.gen_total - a.gen_len) * vecs;
+    for (int i = lane; i < n; i += 32) {
+        const int u = i / vecs, v = i - u * vecs;
+        const size_t src = (static_cast<size_t>(u) * a.Hkv + kvh) * vecs + v;
+        const size_t dst = (static_cast<size_t>(a.gen_len + u) * a.Hkv + kvh) * vecs + v;
+        a.Kgen[dst] = a.Knew[src];
+        a.Vgen[dst] = a.Vnew[src];
+    }
+    fence_proxy_async_global();
+    __syncwarp();
 }
 
 // Row maximum of 128 raw logits (3-input max, four independent chains).
@@ -584,6 +597,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 Item it;
                 decode_item(a, vt, idx, it);
                 if (it.bad_length && lane == 0) report(a.status, PULSAR_DEV_BAD_LENGTH);
+                if (kSingle && it.gen_base >= 0 && a.Knew != nullptr) append_head(a, it.kvh, D, lane);
                 const int x = it.kvh * D;
                 // query tile 0
                 ok = mbar_wait_a(bar0 + 8 * (SL::bQEmpty + 0), (q_use0 & 1) ^ 1, abort_flag, a.status);
@@ -1543,7 +1557,6 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
     a.pack = g;
     a.split_len = static_cast<int>(phase2_split_len(L, n_splits));
     a.kv_len = static_cast<int>(L);
-    a.n_ctx_parts = n_splits;
     a.quad = quad ? 1 : 0;
     a.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
     a.O = O;
@@ -1579,7 +1592,7 @@ extern "C" size_t pulsar_phase2_generate_workspace_bytes(int32_t n_new, int32_t 
                                                          int32_t Hkv, int32_t d, int32_t n_splits) {
     size_t a, b;
     if (plan_phase2(n_new, B, block_size, Hq, Hkv, d, n_splits, a, b) != PULSAR_OK) return 0;
-    // one more part than the context has: the generation shard; four partials per part for decode shapes
+    // room for a part of its own for the generation shard; four partials per part for decode shapes
     const size_t parts = static_cast<size_t>(n_splits + 1) * (phase2_quad(n_new, Hq / Hkv) ? 4 : 1);
     return round_up(parts * n_new * Hq * d * 4, 256) + round_up(parts * n_new * Hq * 4, 256);
 }
@@ -1601,7 +1614,15 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
         !aligned(Kgen, 16) || !aligned(Vgen, 16) || !aligned(O, 16) || (LSE && !aligned(LSE, 4)) ||
         !aligned(workspace, 256))
         return PULSAR_ERR_ALIGNMENT;
-    const int n_parts = n_splits + 1;
+    // Parts of equally many key tiles over context and shard.  The shard goes in front of the last part's context
+    // keys, or is a part of its own where the parts before it already hold the whole context.  (As a part of its own
+    // in any case it made 152 work items of 144 for 148 SMs at 8 KV heads and 18 parts.)
+    const int64_t L_ctx = static_cast<int64_t>(B) * block_size;
+    const int64_t ctx_tiles = (L_ctx + kTileN - 1) / kTileN, gen_tiles = (static_cast<int64_t>(gen_len) + n_new + kTileN - 1) / kTileN;
+    const int64_t part_tiles = (ctx_tiles + gen_tiles + n_splits - 1) / n_splits;
+    const int64_t ctx_parts = (ctx_tiles + part_tiles - 1) / part_tiles;
+    const bool own_part = ctx_tiles - (ctx_parts - 1) * part_tiles + gen_tiles > part_tiles;
+    const int n_parts = static_cast<int>(ctx_parts + (own_part ? 1 : 0));       // at most n_splits
     const bool quad = phase2_quad(n_new, Hq / Hkv);
     const int copies = quad ? 4 : 1;
     const size_t po_bytes = round_up(static_cast<size_t>(n_parts) * copies * n_new * Hq * d * 4, 256);
@@ -1625,16 +1646,6 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
         !make_map_2d(&tmVg, Vgen, static_cast<int64_t>(gen_len) + n_new, static_cast<int64_t>(Hkv) * d))
         return PULSAR_ERR_CUDA;
 
-    // append KV(q) to the generation shard (Algorithm 1 line 15), then attend
-    {
-        const int vecs = static_cast<int>(n_new * row_bytes / 16);
-        PULSAR_CUDA_OK(launch_kernel(append_kv_kernel, dim3((vecs + 255) / 256), dim3(256), 0, stream, true,
-                                     reinterpret_cast<const uint4*>(Knew), reinterpret_cast<const uint4*>(Vnew),
-                                     reinterpret_cast<uint4*>(reinterpret_cast<char*>(Kgen) + gen_len * row_bytes),
-                                     reinterpret_cast<uint4*>(reinterpret_cast<char*>(Vgen) + gen_len * row_bytes), vecs));
-        count_launch();
-    }
-
     float* pO = static_cast<float*>(workspace);
     float* pL = reinterpret_cast<float*>(static_cast<char*>(workspace) + po_bytes);
     AttnArgs a{};
@@ -1643,9 +1654,9 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     a.Hq = Hq;
     a.g = g;
     a.pack = g;
-    a.split_len = static_cast<int>(phase2_split_len(L, n_splits));
+    a.split_len = static_cast<int>(part_tiles * kTileN);
     a.kv_len = static_cast<int>(L);
-    a.n_ctx_parts = n_splits;
+    a.gen_part = n_parts - 1;
     a.gen_len = gen_len;
     a.gen_total = gen_len + n_new;
     a.quad = quad ? 1 : 0;
@@ -1659,6 +1670,20 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     const int row_tiles = (n_new + tokens_per_tile - 1) / tokens_per_tile;
     a.Hkv = Hkv;
     a.single = row_tiles == 1 ? 1 : 0;               // includes every decode shape (quad)
+    // KV(q) is appended to the generation shard first (Algorithm 1 line 15)
+    if (a.single) {
+        a.Knew = reinterpret_cast<const uint4*>(Knew);
+        a.Vnew = reinterpret_cast<const uint4*>(Vnew);
+        a.Kgen = reinterpret_cast<uint4*>(Kgen);
+        a.Vgen = reinterpret_cast<uint4*>(Vgen);
+    } else {
+        const int vecs = static_cast<int>(n_new * row_bytes / 16);
+        PULSAR_CUDA_OK(launch_kernel(append_kv_kernel, dim3((vecs + 255) / 256), dim3(256), 0, stream, true,
+                                     reinterpret_cast<const uint4*>(Knew), reinterpret_cast<const uint4*>(Vnew),
+                                     reinterpret_cast<uint4*>(reinterpret_cast<char*>(Kgen) + gen_len * row_bytes),
+                                     reinterpret_cast<uint4*>(reinterpret_cast<char*>(Vgen) + gen_len * row_bytes), vecs));
+        count_launch();
+    }
     a.pairs = (row_tiles + 1) / 2;
     a.n_items = a.pairs * Hkv * n_parts;
     rc = d == 128 ? launch_attn<128>(tmQ, tmK, tmV, tmKg, tmVg, a, stream)

@@ -116,3 +116,28 @@ def test_step_captured_as_a_cuda_graph_replays_to_the_same_results():
                                           gen_len)
         print(check_attention(O_replay, LSE_replay, Oref, Lref, f"graph replay fresh={fresh}"))
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("n_new", [1, 3, 9, 32, 33])
+@pytest.mark.parametrize("L,gen_len,n_splits", [(1, 0, 1), (128, 127, 1), (129, 128, 2), (1000, 700, 3), (300, 900, 2), (2049, 5, 17), (640, 0, 5)])
+def test_shard_beside_the_last_part_of_the_context(L, gen_len, n_splits, n_new):
+    """The shard shares the last context part, or has a part of its own when the others hold the whole context; its new
+    rows are appended by the attention kernel (one query tile) or by a launch before it (33 tokens of 4 heads)."""
+    Hq, Hkv, d = 8, 2, 64
+    gen = torch.Generator().manual_seed(L + gen_len + n_new)
+    K, V = (torch.randn(L, Hkv, d, generator=gen).to(torch.bfloat16) for _ in range(2))
+    cap = gen_len + n_new + 3
+    Kg, Vg = (torch.randn(cap, Hkv, d, generator=gen).to(torch.bfloat16) for _ in range(2))
+    Qn = (2 * torch.randn(n_new, Hq, d, generator=gen)).to(torch.bfloat16)
+    Kn, Vn = (torch.randn(n_new, Hkv, d, generator=gen).to(torch.bfloat16) for _ in range(2))
+    Kg_d, Vg_d = Kg.to(DEV), Vg.to(DEV)
+    status = binding.new_status(DEV)
+    O, LSE = binding.pulsar_phase2_generate_step(Qn.to(DEV), Kn.to(DEV), Vn.to(DEV), K.to(DEV), V.to(DEV), 1, L, Kg_d, Vg_d,
+                                                 gen_len, n_splits=n_splits, status=status)
+    Kg_o, Vg_o = (x.view(torch.int16).numpy().view(np.uint16).copy() for x in (Kg, Vg))
+    Oref, Lref = oracle.generate_step(Qn, Kn, Vn, K, V, Kg_o, Vg_o, gen_len)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    check_attention(O, LSE, Oref, Lref, f"L={L} gen_len={gen_len} parts={n_splits} n_new={n_new}")
+    for got, want in ((Kg_d, Kg_o), (Vg_d, Vg_o)):             # the rows beyond the new ones stay as they were
+        np.testing.assert_array_equal(got.cpu().view(torch.int16).numpy().view(np.uint16), want)
