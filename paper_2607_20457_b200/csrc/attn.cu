@@ -17,6 +17,8 @@
 //            one more part, causal by token.
 //   Assembled inputs (Algorithm 1 l.8 as the paper runs it): sequences of any lengths packed back
 //            to back, every token a query, plain causal attention inside each.
+#include <type_traits>
+
 #include <cuda.h>
 
 #include "common.cuh"
@@ -38,8 +40,14 @@ enum : int { kModePhase1 = 0, kModePhase2 = 1, kModeVarlen = 2 };
 constexpr int kMaxVarlenSeqs = 64;
 struct VarlenTable {
     int start[kMaxVarlenSeqs + 1];      // first row of sequence j; start[n] = total rows
-    int pair_cum[kMaxVarlenSeqs + 1];   // tile pairs of the sequences n-1, n-2, ... j summed (scheduling order)
+    int pair_cum[kMaxVarlenSeqs + 1];   // work items per head of the sequences n-1, n-2, ... j summed (scheduling order)
     int n_seq;
+};
+
+// Stands in for the table in the decode-shaped instance, which has no sequences (a kilobyte of parameters costs a
+// launch about 1.2 us on the host).
+struct NoTable {
+    int start[1], pair_cum[1], n_seq;
 };
 
 struct AttnArgs {
@@ -47,7 +55,6 @@ struct AttnArgs {
     int n_tokens;          // L (phase 1) or nq (phase 2): tokens that exist, for the store guard
     int Hq, g, pack;       // query heads, heads per KV head, rows per token in a tile (1 or g)
     int block_size;        // phase 1: tokens per block
-    int tiles_per_block;   // phase 1: ceil(block_size / 128)
     int prefix_total;      // phase 1: rows in the gathered prefix buffers
     const int32_t* prefix_len;
     int split_len;         // phase 2: keys per KV part (the last part may be shorter)
@@ -61,13 +68,14 @@ struct AttnArgs {
     uint4* Vgen;
     int quad;              // phase 2, at most 32 query rows per KV head: the rows are replicated into the four
                            // lane quarters of the tile and each softmax warp takes one quarter of the keys
-    int single;            // phase 2, one query tile per KV head (at most 128 rows): the tile's logits alternate
-                           // between the two S buffers so that S of the next key tile is formed during the softmax
-                           // of this one (set with quad as well)
+    int single;            // work items of one query tile: the tile's logits alternate between the two S buffers so
+                           // that S of the next key tile is formed during the softmax of this one.  Phase 2 with
+                           // one query tile per KV head (set with quad as well), causal attention with few items
     int Hkv;
-    int pairs;             // phase 1: query-tile pairs per full block; phase 2: query-tile pairs per KV head
+    int pairs;             // phase 1: work items (query-tile pairs, or tiles if single) per full block and head;
+                           // phase 2: per KV head and part
     int last_len;          // phase 1: tokens of the last block (block_size unless the sequence ends inside it)
-    int pairs_last;        // phase 1: query-tile pairs of the last block
+    int pairs_last;        // phase 1: the same for the last block
     int n_items;           // work items in total
     int n_blocks;          // phase 1
     int32_t* counter;      // work counter (zeroed before the launch): items are drawn in index order as CTAs
@@ -320,7 +328,10 @@ __device__ __forceinline__ int item_of_round(int round, int n_items) {
     return idx < n_items ? idx : -1;
 }
 
-__device__ __forceinline__ void decode_item(const AttnArgs& a, const VarlenTable& vt, int idx, Item& it) {
+// (Table: the sequence table, or NoTable where the launch has no sequences.)
+template <typename Table>
+__device__ __forceinline__ void decode_item(const AttnArgs& a, const Table& vt, int idx, Item& it) {
+    const int per_item = a.single ? 1 : 2;                     // causal attention: query tiles per work item
     if (a.mode == kModeVarlen) {
         // Independent sequences of different lengths, plain causal attention inside each.
         // Items run from the last sequence down and, inside a sequence, from its last tile
@@ -333,10 +344,10 @@ __device__ __forceinline__ void decode_item(const AttnArgs& a, const VarlenTable
         while (k + 1 < vt.n_seq && vt.pair_cum[k + 1] <= rank) ++k;
         const int seq = vt.n_seq - 1 - k;
         const int start = vt.start[seq], len = vt.start[seq + 1] - start;
-        const int tiles = (len + kTileM - 1) / kTileM, pairs = (tiles + 1) / 2;
+        const int tiles = (len + kTileM - 1) / kTileM, pairs = (tiles + per_item - 1) / per_item;
         const int pair = pairs - 1 - (rank - vt.pair_cum[k]);
-        const int qt0 = 2 * pair;
-        it.has1 = (qt0 + 1 < tiles) ? 1 : 0;
+        const int qt0 = per_item * pair;
+        it.has1 = (per_item == 2 && qt0 + 1 < tiles) ? 1 : 0;
         it.row0_a = qt0 * kTileM;
         it.row0_b = (qt0 + 1) * kTileM;
         it.token0_a = start + it.row0_a;
@@ -370,8 +381,8 @@ __device__ __forceinline__ void decode_item(const AttnArgs& a, const VarlenTable
             pair = a.pairs - 1 - r2 % a.pairs;
             len = a.block_size;
         }
-        const int qt0 = 2 * pair;
-        it.has1 = (qt0 + 1 < (len + kTileM - 1) / kTileM) ? 1 : 0;
+        const int qt0 = per_item * pair;
+        it.has1 = (per_item == 2 && qt0 + 1 < (len + kTileM - 1) / kTileM) ? 1 : 0;
         it.row0_a = qt0 * kTileM;
         it.row0_b = (qt0 + 1) * kTileM;
         it.token0_a = blk * a.block_size + it.row0_a;
@@ -492,7 +503,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKp,
             const __grid_constant__ CUtensorMap tmVp, const AttnArgs a,
-            const __grid_constant__ VarlenTable vt) {
+            const __grid_constant__ std::conditional_t<kQuad, NoTable, VarlenTable> vt) {
     using SL = SmemLayout<D>;
     static_assert(kSingle || !kQuad, "the decode-shaped instance has one query tile per item");
     extern __shared__ uint8_t smem_raw[];
@@ -1179,12 +1190,8 @@ int32_t launch_attn(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMa
     constexpr int smem = SmemLayout<D>::kDynBytes;
     // The opt-in to more than 48 KB of dynamic shared memory is a per-device function attribute;
     // setting it on every launch keeps multi-device processes correct and costs well under a microsecond.
-    auto kernel = a.quad ? attn_kernel<D, true, true>
-                         : (a.single ? attn_kernel<D, false, true> : attn_kernel<D, false, false>);
-    PULSAR_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int grid = a.n_items < sm_count() ? a.n_items : sm_count();     // one persistent CTA per SM
     if (grid <= 0) return PULSAR_OK;
-    static const VarlenTable kNoTable{};
     a.out_wide = aligned(a.part_O != nullptr ? static_cast<const void*>(a.part_O) : a.O, 32) ? 1 : 0;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
@@ -1196,18 +1203,31 @@ int32_t launch_attn(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMa
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    PULSAR_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, q, k, v, kp, vp, a, table ? *table : kNoTable));
-    PULSAR_CUDA_OK(cudaGetLastError());
+    const auto launch = [&](auto kernel, const auto& tab) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, kernel, q, k, v, kp, vp, a, tab);
+    };
+    static const VarlenTable kNoSequences{};
+    const VarlenTable& tab = table ? *table : kNoSequences;
+    PULSAR_CUDA_OK(a.quad ? launch(attn_kernel<D, true, true>, NoTable{})
+                          : (a.single ? launch(attn_kernel<D, false, true>, tab) : launch(attn_kernel<D, false, false>, tab)));
     count_launch();
     return PULSAR_OK;
 }
 
 struct Phase1Plan {
-    int n_blocks, tiles_per_block, pairs_per_block;
-    int last_len, pairs_last;                 // the last block: its tokens and its tile pairs
+    int n_blocks;
+    int last_len;                             // tokens of the last block
+    int single, items_block, items_last;      // one query tile per work item; items per head of a full and of the last block
     int n_items;
     size_t pref_rows, pref_bytes, total;
 };
+
+// Causal attention with so few pairs of query tiles that they would not fill the SMs once takes work items of one
+// tile: twice the items, and a key tile costs the chain of one tile (about 1.2 us) instead of two interleaved ones
+// (1.8 us).  With more items than that the pair is the better unit (0.9 us per tile and key tile).
+// 4096 tokens in 4 blocks of 4 heads, d = 64 (64 pairs, up to 10 key tiles): 24 -> 17 us.
+bool causal_single(int64_t pair_items) { return pair_items <= sm_count(); }
 
 // whole_only: the entry point takes only sequences made of whole blocks.
 int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block_size, int32_t prefix_total,
@@ -1219,15 +1239,22 @@ int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block
     if (B > 65535 || Hq > 65535) return PULSAR_ERR_SHAPE;
     if (prefix_total > (1 << 30)) return PULSAR_ERR_SHAPE;
     p.n_blocks = static_cast<int>(B);
-    p.tiles_per_block = (block_size + kTileM - 1) / kTileM;
     p.pref_rows = static_cast<size_t>(prefix_total > 0 ? prefix_total : 1);
-    p.pairs_per_block = (p.tiles_per_block + 1) / 2;
     p.last_len = static_cast<int>(L - (B - 1) * block_size);
-    p.pairs_last = ((p.last_len + kTileM - 1) / kTileM + 1) / 2;
     p.pref_bytes = round_up(p.pref_rows * Hkv * d * 2, 256);
     p.total = 2 * p.pref_bytes + 256;                        // gathered prefix K, V and the work counter
-    const int64_t items = ((B - 1) * p.pairs_per_block + p.pairs_last) * Hq;
+    const int tiles_block = static_cast<int>((static_cast<int64_t>(block_size) + kTileM - 1) / kTileM);
+    const int tiles_last = (p.last_len + kTileM - 1) / kTileM;
+    p.items_block = (tiles_block + 1) / 2;
+    p.items_last = (tiles_last + 1) / 2;
+    int64_t items = ((B - 1) * p.items_block + p.items_last) * Hq;
     if (items >= (1ll << 31)) return PULSAR_ERR_SHAPE;
+    p.single = causal_single(items) ? 1 : 0;
+    if (p.single) {
+        p.items_block = tiles_block;
+        p.items_last = tiles_last;
+        items = ((B - 1) * p.items_block + p.items_last) * Hq;
+    }
     p.n_items = static_cast<int>(items);
     return PULSAR_OK;
 }
@@ -1335,9 +1362,10 @@ extern "C" int32_t pulsar_phase1_attn(const uint16_t* Q, const uint16_t* K, cons
     AttnArgs a{};
     a.mode = kModePhase1;
     a.Hkv = Hkv;
-    a.pairs = p.pairs_per_block;
+    a.single = p.single;
+    a.pairs = p.items_block;
     a.last_len = p.last_len;
-    a.pairs_last = p.pairs_last;
+    a.pairs_last = p.items_last;
     a.n_items = p.n_items;
     a.n_blocks = p.n_blocks;
     a.counter = counter;
@@ -1346,7 +1374,6 @@ extern "C" int32_t pulsar_phase1_attn(const uint16_t* Q, const uint16_t* K, cons
     a.g = Hq / Hkv;
     a.pack = 1;
     a.block_size = block_size;
-    a.tiles_per_block = p.tiles_per_block;
     a.prefix_total = prefix_total;
     a.prefix_len = prefix_len;
     a.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
@@ -1452,9 +1479,10 @@ extern "C" int32_t pulsar_phase1_attn_sharded(const uint16_t* Q, const uint16_t*
     AttnArgs a{};
     a.mode = kModePhase1;
     a.Hkv = Hkv;
-    a.pairs = p.pairs_per_block;
+    a.single = p.single;
+    a.pairs = p.items_block;
     a.last_len = p.last_len;
-    a.pairs_last = p.pairs_last;
+    a.pairs_last = p.items_last;
     a.n_items = p.n_items;
     a.n_blocks = p.n_blocks;
     a.counter = counter;
@@ -1463,7 +1491,6 @@ extern "C" int32_t pulsar_phase1_attn_sharded(const uint16_t* Q, const uint16_t*
     a.g = Hq / Hkv;
     a.pack = 1;
     a.block_size = block_size;
-    a.tiles_per_block = p.tiles_per_block;
     a.prefix_total = prefix_total;
     a.prefix_len = prefix_len_local;
     a.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
@@ -1720,13 +1747,19 @@ extern "C" int32_t pulsar_causal_varlen_attn(const uint16_t* Q, const uint16_t* 
     vt.n_seq = n_seq;
     for (int j = 0; j <= n_seq; ++j) vt.start[j] = cu_seqlens_host[j];
     int64_t pairs_total = 0;
-    for (int k = 0; k < n_seq; ++k) {
-        vt.pair_cum[k] = static_cast<int>(pairs_total);
-        const int len = vt.start[n_seq - k] - vt.start[n_seq - 1 - k];
-        pairs_total += ((len + kTileM - 1) / kTileM + 1) / 2;
+    int single = 0;
+    for (int per_item = 2; per_item >= 1; --per_item) {
+        pairs_total = 0;
+        for (int k = 0; k < n_seq; ++k) {
+            vt.pair_cum[k] = static_cast<int>(pairs_total);
+            const int len = vt.start[n_seq - k] - vt.start[n_seq - 1 - k];
+            pairs_total += ((len + kTileM - 1) / kTileM + per_item - 1) / per_item;
+        }
+        vt.pair_cum[n_seq] = static_cast<int>(pairs_total);
+        if (pairs_total * Hq >= (1ll << 31)) return PULSAR_ERR_SHAPE;
+        if (per_item == 2 && !causal_single(pairs_total * Hq)) break;
+        single = per_item == 1 ? 1 : 0;
     }
-    vt.pair_cum[n_seq] = static_cast<int>(pairs_total);
-    if (pairs_total * Hq >= (1ll << 31)) return PULSAR_ERR_SHAPE;
 
     CUtensorMap tmQ, tmK, tmV;
     if (!make_map_3d(&tmQ, Q, total_rows, Hq, d, 1, kTileM) ||
@@ -1744,6 +1777,7 @@ extern "C" int32_t pulsar_causal_varlen_attn(const uint16_t* Q, const uint16_t* 
     a.g = Hq / Hkv;
     a.pack = 1;
     a.Hkv = Hkv;
+    a.single = single;
     a.n_items = static_cast<int>(pairs_total) * Hq;
     a.counter = counter;
     a.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;

@@ -107,3 +107,21 @@ def test_kv_discard_keeps_each_blocks_own_rows():
     assert torch.equal(Kr.cpu(), K) and torch.equal(Vr.cpu(), V)
     with pytest.raises(binding.PulsarError):
         binding.pulsar_retain_block_kv(Ka, Va, cu, w.block_size + cu[1] + 1)       # longer than the first input
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n_seq,length", [(1, 1), (2, 129), (36, 300), (37, 300), (3, 1500)])
+def test_few_and_many_work_items(n_seq, length, d):
+    """Up to one pair of query tiles per SM the work items are single tiles (36 sequences of two pairs and two heads: 144
+    pairs), beyond that pairs (37: 148 on 148 SMs, and with lengths that differ more)."""
+    gen = torch.Generator().manual_seed(n_seq * length)
+    lens = [length + 7 * (j % 3) for j in range(n_seq)]
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    Q = (2 * torch.randn(int(cu[-1]), 2, d, generator=gen)).to(torch.bfloat16)
+    K, V = (torch.randn(int(cu[-1]), 1, d, generator=gen).to(torch.bfloat16) for _ in range(2))
+    status = binding.new_status(DEV)
+    O, LSE = binding.pulsar_causal_varlen_attn(Q.to(DEV), K.to(DEV), V.to(DEV), cu.tolist(), status=status)
+    Oref, Lref = oracle.causal_varlen_attn(Q, K, V, cu)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    check_attention(O, LSE, Oref, Lref, f"{n_seq} x {length} d={d}")
