@@ -237,7 +237,7 @@ pack_summary_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, co
 // P_s (bf16 pairs) overwrites the first 64 columns of S_s.  The running maximum is only moved
 // when it grows by more than 2^8 (the stale maximum is used consistently for P, O and the row
 // sum, so the result is unchanged); the rare rescale of O is done by the softmax warpgroup.
-// P goes to the issuer in two halves of 64 keys (two barriers), so the first half of PV runs while
+// P goes to the issuer in two pieces (96 and 32 keys, two barriers), so the first piece of PV runs while
 // the second half of the row is exponentiated.  The loader publishes the CTA's work items through
 // a small shared-memory queue; all device waits are bounded (see mbar_wait).
 // ---------------------------------------------------------------------------------------------
@@ -248,6 +248,9 @@ pack_summary_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, co
 constexpr int kStages = 5;
 constexpr int kItemQueue = 4;     // work items the loader may publish ahead of the slowest consumer
 constexpr int kAttnThreads = 384;             // warps 10 and 11 only take part in the register hand-back
+// Keys of the first of the two pieces in which P is handed over: PV of the first piece runs while the second is exponentiated,
+// and the shorter the second, the sooner the next S follows it (64 keys: 16K +0.1..2 %, 32 or 128: 1.5..3 % slower).
+constexpr int kFirstKeys = 96;
 constexpr int kMmaWarp = 8;
 constexpr int kLoadWarp = 9;
 constexpr float kRescaleThreshold = 8.0f;      // in log2 units
@@ -260,22 +263,14 @@ constexpr float kRescaleThreshold = 8.0f;      // in log2 units
 #ifndef PULSAR_POLY_PAIRS
 #define PULSAR_POLY_PAIRS 0
 #endif
-#ifndef PULSAR_EARLY_RELEASE
-#define PULSAR_EARLY_RELEASE 1
-#endif
-// Hand a query tile's shared memory back to the loader when its last S product has been issued (the PV
-// products that follow do not read Q), and the O accumulator back to the issuer as soon as the epilogue has
-// read it into registers (before the rows are scaled and stored): both shorten the gap between work items.
-constexpr bool kEarlyRelease = PULSAR_EARLY_RELEASE;
 // Two more variants were built, measured at the 128K step and taken out again: the two softmax warps of a
 // scheduler taking turns at a key tile's exponentials instead of interleaving them on the MUFU pipe (Phase 1
 // 17.09 ms against 15.75 ms: one warp alone does not fill the pipe, two interleaved warps hide each other's
 // latencies), and reading S from TMEM in two halves with the first half's maximum formed while the second
 // arrives (0.6-1 % slower at the power limit).
 constexpr int kPolyPairs128 = PULSAR_POLY_PAIRS;  // of every four column pairs, how many use the polynomial exp2 (d = 128)
-// Head dimension 64 halves the tensor work per exponential, the GPU stays below its power limit there,
-// and one polynomial pair in four is 3.6 % faster (32K shape with d = 64: 1.228 against 1.272 ms; two pairs
-// in four: 1.309 ms).
+// Head dimension 64 halves the tensor work per exponential and the GPU stays below its power limit there: one pair in
+// four of the second piece of P (the one the next S waits for) takes the polynomial.
 #ifndef PULSAR_POLY_PAIRS_D64
 #define PULSAR_POLY_PAIRS_D64 1
 #endif
@@ -303,7 +298,7 @@ struct SmemLayout {
     static constexpr int kAbort = kTmemPtr + 4;
     static constexpr int kItemQ = kAbort + 4;                      // int [kItemQueue]: published work items
     static constexpr int kTotal = kItemQ + 4 * kItemQueue;
-    static constexpr int kDynBytes = kTotal + 1024;                // room to align the base to 1024 bytes
+    static constexpr int kDynBytes = kTotal;
 };
 
 // What one work item covers; every role decodes it the same way.
@@ -506,15 +501,18 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             const __grid_constant__ std::conditional_t<kQuad, NoTable, VarlenTable> vt) {
     using SL = SmemLayout<D>;
     static_assert(kSingle || !kQuad, "the decode-shaped instance has one query tile per item");
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // The swizzled tiles want 1024-byte alignment.  Declared, not computed: tile addresses and descriptors are constants
+    // then, which takes them out of the registers of the issuer.
+    extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sQ = smem + SL::kQ;
     uint8_t* sKV = smem + SL::kKV;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SL::kBars);
     uint32_t* tmem_ptr = reinterpret_cast<uint32_t*>(smem + SL::kTmemPtr);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::kAbort);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    // Broadcast, so that the compiler knows the branches into the roles to be warp-uniform.
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
 
     if (tid == 0) {
         *abort_flag = 0;
@@ -702,14 +700,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         }                                                                                                 \
         if (leader) umma_commit_a(bar0 + 8 * (SL::bSFull + (s_)));                                        \
     } while (0)
-// P arrives in two halves of 64 keys, each with its own barrier.
+// P arrives in two pieces (kFirstKeys keys, then the rest), each with its own barrier.
 #define PULSAR_ISSUE_PV(tO, tP, dv, acc, s_, par)                                                         \
     do {                                                                                                  \
         _Pragma("unroll") for (int half = 0; half < 2; ++half) {                                          \
             ok = ok && mbar_wait_a(bar0 + 8 * ((half ? SL::bPFull2 : SL::bPFull) + (s_)), par, abort_flag, \
                                    a.status);                                                             \
             tc_fence_after();                                                                             \
-            _Pragma("unroll") for (int kk = half * 4; kk < half * 4 + 4; ++kk)                            \
+            _Pragma("unroll") for (int kk = half ? kFirstKeys / 16 : 0; kk < (half ? kTileN : kFirstKeys) / 16; ++kk) \
                 if (leader && ok)                                                                         \
                     umma_ts(tO, (tP) + kk * 8, (dv) + static_cast<uint64_t>(kk * 128), kIdescPV,          \
                             ((acc) || kk > 0) ? 1u : 0u);                                                 \
@@ -790,21 +788,29 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 if (!ok) break;
                 tc_fence_after();
                 PULSAR_ISSUE_S(tS0, descQ0, descK + static_cast<uint64_t>(ks * kStageStep), 0);
-                if (kEarlyRelease && n0 == 1 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 0));
+                if (n0 == 1 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 0));
                 if (it.has1) {
                     ok = mbar_wait_a(bar0 + 8 * (SL::bQFull + 1), q_use1 & 1, abort_flag, a.status);
                     ++q_use1;
                     if (!ok) break;
                     tc_fence_after();
                     PULSAR_ISSUE_S(tS1, descQ1, descK + static_cast<uint64_t>(ks * kStageStep), 1);
-                    if (kEarlyRelease && n1 == 1 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 1));
+                    if (n1 == 1 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 1));
                 }
                 if (leader) umma_commit_a(bar0 + 8 * (SL::bKvEmpty + ks));
-                for (int t = 0; t < it.n_load; ++t) {
+                // Key tile t: PV_0(t), S_0(t+1), PV_1(t), S_1(t+1).  The issuer's own time is part of the chain that sets
+                // the pace (a barrier test takes 100-300 cycles while the softmax warps of its scheduler keep the
+                // queue that special functions and shared memory share full), so everything that can be waited for
+                // early is waited for before PV_0, and the key tiles in the middle of an item, for which none of the
+                // conditions below can fail, run without them (kMid).  With the constants and the uniform role branch
+                // above, and no register spilled any more: Phase 1 at 64K 5.94 -> 5.53 ms (4.82 before the power
+                // limit bites), at 16K 0.685 -> 0.638 ms, 45K ragged with d = 64 1.04 -> 0.96 ms.
+                const auto key_tile = [&](auto mid, int t) {
+                    constexpr bool kMid = decltype(mid)::value;
                     __syncwarp();
                     const uint32_t vs = stage, vp = phase;                 // V_t
                     PULSAR_RING_NEXT(stage, phase);
-                    const bool more = t + 1 < it.n_load;
+                    const bool more = kMid || t + 1 < it.n_load;
                     if (more) {                                            // K_{t+1}
                         ks = stage;
                         kp = phase;
@@ -813,52 +819,49 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     const uint64_t dv = descV + static_cast<uint64_t>(vs * kStageStep);
                     const uint64_t dk = descK + static_cast<uint64_t>(ks * kStageStep);
                     ok = mbar_wait_a(bar0 + 8 * (SL::bKvFull + vs), vp, abort_flag, a.status);
-                    if (!ok) break;
-                    if (t < n0) {
-                        if (t == 0) {
+                    if (!ok) return;
+                    if (more) {
+                        ok = mbar_wait_a(bar0 + 8 * (SL::bKvFull + ks), kp, abort_flag, a.status);
+                        if (!ok) return;
+                    }
+                    if (kMid || t < n0) {
+                        if (!kMid && t == 0) {
                             ok = mbar_wait_a(bar0 + 8 * (SL::bOEmpty + 0), (o_use0 & 1) ^ 1, abort_flag, a.status);
                             ++o_use0;
                         }
-                        PULSAR_ISSUE_PV(tO0, tS0, dv, t > 0, 0, p_cnt0 & 1);
+                        PULSAR_ISSUE_PV(tO0, tS0, dv, kMid || t > 0, 0, p_cnt0 & 1);
                         ++p_cnt0;
-                        if (!ok) break;
-                        if (t == n0 - 1) {
-                            if (leader) umma_commit_a(bar0 + 8 * (SL::bOFull + 0));
-                            if (!kEarlyRelease && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 0));
-                        }
+                        if (!ok) return;
+                        if (!kMid && t == n0 - 1 && leader) umma_commit_a(bar0 + 8 * (SL::bOFull + 0));
                     }
-                    if (more) {
-                        ok = mbar_wait_a(bar0 + 8 * (SL::bKvFull + ks), kp, abort_flag, a.status);
-                        if (!ok) break;
-                        tc_fence_after();
-                        if (t + 1 < n0) {
-                            PULSAR_ISSUE_S(tS0, descQ0, dk, 0);
-                            // the tile's last S: nothing reads its Q any more
-                            if (kEarlyRelease && t + 2 == n0 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 0));
-                        }
+                    if (kMid || t + 1 < n0) {
+                        PULSAR_ISSUE_S(tS0, descQ0, dk, 0);
+                        // the tile's last S: nothing reads its Q any more
+                        if (!kMid && t + 2 == n0 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 0));
                     }
-                    if (t < n1) {
-                        if (t == 0) {
+                    if (kMid || t < n1) {
+                        if (!kMid && t == 0) {
                             ok = mbar_wait_a(bar0 + 8 * (SL::bOEmpty + 1), (o_use1 & 1) ^ 1, abort_flag, a.status);
                             ++o_use1;
                         }
-                        PULSAR_ISSUE_PV(tO1, tS1, dv, t > 0, 1, p_cnt1 & 1);
+                        PULSAR_ISSUE_PV(tO1, tS1, dv, kMid || t > 0, 1, p_cnt1 & 1);
                         ++p_cnt1;
-                        if (!ok) break;
-                        if (t == n1 - 1) {
-                            if (leader) umma_commit_a(bar0 + 8 * (SL::bOFull + 1));
-                            if (!kEarlyRelease && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 1));
-                        }
+                        if (!ok) return;
+                        if (!kMid && t == n1 - 1 && leader) umma_commit_a(bar0 + 8 * (SL::bOFull + 1));
                     }
                     if (leader) umma_commit_a(bar0 + 8 * (SL::bKvEmpty + vs));
                     if (more) {
-                        if (t + 1 < n1) {
+                        if (kMid || t + 1 < n1) {
                             PULSAR_ISSUE_S(tS1, descQ1, dk, 1);
-                            if (kEarlyRelease && t + 2 == n1 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 1));
+                            if (!kMid && t + 2 == n1 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 1));
                         }
                         if (leader) umma_commit_a(bar0 + 8 * (SL::bKvEmpty + ks));
                     }
-                }
+                };
+                int t = 0;
+                key_tile(std::false_type{}, t++);
+                for (const int t_mid = min(n0, n1) - 2; ok && t < t_mid; ++t) key_tile(std::true_type{}, t);
+                for (; ok && t < it.n_load; ++t) key_tile(std::false_type{}, t);
             }
 #undef PULSAR_ISSUE_S
 #undef PULSAR_ISSUE_PV
@@ -1048,17 +1051,17 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     }
                 }
                 const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
-                // P goes to the MMA issuer in two halves of 64 keys, so that the first half
-                // of the PV product runs while the second half of the row is exponentiated.
+                // P goes to the MMA issuer in two pieces, so that the first piece of the PV product runs while the
+                // rest of the row is exponentiated.
                 // (The rescale above has stored its O columns before the first hand-over.)
-                if (masked) l_run += exp_row128<0, 0, 64>(r, a.scale_log2, neg_m, tS);
-                else l_run += exp_row128<kPolyPairsFor<D>, 0, 64>(r, a.scale_log2, neg_m, tS);
+                if (masked) l_run += exp_row128<0, 0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
+                else l_run += exp_row128<kPolyPairs128, 0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_p);
-                if (masked) l_run += exp_row128<0, 64, 128>(r, a.scale_log2, neg_m, tS);
-                else l_run += exp_row128<kPolyPairsFor<D>, 64, 128>(r, a.scale_log2, neg_m, tS);
+                if (masked) l_run += exp_row128<0, kFirstKeys, 128>(r, a.scale_log2, neg_m, tS);
+                else l_run += exp_row128<kPolyPairsFor<D>, kFirstKeys, 128>(r, a.scale_log2, neg_m, tS);
 
                 tmem_wait_st();
                 tc_fence_before();
@@ -1087,11 +1090,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 #pragma unroll
                 for (int c0 = 0; c0 < D; c0 += 32) PULSAR_TMEM_LD32_AT(tO + c0, o, c0);
                 tmem_wait_ld();
-                if (kEarlyRelease) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_oe);
-                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_oe);
                 if (store) {
                     // A row per lane: every store instruction touches 32 rows.  With 16-byte stores each sector went
                     // out in two halves and an item's rows took about 5000 cycles; whole 32-byte sectors per store:
@@ -1119,11 +1120,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                         if (a.LSE != nullptr) a.LSE[orow] = lse;
                     }
                 }
-            }
-            if (!kEarlyRelease) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_oe);
             }
         }
     }
