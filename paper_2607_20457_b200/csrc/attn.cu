@@ -254,33 +254,35 @@ constexpr int kFirstKeys = 96;
 constexpr int kMmaWarp = 8;
 constexpr int kLoadWarp = 9;
 constexpr float kRescaleThreshold = 8.0f;      // in log2 units
-// Tuning knobs (overridable at build time with -D).  Measured on a 1000 W B200 running the 128K
-// step back to back (power-capped, SM clock ~1.56 GHz): without the polynomial exponential 1060 TFLOP/s,
-// with one pair in four 1032 -- under the power cap the variant that executes the fewest instructions
-// wins, although the option shortens the per-tile latency in short runs.  (Forming the first half of P
-// with the maximum in use while the tile maximum is computed alongside was a second such option: 1048,
-// and 1020 with both; taken out of the source.)
-#ifndef PULSAR_POLY_PAIRS
-#define PULSAR_POLY_PAIRS 0
-#endif
-// Two more variants were built, measured at the 128K step and taken out again: the two softmax warps of a
-// scheduler taking turns at a key tile's exponentials instead of interleaving them on the MUFU pipe (Phase 1
-// 17.09 ms against 15.75 ms: one warp alone does not fill the pipe, two interleaved warps hide each other's
-// latencies), and reading S from TMEM in two halves with the first half's maximum formed while the second
-// arrives (0.6-1 % slower at the power limit).
-constexpr int kPolyPairs128 = PULSAR_POLY_PAIRS;  // of every four column pairs, how many use the polynomial exp2 (d = 128)
-// Head dimension 64 halves the tensor work per exponential and the GPU stays below its power limit there: one pair in
-// four of the second piece of P (the one the next S waits for) takes the polynomial.
-#ifndef PULSAR_POLY_PAIRS_D64
-#define PULSAR_POLY_PAIRS_D64 1
-#endif
-template <int D> constexpr int kPolyPairsFor = D == 64 ? PULSAR_POLY_PAIRS_D64 : kPolyPairs128;
+constexpr float kPieceSumBound = 256.f * kFirstKeys;   // of a piece formed with an old maximum, all at the threshold
+// Measured and not kept: a polynomial exponential on the FMA pipe for part of the columns (2.5-4 % slower with d = 128, no
+// difference with d = 64), the two softmax warps of a scheduler taking turns at a key tile's exponentials (8.5 %
+// slower: one warp alone does not fill the MUFU pipe), reading S from TMEM in two halves (2 % slower).
 // Registers per thread: the kernel is compiled for 168 (twelve warps).  setmaxnreg moves
 // registers inside the CTA's own pool of 12 * 168 per lane slot and acts on whole warpgroups:
 // warpgroup 2 (MMA issuer, TMA loader and two spare warps) hands back all but kRegsIssuer,
 // the eight softmax warps grow to kRegsSoftmax:  4 * 88 + 8 * 208 = 2016 = 12 * 168.
 constexpr int kRegsIssuer = 88;
 constexpr int kRegsSoftmax = 208;
+
+// What one work item covers.  The loader decodes it and hands it to the issuer and the softmax warps through a queue in
+// shared memory; they read what they need rarely where they need it, which leaves the registers to the logits.
+struct __align__(16) Item {
+    int valid;                   // 0: no further work items
+
+    int token0_a, token0_b;      // first token of each query tile
+    int head0, kvh, part;
+    int has1;                    // second query tile exists
+    int n_tiles_a, n_tiles_b;    // key tiles each query tile walks
+    int n_load;                  // key tiles to stage = max of the two
+    int n_pref_tiles, pref_len;
+    int main_row0, main_len;
+    int row0_a, row0_b;          // first row of each query tile within its block (phase 1)
+    int bad_length;              // phase 1: prefix_len of the block was outside [0, prefix_total] (clamped)
+    int gen_base;                // >= 0: generation shard, token u sees its rows [0, gen_base + u]; -1 otherwise
+    int pad_;
+};
+static_assert(sizeof(Item) == 80, "whole 16-byte words");
 
 template <int D>
 struct SmemLayout {
@@ -296,23 +298,9 @@ struct SmemLayout {
     static constexpr int kNumBars = bItemEmpty + kItemQueue;
     static constexpr int kTmemPtr = kBars + kNumBars * 8;
     static constexpr int kAbort = kTmemPtr + 4;
-    static constexpr int kItemQ = kAbort + 4;                      // int [kItemQueue]: published work items
-    static constexpr int kTotal = kItemQ + 4 * kItemQueue;
+    static constexpr int kItemQ = (kAbort + 4 + 15) / 16 * 16;     // Item [kItemQueue]: published work items
+    static constexpr int kTotal = kItemQ + static_cast<int>(sizeof(Item)) * kItemQueue;
     static constexpr int kDynBytes = kTotal;
-};
-
-// What one work item covers; every role decodes it the same way.
-struct Item {
-    int token0_a, token0_b;      // first token of each query tile
-    int head0, kvh, part;
-    int has1;                    // second query tile exists
-    int n_tiles_a, n_tiles_b;    // key tiles each query tile walks
-    int n_load;                  // key tiles to stage = max of the two
-    int n_pref_tiles, pref_len;
-    int main_row0, main_len;
-    int row0_a, row0_b;          // first row of each query tile within its block (phase 1)
-    int bad_length;              // phase 1: prefix_len of the block was outside [0, prefix_total] (clamped)
-    int gen_base;                // >= 0: generation shard, token u sees its rows [0, gen_base + u]; -1 otherwise
 };
 
 // Work item of this CTA in a given round.  Items are sorted costliest first; rounds alternate
@@ -326,6 +314,7 @@ __device__ __forceinline__ int item_of_round(int round, int n_items) {
 // (Table: the sequence table, or NoTable where the launch has no sequences.)
 template <typename Table>
 __device__ __forceinline__ void decode_item(const AttnArgs& a, const Table& vt, int idx, Item& it) {
+    it.valid = 1;
     const int per_item = a.single ? 1 : 2;                     // causal attention: query tiles per work item
     if (a.mode == kModeVarlen) {
         // Independent sequences of different lengths, plain causal attention inside each.
@@ -450,10 +439,8 @@ __device__ __forceinline__ float row_max128(const uint32_t (&r)[kTileN]) {
 }
 
 // p_c = 2^(s_c * scale + neg_m) for logits [kBegin, kEnd) of a row, rounded to bf16 pairs and written
-// to TMEM as the A operand of the PV product; returns the fp32 row sum.  kPoly of every four
-// column pairs take the polynomial exp2 (FMA pipe) instead of MUFU.  kPoly must be 0 when
-// logits may be -inf (masked tiles).
-template <int kPoly, int kBegin = 0, int kEnd = kTileN>
+// to TMEM as the A operand of the PV product; returns the fp32 row sum.
+template <int kBegin, int kEnd>
 __device__ __forceinline__ float exp_row128(const uint32_t (&r)[kTileN], float scale, float neg_m, uint32_t tP) {
     float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
     const float2 sc = make_float2(scale, scale), nm = make_float2(neg_m, neg_m);
@@ -465,12 +452,8 @@ __device__ __forceinline__ float exp_row128(const uint32_t (&r)[kTileN], float s
             const float2 x =
                 __ffma2_rn(make_float2(__uint_as_float(r[c0 + c]), __uint_as_float(r[c0 + c + 1])), sc, nm);
             float2 pv;
-            if (((c >> 1) & 3) >= 4 - kPoly) {
-                pv = ex2_poly2(x);
-            } else {
-                pv.x = ex2(x.x);
-                pv.y = ex2(x.y);
-            }
+            pv.x = ex2(x.x);
+            pv.y = ex2(x.y);
             if ((c >> 1) & 1) acc1 = __fadd2_rn(acc1, pv);
             else acc0 = __fadd2_rn(acc0, pv);
             pk[c >> 1] = pack_bf16x2(pv.x, pv.y);
@@ -561,6 +544,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     // Ring bookkeeping shared by the two issuer roles: `stage` walks 0..kStages-1, `phase`
     // flips at every wrap.  Barrier i lives at bar0 + 8 * i.
     const uint32_t bar0 = smem_u32(bars);
+    Item* item_q = reinterpret_cast<Item*>(smem + SL::kItemQ);
 #define PULSAR_RING_NEXT(stage, phase) \
     do { if (++(stage) == kStages) { (stage) = 0; (phase) ^= 1u; } } while (0)
 
@@ -575,7 +559,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             uint32_t stage = 0, phase = 0;           // next ring slot to fill
             uint32_t q_use0 = 0, q_use1 = 0;
             bool ok = true;
-            volatile int* item_q = reinterpret_cast<volatile int*>(smem + SL::kItemQ);
             for (uint32_t seq = 0; ok; ++seq) {
                 // Reconverge once per iteration: every barrier is waited on at most once per
                 // iteration, so a lane that is still polling can never be more than one phase behind
@@ -598,13 +581,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     idx = static_cast<int>(seq) * static_cast<int>(gridDim.x) < a.n_items
                               ? item_of_round(static_cast<int>(seq), a.n_items) : -1;
                 }
+                Item it;
+                it.valid = 0;
+                if (idx >= 0) decode_item(a, vt, idx, it);
                 if (lane == 0) {
-                    item_q[slot] = idx;
+                    item_q[slot] = it;
                     mbar_arrive(bars + SL::bItemFull + slot);
                 }
                 if (idx < 0) break;
-                Item it;
-                decode_item(a, vt, idx, it);
                 if (it.bad_length && lane == 0) report(a.status, PULSAR_DEV_BAD_LENGTH);
                 if (kSingle && it.gen_base >= 0 && a.Knew != nullptr) append_head(a, it.kvh, D, lane);
                 const int x = it.kvh * D;
@@ -714,18 +698,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         }                                                                                                 \
     } while (0)
 
-            volatile int* item_q = reinterpret_cast<volatile int*>(smem + SL::kItemQ);
             for (uint32_t seq = 0; ok; ++seq) {
                 __syncwarp();              // see the loader: lanes stay within one barrier phase of each other
                 const uint32_t slot = seq % kItemQueue;
                 ok = mbar_wait_a(bar0 + 8 * (SL::bItemFull + slot), (seq / kItemQueue) & 1, abort_flag, a.status);
                 if (!ok) break;
-                const int idx = item_q[slot];
+                const int valid = item_q[slot].valid, n0 = item_q[slot].n_tiles_a, n1 = item_q[slot].n_tiles_b;
+                __syncwarp();
                 if (leader) mbar_arrive(bars + SL::bItemEmpty + slot);
-                if (idx < 0) break;
-                Item it;
-                decode_item(a, vt, idx, it);
-                const int n0 = it.n_tiles_a, n1 = it.n_tiles_b;
+                if (!valid) break;
+                const int n_load = max(n0, n1);
                 if (kSingle) {
                     // Ring slots: K_t at position 2t of the item, V_t at 2t + 1 (the loader's order); the
                     // issuer consumes K_t+1 before V_t.
@@ -789,7 +771,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 tc_fence_after();
                 PULSAR_ISSUE_S(tS0, descQ0, descK + static_cast<uint64_t>(ks * kStageStep), 0);
                 if (n0 == 1 && leader) umma_commit_a(bar0 + 8 * (SL::bQEmpty + 0));
-                if (it.has1) {
+                if (n1 > 0) {
                     ok = mbar_wait_a(bar0 + 8 * (SL::bQFull + 1), q_use1 & 1, abort_flag, a.status);
                     ++q_use1;
                     if (!ok) break;
@@ -810,7 +792,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     __syncwarp();
                     const uint32_t vs = stage, vp = phase;                 // V_t
                     PULSAR_RING_NEXT(stage, phase);
-                    const bool more = kMid || t + 1 < it.n_load;
+                    const bool more = kMid || t + 1 < n_load;
                     if (more) {                                            // K_{t+1}
                         ks = stage;
                         kp = phase;
@@ -861,7 +843,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 int t = 0;
                 key_tile(std::false_type{}, t++);
                 for (const int t_mid = min(n0, n1) - 2; ok && t < t_mid; ++t) key_tile(std::true_type{}, t);
-                for (; ok && t < it.n_load; ++t) key_tile(std::false_type{}, t);
+                for (; ok && t < n_load; ++t) key_tile(std::false_type{}, t);
             }
 #undef PULSAR_ISSUE_S
 #undef PULSAR_ISSUE_PV
@@ -882,41 +864,35 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         uint32_t s_cnt = 0, o_cnt = 0;
         bool ok = true;
 
-        volatile int* item_q = reinterpret_cast<volatile int*>(smem + SL::kItemQ);
         for (uint32_t seq = 0; ok; ++seq) {
             const uint32_t slot = seq % kItemQueue;
             ok = __all_sync(0xffffffffu, mbar_wait(bars + SL::bItemFull + slot, (seq / kItemQueue) & 1, abort_flag, a.status));
             if (!ok) break;
-            const int idx = item_q[slot];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bars + SL::bItemEmpty + slot);
-            if (idx < 0) break;
-            Item it;
-            decode_item(a, vt, idx, it);
+            const volatile Item& it = item_q[slot];            // handed back at the end of the item
+            if (!it.valid) break;
             const int n = s ? it.n_tiles_b : it.n_tiles_a;
-            if (n == 0) continue;
+            const int pref_len = it.pref_len;
             float m_used = -INFINITY, l_run = 0.f;
-            const int my_row_in_block = (s ? it.row0_b : it.row0_a) + row;
             const int row_t = kQuad ? lane : row;             // row as far as token and head are concerned
 
             for (int t = 0; t < n; ++t) {
                 // visible key columns of this tile for this row: [0, n_vis)
                 int n_vis = kTileN;
                 bool masked = false;
-                if (t < it.n_pref_tiles) {
-                    const int valid = it.pref_len - t * kTileN;
-                    if (valid < kTileN) { n_vis = valid; masked = true; }
+                const int pref_left = pref_len - t * kTileN;
+                if (pref_left > 0) {
+                    if (pref_left < kTileN) { n_vis = pref_left; masked = true; }
                     if (it.gen_base >= 0) {                   // generation shard: causal by token
                         const int token = (s ? it.token0_b : it.token0_a) + row_t / a.pack;
                         n_vis = min(n_vis, it.gen_base + token + 1 - t * kTileN);
                         masked = true;
                     }
                 } else {
-                    const int j = t - it.n_pref_tiles;
+                    const int j = t - (pref_len + kTileN - 1) / kTileN;
                     const int valid = it.main_len - j * kTileN;
                     if (valid < kTileN) { n_vis = valid; masked = true; }
                     if (a.mode != kModePhase2 && t == n - 1) {
-                        n_vis = min(n_vis, my_row_in_block - j * kTileN + 1);
+                        n_vis = min(n_vis, (s ? it.row0_b : it.row0_a) + row - j * kTileN + 1);
                         masked = true;
                     }
                 }
@@ -1022,46 +998,61 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     for (int c = 0; c < kTileN; ++c)
                         if (c >= n_vis) r[c] = 0xff800000u;          // -inf
                 }
-                const float m_tile = row_max128(r) * a.scale_log2;
-                const bool need = m_tile > m_used + kRescaleThreshold;   // always true on the first tile
-                if (__any_sync(0xffffffffu, need)) {
-                    if (kSingle && t > 0) {
-                        // O may be rescaled once the PV product of the previous key tile is complete.
-                        // This is key tile g_tile - 1 of the CTA; completions 0 .. g_tile - 3 are certain
-                        // (this tile's S was issued after them), so the barrier is in phase g_tile - 2
-                        // or g_tile - 1 and the parity of g_tile - 2 tells the two apart.
-                        ok = __all_sync(0xffffffffu, mbar_wait(bar_pv, g_tile & 1u, abort_flag, a.status));
-                        if (!ok) break;
-                        tc_fence_after();
-                    }
-                    const float m_new = need ? m_tile : m_used;
-                    const float alpha = (m_new == -INFINITY) ? 1.f : ex2(m_used - m_new);
-                    l_run *= alpha;
-                    m_used = m_new;
-                    if (t > 0) {
+                // After the first key tile the running maximum is nearly always good enough, so the first piece of P is
+                // formed with it at once, and whether it was is seen afterwards: its own sum bounds every one of its
+                // probabilities, the logits of the second piece are compared.  If it was not (or the tile is masked),
+                // the row maximum is taken over the whole tile, O is rescaled and the piece is formed again.  The
+                // maximum and the vote took 520 of the 3250 cycles of a key tile before anything could be
+                // exponentiated: Phase 1 at 64K 5.46 -> 5.37 ms, d = 64 0.944 -> 0.918 ms.
+                float s1 = 0.f, neg_m = -m_used;
+                bool fast = !masked && t > 0;
+                if (fast) {
+                    s1 = exp_row128<0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
+                    float m2 = -INFINITY;
 #pragma unroll
-                        for (int c0 = 0; c0 < D; c0 += 32) {
-                            uint32_t o[32];
-                            tmem_ld32(tO + c0, o);
-                            tmem_wait_ld();
+                    for (int c = kFirstKeys; c < kTileN; c += 2) m2 = max3(m2, __uint_as_float(r[c]), __uint_as_float(r[c + 1]));
+                    fast = !__any_sync(0xffffffffu, !(s1 <= kPieceSumBound) || m2 * a.scale_log2 > m_used + kRescaleThreshold);
+                }
+                if (!fast) {
+                    const float m_tile = row_max128(r) * a.scale_log2;
+                    const bool need = m_tile > m_used + kRescaleThreshold;   // always true on the first tile
+                    if (__any_sync(0xffffffffu, need)) {
+                        if (kSingle && t > 0) {
+                            // O may be rescaled once the PV product of the previous key tile is complete.
+                            // This is key tile g_tile - 1 of the CTA; completions 0 .. g_tile - 3 are certain
+                            // (this tile's S was issued after them), so the barrier is in phase g_tile - 2
+                            // or g_tile - 1 and the parity of g_tile - 2 tells the two apart.
+                            ok = __all_sync(0xffffffffu, mbar_wait(bar_pv, g_tile & 1u, abort_flag, a.status));
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
+                        const float m_new = need ? m_tile : m_used;
+                        const float alpha = (m_new == -INFINITY) ? 1.f : ex2(m_used - m_new);
+                        l_run *= alpha;
+                        m_used = m_new;
+                        if (t > 0) {
 #pragma unroll
-                            for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
-                            tmem_st32(tO + c0, o);
+                            for (int c0 = 0; c0 < D; c0 += 32) {
+                                uint32_t o[32];
+                                tmem_ld32(tO + c0, o);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
+                                tmem_st32(tO + c0, o);
+                            }
                         }
                     }
+                    neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
+                    s1 = exp_row128<0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
                 }
-                const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
+                l_run += s1;
                 // P goes to the MMA issuer in two pieces, so that the first piece of the PV product runs while the
-                // rest of the row is exponentiated.
-                // (The rescale above has stored its O columns before the first hand-over.)
-                if (masked) l_run += exp_row128<0, 0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
-                else l_run += exp_row128<kPolyPairs128, 0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
+                // rest of the row is exponentiated.  (A rescale has stored its O columns before the first hand-over.)
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_p);
-                if (masked) l_run += exp_row128<0, kFirstKeys, 128>(r, a.scale_log2, neg_m, tS);
-                else l_run += exp_row128<kPolyPairsFor<D>, kFirstKeys, 128>(r, a.scale_log2, neg_m, tS);
+                l_run += exp_row128<kFirstKeys, 128>(r, a.scale_log2, neg_m, tS);
 
                 tmem_wait_st();
                 tc_fence_before();
@@ -1071,16 +1062,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             if (!ok) break;
 
             // ---- epilogue: normalise and store this thread's row ----
-            ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_of, o_cnt & 1, abort_flag, a.status));
-            ++o_cnt;
-            if (!ok) break;
-            tc_fence_after();
-            {
+            if (n > 0) {
+                ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_of, o_cnt & 1, abort_flag, a.status));
+                ++o_cnt;
+                if (!ok) break;
+                tc_fence_after();
                 const int token = (s ? it.token0_b : it.token0_a) + row_t / a.pack;
                 const int head = it.head0 + row_t % a.pack;
                 const int part = kQuad ? it.part * 4 + (warp & 3) : it.part;
                 bool store = token < a.n_tokens;
-                if (a.mode != kModePhase2) store = store && my_row_in_block < it.main_len;
+                if (a.mode != kModePhase2) store = store && (s ? it.row0_b : it.row0_a) + row < it.main_len;
                 const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
                 const float lse = (l_run > 0.f) ? (m_used + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
                 const size_t orow = static_cast<size_t>(token) * a.Hq + head;
@@ -1121,6 +1112,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     }
                 }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bars + SL::bItemEmpty + slot);
         }
     }
 

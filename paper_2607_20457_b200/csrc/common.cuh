@@ -374,25 +374,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
-// 2^x for two values on the FMA and integer pipes only (no MUFU): round-to-nearest split
-// x = n + f, |f| <= 0.5, a minimax cubic for 2^f (max relative error 7.5e-5, far below the
-// bf16 rounding of the probabilities), and n added into the exponent field.  Inputs are
-// clamped below at -126; valid for x <= 120.
-__device__ __forceinline__ float2 ex2_poly2(float2 x) {
-    x.x = fmaxf(x.x, -126.f);
-    x.y = fmaxf(x.y, -126.f);
-    const float2 magic = make_float2(12582912.f, 12582912.f);           // 1.5 * 2^23
-    const float2 t = __fadd2_rn(x, magic);                              // integer part in the low mantissa bits
-    const float2 n = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
-    const float2 f = __ffma2_rn(n, make_float2(-1.f, -1.f), x);
-    float2 q = __ffma2_rn(make_float2(0.0551716685f, 0.0551716685f), f, make_float2(0.242611125f, 0.242611125f));
-    q = __ffma2_rn(q, f, make_float2(0.693260968f, 0.693260968f));
-    q = __ffma2_rn(q, f, make_float2(0.999928057f, 0.999928057f));
-    float2 r;
-    r.x = __int_as_float(__float_as_int(q.x) + (__float_as_int(t.x) << 23));
-    r.y = __int_as_float(__float_as_int(q.y) + (__float_as_int(t.y) << 23));
-    return r;
-}
 // 32 bytes in one store where the address allows it (wide), in two otherwise.
 __device__ __forceinline__ void store_32b(void* dst, const uint32_t (&v)[8], bool wide) {
     if (wide) {

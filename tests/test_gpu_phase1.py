@@ -202,3 +202,23 @@ def test_outputs_at_a_16_byte_aligned_base(d):
     pL2 = torch.empty_like(pL)
     binding.pulsar_phase2_attn(Qq, K, V, 1, w.L, n_splits=3, partials=(podd, pL2))
     assert torch.equal(podd, pO) and torch.equal(pL2, pL)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("Hq", [2, 48])                    # work items of one query tile, and of two
+@pytest.mark.parametrize("where", ["first piece", "second piece", "creeping"])
+def test_running_maximum_moves_inside_a_key_tile(where, Hq, d):
+    """P is formed with the maximum of earlier key tiles and formed again when that was too small: one key of a tile far
+    above everything before it (in the first 96 keys or in the last 32), and logits that grow a little in every
+    tile, so that the maximum lags behind by less and then by more than the threshold."""
+    w = W.shrink(W.CONFIGS["tiny"], L=2048, block_size=1024, chunk=16, k=4, sink=64, Hq=Hq, Hkv=2, d=d)
+    Q, K, V = W.qkv(w, seed=41)
+    Kf = K.float()
+    if where == "creeping":
+        Kf *= (1.0 + torch.arange(w.L, dtype=torch.float32) / 128 * 0.8)[:, None, None]
+    else:
+        for j, t in enumerate((1, 3, 4, 9, 11, 13)):
+            Kf[128 * t + (17 if where == "first piece" else 101) + j] *= 6.0 + 9.0 * j
+    rows = W.sample_rows(w, per_block=96)
+    pidx, plen = W.first_k_prefix(w)
+    print(run_phase1(w, Q, Kf.bfloat16(), V, pidx, plen, rows=rows, what=f"{where} Hq={Hq} d={d}"))
