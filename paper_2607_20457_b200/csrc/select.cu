@@ -265,8 +265,12 @@ topk_kernel(const uint16_t* __restrict__ level_all, int n_blocks, int64_t L, int
 constexpr int kMaxScoreBlocks = 1024;
 constexpr int kMaxScoreChunk = 1024;
 constexpr int kMaxScoreChunksPerBlock = 4096;
+// kBlocks: room for df = 0 .. kBlocks.  A kernel parameter costs the host about 1.2 us a kilobyte at every launch (20.6
+// against 18.1 us for the whole BM25 selection over 16 blocks), so there are two sizes.
+constexpr int kFewScoreBlocks = 64;
+template <int kBlocks>
 struct ScoreTable {
-    double by_df[kMaxScoreBlocks + 1];   // Eq. 5 (TF-IDF, Max-IDF) or the BM25 IDF of Eq. 7, per df
+    double by_df[kBlocks + 1];           // Eq. 5 (TF-IDF, Max-IDF) or the BM25 IDF of Eq. 7, per df
     double k1_plus_1, k1, b, one_minus_b, mean_len;   // BM25: D(C) = (1 - b) + b * (|C| / mean chunk length)
 };
 
@@ -280,11 +284,11 @@ struct ScoreTable {
 // this form and the four launches chained as programmatic dependents).
 constexpr int kScoreWarps = 4;
 
-template <int kMode>
+template <int kMode, int kBlocks>
 __global__ void __launch_bounds__(kScoreWarps * 32)
 chunk_score_kernel(const uint32_t* __restrict__ ids, const uint16_t* __restrict__ df_table, int64_t L,
                    int block_size, int chunks_per_block, int n_slots_total, int chunk, int vocab_size,
-                   const __grid_constant__ ScoreTable tab, double* __restrict__ score) {
+                   const __grid_constant__ ScoreTable<kBlocks> tab, double* __restrict__ score) {
     extern __shared__ double smem_d[];                     // per warp: a term and a token per position
     grid_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -534,6 +538,37 @@ int32_t plan_score(int64_t L, int32_t vocab_size, int32_t block_size, int32_t ch
     p.topk_smem = static_cast<size_t>(p.base.C) * 8 + static_cast<size_t>(k) * 4;
     return PULSAR_OK;
 }
+
+template <int kBlocks>
+cudaError_t launch_scores(const SelectPlan& b, int32_t score_mode, const uint32_t* token_ids, const uint16_t* df_table, int64_t L,
+                          int32_t block_size, int32_t chunk, int32_t vocab_size, double* score, cudaStream_t stream) {
+    // The logarithms of Eq. 5 / Eq. 7 for every possible df, in float64 from the host's libm.
+    ScoreTable<kBlocks> tab;
+    const double N = static_cast<double>(b.n_blocks);
+    for (int f = 0; f <= b.n_blocks; ++f) {
+        const double fd = static_cast<double>(f);
+        tab.by_df[f] = score_mode == PULSAR_SCORE_BM25 ? std::log((N - fd + 0.5) / (fd + 0.5) + 1.0)
+                                                       : std::log(N / static_cast<double>(f > 1 ? f : 1));
+    }
+    const double k1 = 1.2, bb = 0.75;
+    // mean chunk length over the sequence: full blocks have C chunks, a short last block what it needs
+    const int64_t last_len = L - static_cast<int64_t>(b.n_blocks - 1) * block_size;
+    const int64_t n_chunks = static_cast<int64_t>(b.n_blocks - 1) * b.C + (last_len + chunk - 1) / chunk;
+    tab.k1_plus_1 = k1 + 1.0;
+    tab.k1 = k1;
+    tab.b = bb;
+    tab.one_minus_b = 1.0 - bb;
+    tab.mean_len = static_cast<double>(L) / static_cast<double>(n_chunks);
+
+    auto kernel = score_mode == PULSAR_SCORE_MAX_IDF ? chunk_score_kernel<PULSAR_SCORE_MAX_IDF, kBlocks>
+                : score_mode == PULSAR_SCORE_TF_IDF  ? chunk_score_kernel<PULSAR_SCORE_TF_IDF, kBlocks>
+                : score_mode == PULSAR_SCORE_BM25    ? chunk_score_kernel<PULSAR_SCORE_BM25, kBlocks>
+                                                     : chunk_score_kernel<PULSAR_SCORE_TYPE_TOKEN, kBlocks>;
+    const int n_chunks_total = b.n_blocks * b.C;
+    const size_t smem = static_cast<size_t>(kScoreWarps) * chunk * (sizeof(double) + sizeof(uint32_t));
+    return launch_kernel(kernel, dim3((n_chunks_total + kScoreWarps - 1) / kScoreWarps), dim3(kScoreWarps * 32), smem, stream,
+                         true, token_ids, df_table, L, block_size, b.C, n_chunks_total, chunk, vocab_size, tab, score);
+}
 }  // namespace
 
 extern "C" size_t pulsar_chunk_select_workspace_bytes(int64_t L, int32_t vocab_size, int32_t block_size,
@@ -566,24 +601,6 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
     double* score = score_out ? score_out
                               : reinterpret_cast<double*>(static_cast<char*>(workspace) + b.bitmap_bytes + b.df_bytes);
 
-    // The logarithms of Eq. 5 / Eq. 7 for every possible df, in float64 from the host's libm.
-    ScoreTable tab;
-    const double N = static_cast<double>(b.n_blocks);
-    for (int f = 0; f <= b.n_blocks; ++f) {
-        const double fd = static_cast<double>(f);
-        tab.by_df[f] = score_mode == PULSAR_SCORE_BM25 ? std::log((N - fd + 0.5) / (fd + 0.5) + 1.0)
-                                                       : std::log(N / static_cast<double>(f > 1 ? f : 1));
-    }
-    const double k1 = 1.2, bb = 0.75;
-    // mean chunk length over the sequence: full blocks have C chunks, a short last block what it needs
-    const int64_t last_len = L - static_cast<int64_t>(b.n_blocks - 1) * block_size;
-    const int64_t n_chunks = static_cast<int64_t>(b.n_blocks - 1) * b.C + (last_len + chunk - 1) / chunk;
-    tab.k1_plus_1 = k1 + 1.0;
-    tab.k1 = k1;
-    tab.b = bb;
-    tab.one_minus_b = 1.0 - bb;
-    tab.mean_len = static_cast<double>(L) / static_cast<double>(n_chunks);
-
     if (b.presence_smem > 48 * 1024)
         PULSAR_CUDA_OK(cudaFuncSetAttribute(presence_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             static_cast<int>(b.presence_smem)));
@@ -594,15 +611,9 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
     PULSAR_CUDA_OK(launch_kernel(df_idf_kernel, dim3((vocab_size + 255) / 256), dim3(256), 0, stream, true, bitmaps,
                                  b.n_blocks, b.words, vocab_size, df_table, nullptr, nullptr));
     count_launch();
-    const int n_chunks_total = b.n_blocks * b.C;
-    auto score_kernel = score_mode == PULSAR_SCORE_MAX_IDF ? chunk_score_kernel<PULSAR_SCORE_MAX_IDF>
-                      : score_mode == PULSAR_SCORE_TF_IDF  ? chunk_score_kernel<PULSAR_SCORE_TF_IDF>
-                      : score_mode == PULSAR_SCORE_BM25    ? chunk_score_kernel<PULSAR_SCORE_BM25>
-                                                           : chunk_score_kernel<PULSAR_SCORE_TYPE_TOKEN>;
-    const size_t score_smem = static_cast<size_t>(kScoreWarps) * chunk * (sizeof(double) + sizeof(uint32_t));
-    PULSAR_CUDA_OK(launch_kernel(score_kernel, dim3((n_chunks_total + kScoreWarps - 1) / kScoreWarps), dim3(kScoreWarps * 32),
-                                 score_smem, stream, true, token_ids, df_table, L, block_size, b.C, n_chunks_total, chunk,
-                                 vocab_size, tab, score));
+    PULSAR_CUDA_OK(b.n_blocks <= kFewScoreBlocks
+                       ? launch_scores<kFewScoreBlocks>(b, score_mode, token_ids, df_table, L, block_size, chunk, vocab_size, score, stream)
+                       : launch_scores<kMaxScoreBlocks>(b, score_mode, token_ids, df_table, L, block_size, chunk, vocab_size, score, stream));
     count_launch();
     PULSAR_CUDA_OK(launch_kernel(topk_score_kernel, dim3(b.n_blocks), dim3(kTopkThreads), p.topk_smem, stream, true, score,
                                  b.n_blocks, L, block_size, chunk, k, sink, sel_chunks, prefix_idx, prefix_len));

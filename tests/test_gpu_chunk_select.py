@@ -101,3 +101,11 @@ def test_chunk_lengths_around_a_warp(chunk, mode):
     block = 2 * chunk + max(1, chunk // 2)
     ids = rng.integers(0, max(3, chunk // 2), size=3 * block + chunk).astype(np.uint32)
     run_and_compare(ids, 2000, block, chunk, 2, min(5, block), mode)
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("n_blocks", [64, 65])
+def test_block_counts_around_the_small_score_table(n_blocks, mode):
+    rng = np.random.default_rng(n_blocks)
+    ids = np.concatenate([rng.integers(0, 40, size=48) * rng.integers(1, 6) for _ in range(n_blocks)]).astype(np.uint32)
+    run_and_compare(ids, 300, 48, 12, 2, 5, mode)
