@@ -53,7 +53,8 @@ struct NoTable {
 struct AttnArgs {
     int mode;
     int n_tokens;          // L (phase 1) or nq (phase 2): tokens that exist, for the store guard
-    int Hq, g, pack;       // query heads, heads per KV head, rows per token in a tile (1 or g)
+    int Hq, g;             // query heads, heads per KV head
+    int pack_shift;        // log2 of the rows a token has in a tile (1, or the g heads of one KV head)
     int block_size;        // phase 1: tokens per block
     int prefix_total;      // phase 1: rows in the gathered prefix buffers
     const int32_t* prefix_len;
@@ -315,89 +316,76 @@ __device__ __forceinline__ int item_of_round(int round, int n_items) {
 template <typename Table>
 __device__ __forceinline__ void decode_item(const AttnArgs& a, const Table& vt, int idx, Item& it) {
     it.valid = 1;
-    const int per_item = a.single ? 1 : 2;                     // causal attention: query tiles per work item
-    if (a.mode == kModeVarlen) {
-        // Independent sequences of different lengths, plain causal attention inside each.
-        // Items run from the last sequence down and, inside a sequence, from its last tile
-        // pair down (for assembled Pulsar inputs the later blocks are the longer ones).
-        const int rank = idx / a.Hq;
-        it.head0 = idx - rank * a.Hq;
-        it.kvh = it.head0 / a.g;
-        it.part = 0;
-        int k = 0;                                             // k-th sequence from the end
-        while (k + 1 < vt.n_seq && vt.pair_cum[k + 1] <= rank) ++k;
-        const int seq = vt.n_seq - 1 - k;
-        const int start = vt.start[seq], len = vt.start[seq + 1] - start;
-        const int tiles = (len + kTileM - 1) / kTileM, pairs = (tiles + per_item - 1) / per_item;
-        const int pair = pairs - 1 - (rank - vt.pair_cum[k]);
-        const int qt0 = per_item * pair;
-        it.has1 = (per_item == 2 && qt0 + 1 < tiles) ? 1 : 0;
-        it.row0_a = qt0 * kTileM;
-        it.row0_b = (qt0 + 1) * kTileM;
+    it.bad_length = 0;
+    it.part = 0;
+    it.gen_base = -1;
+    const int tpt = kTileM >> a.pack_shift;                    // tokens per query tile
+    if (a.mode != kModePhase2) {
+        const int per_item = a.single ? 1 : 2;                 // query tiles per work item
+        const int heads = a.pack_shift ? a.Hkv : a.Hq;         // work items per run of tokens
+        const int rank = idx / heads, h = idx - rank * heads;
+        it.head0 = a.pack_shift ? h * a.g : h;
+        it.kvh = a.pack_shift ? h : h / a.g;
+        int pair, len, start;
+        if (a.mode == kModeVarlen) {
+            // Independent sequences of different lengths, plain causal attention inside each.
+            // Items run from the last sequence down and, inside a sequence, from its last tokens
+            // down (for assembled Pulsar inputs the later blocks are the longer ones).
+            int k = 0;                                             // k-th sequence from the end
+            while (k + 1 < vt.n_seq && vt.pair_cum[k + 1] <= rank) ++k;
+            const int seq = vt.n_seq - 1 - k;
+            start = vt.start[seq];
+            len = vt.start[seq + 1] - start;
+            pair = (len + per_item * tpt - 1) / (per_item * tpt) - 1 - (rank - vt.pair_cum[k]);
+            it.pref_len = 0;
+        } else {
+            // Items run block-major from the last block (longest prefix) down and, within a block,
+            // from the last tokens (most causal tiles) down; the heads of one run of tokens are
+            // adjacent.  CTAs that run at the same time therefore read the same K/V rows (L2 hits),
+            // and the costliest items are handed out first.
+            // The last block may be shorter than the others: it then has fewer items.
+            int blk;
+            if (rank < a.pairs_last) {
+                blk = a.n_blocks - 1;
+                pair = a.pairs_last - 1 - rank;
+                len = a.last_len;
+            } else {
+                const int r2 = rank - a.pairs_last;
+                blk = a.n_blocks - 2 - r2 / a.pairs;
+                pair = a.pairs - 1 - r2 % a.pairs;
+                len = a.block_size;
+            }
+            start = blk * a.block_size;
+            int pl = a.prefix_len[blk];
+            it.bad_length = (pl < 0 || pl > a.prefix_total) ? 1 : 0;
+            it.pref_len = max(0, min(pl, a.prefix_total));
+        }
+        it.n_pref_tiles = (it.pref_len + kTileN - 1) / kTileN;
+        it.row0_a = per_item * pair * tpt;
+        it.row0_b = it.row0_a + tpt;
+        it.has1 = (per_item == 2 && it.row0_b < len) ? 1 : 0;
         it.token0_a = start + it.row0_a;
         it.token0_b = start + it.row0_b;
-        it.bad_length = 0;
-        it.pref_len = 0;
-        it.n_pref_tiles = 0;
         it.main_row0 = start;
         it.main_len = len;
-        it.gen_base = -1;
-        it.n_tiles_a = qt0 + 1;
-        it.n_tiles_b = it.has1 ? qt0 + 2 : 0;
-    } else if (a.mode == kModePhase1) {
-        // Items run block-major from the last block (longest prefix) down and, within a block,
-        // from the last tile pair (most causal tiles) down; the heads of one (block, pair) are
-        // adjacent.  CTAs that run at the same time therefore read the same K/V rows (L2 hits),
-        // and the costliest items are handed out first.
-        // The last block may be shorter than the others: it then has fewer tile pairs.
-        const int rank = idx / a.Hq;
-        it.head0 = idx - rank * a.Hq;
-        it.kvh = it.head0 / a.g;
-        it.part = 0;
-        int blk, pair, len;
-        if (rank < a.pairs_last) {
-            blk = a.n_blocks - 1;
-            pair = a.pairs_last - 1 - rank;
-            len = a.last_len;
-        } else {
-            const int r2 = rank - a.pairs_last;
-            blk = a.n_blocks - 2 - r2 / a.pairs;
-            pair = a.pairs - 1 - r2 % a.pairs;
-            len = a.block_size;
-        }
-        const int qt0 = per_item * pair;
-        it.has1 = (per_item == 2 && qt0 + 1 < (len + kTileM - 1) / kTileM) ? 1 : 0;
-        it.row0_a = qt0 * kTileM;
-        it.row0_b = (qt0 + 1) * kTileM;
-        it.token0_a = blk * a.block_size + it.row0_a;
-        it.token0_b = blk * a.block_size + it.row0_b;
-        int pl = a.prefix_len[blk];
-        it.bad_length = (pl < 0 || pl > a.prefix_total) ? 1 : 0;
-        pl = max(0, min(pl, a.prefix_total));
-        it.pref_len = pl;
-        it.n_pref_tiles = (pl + kTileN - 1) / kTileN;
-        it.main_row0 = blk * a.block_size;
-        it.main_len = len;
-        it.gen_base = -1;
-        it.n_tiles_a = it.n_pref_tiles + qt0 + 1;
-        it.n_tiles_b = it.has1 ? it.n_pref_tiles + qt0 + 2 : 0;
+        // key tiles up to the one with the tile's last row
+        it.n_tiles_a = it.n_pref_tiles + (min(it.row0_a + tpt, len) + kTileN - 1) / kTileN;
+        it.n_tiles_b = it.has1 ? it.n_pref_tiles + (min(it.row0_b + tpt, len) + kTileN - 1) / kTileN : 0;
     } else {
         const int rp = idx % a.pairs;
         const int rest = idx / a.pairs;
         it.kvh = rest % a.Hkv;
         it.part = rest / a.Hkv;
         it.head0 = it.kvh * a.g;
-        const int tokens_per_tile = kTileM / a.pack;
-        it.token0_a = (2 * rp) * tokens_per_tile;
-        it.token0_b = (2 * rp + 1) * tokens_per_tile;
+        it.token0_a = (2 * rp) * tpt;
+        it.token0_b = (2 * rp + 1) * tpt;
         it.has1 = (it.token0_b < a.n_tokens) ? 1 : 0;
         it.row0_a = it.row0_b = 0;
-        it.bad_length = 0;
         // the generation shard: read through the second pair of tensor maps, causal by token
         const bool shard = a.gen_total > 0 && it.part == a.gen_part;
         it.pref_len = shard ? a.gen_total : 0;
         it.n_pref_tiles = (it.pref_len + kTileN - 1) / kTileN;
-        it.gen_base = shard ? a.gen_len : -1;
+        if (shard) it.gen_base = a.gen_len;
         it.main_row0 = it.part * a.split_len;
         it.main_len = max(0, min(a.split_len, a.kv_len - it.main_row0));
         const int n = it.n_pref_tiles + (it.main_len + kTileN - 1) / kTileN;
@@ -883,7 +871,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 if (pref_left > 0) {
                     if (pref_left < kTileN) { n_vis = pref_left; masked = true; }
                     if (it.gen_base >= 0) {                   // generation shard: causal by token
-                        const int token = (s ? it.token0_b : it.token0_a) + row_t / a.pack;
+                        const int token = (s ? it.token0_b : it.token0_a) + (row_t >> a.pack_shift);
                         n_vis = min(n_vis, it.gen_base + token + 1 - t * kTileN);
                         masked = true;
                     }
@@ -892,7 +880,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     const int valid = it.main_len - j * kTileN;
                     if (valid < kTileN) { n_vis = valid; masked = true; }
                     if (a.mode != kModePhase2 && t == n - 1) {
-                        n_vis = min(n_vis, (s ? it.row0_b : it.row0_a) + row - j * kTileN + 1);
+                        n_vis = min(n_vis, (s ? it.row0_b : it.row0_a) + (row_t >> a.pack_shift) - j * kTileN + 1);
                         masked = true;
                     }
                 }
@@ -1067,11 +1055,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 ++o_cnt;
                 if (!ok) break;
                 tc_fence_after();
-                const int token = (s ? it.token0_b : it.token0_a) + row_t / a.pack;
-                const int head = it.head0 + row_t % a.pack;
+                const int in_tile = row_t >> a.pack_shift, token = (s ? it.token0_b : it.token0_a) + in_tile;
+                const int head = it.head0 + (row_t & ((1 << a.pack_shift) - 1));
                 const int part = kQuad ? it.part * 4 + (warp & 3) : it.part;
                 bool store = token < a.n_tokens;
-                if (a.mode != kModePhase2) store = store && (s ? it.row0_b : it.row0_a) + row < it.main_len;
+                if (a.mode != kModePhase2) store = store && (s ? it.row0_b : it.row0_a) + in_tile < it.main_len;
                 const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
                 const float lse = (l_run > 0.f) ? (m_used + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
                 const size_t orow = static_cast<size_t>(token) * a.Hq + head;
@@ -1207,10 +1195,29 @@ int32_t launch_attn(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMa
 struct Phase1Plan {
     int n_blocks;
     int last_len;                             // tokens of the last block
-    int single, items_block, items_last;      // one query tile per work item; items per head of a full and of the last block
+    int pack_shift;                           // log2 of the query rows a token has in a tile
+    int single, items_block, items_last;      // one query tile per work item; items per head (group) of a full and of the last block
     int n_items;
     size_t pref_rows, pref_bytes, total;
 };
+
+// log2 of a power of two
+int log2_of(int g) {
+    int s = 0;
+    while ((1 << s) < g) ++s;
+    return s;
+}
+
+// log2 of the heads of a KV head that share a query tile of causal attention.  With all g heads of 128/g tokens in a tile,
+// both tiles of a work item end in the same key tile; with 128 tokens of one head the second needs one more, which
+// it walks alone.  Half a key tile per item is saved, but the items that run at the same time then cover g times as
+// many tokens and no longer read the same K/V tiles in step.  With d = 64, where a tile is half as large and the GPU is
+// below its power limit, packing gains 3.5 % (45K ragged 0.916 -> 0.884 ms); with d = 128 it costs 0.7-1 % from 32K on
+// (64K 5.33 -> 5.37 ms, 128K 14.12 -> 14.27 ms; 16K the same).  The group must be a power of two up to 16.
+int causal_pack_shift(int32_t Hq, int32_t Hkv, int32_t d) {
+    const int g = Hq / Hkv;
+    return d == 64 && g <= 16 && (g & (g - 1)) == 0 ? log2_of(g) : 0;
+}
 
 // Causal attention with so few pairs of query tiles that they would not fill the SMs once takes work items of one
 // tile: twice the items, and a key tile costs the chain of one tile (about 1.2 us) instead of two interleaved ones
@@ -1232,17 +1239,17 @@ int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block
     p.last_len = static_cast<int>(L - (B - 1) * block_size);
     p.pref_bytes = round_up(p.pref_rows * Hkv * d * 2, 256);
     p.total = 2 * p.pref_bytes + 256;                        // gathered prefix K, V and the work counter
-    const int tiles_block = static_cast<int>((static_cast<int64_t>(block_size) + kTileM - 1) / kTileM);
-    const int tiles_last = (p.last_len + kTileM - 1) / kTileM;
-    p.items_block = (tiles_block + 1) / 2;
-    p.items_last = (tiles_last + 1) / 2;
-    int64_t items = ((B - 1) * p.items_block + p.items_last) * Hq;
-    if (items >= (1ll << 31)) return PULSAR_ERR_SHAPE;
-    p.single = causal_single(items) ? 1 : 0;
-    if (p.single) {
-        p.items_block = tiles_block;
-        p.items_last = tiles_last;
-        items = ((B - 1) * p.items_block + p.items_last) * Hq;
+    p.pack_shift = causal_pack_shift(Hq, Hkv, d);
+    const int64_t heads = p.pack_shift ? Hkv : Hq;
+    int64_t items = 0;
+    for (int per_item = 2; per_item >= 1; --per_item) {
+        const int64_t tokens = static_cast<int64_t>(per_item) * (kTileM >> p.pack_shift);
+        p.single = per_item == 1 ? 1 : 0;
+        p.items_block = static_cast<int>((block_size + tokens - 1) / tokens);
+        p.items_last = static_cast<int>((p.last_len + tokens - 1) / tokens);
+        items = ((B - 1) * p.items_block + p.items_last) * heads;
+        if (items >= (1ll << 31)) return PULSAR_ERR_SHAPE;
+        if (per_item == 2 && !causal_single(items)) break;
     }
     p.n_items = static_cast<int>(items);
     return PULSAR_OK;
@@ -1332,7 +1339,7 @@ extern "C" int32_t pulsar_phase1_attn(const uint16_t* Q, const uint16_t* K, cons
     int32_t* counter = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + 2 * p.pref_bytes);
 
     CUtensorMap tmQ, tmK, tmV, tmKp, tmVp;
-    if (!make_map_3d(&tmQ, Q, L, Hq, d, 1, kTileM) || !make_map_2d(&tmK, K, L, static_cast<int64_t>(Hkv) * d) ||
+    if (!make_map_3d(&tmQ, Q, L, Hq, d, 1 << p.pack_shift, kTileM >> p.pack_shift) || !make_map_2d(&tmK, K, L, static_cast<int64_t>(Hkv) * d) ||
         !make_map_2d(&tmV, V, L, static_cast<int64_t>(Hkv) * d) ||
         !make_map_2d(&tmKp, Kp, static_cast<int64_t>(p.pref_rows), static_cast<int64_t>(Hkv) * d) ||
         !make_map_2d(&tmVp, Vp, static_cast<int64_t>(p.pref_rows), static_cast<int64_t>(Hkv) * d))
@@ -1361,7 +1368,7 @@ extern "C" int32_t pulsar_phase1_attn(const uint16_t* Q, const uint16_t* K, cons
     a.n_tokens = static_cast<int>(L);
     a.Hq = Hq;
     a.g = Hq / Hkv;
-    a.pack = 1;
+    a.pack_shift = p.pack_shift;
     a.block_size = block_size;
     a.prefix_total = prefix_total;
     a.prefix_len = prefix_len;
@@ -1456,7 +1463,7 @@ extern "C" int32_t pulsar_phase1_attn_sharded(const uint16_t* Q, const uint16_t*
     const uint16_t* Kp = prefix_total > 0 ? K_prefix : K;
     const uint16_t* Vp = prefix_total > 0 ? V_prefix : V;
     CUtensorMap tmQ, tmK, tmV, tmKp, tmVp;
-    if (!make_map_3d(&tmQ, Q, L_local, Hq, d, 1, kTileM) ||
+    if (!make_map_3d(&tmQ, Q, L_local, Hq, d, 1 << p.pack_shift, kTileM >> p.pack_shift) ||
         !make_map_2d(&tmK, K, L_local, static_cast<int64_t>(Hkv) * d) ||
         !make_map_2d(&tmV, V, L_local, static_cast<int64_t>(Hkv) * d) ||
         !make_map_2d(&tmKp, Kp, static_cast<int64_t>(p.pref_rows), static_cast<int64_t>(Hkv) * d) ||
@@ -1478,7 +1485,7 @@ extern "C" int32_t pulsar_phase1_attn_sharded(const uint16_t* Q, const uint16_t*
     a.n_tokens = static_cast<int>(L_local);
     a.Hq = Hq;
     a.g = Hq / Hkv;
-    a.pack = 1;
+    a.pack_shift = p.pack_shift;
     a.block_size = block_size;
     a.prefix_total = prefix_total;
     a.prefix_len = prefix_len_local;
@@ -1570,7 +1577,7 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
     a.n_tokens = nq;
     a.Hq = Hq;
     a.g = g;
-    a.pack = g;
+    a.pack_shift = log2_of(g);
     a.split_len = static_cast<int>(phase2_split_len(L, n_splits));
     a.kv_len = static_cast<int>(L);
     a.quad = quad ? 1 : 0;
@@ -1669,7 +1676,7 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     a.n_tokens = n_new;
     a.Hq = Hq;
     a.g = g;
-    a.pack = g;
+    a.pack_shift = log2_of(g);
     a.split_len = static_cast<int>(part_tiles * kTileN);
     a.kv_len = static_cast<int>(L);
     a.gen_part = n_parts - 1;
@@ -1735,23 +1742,25 @@ extern "C" int32_t pulsar_causal_varlen_attn(const uint16_t* Q, const uint16_t* 
     VarlenTable vt{};
     vt.n_seq = n_seq;
     for (int j = 0; j <= n_seq; ++j) vt.start[j] = cu_seqlens_host[j];
+    const int pack_shift = causal_pack_shift(Hq, Hkv, d), heads = pack_shift ? Hkv : Hq;
     int64_t pairs_total = 0;
     int single = 0;
     for (int per_item = 2; per_item >= 1; --per_item) {
+        const int tokens = per_item * (kTileM >> pack_shift);
         pairs_total = 0;
         for (int k = 0; k < n_seq; ++k) {
             vt.pair_cum[k] = static_cast<int>(pairs_total);
             const int len = vt.start[n_seq - k] - vt.start[n_seq - 1 - k];
-            pairs_total += ((len + kTileM - 1) / kTileM + per_item - 1) / per_item;
+            pairs_total += (len + tokens - 1) / tokens;
         }
         vt.pair_cum[n_seq] = static_cast<int>(pairs_total);
-        if (pairs_total * Hq >= (1ll << 31)) return PULSAR_ERR_SHAPE;
-        if (per_item == 2 && !causal_single(pairs_total * Hq)) break;
+        if (pairs_total * heads >= (1ll << 31)) return PULSAR_ERR_SHAPE;
+        if (per_item == 2 && !causal_single(pairs_total * heads)) break;
         single = per_item == 1 ? 1 : 0;
     }
 
     CUtensorMap tmQ, tmK, tmV;
-    if (!make_map_3d(&tmQ, Q, total_rows, Hq, d, 1, kTileM) ||
+    if (!make_map_3d(&tmQ, Q, total_rows, Hq, d, 1 << pack_shift, kTileM >> pack_shift) ||
         !make_map_2d(&tmK, K, total_rows, static_cast<int64_t>(Hkv) * d) ||
         !make_map_2d(&tmV, V, total_rows, static_cast<int64_t>(Hkv) * d))
         return PULSAR_ERR_CUDA;
@@ -1764,10 +1773,10 @@ extern "C" int32_t pulsar_causal_varlen_attn(const uint16_t* Q, const uint16_t* 
     a.n_tokens = static_cast<int>(total_rows);
     a.Hq = Hq;
     a.g = Hq / Hkv;
-    a.pack = 1;
+    a.pack_shift = pack_shift;
     a.Hkv = Hkv;
     a.single = single;
-    a.n_items = static_cast<int>(pairs_total) * Hq;
+    a.n_items = static_cast<int>(pairs_total) * heads;
     a.counter = counter;
     a.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
     a.O = O;

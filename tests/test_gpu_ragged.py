@@ -146,3 +146,20 @@ def test_whole_step_through_the_encoder():
     check_attention(res["O1"], res["LSE1"], Oref, Lref, "encoder phase 1")
     O2ref, L2ref = oracle.phase2_attn(Qq, K, V, 1, w.L)
     check_attention(res["O2"], res["LSE2"], O2ref, L2ref, "encoder phase 2")
+
+
+@pytest.mark.parametrize("Hq,Hkv", [(1, 1), (6, 2), (8, 4), (16, 1), (32, 1), (40, 5)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_head_groups_in_a_query_tile(Hq, Hkv, d):
+    """A query tile holds the heads of a group for 128/g tokens (d = 64, g a power of two up to 16) or 128 tokens of one
+    head; blocks and a last block that end inside a tile of either."""
+    w = W.shrink(W.CONFIGS["tiny"], L=1111, block_size=333, chunk=9, k=5, sink=21, Hq=Hq, Hkv=Hkv, d=d, nq=5)
+    Q, K, V = W.qkv(w, q_scale=2.0)
+    pidx, plen = W.first_k_prefix(w)
+    status = binding.new_status(DEV)
+    O, LSE, _, _ = binding.pulsar_phase1_attn(Q.to(DEV), K.to(DEV), V.to(DEV), w.block_size, torch.from_numpy(pidx).to(DEV),
+                                              torch.from_numpy(plen).to(DEV), status=status)
+    Oref, Lref = oracle.phase1_attn(Q, K, V, w.block_size, pidx, plen)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    check_attention(O, LSE, Oref, Lref, f"Hq={Hq} Hkv={Hkv} d={d}")
