@@ -636,7 +636,7 @@ def run_extras(binding, w, dev, K_d, V_d, peaks):
                                             frac_of_measured_hbm=nbytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                                             ms_after_write_only_flush=ms_dirty,
                                             frac_after_write_only_flush=nbytes / (ms_dirty * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                                            launches="append + attention + merge", l2=how)
+                                            launches="attention (appends the new rows) + merge", l2=how)
     del flush_words
     del flush
     w4 = W.CONFIGS["64k"]
