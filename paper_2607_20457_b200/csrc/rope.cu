@@ -2,10 +2,10 @@
 //
 //   assemble_positions_kernel  one CTA column per assembled input: the prefix entries keep their
 //                              global positions (sparse) or everything is renumbered (contiguous)
-//   rope_kernel                a CTA takes eight rows at a time: each row's d/2 (cos, sin) pairs are
-//                              formed once in shared memory -- angle in float64, reduced to [-pi, pi],
-//                              then sincosf -- and applied to every head with 16-byte loads and
-//                              stores.  A pure stream over the rows: HBM-bound.
+//   rope_kernel                a thread owns one 16-byte vector position of one row, holds its eight
+//                              (cos, sin) pairs in registers -- angle in float64, reduced to [-pi, pi],
+//                              then sincosf, each formed once -- and walks the heads.  A pure stream
+//                              over the rows: HBM-bound.
 #include <cmath>
 
 #include "common.cuh"
@@ -52,90 +52,98 @@ assemble_positions_kernel(const int32_t* __restrict__ prefix_idx, const int32_t*
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-// Measured on B200 (80,320 rows of 32 + 8 heads, d = 128, two launches): 8 rows, 2 loads in flight,
-// 4 CTAs per SM 5.25 TB/s; 16 rows 5.09; 4 loads in flight (spills at 64 registers) 4.88; 6 CTAs per SM
-// 4.77.  The 32-head pass alone streams at 6.4 TB/s; the 8-head pass is bound by the sines and cosines
-// (same work per row, a quarter of the bytes), which is why Q and K can share one launch.
-constexpr int kRopeRows = 8;                        // rows a CTA takes at a time
-constexpr int kRopeUnroll = 2;                      // tasks (2 x 16-byte loads each) in flight per thread
-constexpr int kRopeCtasPerSm = 4;
+// Measured on B200 against a persistent kernel that took eight rows between two barriers and read the pairs from shared
+// memory for every vector (us, Q + K heads x d): 80,320 rows of 32 + 8 x 128 259 -> 257; 37,003 of 16 + 4 x 64 46 -> 38;
+// 50,000 of 4 + 1 x 32 16.9 -> 11.4; 65 of 32 + 8 x 128 8.7 -> 4.6.  Six heads in flight 1.5 %, four 3 % slower with 40
+// heads; loads issued ahead of the barrier of the shared form 15-50 % slower.
+constexpr int kRopeThreads = 128;
+constexpr int kRopeUnroll = 8;                      // heads (2 x 16-byte loads each) in flight per thread
+constexpr int kRopePairs = kRopeThreads * 8;        // a vector holds eight pairs' first or second halves
 
 // X2/Y2/H2 describe an optional second tensor with the same rows and head size (K beside Q): it
-// shares the rows' cosines and sines; H2 = 0 when there is none.
-__global__ void __launch_bounds__(256, kRopeCtasPerSm)
+// shares the rows' cosines and sines; H2 = 0 when there is none.  `groups` threads share a vector position of a row and
+// take every groups-th head.
+// kShared: the CTA's threads form the pairs together; one thread's eight in a row take 2 us, most of a small call.
+template <bool kShared>
+__global__ void __launch_bounds__(kRopeThreads)
 rope_kernel(const uint4* __restrict__ X1, uint4* __restrict__ Y1, int H1, const uint4* __restrict__ X2,
-            uint4* __restrict__ Y2, int H2, int64_t rows, int d, const int32_t* __restrict__ positions,
+            uint4* __restrict__ Y2, int H2, int64_t rows, int d, int groups, const int32_t* __restrict__ positions,
             const __grid_constant__ RopeFreq f, int32_t* status) {
-    __shared__ float s_cos[kRopeRows][kMaxHalf], s_sin[kRopeRows][kMaxHalf];
     const int half = d >> 1;
     const int vec_half = half >> 3;                 // 16-byte vectors per half row of a head
     const int head_vecs = d >> 3;
-    const int tasks1 = H1 * vec_half;               // per row: one task = vector v of both halves of head h
-    const int tasks = tasks1 + H2 * vec_half;
-    const int64_t n_groups = (rows + kRopeRows - 1) / kRopeRows;
-    for (int64_t grp = blockIdx.x; grp < n_groups; grp += gridDim.x) {
-        const int64_t row0 = grp * kRopeRows;
-        const int nr = static_cast<int>(min(static_cast<int64_t>(kRopeRows), rows - row0));
-        for (int e = threadIdx.x; e < nr * half; e += blockDim.x) {
-            const int r = e / half, j = e - r * half;
-            int p = positions[row0 + r];
-            if (p < 0) {
-                report(status, PULSAR_DEV_BAD_POSITION);
-                p = 0;
-            }
-            // angle / 2pi in float64, reduced to [-1/2, 1/2] turns, then float32 sincos of at most pi
-            const double turns = static_cast<double>(p) * f.inv_freq[j] * 0.15915494309189535;
-            const double frac = turns - rint(turns);
-            float sn, cs;
-            sincosf(static_cast<float>(frac * 6.283185307179586), &sn, &cs);
-            s_cos[r][j] = cs;
-            s_sin[r][j] = sn;
-        }
-        __syncthreads();
-        const int total = nr * tasks;
-        for (int t0 = threadIdx.x; t0 < total; t0 += blockDim.x * kRopeUnroll) {
-            uint4 a[kRopeUnroll], b[kRopeUnroll];
-            int rr[kRopeUnroll], vv[kRopeUnroll];
-            uint4* dst[kRopeUnroll];
+    const int rows_cta = kRopeThreads / vec_half / groups;
+    const int64_t row0 = static_cast<int64_t>(blockIdx.x) * rows_cta;
+    const int nr = static_cast<int>(min(static_cast<int64_t>(rows_cta), rows - row0));
+    const int slot = threadIdx.x / vec_half, v = threadIdx.x - slot * vec_half;
+    const int r = slot / groups;
+    const bool active = r < nr;
+    const int heads = active ? H1 + H2 : 0;
+    const int64_t at1 = (row0 + r) * H1 * head_vecs + v, at2 = (row0 + r) * H2 * head_vecs + v;
+
+    uint4 a[kRopeUnroll], b[kRopeUnroll];
+    auto load = [&](int h0) {
 #pragma unroll
-            for (int u = 0; u < kRopeUnroll; ++u) {
-                const int t = t0 + u * blockDim.x;
-                if (t < total) {
-                    const int r = t / tasks;
-                    int rem = t - r * tasks;
-                    const bool second = rem >= tasks1;
-                    if (second) rem -= tasks1;
-                    const int h = rem / vec_half, v = rem - h * vec_half;
-                    const int64_t lo = (row0 + r) * (static_cast<int64_t>(second ? H2 : H1) * head_vecs) + h * head_vecs + v;
-                    const uint4* src = (second ? X2 : X1) + lo;
-                    rr[u] = r;
-                    vv[u] = v;
-                    dst[u] = (second ? Y2 : Y1) + lo;
-                    a[u] = src[0];
-                    b[u] = src[vec_half];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kRopeUnroll; ++u) {
-                const int t = t0 + u * blockDim.x;
-                if (t < total) {
-                    const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
-                    uint32_t ya[4], yb[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int j = vv[u] * 8 + 2 * k;
-                        const float c0 = s_cos[rr[u]][j], s0 = s_sin[rr[u]][j];
-                        const float c1 = s_cos[rr[u]][j + 1], s1 = s_sin[rr[u]][j + 1];
-                        const float a0 = bf16_lo(aw[k]), a1 = bf16_hi(aw[k]), b0 = bf16_lo(bw[k]), b1 = bf16_hi(bw[k]);
-                        ya[k] = pack_bf16x2(a0 * c0 - b0 * s0, a1 * c1 - b1 * s1);
-                        yb[k] = pack_bf16x2(b0 * c0 + a0 * s0, b1 * c1 + a1 * s1);
-                    }
-                    dst[u][0] = make_uint4(ya[0], ya[1], ya[2], ya[3]);
-                    dst[u][vec_half] = make_uint4(yb[0], yb[1], yb[2], yb[3]);
-                }
+        for (int u = 0; u < kRopeUnroll; ++u) {
+            const int h = h0 + u * groups;
+            if (h < heads) {
+                const uint4* src = h < H1 ? X1 + at1 + h * head_vecs : X2 + at2 + (h - H1) * head_vecs;
+                a[u] = src[0];
+                b[u] = src[vec_half];
             }
         }
+    };
+    int h0 = slot - r * groups;
+    float cs[8], sn[8];
+    auto pair = [&](int64_t row, int j, float* sine, float* cosine) {
+        int p = positions[row];
+        if (p < 0) {
+            report(status, PULSAR_DEV_BAD_POSITION);
+            p = 0;
+        }
+        // angle / 2pi in float64, reduced to [-1/2, 1/2] turns, then float32 sincos of at most pi
+        const double turns = static_cast<double>(p) * f.inv_freq[j] * 0.15915494309189535;
+        const double frac = turns - rint(turns);
+        sincosf(static_cast<float>(frac * 6.283185307179586), sine, cosine);
+    };
+    if constexpr (kShared) {
+        __shared__ __align__(16) float s_cos[kRopePairs], s_sin[kRopePairs];
+        for (int e = threadIdx.x; e < nr * half; e += kRopeThreads) {
+            const int er = e / half;
+            pair(row0 + er, e - er * half, &s_sin[e], &s_cos[e]);
+        }
         __syncthreads();
+        if (!active) return;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            cs[k] = s_cos[r * half + v * 8 + k];
+            sn[k] = s_sin[r * half + v * 8 + k];
+        }
+    } else {
+        if (!active) return;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) pair(row0 + r, v * 8 + k, &sn[k], &cs[k]);
+    }
+    for (; h0 < heads; h0 += kRopeUnroll * groups) {
+        load(h0);
+#pragma unroll
+        for (int u = 0; u < kRopeUnroll; ++u) {
+            const int h = h0 + u * groups;
+            if (h < heads) {
+                uint4* dst = h < H1 ? Y1 + at1 + h * head_vecs : Y2 + at2 + (h - H1) * head_vecs;
+                const uint32_t aw[4] = {a[u].x, a[u].y, a[u].z, a[u].w}, bw[4] = {b[u].x, b[u].y, b[u].z, b[u].w};
+                uint32_t ya[4], yb[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float c0 = cs[2 * k], s0 = sn[2 * k], c1 = cs[2 * k + 1], s1 = sn[2 * k + 1];
+                    const float a0 = bf16_lo(aw[k]), a1 = bf16_hi(aw[k]), b0 = bf16_lo(bw[k]), b1 = bf16_hi(bw[k]);
+                    ya[k] = pack_bf16x2(a0 * c0 - b0 * s0, a1 * c1 - b1 * s1);
+                    yb[k] = pack_bf16x2(b0 * c0 + a0 * s0, b1 * c1 + a1 * s1);
+                }
+                dst[0] = make_uint4(ya[0], ya[1], ya[2], ya[3]);
+                dst[vec_half] = make_uint4(yb[0], yb[1], yb[2], yb[3]);
+            }
+        }
     }
 }
 
@@ -152,10 +160,19 @@ int32_t launch_rope(const uint16_t* X1, uint16_t* Y1, int32_t H1, const uint16_t
     if (rc != PULSAR_OK) return rc;
     RopeFreq f;
     for (int j = 0; j < d / 2; ++j) f.inv_freq[j] = std::pow(theta, -2.0 * static_cast<double>(j) / static_cast<double>(d));
-    const int64_t ctas = std::min<int64_t>((rows + kRopeRows - 1) / kRopeRows, static_cast<int64_t>(sm_count()) * kRopeCtasPerSm);
-    rope_kernel<<<static_cast<unsigned>(ctas), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+    // Few rows: the threads of a CTA split the heads instead of taking more rows, as long as the chip then has no more than
+    // the four CTAs per SM that fit (113 registers); a power of two leaves no slot idle.  32 + 8 heads x 128, us with a
+    // target of one / two / four / eight CTAs per SM: 1500 rows 12.8 / 10.7 / 8.7 / 8.9, 4000 rows 16.9 / 16.9 / 14.8 / 16.8.
+    const int slots = kRopeThreads / (d / 16);       // vector positions of whole rows per CTA, at least 8
+    const int64_t want = static_cast<int64_t>(sm_count()) * 4 * slots / rows;
+    int groups = 1;
+    while (2 * groups <= std::min<int64_t>(want, std::min(slots, H1 + H2))) groups *= 2;
+    const int64_t ctas = (rows + slots / groups - 1) / (slots / groups);
+    if (ctas > INT32_MAX) return PULSAR_ERR_SHAPE;
+    auto kernel = groups > 1 ? rope_kernel<true> : rope_kernel<false>;
+    kernel<<<static_cast<unsigned>(ctas), kRopeThreads, 0, static_cast<cudaStream_t>(stream)>>>(
         reinterpret_cast<const uint4*>(X1), reinterpret_cast<uint4*>(Y1), H1, reinterpret_cast<const uint4*>(X2),
-        reinterpret_cast<uint4*>(Y2), H2, rows, d, positions, f, device_status);
+        reinterpret_cast<uint4*>(Y2), H2, rows, d, groups, positions, f, device_status);
     PULSAR_CUDA_OK(cudaGetLastError());
     count_launch();
     return PULSAR_OK;

@@ -40,6 +40,16 @@ def test_rope_matches_oracle(H, d):
     check_rope(X, pos, 500000.0 if d != 64 else 10000.0)
 
 
+@pytest.mark.parametrize("rows,H,d", [(1, 1, 128), (1, 40, 128), (17, 9, 128), (4736, 2, 128), (4737, 2, 128),
+                                      (5, 17, 48), (43, 3, 48), (12432, 2, 48), (12433, 2, 48), (9, 8, 256)])
+def test_rope_few_and_many_rows(rows, H, d):
+    """On 148 SMs a CTA's threads split the heads up to 148 * 4 * (128 // (d / 16)) / 2 rows (4736 with d = 128, 12432 with
+    d = 48, where two of 128 threads have no vector); beyond that every thread forms its own sines."""
+    g = torch.Generator().manual_seed(rows + H)
+    pos = torch.randint(0, 131072, (rows,), generator=g, dtype=torch.int32).numpy()
+    check_rope(torch.randn((rows, H, d), generator=g).bfloat16(), pos, 500000.0)
+
+
 def test_rope_in_place_and_sparse_positions_of_an_assembled_input():
     w = W.CONFIGS["16k"]
     ids = W.needle_ids(w)
