@@ -53,8 +53,8 @@ __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w 
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
 // Measured on B200 against a persistent kernel that took eight rows between two barriers and read the pairs from shared
-// memory for every vector (us, Q + K heads x d): 80,320 rows of 32 + 8 x 128 259 -> 257; 37,003 of 16 + 4 x 64 46 -> 38;
-// 50,000 of 4 + 1 x 32 16.9 -> 11.4; 65 of 32 + 8 x 128 8.7 -> 4.6.  Six heads in flight 1.5 %, four 3 % slower with 40
+// memory for every vector (us, Q + K heads x d): 80,320 rows of 32 + 8 x 128 260 -> 258; 37,003 of 16 + 4 x 64 46 -> 39;
+// 50,000 of 4 + 1 x 32 16.9 -> 11.4; 65 of 32 + 8 x 128 8.7 -> 4.6.  Six heads in flight 1.5 %, four 2-4 % slower with 40
 // heads; loads issued ahead of the barrier of the shared form 15-50 % slower.
 constexpr int kRopeThreads = 128;
 constexpr int kRopeUnroll = 8;                      // heads (2 x 16-byte loads each) in flight per thread
