@@ -395,17 +395,20 @@ int32_t pulsar_phase2_attn(const uint16_t *Qq, int32_t nq,
  * The n_new newest tokens (the whole query on the first step, one generated token afterwards)
  * have their keys and values appended to the "designated generation shard" (Alg. 1 l.15) and
  * then attend to (1) all B*block_size retained context keys, without mask, and (2) the
- * generation shard causally: new token u sees shard rows [0, gen_len + u].  The context is cut
- * into n_splits parts as in pulsar_phase2_attn; the generation shard is one more part; all parts
- * are merged exactly through their log-sum-exp (Appendix H), so the result equals one softmax
- * over the concatenation [context | generation shard up to the token].
+ * generation shard causally: new token u sees shard rows [0, gen_len + u].  Context and shard are
+ * cut into parts, whichever way is expected to take less time: the context into
+ * n_splits parts as in pulsar_phase2_attn and the shard as one more part, or both together into at
+ * most n_splits parts, the shard in front of the last part's context keys or a part beside them.
+ * All parts are merged exactly through their log-sum-exp (Appendix H), so the result equals one
+ * softmax over the concatenation [context | generation shard up to the token] however it is cut.
  *
  *   Qnew        in  [n_new, Hq, d] bf16       Knew, Vnew  in [n_new, Hkv, d] bf16
  *   Kblocks, Vblocks in [B*block_size, Hkv, d] bf16 (retained context KV)
  *   Kgen, Vgen  in/out [gen_capacity, Hkv, d] bf16: rows [0, gen_len) hold the earlier query /
  *               generated tokens; rows [gen_len, gen_len + n_new) are written by this call;
  *               rows from gen_len + n_new on are never read (they may hold anything, NaN included)
- *   n_splits    parts of the context KV: 0 = library's choice, else as in pulsar_phase2_attn
+ *   n_splits    0 = library's choice, else the parts the context alone would be cut into (a count that
+ *               would leave one of them empty is rejected as in pulsar_phase2_attn)
  *   O           out [n_new, Hq, d] bf16       LSE out [n_new, Hq] float32 or NULL
  *
  * Requirements as for pulsar_phase2_attn, plus gen_len >= 0 and gen_len + n_new <= gen_capacity

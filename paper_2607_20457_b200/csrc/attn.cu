@@ -13,10 +13,11 @@
 //            contiguous part of the retained KV, no mask; output is the fp32 partial (A_j, l_j)
 //            or, with a single part, the final bf16 result.  With at most 32 such rows (decode)
 //            the rows are replicated into the four lane quarters of the tile and each softmax
-//            warp takes a quarter of the keys; the generation shard of Algorithm 1 l.11-16 is
-//            one more part, causal by token.
+//            warp takes a quarter of the keys; the generation shard of Algorithm 1 l.11-16, causal by
+//            token, is one more part or stands in front of the last part's context keys.
 //   Assembled inputs (Algorithm 1 l.8 as the paper runs it): sequences of any lengths packed back
 //            to back, every token a query, plain causal attention inside each.
+#include <algorithm>
 #include <type_traits>
 
 #include <cuda.h>
@@ -60,6 +61,7 @@ struct AttnArgs {
     const int32_t* prefix_len;
     int split_len;         // phase 2: keys per KV part (the last part may be shorter)
     int kv_len;            // phase 2: context keys in total
+    int ctx_part0;         // phase 2: the first part with context keys (1 where part 0 is the generation shard)
     int gen_part;          // phase 2: the part that has the generation shard in front of its context keys (if any)
     int gen_len;           // phase 2: rows of the generation shard that precede the new tokens
     int gen_total;         // phase 2: gen_len + new tokens (0 = no generation shard)
@@ -69,6 +71,7 @@ struct AttnArgs {
     uint4* Vgen;
     int quad;              // phase 2, at most 32 query rows per KV head: the rows are replicated into the four
                            // lane quarters of the tile and each softmax warp takes one quarter of the keys
+    int tile_max;          // phase 2: P of a key tile is formed with that tile's own maximum (see cut_generate, next_max)
     int single;            // work items of one query tile: the tile's logits alternate between the two S buffers so
                            // that S of the next key tile is formed during the softmax of this one.  Phase 2 with
                            // one query tile per KV head (set with quad as well), causal attention with few items
@@ -386,8 +389,8 @@ __device__ __forceinline__ void decode_item(const AttnArgs& a, const Table& vt, 
         it.pref_len = shard ? a.gen_total : 0;
         it.n_pref_tiles = (it.pref_len + kTileN - 1) / kTileN;
         if (shard) it.gen_base = a.gen_len;
-        it.main_row0 = it.part * a.split_len;
-        it.main_len = max(0, min(a.split_len, a.kv_len - it.main_row0));
+        it.main_row0 = (it.part - a.ctx_part0) * a.split_len;
+        it.main_len = it.main_row0 < 0 ? 0 : min(a.split_len, a.kv_len - it.main_row0);
         const int n = it.n_pref_tiles + (it.main_len + kTileN - 1) / kTileN;
         it.n_tiles_a = n;
         it.n_tiles_b = it.has1 ? n : 0;
@@ -411,6 +414,15 @@ __device__ __forceinline__ void append_head(const AttnArgs& a, int kvh, int d, i
     }
     fence_proxy_async_global();
     __syncwarp();
+}
+
+// The maximum that the P of a key tile is formed with.  It moves up when the tile's maximum is more than the threshold
+// above it, always on the first tile.  With tile_max it follows the tile's maximum down as well (by at most the
+// threshold at a time, and only while the row sum shows that no earlier probability is far above 1), so that the
+// largest probability of every tile is 1 and has no rounding error.
+__device__ __forceinline__ float next_max(float m_tile, float m_used, float l_run, bool tile_max) {
+    if (tile_max && (m_tile > m_used || l_run < 256.f)) return fmaxf(m_tile, m_used - kRescaleThreshold);
+    return m_tile > m_used + kRescaleThreshold ? m_tile : m_used;
 }
 
 // Row maximum of 128 raw logits (3-input max, four independent chains).
@@ -860,6 +872,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             if (!it.valid) break;
             const int n = s ? it.n_tiles_b : it.n_tiles_a;
             const int pref_len = it.pref_len;
+            const bool tile_max = a.tile_max && it.main_len > 0;
             float m_used = -INFINITY, l_run = 0.f;
             const int row_t = kQuad ? lane : row;             // row as far as token and head are concerned
 
@@ -915,8 +928,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 #pragma unroll
                     for (int c = 0; c < 32; c += 2) mq = max3(mq, __uint_as_float(rq[c]), __uint_as_float(rq[c + 1]));
                     const float m_tile = mq * a.scale_log2;
-                    const bool need = m_tile > m_used + kRescaleThreshold;
-                    if (__any_sync(0xffffffffu, need)) {
+                    const float m_new = next_max(m_tile, m_used, l_run, tile_max);
+                    if (__any_sync(0xffffffffu, m_new != m_used)) {
                         if (kSingle && t > 0) {
                             // O may be rescaled once the PV product of the previous key tile is complete.
                             // This is key tile g_tile - 1 of the CTA; completions 0 .. g_tile - 3 are certain
@@ -926,7 +939,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                             if (!ok) break;
                             tc_fence_after();
                         }
-                        const float m_new = need ? m_tile : m_used;
                         const float alpha = (m_new == -INFINITY) ? 1.f : ex2(m_used - m_new);
                         l_run *= alpha;
                         m_used = m_new;
@@ -993,7 +1005,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 // maximum and the vote took 520 of the 3250 cycles of a key tile before anything could be
                 // exponentiated: Phase 1 at 64K 5.46 -> 5.37 ms, d = 64 0.944 -> 0.918 ms.
                 float s1 = 0.f, neg_m = -m_used;
-                bool fast = !masked && t > 0;
+                bool fast = !masked && t > 0 && !tile_max;
                 if (fast) {
                     s1 = exp_row128<0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
                     float m2 = -INFINITY;
@@ -1003,8 +1015,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 }
                 if (!fast) {
                     const float m_tile = row_max128(r) * a.scale_log2;
-                    const bool need = m_tile > m_used + kRescaleThreshold;   // always true on the first tile
-                    if (__any_sync(0xffffffffu, need)) {
+                    const float m_new = next_max(m_tile, m_used, l_run, tile_max);
+                    if (__any_sync(0xffffffffu, m_new != m_used)) {
                         if (kSingle && t > 0) {
                             // O may be rescaled once the PV product of the previous key tile is complete.
                             // This is key tile g_tile - 1 of the CTA; completions 0 .. g_tile - 3 are certain
@@ -1014,7 +1026,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                             if (!ok) break;
                             tc_fence_after();
                         }
-                        const float m_new = need ? m_tile : m_used;
                         const float alpha = (m_new == -INFINITY) ? 1.f : ex2(m_used - m_new);
                         l_run *= alpha;
                         m_used = m_new;
@@ -1297,6 +1308,39 @@ int64_t phase2_split_len(int64_t L, int32_t n_splits) {
     const int64_t tiles_per_part = (kv_tiles + n_splits - 1) / n_splits;
     if ((kv_tiles + tiles_per_part - 1) / tiles_per_part != n_splits) return 0;
     return tiles_per_part * kTileN;
+}
+
+// How a generation step cuts context and shard.
+struct GenerateCut {
+    int n_parts;
+    int64_t split_len;        // context keys per part
+    bool shard_apart;         // the shard is part 0; otherwise it stands in front of the last part's context keys
+    bool lengthened;          // parts of fewer than four key tiles became longer than n_splits parts of the context are: P
+                              // is then formed with every tile's own maximum, as it is in parts of one tile (with a
+                              // maximum that lags it is 8-10 % further from float64 in decode shapes, 3-5 % in others;
+                              // from four tiles on one tile more is worth 1 % and less, and the rescaling of O would cost 7 %)
+};
+
+// Either the context in n_splits parts and the shard as one more (J + 1 parts), or context and shard together in parts of
+// equally many key tiles, at most n_splits of them, with the shard in front of the last part's context keys where
+// it fits there.  The second form has fewer partials and keeps the work items at one per SM where the first opens
+// another round (1024 key tiles, 8 KV heads: 152 items on 148 SMs, 97 us against 92; 72 tiles, 4 KV heads: 11.8 against
+// 10.6 us), so it is taken unless its longest chain of key tiles is clearly the longer one (n_splits = 1 with 32
+// tiles on each side: 53 us against 37).  An item beyond the first of a CTA costs about three tiles more.
+GenerateCut cut_generate(int64_t L_ctx, int64_t gen_rows, int64_t items_per_part, int32_t n_splits) {
+    const int64_t ctx = (L_ctx + kTileN - 1) / kTileN, gen = (gen_rows + kTileN - 1) / kTileN;      // key tiles
+    const int64_t J = n_splits, sms = sm_count();
+    const auto chain = [&](int64_t parts, int64_t tiles, int64_t shard_tiles) {
+        const int64_t rounds = (parts * items_per_part + sms - 1) / sms;
+        return std::max(rounds * (tiles + 3) - 3, shard_tiles);
+    };
+    const int64_t own = (ctx + J - 1) / J, own_chain = chain(J + 1, own, gen);
+    const int64_t joint = (ctx + gen + J - 1) / J, parts = (ctx + joint - 1) / joint;
+    const bool fits = ctx - (parts - 1) * joint + gen <= joint;
+    const int64_t joint_chain = fits ? chain(parts, joint, 0) : chain(parts + 1, joint, gen);
+    if (joint_chain > own_chain + std::max<int64_t>(2, own_chain / 8))
+        return {static_cast<int>(J + 1), phase2_split_len(L_ctx, n_splits), true, false};
+    return {static_cast<int>(fits ? parts : parts + 1), joint * kTileN, !fits, joint > own && own < 4};
 }
 
 }  // namespace
@@ -1615,7 +1659,7 @@ extern "C" size_t pulsar_phase2_generate_workspace_bytes(int32_t n_new, int32_t 
                                                          int32_t Hkv, int32_t d, int32_t n_splits) {
     size_t a, b;
     if (plan_phase2(n_new, B, block_size, Hq, Hkv, d, n_splits, a, b) != PULSAR_OK) return 0;
-    // room for a part of its own for the generation shard; four partials per part for decode shapes
+    // one more part than the context has: the generation shard; four partials per part for decode shapes
     const size_t parts = static_cast<size_t>(n_splits + 1) * (phase2_quad(n_new, Hq / Hkv) ? 4 : 1);
     return round_up(parts * n_new * Hq * d * 4, 256) + round_up(parts * n_new * Hq * 4, 256);
 }
@@ -1637,15 +1681,10 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
         !aligned(Kgen, 16) || !aligned(Vgen, 16) || !aligned(O, 16) || (LSE && !aligned(LSE, 4)) ||
         !aligned(workspace, 256))
         return PULSAR_ERR_ALIGNMENT;
-    // Parts of equally many key tiles over context and shard.  The shard goes in front of the last part's context
-    // keys, or is a part of its own where the parts before it already hold the whole context.  (As a part of its own
-    // in any case it made 152 work items of 144 for 148 SMs at 8 KV heads and 18 parts.)
     const int64_t L_ctx = static_cast<int64_t>(B) * block_size;
-    const int64_t ctx_tiles = (L_ctx + kTileN - 1) / kTileN, gen_tiles = (static_cast<int64_t>(gen_len) + n_new + kTileN - 1) / kTileN;
-    const int64_t part_tiles = (ctx_tiles + gen_tiles + n_splits - 1) / n_splits;
-    const int64_t ctx_parts = (ctx_tiles + part_tiles - 1) / part_tiles;
-    const bool own_part = ctx_tiles - (ctx_parts - 1) * part_tiles + gen_tiles > part_tiles;
-    const int n_parts = static_cast<int>(ctx_parts + (own_part ? 1 : 0));       // at most n_splits
+    const GenerateCut cut = cut_generate(L_ctx, static_cast<int64_t>(gen_len) + n_new,
+                                         (static_cast<int64_t>(n_new) * (Hq / Hkv) + 2 * kTileM - 1) / (2 * kTileM) * Hkv, n_splits);
+    const int n_parts = cut.n_parts;
     const bool quad = phase2_quad(n_new, Hq / Hkv);
     const int copies = quad ? 4 : 1;
     const size_t po_bytes = round_up(static_cast<size_t>(n_parts) * copies * n_new * Hq * d * 4, 256);
@@ -1677,9 +1716,11 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     a.Hq = Hq;
     a.g = g;
     a.pack_shift = log2_of(g);
-    a.split_len = static_cast<int>(part_tiles * kTileN);
+    a.split_len = static_cast<int>(cut.split_len);
+    a.ctx_part0 = cut.shard_apart ? 1 : 0;
     a.kv_len = static_cast<int>(L);
-    a.gen_part = n_parts - 1;
+    a.gen_part = cut.shard_apart ? 0 : n_parts - 1;
+    a.tile_max = cut.lengthened ? 1 : 0;
     a.gen_len = gen_len;
     a.gen_total = gen_len + n_new;
     a.quad = quad ? 1 : 0;

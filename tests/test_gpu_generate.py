@@ -141,3 +141,33 @@ def test_shard_beside_the_last_part_of_the_context(L, gen_len, n_splits, n_new):
     check_attention(O, LSE, Oref, Lref, f"L={L} gen_len={gen_len} parts={n_splits} n_new={n_new}")
     for got, want in ((Kg_d, Kg_o), (Vg_d, Vg_o)):             # the rows beyond the new ones stay as they were
         np.testing.assert_array_equal(got.cpu().view(torch.int16).numpy().view(np.uint16), want)
+
+
+@pytest.mark.parametrize("L,n_new,gen_len,Hq,Hkv", [(6001, 1, 33, 8, 2), (4416, 1, 58, 16, 4), (3271, 1, 642, 8, 2),
+                                                    (6314, 1, 163, 16, 2), (4416, 12, 77, 8, 2), (2500, 64, 200, 16, 4)])
+def test_parts_longer_than_the_contexts_cost_no_accuracy(L, n_new, gen_len, Hq, Hkv):
+    """Where context and shard are cut together the parts are longer than n_splits parts of the context alone (two key tiles
+    instead of one here).  P's rounding error is smallest in short parts (the largest probability of a part's first
+    key tile is exactly 1): formed with a maximum that lags behind, P is 8-10 % further from float64 with two tiles
+    (4-5 % with more than 32 query rows, two estimates of 16,000 outputs or more, each good to 1 %)."""
+    d, dev = 128, DEV
+    tiles = lambda n: (n + 127) // 128
+    n_splits = binding.phase2_choose_splits(n_new, 1, L, Hq, Hkv, d)
+    assert n_splits == tiles(L)
+    gen = torch.Generator(device=dev).manual_seed(L)
+    rnd = lambda n, h: torch.randn(n, h, d, generator=gen, device=dev, dtype=torch.bfloat16)
+    err = torch.zeros(2, dtype=torch.float64, device=dev)
+    for _ in range(max(4, 16 // n_new)):
+        K, V, Kg, Vg = rnd(L, Hkv), rnd(L, Hkv), rnd(gen_len + n_new, Hkv), rnd(gen_len + n_new, Hkv)
+        Q, Kn, Vn = rnd(n_new, Hq), rnd(n_new, Hkv), rnd(n_new, Hkv)
+        O, _ = binding.pulsar_phase2_generate_step(Q, Kn, Vn, K, V, 1, L, Kg, Vg, gen_len)
+        Kc, Vc = torch.cat([K, Kg]), torch.cat([V, Vg])          # the shard has its new rows by now
+        n = Kc.shape[0]
+        O2, _ = binding.pulsar_phase2_attn(Q, Kc, Vc, 1, n, n_splits=tiles(n))
+        s = torch.einsum("nhgd,mhd->nhgm", Q.view(n_new, Hkv, Hq // Hkv, d).double(), Kc.double()) / d ** 0.5
+        later = torch.arange(n, device=dev) > L + gen_len + torch.arange(n_new, device=dev)[:, None]
+        ref = lambda s: torch.einsum("nhgm,mhd->nhgd", s.softmax(-1), Vc.double()).reshape(n_new, Hq, d)
+        refs = ref(s.masked_fill(later[:, None, None], float("-inf"))), ref(s)
+        err += torch.stack([(x.double() - r).square().sum() for x, r in zip((O, O2), refs)])
+    a, b = err.sqrt().tolist()
+    assert a <= 1.025 * b, (a, b)
