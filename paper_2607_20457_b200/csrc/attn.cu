@@ -1014,6 +1014,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     fast = !__any_sync(0xffffffffu, !(s1 <= kPieceSumBound) || m2 * a.scale_log2 > m_used + kRescaleThreshold);
                 }
                 if (!fast) {
+                    tmem_wait_st();          // stores to the same columns have no order among themselves
                     const float m_tile = row_max128(r) * a.scale_log2;
                     const float m_new = next_max(m_tile, m_used, l_run, tile_max);
                     if (__any_sync(0xffffffffu, m_new != m_used)) {

@@ -255,3 +255,25 @@ def test_merge_at_the_edges_of_its_splits(J, rows, d):
     assert (lse[~empty] - l[~empty]).abs().max().item() <= 5e-6 if (~empty).any() else True
     O, _ = binding.pulsar_lse_merge(pO, pL)
     assert torch.equal(O, out.bfloat16())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("nq", [20, 40])                     # 80 query rows per KV head: one query tile; 160: two
+@pytest.mark.parametrize("where", ["first piece", "second piece"])
+def test_running_maximum_moves_inside_a_key_tile_of_a_part(where, nq, d):
+    """The first 96 keys' P is formed with the maximum of earlier key tiles and written a second time, over the first, when
+    one key of the tile lies far above it: with the old P left in place an output would be off by powers of two."""
+    w = W.shrink(W.CONFIGS["tiny"], L=4096, block_size=1024, Hq=8, Hkv=2, d=d, nq=nq)
+    _, K, V = W.qkv(w, seed=43)
+    Kf = K.float()
+    for j, t in enumerate(range(1, 32, 3)):
+        Kf[128 * t + (17 if where == "first piece" else 101) + j] *= 5.0 + 3.0 * (j % 6)
+    Kf = Kf.bfloat16()
+    Qq = W.phase2_query(w)
+    Oref, Lref = oracle.phase2_attn(Qq, Kf, V, 1, w.L)
+    args = Qq.to(DEV), Kf.to(DEV), V.to(DEV), 1, w.L
+    for n_splits in (1, 3, 0):
+        O, LSE = binding.pulsar_phase2_attn(*args, n_splits=n_splits)
+        check_attention(O, LSE, Oref, Lref, f"{where} nq={nq} d={d} parts={n_splits}")
+        again = binding.pulsar_phase2_attn(*args, n_splits=n_splits)
+        assert torch.equal(O, again[0]) and torch.equal(LSE, again[1])
