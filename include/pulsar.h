@@ -431,7 +431,8 @@ int32_t pulsar_phase2_generate_step(const uint16_t *Qnew, const uint16_t *Knew, 
 /* ------------------------------------------------------------------------------------------
  * Online-softmax merge (Appendix H, Eq. 12-13), in its order-free closed form:
  *   l = m + ln sum_j e^{l_j - m} (m = max_j l_j),  O = sum_j e^{l_j - l} A_j.
- * A part with l_j = -inf has weight 0.  Also the entry point for merging partials gathered
+ * A part with l_j = -inf has weight 0 (undefined values in it still make the result undefined, unless
+ * all parts of the row are empty: then it is 0).  Also the entry point for merging partials gathered
  * from several GPUs.
  *
  *   part_O   in  [n_parts, rows, d] float32     part_LSE in [n_parts, rows] float32

@@ -98,20 +98,19 @@ lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict_
         float m_new = m;
 #pragma unroll
         for (int i = 0; i < kInFlight; ++i) m_new = fmaxf(m_new, l[i]);
-        if (m_new > -INFINITY) {
-            const float keep = (m == -INFINITY) ? 0.f : __expf(m - m_new);
-            denom *= keep;
+        // (A part without keys, l = -inf, weighs nothing, but an undefined row in it stays undefined in the result.)
+        const float keep = (m == -INFINITY) ? 0.f : __expf(m - m_new);
+        denom *= keep;
 #pragma unroll
-            for (int k = 0; k < kVec; ++k) acc[k] *= keep;
+        for (int k = 0; k < kVec; ++k) acc[k] *= keep;
 #pragma unroll
-            for (int i = 0; i < kInFlight; ++i) {
-                const float w = (l[i] == -INFINITY) ? 0.f : __expf(l[i] - m_new);
-                denom += w;
+        for (int i = 0; i < kInFlight; ++i) {
+            const float w = (l[i] == -INFINITY) ? 0.f : __expf(l[i] - m_new);
+            denom += w;
 #pragma unroll
-                for (int k = 0; k < kVec; ++k) acc[k] += w * o[i][k];
-            }
-            m = m_new;
+            for (int k = 0; k < kVec; ++k) acc[k] += w * o[i][k];
         }
+        m = m_new;
     }
     if (kWarps > 1) {
         __shared__ float s_m[kWarps], s_denom[kWarps], s_acc[kWarps][kD];
@@ -138,11 +137,9 @@ lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict_
             }
         }
     }
-    if (m > -INFINITY) {
-        const float inv = 1.f / denom;
+    const float inv = 1.f / denom;
 #pragma unroll
-        for (int k = 0; k < kVec; ++k) acc[k] *= inv;
-    }
+    for (int k = 0; k < kVec; ++k) acc[k] = (m > -INFINITY) ? acc[k] * inv : 0.f;
     const int64_t at = row * kD + lane * kVec;
     if (kF32) {
         float* dst = static_cast<float*>(O_) + at;

@@ -277,3 +277,23 @@ def test_running_maximum_moves_inside_a_key_tile_of_a_part(where, nq, d):
         check_attention(O, LSE, Oref, Lref, f"{where} nq={nq} d={d} parts={n_splits}")
         again = binding.pulsar_phase2_attn(*args, n_splits=n_splits)
         assert torch.equal(O, again[0]) and torch.equal(LSE, again[1])
+
+
+@pytest.mark.parametrize("d", [64, 128, 192])
+@pytest.mark.parametrize("J,rows", [(4, 7), (16, 5), (32, 5), (64, 3), (130, 2), (300, 1), (20, 20000)])
+def test_undefined_rows_of_empty_parts_show_in_the_merge(J, rows, d):
+    """A key that is not a number leaves its part with l = -inf and an undefined row.  The merged row is undefined too,
+    whichever warp or round the part falls to and whatever else falls there; only a row without any key is 0."""
+    gen = torch.Generator(device=DEV).manual_seed(J + rows)
+    j = torch.arange(J, device=DEV)
+    lost = [j % s == s - 1 for s in (2, 4, 8, 16) if s <= J] + [j < 8 * s for s in (1, 2, 4, 16) if 8 * s < J]
+    for bad in lost:
+        pO = torch.randn(J, rows, d, generator=gen, device=DEV)
+        pL = torch.randn(J, rows, generator=gen, device=DEV)
+        pO[bad], pL[bad] = float("nan"), float("-inf")
+        pL[:, rows // 2] = float("-inf")
+        out, lse = torch.empty(rows, d, device=DEV), torch.empty(rows, device=DEV)
+        binding.pulsar_lse_merge_strided(pO, pL, J, rows * d, rows, rows, d, out, lse)
+        empty = torch.isneginf(pL).all(0)
+        assert out[~empty].isnan().all() and (out[empty] == 0).all()
+        assert torch.equal(torch.isneginf(lse), empty) and not lse.isnan().any()
