@@ -1,7 +1,7 @@
 // Online-softmax merge of attention partials (Appendix H, Eq. 12-13) in closed form:
 //   l = m + ln sum_j exp(l_j - m),  O = sum_j exp(l_j - l) A_j,  m = max_j l_j.
-// For the head sizes of the attention kernels a warp owns an output row and its parts are spread over the warps of
-// a CTA; other row sizes take one thread per four consecutive output elements.
+// For the head sizes of the attention kernels and few rows a warp owns an output row and its parts are spread over
+// the warps of a CTA; otherwise one thread takes four consecutive output elements (merge_warps).
 #include "common.cuh"
 
 namespace pulsar {
@@ -14,6 +14,7 @@ lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ par
                  int64_t stride_O, int64_t stride_L, int64_t rows, int d, void* __restrict__ O_,
                  float* __restrict__ LSE) {
     grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
+    grid_launch_dependents();
     const int vec_per_row = d >> 2;
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= rows * vec_per_row) return;
@@ -56,7 +57,7 @@ lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ par
 // the row pieces, which do not depend on them) before it uses any, and there are enough warps per row that one or
 // two such rounds cover all parts.  The order of the sums is fixed, so the result is reproducible.
 // Measured tail from the end of the attention launch to the end of the merge: 384 rows of 19 parts
-// 8.5 us with one thread per four outputs, 3.4 us with this form; 1600 rows of 18 parts 10 -> 8 us.
+// 8.5 us with one thread per four outputs, 3.4 us with this form.
 template <bool kF32, int kVec, int kWarps, int kRows>
 __global__ void __launch_bounds__(32 * kWarps * kRows)
 lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict__ part_LSE, int n_parts,
@@ -214,14 +215,26 @@ auto merge_rows_kernel(int warps) {
                         : lse_merge_rows_kernel<kF32, kVec, 1, 8>;
 }
 
+// Warps that share an output row; 0: one thread per four outputs (lse_merge_kernel).  That form loads eight parts at a
+// time too, but one group after the other (3 us and 0.11 us more per part, a remainder of the groups of eight part by
+// part), and it streams many rows better, since a row needs no CTA or barrier of its own.  So: as many warps as
+// leave each of them one round of eight parts, while the rows' warps fit the chip at once (2048 warps with several warps a
+// row, 1600 rows in all); beyond that four or two warps for more than 64 parts, one thread per four outputs otherwise.
+// Measured in us, rows / thread form, d = 64: 2 parts of 65536 rows 26 / 10, 9 of 16384 11.8 / 5.9, 18 of 1024 3.5 / 4.0,
+// 18 of 4096 5.7 / 4.3, 48 of 512 3.7 / 7.1, 96 of 4096 20.9 / 32; d = 128: 33 of 4096 14 / 7.1, 96 of 6144 64 / 53.
+int merge_warps(int32_t n_parts, int64_t rows, int32_t d) {
+    if (n_parts <= 8) return n_parts > 4 && (rows * d <= 4096 * 64 || (n_parts < 8 && d == 128)) ? 1 : 0;
+    if (rows > 1600) return n_parts <= 64 ? 0 : rows <= 4096 ? 4 : d == 64 ? 2 : 0;
+    int warps = n_parts > 64 ? 16 : n_parts > 32 ? 8 : n_parts > 16 ? 4 : 2;
+    while (warps > 2 && rows * warps > 2048) warps /= 2;
+    return warps;
+}
+
 int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t stride_O, int64_t stride_L,
                      int64_t rows, int32_t d, void* O, bool f32, float* LSE, cudaStream_t stream) {
     if (rows == 0) return PULSAR_OK;
-    if (d == 64 || d == 128) {
-        // Warps per row: as many as leave a warp four to eight parts (one round of loads), while all of them fit the
-        // chip about once (148 SMs of 64 warps); with more rows than that the rows themselves fill it.
-        int warps = n_parts > 64 ? 16 : n_parts > 32 ? 8 : n_parts > 16 ? 4 : n_parts > 8 ? 2 : 1;
-        while (warps > 1 && rows * warps > 2 * 148 * 64) warps /= 2;
+    const int warps = (d == 64 || d == 128) ? merge_warps(n_parts, rows, d) : 0;
+    if (warps > 0) {
         const int64_t blocks = warps == 1 ? (rows + 7) / 8 : rows;
         if (blocks > 0x7fffffffll) return PULSAR_ERR_SHAPE;
         auto kernel = d == 128 ? (f32 ? merge_rows_kernel<true, 4>(warps) : merge_rows_kernel<false, 4>(warps))

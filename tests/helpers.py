@@ -35,3 +35,15 @@ def check_attention(O_gpu, LSE_gpu, O_ref, LSE_ref, what=""):
     assert worst <= 1.0, msg + f" (worst element at {worst:.2f} of its bound)"
     assert rel <= TOL_O_REL_L2, msg
     return msg
+
+
+def kernel_names(fn):
+    """Names (with their template arguments) of the kernels that ``fn`` launches, in order."""
+    from torch.profiler import ProfilerActivity, profile
+    fn()                                             # a first call outside: module loading is not part of the record
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        fn()
+        torch.cuda.synchronize()
+    ev = [e for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA]
+    return [e.name for e in sorted(ev, key=lambda e: e.time_range.start)]

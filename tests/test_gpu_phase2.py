@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import check_attention, TOL_LSE_ABS
+from helpers import check_attention, kernel_names, TOL_LSE_ABS
 from paper_2607_20457_b200 import binding, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -297,3 +297,22 @@ def test_undefined_rows_of_empty_parts_show_in_the_merge(J, rows, d):
         empty = torch.isneginf(pL).all(0)
         assert out[~empty].isnan().all() and (out[empty] == 0).all()
         assert torch.equal(torch.isneginf(lse), empty) and not lse.isnan().any()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("J,rows,warps", [(2, 65536, 0), (4, 7, 0), (5, 2048, 1), (8, 2048, 1), (8, 4097, 0), (9, 1600, 2),
+                                          (9, 1601, 0), (18, 512, 4), (18, 513, 2), (33, 256, 8), (64, 1601, 0), (65, 128, 16),
+                                          (65, 129, 8), (65, 1601, 4), (65, 4097, None)])
+def test_merge_on_both_sides_of_its_rule(J, rows, warps, d):
+    """Warps per row for few rows, one thread per four outputs for many (9 parts of 16384 rows: 5.9 us against 11.8)."""
+    if warps is None:
+        warps = 2 if d == 64 else 0
+    pO, pL = torch.zeros(J, rows, d, device=DEV), torch.zeros(J, rows, device=DEV)
+    names = kernel_names(lambda: binding.pulsar_lse_merge(pO, pL))
+    got = [n for n in names if "lse_merge" in n]
+    assert len(got) == 1
+    if warps:
+        assert f"lse_merge_rows_kernel<false, {d // 32}, {warps}, " in got[0], got
+    else:
+        assert "lse_merge_kernel<false>" in got[0], got
+    test_merge_at_the_edges_of_its_splits(J, rows, d)
