@@ -215,18 +215,21 @@ auto merge_rows_kernel(int warps) {
                         : lse_merge_rows_kernel<kF32, kVec, 1, 8>;
 }
 
-// Warps that share an output row; 0: one thread per four outputs (lse_merge_kernel).  That form loads eight parts at a
-// time too, but one group after the other (3 us and 0.11 us more per part, a remainder of the groups of eight part by
-// part), and it streams many rows better, since a row needs no CTA or barrier of its own.  So: as many warps as
-// leave each of them one round of eight parts, while the rows' warps fit the chip at once (2048 warps with several warps a
-// row, 1600 rows in all); beyond that four or two warps for more than 64 parts, one thread per four outputs otherwise.
-// Measured in us, rows / thread form, d = 64: 2 parts of 65536 rows 26 / 10, 9 of 16384 11.8 / 5.9, 18 of 1024 3.5 / 4.0,
-// 18 of 4096 5.7 / 4.3, 48 of 512 3.7 / 7.1, 96 of 4096 20.9 / 32; d = 128: 33 of 4096 14 / 7.1, 96 of 6144 64 / 53.
+// Warps that share an output row; 0: one thread per four outputs (lse_merge_kernel).  That form reads the l_j before
+// it can use an output row, and eight parts at a time: 6 us of latency for 18 parts fresh from another kernel, 10 for 48 (a
+// remainder of the eights part by part).  Rows over warps take a third of that, but every row costs its warps: with several
+// a row up to 3200 warps in all, with one up to 3200 rows; from 48 parts on one warp a row is the better form for any
+// number of rows (more than two if there are more than 64 parts and few rows).  Measured behind a kernel that writes the parts, us, rows
+// form / thread form, d = 128: 18 parts of 512 rows 3.1 / 5.7, of 1600 4.8 / 6.0, of 2048 6.0 / 6.1, of 4096 8.0 / 7.1;
+// 33 of 512 4.0 / 8.4, of 4096 14.7 / 15.9; 4 of 1024 2.9 / 3.6, of 8192 5.5 / 6.2; d = 64: 9 of 4096 4.5 / 3.8, of 16384
+// 13.4 / 8.4; 96 of 4096 19 / 40; alone and in cache the thread form gains earlier (9 of 4096 4.3 / 3.2).
 int merge_warps(int32_t n_parts, int64_t rows, int32_t d) {
-    if (n_parts <= 8) return n_parts > 4 && (rows * d <= 4096 * 64 || (n_parts < 8 && d == 128)) ? 1 : 0;
-    if (rows > 1600) return n_parts <= 64 ? 0 : rows <= 4096 ? 4 : d == 64 ? 2 : 0;
-    int warps = n_parts > 64 ? 16 : n_parts > 32 ? 8 : n_parts > 16 ? 4 : 2;
-    while (warps > 2 && rows * warps > 2048) warps /= 2;
+    constexpr int64_t kMost = 3200;
+    if (n_parts > 4 && n_parts < 8 && (d == 128 || rows <= 8192)) return 1;     // the thread form's eights are all remainder
+    if (n_parts == 1 || (n_parts < 48 && rows > kMost)) return 0;
+    if (rows > kMost) return 1;
+    int warps = n_parts > 64 ? 16 : n_parts > 32 ? 8 : n_parts > 16 ? 4 : n_parts > 8 ? 2 : 1;
+    while (warps > (n_parts > 64 ? 2 : 1) && rows * warps > kMost) warps /= 2;
     return warps;
 }
 

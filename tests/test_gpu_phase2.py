@@ -300,13 +300,12 @@ def test_undefined_rows_of_empty_parts_show_in_the_merge(J, rows, d):
 
 
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("J,rows,warps", [(2, 65536, 0), (4, 7, 0), (5, 2048, 1), (8, 2048, 1), (8, 4097, 0), (9, 1600, 2),
-                                          (9, 1601, 0), (18, 512, 4), (18, 513, 2), (33, 256, 8), (64, 1601, 0), (65, 128, 16),
-                                          (65, 129, 8), (65, 1601, 4), (65, 4097, None)])
+@pytest.mark.parametrize("J,rows,warps", [(1, 300, 0), (2, 65536, 0), (4, 3200, 1), (4, 3201, 0), (5, 8192, 1), (8, 3201, 0),
+                                          (9, 1600, 2), (9, 1601, 1), (9, 3201, 0), (18, 800, 4), (18, 801, 2), (33, 400, 8),
+                                          (33, 401, 4), (47, 3201, 0), (48, 3201, 1), (65, 200, 16), (65, 201, 8),
+                                          (65, 3200, 2), (65, 3201, 1)])
 def test_merge_on_both_sides_of_its_rule(J, rows, warps, d):
-    """Warps per row for few rows, one thread per four outputs for many (9 parts of 16384 rows: 5.9 us against 11.8)."""
-    if warps is None:
-        warps = 2 if d == 64 else 0
+    """Warps per row for few rows, one thread per four outputs for many."""
     pO, pL = torch.zeros(J, rows, d, device=DEV), torch.zeros(J, rows, device=DEV)
     names = kernel_names(lambda: binding.pulsar_lse_merge(pO, pL))
     got = [n for n in names if "lse_merge" in n]
