@@ -65,8 +65,8 @@ struct AttnArgs {
     int gen_part;          // phase 2: the part that has the generation shard in front of its context keys (if any)
     int gen_len;           // phase 2: rows of the generation shard that precede the new tokens
     int gen_total;         // phase 2: gen_len + new tokens (0 = no generation shard)
-    const uint4* Knew;     // phase 2, one query tile per KV head: KV(q) of the new tokens, appended to the generation shard by
-    const uint4* Vnew;     // the CTA that reads the head's part of it (null: appended by a launch of its own)
+    const uint4* Knew;     // phase 2, one query tile per KV head and few new tokens: their KV(q), appended to the generation
+    const uint4* Vnew;     // shard by the CTA that reads the head's part of it (null: appended by a launch of its own)
     uint4* Kgen;
     uint4* Vgen;
     int quad;              // phase 2, at most 32 query rows per KV head: the rows are replicated into the four
@@ -141,7 +141,7 @@ gather_prefix_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, c
 }
 
 // KV(q) of the new tokens appended to the generation shard: one launch for both tensors, for calls with more than
-// one query tile per KV head (with one, the attention kernel appends: append_head).
+// one query tile per KV head or with many new tokens (otherwise the attention kernel appends: append_head).
 __global__ void __launch_bounds__(256)
 append_kv_kernel(const uint4* __restrict__ Knew, const uint4* __restrict__ Vnew, uint4* __restrict__ Kdst,
                  uint4* __restrict__ Vdst, int vecs) {
@@ -401,16 +401,38 @@ __device__ __forceinline__ void decode_item(const AttnArgs& a, const Table& vt, 
 // KV(q) of the new tokens of one KV head appended to the generation shard by the warp that is about to load the
 // head's shard rows through TMA: written with plain stores, made visible to the async proxy, then loaded.  No other CTA
 // of the launch touches the head's rows.  (As a launch of its own the append cost 2.8 us on the host and 2-3 us on the
-// device of every decoding step.)
+// device of every decoding step.)  The warp's loads are latency, about 0.8 us a round: four vectors of K and of V are
+// under way per lane, and rows that take more than four such rounds (kAppendVecs) come from a launch of their own (64
+// tokens of 8 heads with d = 128 at 65,536: 83 us with one vector at a time, 50 us with that launch; 32 tokens 19.8 -> 15.0).
+constexpr int kAppendVecs = 512;                              // 16-byte vectors of a head's new rows: 32 tokens with d = 128
+
 __device__ __forceinline__ void append_head(const AttnArgs& a, int kvh, int d, int lane) {
     const int vecs = d / 8;                                   // 16-byte vectors of a head's row
     const int n = (a.gen_total - a.gen_len) * vecs;
-    for (int i = lane; i < n; i += 32) {
-        const int u = i / vecs, v = i - u * vecs;
-        const size_t src = (static_cast<size_t>(u) * a.Hkv + kvh) * vecs + v;
-        const size_t dst = (static_cast<size_t>(a.gen_len + u) * a.Hkv + kvh) * vecs + v;
-        a.Kgen[dst] = a.Knew[src];
-        a.Vgen[dst] = a.Vnew[src];
+    const auto at = [&](int i, int row0) {
+        const int u = i / vecs;
+        return (static_cast<size_t>(row0 + u) * a.Hkv + kvh) * vecs + (i - u * vecs);
+    };
+    int i0 = lane;
+    for (; n > 32 && i0 < n; i0 += 128) {
+        uint4 k[4], v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i0 + 32 * j < n) {
+                k[j] = a.Knew[at(i0 + 32 * j, 0)];
+                v[j] = a.Vnew[at(i0 + 32 * j, 0)];
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (i0 + 32 * j < n) {
+                a.Kgen[at(i0 + 32 * j, a.gen_len)] = k[j];
+                a.Vgen[at(i0 + 32 * j, a.gen_len)] = v[j];
+            }
+    }
+    if (i0 < n) {                                             // a row or two: nothing to overlap
+        const uint4 k = a.Knew[at(i0, 0)], v = a.Vnew[at(i0, 0)];
+        a.Kgen[at(i0, a.gen_len)] = k;
+        a.Vgen[at(i0, a.gen_len)] = v;
     }
     fence_proxy_async_global();
     __syncwarp();
@@ -1736,7 +1758,7 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     a.Hkv = Hkv;
     a.single = row_tiles == 1 ? 1 : 0;               // includes every decode shape (quad)
     // KV(q) is appended to the generation shard first (Algorithm 1 line 15)
-    if (a.single) {
+    if (a.single && n_new * (d / 8) <= kAppendVecs) {
         a.Knew = reinterpret_cast<const uint4*>(Knew);
         a.Vnew = reinterpret_cast<const uint4*>(Vnew);
         a.Kgen = reinterpret_cast<uint4*>(Kgen);

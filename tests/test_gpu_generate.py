@@ -171,3 +171,23 @@ def test_parts_longer_than_the_contexts_cost_no_accuracy(L, n_new, gen_len, Hq, 
         err += torch.stack([(x.double() - r).square().sum() for x, r in zip((O, O2), refs)])
     a, b = err.sqrt().tolist()
     assert a <= 1.025 * b, (a, b)
+
+
+@pytest.mark.parametrize("d,n_new,launches", [(128, 1, 2), (128, 2, 2), (128, 3, 2), (128, 17, 2), (128, 32, 2), (128, 33, 3),
+                                              (128, 100, 3), (64, 4, 2), (64, 5, 2), (64, 64, 2), (64, 65, 3)])
+def test_rows_are_appended_by_the_attention_kernel_or_before_it(d, n_new, launches):
+    """One warp appends the new rows of its KV head, 512 vectors of 16 bytes at most; more come from a launch of their own."""
+    L, gen_len, H = 700, 61, 2
+    gen = torch.Generator().manual_seed(d + n_new)
+    rnd = lambda n: torch.randn(n, H, d, generator=gen).to(torch.bfloat16)
+    K, V, Kg, Vg, Qn, Kn, Vn = rnd(L), rnd(L), rnd(gen_len + n_new + 2), rnd(gen_len + n_new + 2), rnd(n_new), rnd(n_new), rnd(n_new)
+    Kg_d, Vg_d = Kg.to(DEV), Vg.to(DEV)
+    args = [t.to(DEV) for t in (Qn, Kn, Vn, K, V)]
+    before = binding.launch_count()
+    O, LSE = binding.pulsar_phase2_generate_step(*args, 1, L, Kg_d, Vg_d, gen_len)
+    assert binding.launch_count() - before == launches
+    Kg_o, Vg_o = (x.view(torch.int16).numpy().view(np.uint16).copy() for x in (Kg, Vg))
+    Oref, Lref = oracle.generate_step(Qn, Kn, Vn, K, V, Kg_o, Vg_o, gen_len)
+    check_attention(O, LSE, Oref, Lref, f"d={d} n_new={n_new}")
+    for got, want in ((Kg_d, Kg_o), (Vg_d, Vg_o)):
+        np.testing.assert_array_equal(got.cpu().view(torch.int16).numpy().view(np.uint16), want)
