@@ -18,6 +18,7 @@
 //   Assembled inputs (Algorithm 1 l.8 as the paper runs it): sequences of any lengths packed back
 //            to back, every token a query, plain causal attention inside each.
 #include <algorithm>
+#include <functional>
 #include <type_traits>
 
 #include <cuda.h>
@@ -1253,11 +1254,57 @@ int causal_pack_shift(int32_t Hq, int32_t Hkv, int32_t d) {
     return d == 64 && g <= 16 && (g & (g - 1)) == 0 ? log2_of(g) : 0;
 }
 
-// Causal attention with so few pairs of query tiles that they would not fill the SMs once takes work items of one
-// tile: twice the items, and a key tile costs the chain of one tile (about 1.2 us) instead of two interleaved ones
-// (1.8 us).  With more items than that the pair is the better unit (0.9 us per tile and key tile).
-// 4096 tokens in 4 blocks of 4 heads, d = 64 (64 pairs, up to 10 key tiles): 24 -> 17 us.
-bool causal_single(int64_t pair_items) { return pair_items <= sm_count(); }
+// Causal attention with few items takes work items of one query tile instead of two: twice the items, and a key tile costs
+// the chain of one tile (0.88 us with d = 64, 0.91 with d = 128; an item 2.2 and 2.8 us more) instead of two interleaved
+// ones (1.39 and 1.51 us, 3.0 and 3.4 us).  While every tile has an SM of its own that is the shorter time, and with more pairs than
+// SMs the pair is the better unit.  Between the two, tiles that cost alike are walked two after the other and lose
+// (one block of 1024 of 32 heads, d = 64, behind 8192 prefix rows: 130 us against 110), tiles that differ are dealt out
+// evenly and win (8 blocks of 512 of 8 heads, prefix growing to 7168 rows: 61 us against 95).  So both are laid out on the
+// SMs in the order in which the items are drawn, and the shorter time decides.  Over 270 shapes that is the better
+// form, or within 4 % of it.
+// A run is a block or a sequence: its prefix rows and its own; in the order in which the items are drawn.
+struct CausalRun {
+    int64_t prefix;
+    int len;
+};
+constexpr int kMaxCausalRuns = 512;             // more runs than that are more pairs than SMs
+
+bool causal_single(const CausalRun* runs, int n_runs, int64_t heads, int tile_tokens, int32_t d) {
+    const int sms = sm_count();
+    struct { int64_t tile, item; } const cost[2] = {{d == 64 ? 882 : 906, d == 64 ? 2185 : 2761},
+                                                    {d == 64 ? 1392 : 1513, d == 64 ? 2986 : 3390}};     // ns, of one tile and of a pair
+    const auto items = [&](int64_t tokens) {
+        int64_t n = 0;
+        for (int r = 0; r < n_runs; ++r) n += (runs[r].len + tokens - 1) / tokens * heads;
+        return n;
+    };
+    if (items(tile_tokens) <= sms) return true;
+    if (items(2 * tile_tokens) > sms || sms > 1024) return false;
+    int64_t time[2];
+    for (int per_item = 1; per_item <= 2; ++per_item) {
+        const int tokens = per_item * tile_tokens;
+        int64_t done[1024];                     // when each SM is free again, the earliest first (a heap)
+        int n = 0;
+        for (int r = 0; r < n_runs; ++r)
+            for (int i = (runs[r].len + tokens - 1) / tokens - 1; i >= 0; --i) {
+                const int rows = std::min(runs[r].len, (i + 1) * tokens);
+                const int64_t t = ((runs[r].prefix + kTileN - 1) / kTileN + (rows + kTileN - 1) / kTileN) * cost[per_item - 1].tile +
+                                  cost[per_item - 1].item;
+                for (int64_t h = 0; h < heads; ++h) {
+                    if (n < sms) {
+                        done[n++] = t;
+                        if (n == sms) std::make_heap(done, done + n, std::greater<int64_t>());
+                        continue;
+                    }
+                    std::pop_heap(done, done + n, std::greater<int64_t>());
+                    done[n - 1] += t;
+                    std::push_heap(done, done + n, std::greater<int64_t>());
+                }
+            }
+        time[per_item - 1] = *std::max_element(done, done + n);
+    }
+    return time[0] < time[1];
+}
 
 // whole_only: the entry point takes only sequences made of whole blocks.
 int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block_size, int32_t prefix_total,
@@ -1275,16 +1322,21 @@ int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block
     p.total = 2 * p.pref_bytes + 256;                        // gathered prefix K, V and the work counter
     p.pack_shift = causal_pack_shift(Hq, Hkv, d);
     const int64_t heads = p.pack_shift ? Hkv : Hq;
-    int64_t items = 0;
-    for (int per_item = 2; per_item >= 1; --per_item) {
-        const int64_t tokens = static_cast<int64_t>(per_item) * (kTileM >> p.pack_shift);
-        p.single = per_item == 1 ? 1 : 0;
-        p.items_block = static_cast<int>((block_size + tokens - 1) / tokens);
-        p.items_last = static_cast<int>((p.last_len + tokens - 1) / tokens);
-        items = ((B - 1) * p.items_block + p.items_last) * heads;
-        if (items >= (1ll << 31)) return PULSAR_ERR_SHAPE;
-        if (per_item == 2 && !causal_single(items)) break;
-    }
+    // How long each block's prefix is stands on the device.  It is taken to grow evenly to prefix_total, as in a whole
+    // context and as blocks are dealt to GPUs in turn or in zigzag; a single block is taken to see all of it.  (Several
+    // blocks that all see a long prefix, the last GPU of a context cut into runs of blocks, would do 1.1-1.2 times
+    // better with pairs; pairs would cost the others up to 1.6 times.)
+    const int tile_tokens = kTileM >> p.pack_shift;
+    CausalRun runs[kMaxCausalRuns];
+    if (B <= kMaxCausalRuns)
+        for (int64_t i = 0; i < B; ++i)
+            runs[i] = {B > 1 ? prefix_total * (B - 1 - i) / (B - 1) : prefix_total, i == 0 ? p.last_len : block_size};
+    p.single = B <= kMaxCausalRuns && causal_single(runs, static_cast<int>(B), heads, tile_tokens, d) ? 1 : 0;
+    const int64_t tokens = static_cast<int64_t>(p.single ? 1 : 2) * tile_tokens;
+    p.items_block = static_cast<int>((block_size + tokens - 1) / tokens);
+    p.items_last = static_cast<int>((p.last_len + tokens - 1) / tokens);
+    const int64_t items = ((B - 1) * p.items_block + p.items_last) * heads;
+    if (items >= (1ll << 31)) return PULSAR_ERR_SHAPE;
     p.n_items = static_cast<int>(items);
     return PULSAR_OK;
 }
@@ -1807,21 +1859,17 @@ extern "C" int32_t pulsar_causal_varlen_attn(const uint16_t* Q, const uint16_t* 
     vt.n_seq = n_seq;
     for (int j = 0; j <= n_seq; ++j) vt.start[j] = cu_seqlens_host[j];
     const int pack_shift = causal_pack_shift(Hq, Hkv, d), heads = pack_shift ? Hkv : Hq;
+    const int tile_tokens = kTileM >> pack_shift;
+    CausalRun runs[kMaxVarlenSeqs];
+    for (int k = 0; k < n_seq; ++k) runs[k] = {0, vt.start[n_seq - k] - vt.start[n_seq - 1 - k]};
+    const int single = causal_single(runs, n_seq, heads, tile_tokens, d) ? 1 : 0, tokens = (single ? 1 : 2) * tile_tokens;
     int64_t pairs_total = 0;
-    int single = 0;
-    for (int per_item = 2; per_item >= 1; --per_item) {
-        const int tokens = per_item * (kTileM >> pack_shift);
-        pairs_total = 0;
-        for (int k = 0; k < n_seq; ++k) {
-            vt.pair_cum[k] = static_cast<int>(pairs_total);
-            const int len = vt.start[n_seq - k] - vt.start[n_seq - 1 - k];
-            pairs_total += (len + tokens - 1) / tokens;
-        }
-        vt.pair_cum[n_seq] = static_cast<int>(pairs_total);
-        if (pairs_total * heads >= (1ll << 31)) return PULSAR_ERR_SHAPE;
-        if (per_item == 2 && !causal_single(pairs_total * heads)) break;
-        single = per_item == 1 ? 1 : 0;
+    for (int k = 0; k < n_seq; ++k) {
+        vt.pair_cum[k] = static_cast<int>(pairs_total);
+        pairs_total += (static_cast<int64_t>(runs[k].len) + tokens - 1) / tokens;
     }
+    vt.pair_cum[n_seq] = static_cast<int>(pairs_total);
+    if (pairs_total * heads >= (1ll << 31)) return PULSAR_ERR_SHAPE;
 
     CUtensorMap tmQ, tmK, tmV;
     if (!make_map_3d(&tmQ, Q, total_rows, Hq, d, 1 << pack_shift, kTileM >> pack_shift) ||

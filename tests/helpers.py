@@ -42,7 +42,7 @@ def kernel_names(fn):
     from torch.profiler import ProfilerActivity, profile
     fn()                                             # a first call outside: module loading is not part of the record
     torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
         fn()
         torch.cuda.synchronize()
     ev = [e for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA]

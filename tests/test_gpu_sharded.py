@@ -8,7 +8,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import check_attention, to_dev_ids
+from helpers import check_attention, kernel_names, to_dev_ids
 from paper_2607_20457_b200 import binding, cost_model as cm, workloads as W
 from paper_2607_20457_b200.sharding import ShardLayout, ShardedContextEncoder
 
@@ -209,3 +209,52 @@ def test_phase1_sharded_at_the_128k_configuration_equals_the_unsharded_call():
     O1, LSE1, _, _ = binding.pulsar_phase1_attn(Q, K, V, w.block_size, sel["prefix_idx"], sel["prefix_len"])
     torch.cuda.synchronize()
     assert torch.equal(O, O1) and torch.equal(LSE, LSE1)
+
+
+def form_of(fn):
+    """Query tiles per work item (1 or 2) of the attention launch in ``fn``: the kernel's last template argument."""
+    names = [n for n in kernel_names(fn) if "attn_kernel" in n]
+    assert len(names) == 1, names
+    return 1 if ", true>" in names[0] else 2
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,block,Hq,prefix,form", [
+    (1, 1024, 32, 0, 1),          # 128 pairs, tiles that differ by up to a factor of eight
+    (1, 1024, 32, 8192, 2),       # the same behind a long prefix: all alike (d = 64: 110 us in pairs, 130 us in tiles)
+    (1, 512, 32, 8192, 1),        # 64 pairs: every tile has an SM of its own
+    (8, 512, 8, 7168, 1),         # a prefix that grows from block to block (d = 64: 61 us in tiles, 95 us in pairs)
+    (4, 1024, 32, 3072, 2),       # 512 pairs
+])
+def test_form_follows_the_time_that_the_items_take(B, block, Hq, prefix, form, d):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the shapes are those of 148 SMs")
+    Hkv = Hq // 4
+    gen = torch.Generator(device=DEV).manual_seed(B * block + prefix)
+    rnd = lambda n, h: torch.randn(n, h, d, generator=gen, device=DEV, dtype=torch.bfloat16)
+    L = B * block
+    Q, K, V = rnd(L, Hq), rnd(L, Hkv), rnd(L, Hkv)
+    Kp, Vp = (rnd(prefix, Hkv), rnd(prefix, Hkv)) if prefix else (None, None)
+    plen = torch.tensor([prefix * i // (B - 1) if B > 1 else prefix for i in range(B)], dtype=torch.int32, device=DEV)
+    O, LSE = binding.pulsar_phase1_attn_sharded(Q, K, V, block, Kp, Vp, plen)
+    assert form_of(lambda: binding.pulsar_phase1_attn_sharded(Q, K, V, block, Kp, Vp, plen)) == form
+    for i in (0, B - 1):
+        for h in (0, Hq - 1):
+            rows, n = slice(i * block, (i + 1) * block), int(plen[i])
+            k, v = K[rows, h // 4].double(), V[rows, h // 4].double()
+            if n:
+                k, v = torch.cat([Kp[:n, h // 4].double(), k]), torch.cat([Vp[:n, h // 4].double(), v])
+            x = Q[rows, h].double() @ k.T / d ** 0.5
+            x.masked_fill_(torch.arange(n + block, device=DEV) > n + torch.arange(block, device=DEV)[:, None], float("-inf"))
+            l = x.logsumexp(1)
+            check_attention(O[rows, h: h + 1], LSE[rows, h: h + 1], ((x - l[:, None]).exp() @ v)[:, None].cpu().numpy(),
+                            l[:, None].cpu().numpy(), f"block {i} head {h}")
+
+
+def test_form_of_assembled_inputs():
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the shapes are those of 148 SMs")
+    for n_seq, length, Hq, form in ((1, 4096, 8, 1), (4, 1024, 8, 2), (16, 300, 8, 2), (2, 1024, 8, 1)):
+        cu = [i * length for i in range(n_seq + 1)]
+        Q, K = (torch.zeros(cu[-1], h, 64, dtype=torch.bfloat16, device=DEV) for h in (Hq, Hq // 4))
+        assert form_of(lambda: binding.pulsar_causal_varlen_attn(Q, K, K, cu)) == form, (n_seq, length, Hq)
