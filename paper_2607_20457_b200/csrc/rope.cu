@@ -167,6 +167,16 @@ int32_t launch_rope(const uint16_t* X1, uint16_t* Y1, int32_t H1, const uint16_t
     const int64_t want = static_cast<int64_t>(sm_count()) * 4 * slots / rows;
     int groups = 1;
     while (2 * groups <= std::min<int64_t>(want, std::min(slots, H1 + H2))) groups *= 2;
+    // Many heads: a thread that walks all of them leaves a warp's rows a whole row apart, and the CTA's threads would come back
+    // to a line long after its other half.  Four threads a row keep the lines together: 16 heads x 16 or 32 heads with
+    // d < 64, and 32 heads of any size once the tensors no longer fit the L2, unless more than a tenth of the slots
+    // would idle (d = 192).  us, 32 + 8 heads unless noted, one / four threads: d = 16, 100,000 rows 89 / 49 (the persistent kernel
+    // 60), d = 32, 50,000 60 / 47 (53), d = 64, 20,000 47 / 41 (42), 64 + 8 x 64, 50,000 155 / 144 (148); below that size
+    // one is better: d = 64, 6000 rows 12.4 / 14.3.
+    const int heads = H1 + H2;
+    const bool past_l2 = 4 * rows * heads * d > 128000000;
+    if ((d == 16 && heads >= 16) || (heads >= 32 && (d < 64 || past_l2) && slots / 4 * 4 * 10 >= slots * 9))
+        groups = std::max(groups, 4);
     const int64_t ctas = (rows + slots / groups - 1) / (slots / groups);
     if (ctas > INT32_MAX) return PULSAR_ERR_SHAPE;
     auto kernel = groups > 1 ? rope_kernel<true> : rope_kernel<false>;

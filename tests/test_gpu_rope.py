@@ -7,7 +7,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import to_dev_ids
+from helpers import kernel_names, to_dev_ids
 from paper_2607_20457_b200 import binding, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -151,3 +151,18 @@ def test_position_ids_of_a_sequence_with_a_short_last_block():
             want += [i * w.block_size + r if mode == "sparse" else P + r for r in range(n)]
         pos = binding.pulsar_assemble_positions(sel["prefix_idx"], sel["prefix_len"], w.n_blocks, w.block_size, total, mode)
         assert pos.cpu().tolist() == want
+
+
+@pytest.mark.parametrize("rows,H,d", [(40001, 15, 16), (40001, 16, 16), (25001, 31, 32), (25001, 32, 32), (9601, 40, 64),
+                                      (13001, 40, 64), (4001, 40, 192), (12001, 33, 48)])
+def test_rope_of_many_heads(rows, H, d):
+    """From 32 heads on (16 with d = 16) four threads of a CTA share a row's vector positions, with d of 64 and more once the
+    tensors have outgrown the L2 (12,500 rows of 40 heads x 64); not with d = 192, where a fifth of the threads would idle."""
+    g = torch.Generator().manual_seed(rows + H)
+    pos = torch.randint(0, 131072, (rows,), generator=g, dtype=torch.int32).numpy()
+    check_rope(torch.randn((rows, H, d), generator=g).bfloat16(), pos, 500000.0)
+    X = torch.randn((rows, H, d), generator=g).bfloat16().to(DEV)
+    p = torch.from_numpy(pos).to(DEV)
+    names = [n for n in kernel_names(lambda: binding.pulsar_rope_apply(X, p)) if "rope_kernel" in n]
+    shared = (d == 16 and H >= 16) or (H >= 32 and (d < 64 or 4 * rows * H * d > 128e6) and d != 192)
+    assert len(names) == 1 and (f"rope_kernel<{'true' if shared else 'false'}>" in names[0])
