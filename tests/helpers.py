@@ -1,4 +1,9 @@
 """Shared helpers of the GPU parity tests: tolerances and error measures."""
+import os
+import re
+import tempfile
+import warnings
+
 import numpy as np
 import torch
 
@@ -38,12 +43,29 @@ def check_attention(O_gpu, LSE_gpu, O_ref, LSE_ref, what=""):
 
 
 def kernel_names(fn):
-    """Names (with their template arguments) of the kernels that ``fn`` launches, in order."""
-    from torch.profiler import ProfilerActivity, profile
-    fn()                                             # a first call outside: module loading is not part of the record
-    torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
+    """(name, template arguments) of every kernel that ``fn`` launches, in order: the calls are recorded as a CUDA graph and
+    its nodes printed.  bool arguments count as 0 and 1; type arguments are left out."""
+    side = torch.cuda.Stream()                       # a first run outside the capture: module loading, kernel attributes
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
         fn()
-        torch.cuda.synchronize()
-    ev = [e for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA]
-    return [e.name for e in sorted(ev, key=lambda e: e.time_range.start)]
+    torch.cuda.current_stream().wait_stream(side)
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        fn()
+    with tempfile.TemporaryDirectory() as tmp, warnings.catch_warnings():
+        warnings.simplefilter("ignore")              # announces the file it writes
+        graph.debug_dump(os.path.join(tmp, "graph.dot"))
+        with open(os.path.join(tmp, "graph.dot")) as f:
+            text = f.read()
+    return parse_kernel_names(text)
+
+
+def parse_kernel_names(dot):
+    """The kernels of a printed CUDA graph: mangled names such as ..16lse_merge_kernelILb0EE.. in its nodes' labels."""
+    names = []
+    for mangled in re.findall(r"topoId: \d+\) \| (_Z\w+)", dot):
+        m = re.search(r"\d([a-z][a-z_]*_kernel)((?:I(?:L[bi]\d+E)+E)?)", mangled)
+        if m:
+            names.append((m.group(1), [int(x) for x in re.findall(r"L[bi](\d+)E", m.group(2))]))
+    return names

@@ -212,10 +212,10 @@ def test_phase1_sharded_at_the_128k_configuration_equals_the_unsharded_call():
 
 
 def form_of(fn):
-    """Query tiles per work item (1 or 2) of the attention launch in ``fn``: the kernel's last template argument."""
-    names = [n for n in kernel_names(fn) if "attn_kernel" in n]
-    assert len(names) == 1, names
-    return 1 if ", true>" in names[0] else 2
+    """Query tiles per work item (1 or 2) of the attention launch in ``fn``: the third template argument of the kernel."""
+    found = [args for name, args in kernel_names(fn) if name == "attn_kernel"]
+    assert len(found) == 1
+    return 1 if found[0][2] else 2
 
 
 @pytest.mark.parametrize("d", [64, 128])
