@@ -280,7 +280,7 @@ struct ScoreTable {
 // compared with all others of the chunk, for a chunk of at most 32 tokens in one warp match -- and
 // lane 0 adds them up in the order of the equations.  A position that carries no term holds 0.0, which
 // leaves the sum's bits as they are.  Latency-bound: one thread per chunk, walking the chunk's pairs
-// of positions serially, took 92 us for 4096 chunks of 32 tokens under BM25 (the whole call 109 us, 38 us with
+// of positions serially, took 92 us for 4096 chunks of 32 tokens under BM25 (the whole call 115 us, 16 us with
 // this form and the four launches chained as programmatic dependents).
 constexpr int kScoreWarps = 4;
 
@@ -290,7 +290,6 @@ chunk_score_kernel(const uint32_t* __restrict__ ids, const uint16_t* __restrict_
                    int block_size, int chunks_per_block, int n_slots_total, int chunk, int vocab_size,
                    const __grid_constant__ ScoreTable<kBlocks> tab, double* __restrict__ score) {
     extern __shared__ double smem_d[];                     // per warp: a term and a token per position
-    grid_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double* term = smem_d + warp * chunk;
     uint32_t* tok = reinterpret_cast<uint32_t*>(smem_d + kScoreWarps * chunk) + warp * chunk;
@@ -302,6 +301,8 @@ chunk_score_kernel(const uint32_t* __restrict__ ids, const uint16_t* __restrict_
     const int len = static_cast<int>(max(static_cast<int64_t>(0),
                                          min(static_cast<int64_t>(chunk), min(lo + block_size, L) - start)));
     const uint32_t V = static_cast<uint32_t>(vocab_size);
+    // The ids may be read before the wait: the presence launch of this call, which let its dependents in only after its own
+    // wait, has found them complete.
     for (int p = lane; p < len; p += 32) tok[p] = ids[start + p];
     __syncwarp();
     grid_dependency_wait();                                // the df table is complete
@@ -356,6 +357,10 @@ chunk_score_kernel(const uint32_t* __restrict__ ids, const uint16_t* __restrict_
         }
     }
     __syncwarp();
+    // The selection's CTAs, one per block and bound by float64 compares, are placed where there is room.  Let in while this grid
+    // still fills the chip they were put several to an SM: 16 blocks of 2048 chunks of 4 tokens under BM25 took 829 us, 190 us
+    // with the dependents let in here.
+    grid_launch_dependents();
     if (lane != 0) return;
     double s = 0.0;
     if (kMode == PULSAR_SCORE_TYPE_TOKEN) {

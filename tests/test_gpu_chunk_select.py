@@ -109,3 +109,28 @@ def test_block_counts_around_the_small_score_table(n_blocks, mode):
     rng = np.random.default_rng(n_blocks)
     ids = np.concatenate([rng.integers(0, 40, size=48) * rng.integers(1, 6) for _ in range(n_blocks)]).astype(np.uint32)
     run_and_compare(ids, 300, 48, 12, 2, 5, mode)
+
+
+def test_selection_is_spread_over_the_chip_under_every_score():
+    """The selection launch waits for the scores on the device.  Its 16 CTAs of 2048 chunks each take the same time under
+    every score (190 us); several to an SM, as they were placed behind a BM25 launch still under way, they took 829 us."""
+    gen = torch.Generator(device=DEV).manual_seed(5)
+    L, block, chunk, vocab = 131072, 8192, 4, 32000
+    ids = (torch.rand(L, generator=gen, device=DEV).pow(4) * vocab).to(torch.int32).clamp_(max=vocab - 1)
+
+    def time_of(mode):
+        call = lambda: binding.pulsar_chunk_select(ids, vocab, block, chunk, 128, 16, mode)
+        for _ in range(3):
+            call()
+        t = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+
+    assert time_of("bm25") <= 2.0 * time_of("tf_idf")
