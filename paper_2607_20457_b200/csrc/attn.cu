@@ -499,7 +499,9 @@ __device__ __forceinline__ float exp_row128(const uint32_t (&r)[kTileN], float s
 // waits for it first.  Measured against the 128K key/value set (131,072 keys, 18 parts, L2 flushed clean
 // before each call): 9 to 32 query tokens of 4 heads per KV head 120-124 us -> 99-103 us (0.69 -> 0.83 of
 // the HBM bandwidth), the 8-token decode shape 101.3 -> 99.4 us.
-template <int D, bool kQuad, bool kSingle>
+// kTileMax: see next_max; generation steps whose parts were made longer.  An instance of its own, since the test alone
+// costs Phase 1 0.4 % (16K 658 -> 661 us).
+template <int D, bool kQuad, bool kSingle, bool kTileMax>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKp,
@@ -895,7 +897,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             if (!it.valid) break;
             const int n = s ? it.n_tiles_b : it.n_tiles_a;
             const int pref_len = it.pref_len;
-            const bool tile_max = a.tile_max && it.main_len > 0;
+            const bool tile_max = kTileMax && it.main_len > 0;
             float m_used = -INFINITY, l_run = 0.f;
             const int row_t = kQuad ? lane : row;             // row as far as token and head are concerned
 
@@ -1221,8 +1223,13 @@ int32_t launch_attn(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMa
     };
     static const VarlenTable kNoSequences{};
     const VarlenTable& tab = table ? *table : kNoSequences;
-    PULSAR_CUDA_OK(a.quad ? launch(attn_kernel<D, true, true>, NoTable{})
-                          : (a.single ? launch(attn_kernel<D, false, true>, tab) : launch(attn_kernel<D, false, false>, tab)));
+    const auto pick = [&](auto tile_max) -> cudaError_t {
+        constexpr bool kTileMax = decltype(tile_max)::value;
+        return a.quad     ? launch(attn_kernel<D, true, true, kTileMax>, NoTable{})
+               : a.single ? launch(attn_kernel<D, false, true, kTileMax>, tab)
+                          : launch(attn_kernel<D, false, false, kTileMax>, tab);
+    };
+    PULSAR_CUDA_OK(a.tile_max ? pick(std::true_type{}) : pick(std::false_type{}));
     count_launch();
     return PULSAR_OK;
 }
