@@ -1771,7 +1771,8 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     const int copies = quad ? 4 : 1;
     const size_t po_bytes = round_up(static_cast<size_t>(n_parts) * copies * n_new * Hq * d * 4, 256);
     const size_t pl_bytes = round_up(static_cast<size_t>(n_parts) * copies * n_new * Hq * 4, 256);
-    if (workspace_bytes < po_bytes + pl_bytes) return PULSAR_ERR_WORKSPACE;
+    // The stated size is asked for however the call is cut: what fits must not depend on the length of the shard.
+    if (workspace_bytes < pulsar_phase2_generate_workspace_bytes(n_new, B, block_size, Hq, Hkv, d, n_splits)) return PULSAR_ERR_WORKSPACE;
     rc = check_device();
     if (rc != PULSAR_OK) return rc;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);

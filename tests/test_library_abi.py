@@ -81,3 +81,15 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(_build, "LIB", str(tmp_path / "absent.so"))
     with pytest.raises(FileNotFoundError):
         binding.load_library()
+
+
+@pytest.mark.parametrize("n_new,L,gen_len,Hq,Hkv,splits", [(1, 6001, 33, 8, 2, 0), (1, 131072, 200, 32, 8, 0), (40, 4096, 0, 8, 8, 4)])
+def test_generation_step_asks_for_the_stated_workspace(lib, n_new, L, gen_len, Hq, Hkv, splits):
+    """One byte less than the stated size is refused however context and shard are cut (nothing is launched, and the pointers
+    are not read: the device check comes later)."""
+    one = ctypes.c_void_p(256)
+    J = splits or lib.pulsar_phase2_choose_splits(n_new, 1, L, Hq, Hkv, 128)
+    stated = lib.pulsar_phase2_generate_workspace_bytes(n_new, 1, L, Hq, Hkv, 128, J)
+    rc = lib.pulsar_phase2_generate_step(one, one, one, n_new, one, one, 1, L, one, one, gen_len, gen_len + n_new, Hq, Hkv, 128,
+                                         0.0, J, one, None, one, stated - 1, None, None)
+    assert stated > 0 and rc == 4
