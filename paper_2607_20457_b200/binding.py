@@ -283,6 +283,8 @@ def pulsar_phase2_attn(Qq, Kblocks, Vblocks, n_blocks: int, block_size: int, sof
     (needs n_splits > 0), also (part_O f32 [J,nq,Hq,d], part_LSE f32 [J,nq,Hq]); ``partials`` may
     give those two tensors preallocated."""
     pO, pL = partials if partials is not None else (None, None)
+    if partials is not None and (pO is None or pL is None):
+        raise TypeError("partials: expected two tensors")
     res = _native_module().phase2_attn(Qq, Kblocks, Vblocks, n_blocks, block_size, softmax_scale, n_splits, want_partials, out,
                                        lse_out, workspace, status, pO, pL)
     return res if want_partials or partials is not None else res[:2]

@@ -156,6 +156,9 @@ template <PyObject* (*F)(Args&)> PyObject* entry(PyObject*, PyObject* const* v, 
 }
 
 // ---- selection ------------------------------------------------------------------------------------------------------
+// The first n entries along the first dimension, fewer if there are not as many (t[:n]).
+at::Tensor head(const at::Tensor& t, int64_t n) { return t.slice(0, 0, n); }
+
 struct SelectShape {
     int32_t V, block, chunk, k, sink;
     int64_t L, B, C;
@@ -190,7 +193,7 @@ PyObject* maxidf_select(Args& a) {
                                       ptr<int32_t>(pidx), ptr<int32_t>(plen), ptr<uint32_t>(df), ptr<float>(idf), ptr<void>(ws),
                                       static_cast<size_t>(ws.numel()), ptr<int32_t>(status), st);
     });
-    return result({sel.narrow(0, 0, z.B * z.k).view({z.B, z.k}), pidx.narrow(0, 0, z.prefix()), plen.narrow(0, 0, z.B)});
+    return result({head(sel, z.B * z.k).view({z.B, z.k}), head(pidx, z.prefix()), head(plen, z.B)});
 }
 
 // (token_ids, vocab, block, chunk, k, sink, mode, want_score, workspace, status)
@@ -208,7 +211,7 @@ PyObject* chunk_select(Args& a) {
                                      ptr<int32_t>(pidx), ptr<int32_t>(plen), ptr<double>(score), ptr<void>(ws),
                                      static_cast<size_t>(ws.numel()), ptr<int32_t>(status), st);
     });
-    return result({sel.narrow(0, 0, z.B * z.k).view({z.B, z.k}), pidx.narrow(0, 0, z.prefix()), plen.narrow(0, 0, z.B), score});
+    return result({head(sel, z.B * z.k).view({z.B, z.k}), head(pidx, z.prefix()), head(plen, z.B), score});
 }
 
 // ---- Phase 1 --------------------------------------------------------------------------------------------------------
@@ -300,10 +303,13 @@ PyObject* causal_varlen_attn(Args& a) {
 
 // (K, V, cu_seqlens, block)
 PyObject* retain_block_kv(Args& a) {
-    at::Tensor K = a.bf16("K", 3), V = a.bf16("V", 3);
+    at::Tensor K = a.bf16("K"), V = a.bf16("V");
+    if (K.dim() < 3) raise(PyExc_ValueError, "K: expected 3 dimensions");
     const std::vector<int32_t> cu = a.sequence();
     const int32_t block = a.i32(), n_seq = static_cast<int32_t>(cu.size()) - 1;
-    at::Tensor Kr = empty({static_cast<int64_t>(n_seq) * block, K.size(1), K.size(2)}, at::kBFloat16, K), Vr = at::empty_like(Kr);
+    std::vector<int64_t> sizes = K.sizes().vec();
+    sizes[0] = static_cast<int64_t>(n_seq) * block;
+    at::Tensor Kr = empty(sizes, at::kBFloat16, K), Vr = at::empty_like(Kr);
     call("pulsar_retain_block_kv", [&, st = stream()] {
         return g.pulsar_retain_block_kv(in16(K), in16(V), K.size(0), cu.data(), n_seq, block, static_cast<int32_t>(K.size(1)),
                                         static_cast<int32_t>(K.size(2)), ptr<uint16_t>(Kr), ptr<uint16_t>(Vr), st);
@@ -430,11 +436,11 @@ PyObject* lse_merge_strided(Args& a) {
 
 // (Q, K, positions, theta, q_out, k_out, status)
 PyObject* rope_apply_qk(Args& a) {
-    at::Tensor Q = a.bf16("Q", 3), K = a.bf16("K", 3), pos = a.i32s("positions");
+    at::Tensor Q = a.bf16("Q", 3), K = a.bf16("K"), pos = a.i32s("positions");
     const double theta = a.real();
     at::Tensor Qo = a.tensor(), Ko = a.tensor(), status = a.tensor();
     const int64_t rows = Q.size(0), d = Q.size(2);
-    if (K.size(0) != rows || K.size(2) != d || pos.numel() != rows)
+    if (K.dim() < 3 || K.size(0) != rows || K.size(2) != d || pos.numel() != rows)
         raise(PyExc_ValueError, "Q, K and positions must cover the same rows and head size");
     if (!Qo.defined()) Qo = at::empty_like(Q);
     if (!Ko.defined()) Ko = at::empty_like(K);

@@ -310,3 +310,12 @@ def test_merge_on_both_sides_of_its_rule(J, rows, warps, d):
     got = [(n, args[:3]) for n, args in kernel_names(lambda: binding.pulsar_lse_merge(pO, pL))]
     assert got == [("lse_merge_rows_kernel", [0, d // 32, warps]) if warps else ("lse_merge_kernel", [0])]
     test_merge_at_the_edges_of_its_splits(J, rows, d)
+
+
+def test_partials_that_are_no_tensors_are_refused():
+    w = W.CONFIGS["tiny"]
+    _, K, V = (t.to(DEV) for t in W.qkv(w))
+    Qq = W.phase2_query(w).to(DEV)
+    for partials in ((None, None), (None, torch.empty(2, w.nq, w.Hq, device=DEV))):
+        with pytest.raises(TypeError):
+            binding.pulsar_phase2_attn(Qq, K, V, 1, w.L, n_splits=2, partials=partials)

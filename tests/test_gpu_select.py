@@ -95,3 +95,17 @@ def test_many_blocks():
     with pytest.raises(binding.PulsarError) as e:            # 65,533 blocks: within the 16-bit levels, beyond shared memory
         binding.pulsar_maxidf_select(ids, 97, 1, 1, 1, 0)
     assert e.value.status == 2
+
+
+def test_output_buffers_of_any_shape():
+    """Buffers of the caller's: sel_chunks as [B, k] or flat, longer than needed or not."""
+    w = W.CONFIGS["tiny"]
+    ids = to_dev_ids(W.needle_ids(w), DEV)
+    want = binding.pulsar_maxidf_select(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink)
+    B, n = w.n_blocks, w.prefix_total
+    new = lambda *s: torch.full(s, -7, dtype=torch.int32, device=DEV)
+    for out in ((new(B, w.k), new(n), new(B)), (new(B * w.k), new(n + 9), new(B + 1)), (new(B + 1, w.k), new(n), new(B))):
+        got = binding.pulsar_maxidf_select(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink, out=out)
+        for name in ("sel_chunks", "prefix_idx", "prefix_len"):
+            assert torch.equal(got[name], want[name])
+        assert got["sel_chunks"].data_ptr() == out[0].data_ptr()

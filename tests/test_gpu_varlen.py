@@ -125,3 +125,11 @@ def test_few_and_many_work_items(n_seq, length, d):
     torch.cuda.synchronize()
     assert int(status.item()) == 0
     check_attention(O, LSE, Oref, Lref, f"{n_seq} x {length} d={d}")
+
+
+def test_kv_discard_takes_values_in_any_shape():
+    """Only K's shape says how many heads of which size a row has; V may come as plain rows."""
+    K, V = (torch.randn(300, 2, 64, device=DEV).bfloat16() for _ in range(2))
+    Kr, Vr = binding.pulsar_retain_block_kv(K, V, [0, 130, 300], 100)
+    K2, V2 = binding.pulsar_retain_block_kv(K, V.view(300, 128), [0, 130, 300], 100)
+    assert torch.equal(Kr, K2) and torch.equal(Vr, V2) and torch.equal(Vr[:100], V[30:130])
