@@ -1,6 +1,7 @@
 """Builds in-tree: the CUDA library ``libpulsar.so`` (sm_100a only) and ``_native.so``, the native half of the binding."""
 from __future__ import annotations
 
+import importlib.metadata
 import os
 import subprocess
 import sysconfig
@@ -10,6 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpulsar.so")
 NATIVE = os.path.join(HERE, "_native.so")
 NATIVE_SOURCE = os.path.join(CSRC, "binding.cpp")
+NATIVE_KEY = os.path.join(HERE, "build", "_native.key")     # what NATIVE was compiled against
 SOURCES = ["api.cu", "select.cu", "merge.cu", "attn.cu", "rope.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(os.path.dirname(HERE), "include", "pulsar.h")]
 NVCC_FLAGS = [
@@ -31,9 +33,21 @@ def needs_build() -> bool:
     return _stale(LIB, [os.path.join(CSRC, s) for s in SOURCES] + HEADERS)
 
 
+def native_key() -> str:
+    """The Python and the torch that a build of the extension module is good for: it uses the ABI of both."""
+    return f"{sysconfig.get_config_var('SOABI')} torch-{importlib.metadata.version('torch')}"
+
+
+def _native_stale() -> bool:
+    if _stale(NATIVE, [NATIVE_SOURCE, HEADERS[1]]) or not os.path.exists(NATIVE_KEY):
+        return True
+    with open(NATIVE_KEY) as f:
+        return f.read() != native_key()
+
+
 def build_native(force: bool = False) -> str:
     """Compile the binding's extension module against the torch that is installed.  Returns its path."""
-    if not force and not _stale(NATIVE, [NATIVE_SOURCE, HEADERS[1]]):
+    if not force and not _native_stale():
         return NATIVE
     import torch
     root = os.path.dirname(torch.__file__)
@@ -46,6 +60,9 @@ def build_native(force: bool = False) -> str:
         "-I" + sysconfig.get_path("include"), "-I" + os.path.join(cuda, "include"), NATIVE_SOURCE, "-o", tmp,
         "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
     os.replace(tmp, NATIVE)
+    os.makedirs(os.path.dirname(NATIVE_KEY), exist_ok=True)
+    with open(NATIVE_KEY, "w") as f:
+        f.write(native_key())
     return NATIVE
 
 

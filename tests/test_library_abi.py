@@ -93,3 +93,10 @@ def test_generation_step_asks_for_the_stated_workspace(lib, n_new, L, gen_len, H
     rc = lib.pulsar_phase2_generate_step(one, one, one, n_new, one, one, 1, L, one, one, gen_len, gen_len + n_new, Hq, Hkv, 128,
                                          0.0, J, one, None, one, stated - 1, None, None)
     assert stated > 0 and rc == 4
+
+
+def test_native_module_is_rebuilt_for_another_torch(lib, monkeypatch):
+    """The extension module uses torch's C++ ABI: file times alone do not say whether a build still fits."""
+    assert not _build._native_stale()
+    monkeypatch.setattr(_build, "native_key", lambda: "another torch")
+    assert _build._native_stale()
