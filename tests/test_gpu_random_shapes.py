@@ -80,3 +80,25 @@ def test_assembled_inputs_and_generation_on_a_random_shape(seed):
         Og_ref, Lg_ref = oracle.generate_step(Qn, Kn, Vn, K, V, Kg_o, Vg_o, gen_len)
         check_attention(Og, Lg, Og_ref, Lg_ref, f"generation step n={n} gen_len={gen_len}")
         gen_len += n
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_phase1_on_a_random_shape_with_many_heads(seed):
+    """As above with so many heads that the work items are pairs of query tiles."""
+    w = random_workload(200 + seed)
+    g = w.Hq // w.Hkv
+    pairs = lambda Hkv: sum(-(-w.block_size // 256) for _ in range(w.n_blocks)) * Hkv * g
+    packed = lambda Hkv: w.n_blocks * -(-w.block_size // max(256 // g, 1)) * Hkv
+    Hkv = next(n for n in range(1, 200) if pairs(n) > 160 and packed(n) > 160)
+    w = W.shrink(w, Hq=Hkv * g, Hkv=Hkv)
+    Q, K, V = W.qkv(w, seed=seed + 3)
+    ids = W.token_ids(w)
+    ref = oracle.maxidf_select(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink)
+    pidx, plen = (torch.from_numpy(np.ascontiguousarray(ref[n])).to(DEV) for n in ("prefix_idx", "prefix_len"))
+    st = binding.new_status(DEV)
+    call = lambda: binding.pulsar_phase1_attn(Q.to(DEV), K.to(DEV), V.to(DEV), w.block_size, pidx, plen, status=st)
+    O, LSE, _, _ = call()
+    O_ref, L_ref = oracle.phase1_attn(Q, K, V, w.block_size, ref["prefix_idx"], ref["prefix_len"])
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    check_attention(O, LSE, O_ref, L_ref, f"phase 1 {w}")

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import check_attention
+from helpers import check_attention, kernel_names
 from paper_2607_20457_b200 import binding, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -112,8 +112,7 @@ def test_kv_discard_keeps_each_blocks_own_rows():
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("n_seq,length", [(1, 1), (2, 129), (36, 300), (37, 300), (3, 1500)])
 def test_few_and_many_work_items(n_seq, length, d):
-    """Up to one pair of query tiles per SM the work items are single tiles (36 sequences of two pairs and two heads: 144
-    pairs), beyond that pairs (37: 148 on 148 SMs, and with lengths that differ more)."""
+    """Fewer pairs of query tiles than SMs (at most 148): work items of one tile, or of two where that is the shorter time."""
     gen = torch.Generator().manual_seed(n_seq * length)
     lens = [length + 7 * (j % 3) for j in range(n_seq)]
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
@@ -133,3 +132,35 @@ def test_kv_discard_takes_values_in_any_shape():
     Kr, Vr = binding.pulsar_retain_block_kv(K, V, [0, 130, 300], 100)
     K2, V2 = binding.pulsar_retain_block_kv(K, V.view(300, 128), [0, 130, 300], 100)
     assert torch.equal(Kr, K2) and torch.equal(Vr, V2) and torch.equal(Vr[:100], V[30:130])
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("Hq,Hkv,lens", [(2, 1, [300 + 7 * (j % 5) for j in range(60)]),     # one or two key tiles, ragged
+                                         (8, 2, [2049, 1000, 3, 1311, 128, 129]), (16, 2, [1500, 777, 1025, 40]),
+                                         (6, 2, [2000, 1100, 900, 260])])                    # a group that is not packed
+def test_pairs_of_query_tiles(Hq, Hkv, lens, d):
+    """More pairs of query tiles than SMs: work items of two tiles, with d = 64 and groups of 2, 4 and 8 heads packed."""
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    gen = torch.Generator().manual_seed(Hq * len(lens))
+    Q = (2 * torch.randn(int(cu[-1]), Hq, d, generator=gen)).to(torch.bfloat16)
+    K, V = (torch.randn(int(cu[-1]), Hkv, d, generator=gen).to(torch.bfloat16) for _ in range(2))
+    Qd, Kd, Vd = Q.to(DEV), K.to(DEV), V.to(DEV)
+    g = Hq // Hkv
+    packed = d == 64 and g in (1, 2, 4, 8, 16)
+    tokens, heads = (256 // g, Hkv) if packed else (256, Hq)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    repeat = sms // (heads * sum(-(-n // tokens) for n in lens)) + 1                 # as often as it takes
+    if repeat > 1:
+        lens = lens * repeat
+        cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        Q, K, V = (x.repeat(repeat, 1, 1) for x in (Q, K, V))
+        Qd, Kd, Vd = (x.repeat(repeat, 1, 1) for x in (Qd, Kd, Vd))
+    assert len(lens) <= 64 and heads * sum(-(-n // tokens) for n in lens) > sms
+    status = binding.new_status(DEV)
+    call = lambda: binding.pulsar_causal_varlen_attn(Qd, Kd, Vd, cu.tolist(), status=status)
+    O, LSE = call()
+    assert [args[:3] for name, args in kernel_names(call) if name == "attn_kernel"] == [[d, 0, 0]]
+    Oref, Lref = oracle.causal_varlen_attn(Q, K, V, cu)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    check_attention(O, LSE, Oref, Lref, f"Hq={Hq} Hkv={Hkv} d={d} {len(lens)} sequences")
