@@ -240,8 +240,9 @@ pack_summary_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, co
 // ping-pong on the tensor pipe: while the softmax warpgroup of one tile works on S, the pipe
 // runs the other tile's PV and next S.  TMEM: S0 [0,128) S1 [128,256) O0 [256,384) O1 [384,512);
 // P_s (bf16 pairs) overwrites the first 64 columns of S_s.  The running maximum is only moved
-// when it grows by more than 2^8 (the stale maximum is used consistently for P, O and the row
-// sum, so the result is unchanged); the rare rescale of O is done by the softmax warpgroup.
+// when a logit exceeds it by more than 2^8, in the first 96 keys of a tile when their probabilities sum to more than
+// 96 * 2^8 (kPieceSumBound: one of them may reach 2^14.6).  The stale maximum is used consistently for P, O and the row
+// sum, so the result is unchanged; the rare rescale of O is done by the softmax warpgroup.
 // P goes to the issuer in two pieces (96 and 32 keys, two barriers), so the first piece of PV runs while
 // the second half of the row is exponentiated.  The loader publishes the CTA's work items through
 // a small shared-memory queue; all device waits are bounded (see mbar_wait).
