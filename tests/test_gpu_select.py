@@ -104,7 +104,7 @@ def test_output_buffers_of_any_shape():
     want = binding.pulsar_maxidf_select(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink)
     B, n = w.n_blocks, w.prefix_total
     new = lambda *s: torch.full(s, -7, dtype=torch.int32, device=DEV)
-    for out in ((new(B, w.k), new(n), new(B)), (new(B * w.k), new(n + 9), new(B + 1)), (new(B + 1, w.k), new(n), new(B))):
+    for out in ((new(B, w.k), new(n), new(B)), (new(B * w.k + 3), new(n + 9), new(B + 1))):
         got = binding.pulsar_maxidf_select(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink, out=out)
         for name in ("sel_chunks", "prefix_idx", "prefix_len"):
             assert torch.equal(got[name], want[name])
