@@ -372,6 +372,69 @@ chunk_score_kernel(const uint32_t* __restrict__ ids, const uint16_t* __restrict_
     score[slot] = kMode == PULSAR_SCORE_BM25 ? s : __ddiv_rn(s, static_cast<double>(len));
 }
 
+// Very many short chunks: one thread per chunk slot walks its tokens, the positions of a type counted where it first occurs.
+// A warp per chunk leaves most of its lanes idle there and needs a warp's start for each.  us of the whole call under BM25,
+// warp / thread form: 262,144 chunks of 4 256 / 197, 131,072 of 8 97 / 67, 125,000 of 4 in 500 blocks 75 / 53, 42,000 of 12
+// in 500 blocks 94 / 89; from 16 tokens on (65,536: 55 against 73 with one thread each) and with few chunks, where one
+// warp each is still all at once, the warp is the better form.
+constexpr int kThreadFormChunk = 12;
+constexpr int kThreadFormSlots = 40000;
+
+template <int kMode, int kBlocks>
+__global__ void __launch_bounds__(128)
+chunk_score_thread_kernel(const uint32_t* __restrict__ ids, const uint16_t* __restrict__ df_table, int64_t L,
+                          int block_size, int chunks_per_block, int n_slots_total, int chunk, int vocab_size,
+                          const __grid_constant__ ScoreTable<kBlocks> tab, double* __restrict__ score) {
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = slot / chunks_per_block, c = slot - b * chunks_per_block;
+    const int64_t lo = static_cast<int64_t>(b) * block_size;
+    const int64_t start = lo + static_cast<int64_t>(c) * chunk;
+    const int len = slot < n_slots_total
+                        ? static_cast<int>(max(static_cast<int64_t>(0), min(static_cast<int64_t>(chunk), min(lo + block_size, L) - start)))
+                        : 0;
+    const uint32_t V = static_cast<uint32_t>(vocab_size);
+    uint32_t tok[kThreadFormChunk];
+#pragma unroll
+    for (int p = 0; p < kThreadFormChunk; ++p) tok[p] = p < len ? ids[start + p] : 0u;    // complete: see the warp form
+    grid_dependency_wait();                                // the df table is complete
+    double s = 0.0;
+    if (kMode == PULSAR_SCORE_MAX_IDF || len == 0) {
+        s = -CUDART_INF;
+#pragma unroll
+        for (int p = 0; p < kThreadFormChunk; ++p)
+            if (p < len && tok[p] < V) s = fmax(s, tab.by_df[df_table[tok[p]]]);
+    } else if (kMode == PULSAR_SCORE_TF_IDF) {
+#pragma unroll
+        for (int p = 0; p < kThreadFormChunk; ++p)
+            if (p < len && tok[p] < V) s = __dadd_rn(s, tab.by_df[df_table[tok[p]]]);
+        s = __ddiv_rn(s, static_cast<double>(len));
+    } else {
+        const double k1_times_D =
+            __dmul_rn(tab.k1, __dadd_rn(tab.one_minus_b, __dmul_rn(tab.b, __ddiv_rn(static_cast<double>(len), tab.mean_len))));
+        int distinct = 0;
+#pragma unroll
+        for (int p = 0; p < kThreadFormChunk; ++p) {
+            int before = 0, tf = 0;
+#pragma unroll
+            for (int q = 0; q < kThreadFormChunk; ++q) {
+                const int eq = q < len && tok[q] == tok[p] ? 1 : 0;
+                tf += eq;
+                before += q < p ? eq : 0;
+            }
+            if (p >= len || before > 0) continue;
+            ++distinct;
+            if (kMode == PULSAR_SCORE_BM25 && tok[p] < V) {
+                const double tfd = static_cast<double>(tf);
+                const double num = __dmul_rn(tab.by_df[df_table[tok[p]]], __dmul_rn(tfd, tab.k1_plus_1));
+                s = __dadd_rn(s, __ddiv_rn(num, __dadd_rn(tfd, k1_times_D)));
+            }
+        }
+        if (kMode == PULSAR_SCORE_TYPE_TOKEN) s = __ddiv_rn(static_cast<double>(distinct), static_cast<double>(len));
+    }
+    grid_launch_dependents();
+    if (slot < n_slots_total) score[slot] = s;
+}
+
 // One CTA per block: chunk c is taken when fewer than k chunks beat it (a larger score, or the
 // same score at a lower index); the taken chunks are compacted in index order.
 __global__ void __launch_bounds__(kTopkThreads)
@@ -565,11 +628,19 @@ cudaError_t launch_scores(const SelectPlan& b, int32_t score_mode, const uint32_
     tab.one_minus_b = 1.0 - bb;
     tab.mean_len = static_cast<double>(L) / static_cast<double>(n_chunks);
 
+    const int n_chunks_total = b.n_blocks * b.C;
+    if (chunk <= kThreadFormChunk && n_chunks_total >= kThreadFormSlots) {
+        auto kernel = score_mode == PULSAR_SCORE_MAX_IDF ? chunk_score_thread_kernel<PULSAR_SCORE_MAX_IDF, kBlocks>
+                    : score_mode == PULSAR_SCORE_TF_IDF  ? chunk_score_thread_kernel<PULSAR_SCORE_TF_IDF, kBlocks>
+                    : score_mode == PULSAR_SCORE_BM25    ? chunk_score_thread_kernel<PULSAR_SCORE_BM25, kBlocks>
+                                                         : chunk_score_thread_kernel<PULSAR_SCORE_TYPE_TOKEN, kBlocks>;
+        return launch_kernel(kernel, dim3((n_chunks_total + 127) / 128), dim3(128), 0, stream, true, token_ids, df_table, L,
+                             block_size, b.C, n_chunks_total, chunk, vocab_size, tab, score);
+    }
     auto kernel = score_mode == PULSAR_SCORE_MAX_IDF ? chunk_score_kernel<PULSAR_SCORE_MAX_IDF, kBlocks>
                 : score_mode == PULSAR_SCORE_TF_IDF  ? chunk_score_kernel<PULSAR_SCORE_TF_IDF, kBlocks>
                 : score_mode == PULSAR_SCORE_BM25    ? chunk_score_kernel<PULSAR_SCORE_BM25, kBlocks>
                                                      : chunk_score_kernel<PULSAR_SCORE_TYPE_TOKEN, kBlocks>;
-    const int n_chunks_total = b.n_blocks * b.C;
     const size_t smem = static_cast<size_t>(kScoreWarps) * chunk * (sizeof(double) + sizeof(uint32_t));
     return launch_kernel(kernel, dim3((n_chunks_total + kScoreWarps - 1) / kScoreWarps), dim3(kScoreWarps * 32), smem, stream,
                          true, token_ids, df_table, L, block_size, b.C, n_chunks_total, chunk, vocab_size, tab, score);

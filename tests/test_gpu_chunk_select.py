@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import to_dev_ids
+from helpers import kernel_names, to_dev_ids
 from paper_2607_20457_b200 import binding, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -134,3 +134,21 @@ def test_selection_is_spread_over_the_chip_under_every_score():
         return min(t)
 
     assert time_of("bm25") <= 2.0 * time_of("tf_idf")
+
+
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("chunk,block,slots", [(1, 200, 40200), (4, 1001, 40160), (11, 1003, 40020), (12, 1000, 39984), (12, 1000, 40068),
+                                               (13, 1000, 40040)])
+def test_very_many_short_chunks(chunk, block, slots, mode):
+    """From 40,000 chunks of up to 12 tokens on a thread takes a chunk: chunks that end inside a block's last one and a short last
+    block, few distinct tokens."""
+    rng = np.random.default_rng(chunk)
+    per_block = -(-block // chunk)
+    n_blocks = slots // per_block
+    assert slots == n_blocks * per_block
+    L = n_blocks * block - block // 3
+    ids = (rng.integers(0, 60, size=L) * rng.integers(1, 5, size=L)).astype(np.uint32)
+    run_and_compare(ids, 240, block, chunk, 3, min(7, block), mode)
+    ids_d = to_dev_ids(ids, DEV)
+    names = [n for n, _ in kernel_names(lambda: binding.pulsar_chunk_select(ids_d, 240, block, chunk, 3, 5, mode))]
+    assert ("chunk_score_thread_kernel" in names) == (chunk <= 12 and slots >= 40000)
