@@ -232,7 +232,7 @@ pack_summary_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, co
 // Attention kernel: persistent, warp-specialised.
 //
 //   warps 0-3   softmax of query tile 0 (one thread per query row, TMEM lane = row)
-//   warps 4-7   softmax of query tile 1
+//   warps 4-7   softmax of query tile 1 (of the other half of the keys where an item has one tile: kHalves)
 //   warp  8     MMA issuer (one elected lane): S_s = Q_s K^T, O_s += P_s V
 //   warp  9     TMA loader (one elected lane): Q tiles and the K/V ring
 //
@@ -449,11 +449,12 @@ __device__ __forceinline__ float next_max(float m_tile, float m_used, float l_ru
     return m_tile > m_used + kRescaleThreshold ? m_tile : m_used;
 }
 
-// Row maximum of 128 raw logits (3-input max, four independent chains).
-__device__ __forceinline__ float row_max128(const uint32_t (&r)[kTileN]) {
+// Row maximum of N raw logits (3-input max, four independent chains).
+template <int N>
+__device__ __forceinline__ float row_max(const uint32_t (&r)[N]) {
     float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
 #pragma unroll
-    for (int c = 0; c < kTileN; c += 8) {
+    for (int c = 0; c < N; c += 8) {
         m0 = max3(m0, __uint_as_float(r[c]), __uint_as_float(r[c + 1]));
         m1 = max3(m1, __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
         m2 = max3(m2, __uint_as_float(r[c + 4]), __uint_as_float(r[c + 5]));
@@ -464,8 +465,8 @@ __device__ __forceinline__ float row_max128(const uint32_t (&r)[kTileN]) {
 
 // p_c = 2^(s_c * scale + neg_m) for logits [kBegin, kEnd) of a row, rounded to bf16 pairs and written
 // to TMEM as the A operand of the PV product; returns the fp32 row sum.
-template <int kBegin, int kEnd>
-__device__ __forceinline__ float exp_row128(const uint32_t (&r)[kTileN], float scale, float neg_m, uint32_t tP) {
+template <int kBegin, int kEnd, int N>
+__device__ __forceinline__ float exp_row(const uint32_t (&r)[N], float scale, float neg_m, uint32_t tP) {
     float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
     const float2 sc = make_float2(scale, scale), nm = make_float2(neg_m, neg_m);
 #pragma unroll
@@ -500,6 +501,12 @@ __device__ __forceinline__ float exp_row128(const uint32_t (&r)[kTileN], float s
 // waits for it first.  Measured against the 128K key/value set (131,072 keys, 18 parts, L2 flushed clean
 // before each call): 9 to 32 query tokens of 4 heads per KV head 120-124 us -> 99-103 us (0.69 -> 0.83 of
 // the HBM bandwidth), the 8-token decode shape 101.3 -> 99.4 us.
+// kHalves (kSingle without kQuad): the two warpgroups share the key tile, 64 keys of every row each, with a maximum, a sum
+// and an accumulator of their own (the absent second tile's), and bring them together when the item ends.  The exponentials of
+// a key tile take the SM's special functions 1024 cycles whoever forms them, but the reads of S, the stores of P and the
+// barriers around them are now under way in two warps per scheduler.  us per key tile of a part, d = 64 0.87 -> 0.80, d = 128
+// 0.88 -> 0.82 (64 key tiles of 64 rows 60.1 -> 55.7 and 61.1 -> 57.4; 4096 causal rows of one head 36.4 -> 34.3 and
+// 36.9 -> 36.0); launches that stream from HBM take what they took.
 // kTileMax: see next_max; generation steps whose parts were made longer.  An instance of its own, since the test alone
 // costs Phase 1 0.4 % (16K 658 -> 661 us).
 template <int D, bool kQuad, bool kSingle, bool kTileMax>
@@ -509,6 +516,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             const __grid_constant__ CUtensorMap tmVp, const AttnArgs a,
             const __grid_constant__ std::conditional_t<kQuad, NoTable, VarlenTable> vt) {
     using SL = SmemLayout<D>;
+    constexpr bool kHalves = kSingle && !kQuad;
+    constexpr int kCols = kHalves ? kTileN / 2 : kTileN;      // logits of a softmax thread per key tile
+    constexpr int kFirst = kHalves ? kCols : kFirstKeys;      // of which it hands over first
     static_assert(kSingle || !kQuad, "the decode-shaped instance has one query tile per item");
     // The swizzled tiles want 1024-byte alignment.  Declared, not computed: tile addresses and descriptors are constants
     // then, which takes them out of the registers of the issuer.
@@ -532,7 +542,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             mbar_init(bars + SL::bPFull + s, 4);        // first half of P: one arrival per softmax warp
             mbar_init(bars + SL::bPFull2 + s, 4);       // second half of P
             mbar_init(bars + SL::bOFull + s, 1);
-            mbar_init(bars + SL::bOEmpty + s, 4);
+            mbar_init(bars + SL::bOEmpty + s, kHalves ? 8 : 4);
         }
         for (int i = 0; i < kItemQueue; ++i) {
             mbar_init(bars + SL::bItemFull + i, 1);
@@ -711,16 +721,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         if (leader) umma_commit_a(bar0 + 8 * (SL::bSFull + (s_)));                                        \
     } while (0)
 // P arrives in two pieces (kFirstKeys keys, then the rest), each with its own barrier.
+// With kHalves they are the two warpgroups': P of keys [64, 128) stands at column 64, and its product goes to the
+// accumulator of the absent second tile.
 #define PULSAR_ISSUE_PV(tO, tP, dv, acc, s_, par)                                                         \
     do {                                                                                                  \
         _Pragma("unroll") for (int half = 0; half < 2; ++half) {                                          \
             ok = ok && mbar_wait_a(bar0 + 8 * ((half ? SL::bPFull2 : SL::bPFull) + (s_)), par, abort_flag, \
                                    a.status);                                                             \
             tc_fence_after();                                                                             \
-            _Pragma("unroll") for (int kk = half ? kFirstKeys / 16 : 0; kk < (half ? kTileN : kFirstKeys) / 16; ++kk) \
+            _Pragma("unroll") for (int kk = half ? kFirst / 16 : 0; kk < (half ? kTileN : kFirst) / 16; ++kk) \
                 if (leader && ok)                                                                         \
-                    umma_ts(tO, (tP) + kk * 8, (dv) + static_cast<uint64_t>(kk * 128), kIdescPV,          \
-                            ((acc) || kk > 0) ? 1u : 0u);                                                 \
+                    umma_ts((tO) + (kHalves && half ? 128 : 0), (tP) + kk * 8 + (kHalves && half ? 32 : 0), \
+                            (dv) + static_cast<uint64_t>(kk * 128), kIdescPV,                             \
+                            ((acc) || kk > (kHalves && half ? kFirst / 16 : 0)) ? 1u : 0u);               \
         }                                                                                                 \
     } while (0)
 
@@ -878,15 +891,22 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     } else if (warp < 8) {
         // =============================== softmax warpgroups ===============================
         reg_alloc<kRegsSoftmax>();
-        const int s = warp >> 2;                               // query tile of this warpgroup
+        const int s = warp >> 2;
         const int row = (warp & 3) * 32 + lane;                // row of the tile = TMEM lane
         const uint32_t lane_sel = static_cast<uint32_t>((warp & 3) * 32) << 16;
-        const uint32_t tS_own = tmem_base + s * 128 + lane_sel;
+        const int tile = kHalves ? 0 : s;                      // query tile of this warpgroup
+        const int key0 = kHalves ? s * kCols : 0;              // its first key of a key tile
+        const uint32_t tS_own = tmem_base + (kHalves ? key0 : s * 128) + lane_sel;
         const uint32_t tO = tmem_base + 256 + s * 128 + lane_sel;
-        uint64_t* bar_of = bars + SL::bOFull + s;
+        const uint32_t tO_other = tmem_base + 256 + (s ^ 1) * 128 + lane_sel;
+        uint64_t* bar_of = bars + SL::bOFull + tile;
         uint64_t* bar_pv = bars + SL::bOFull + 1;              // kSingle: one completion per PV product
         uint32_t g_tile = 0;                                   // kSingle: key tiles this CTA has walked
-        uint64_t* bar_oe = bars + SL::bOEmpty + s;
+        uint64_t* bar_oe = bars + SL::bOEmpty + tile;
+        // kHalves: maximum and sum of each half of a row [2][128], where the second query tile would be, behind a barrier of
+        // their own
+        float2* half_ml = reinterpret_cast<float2*>(sQ + SL::kTileBytes);
+        uint64_t* bar_half = bars + SL::bOEmpty + 1;
         uint32_t s_cnt = 0, o_cnt = 0;
         bool ok = true;
 
@@ -896,7 +916,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
             if (!ok) break;
             const volatile Item& it = item_q[slot];            // handed back at the end of the item
             if (!it.valid) break;
-            const int n = s ? it.n_tiles_b : it.n_tiles_a;
+            const int n = tile ? it.n_tiles_b : it.n_tiles_a;
             const int pref_len = it.pref_len;
             const bool tile_max = kTileMax && it.main_len > 0;
             float m_used = -INFINITY, l_run = 0.f;
@@ -910,7 +930,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 if (pref_left > 0) {
                     if (pref_left < kTileN) { n_vis = pref_left; masked = true; }
                     if (it.gen_base >= 0) {                   // generation shard: causal by token
-                        const int token = (s ? it.token0_b : it.token0_a) + (row_t >> a.pack_shift);
+                        const int token = (tile ? it.token0_b : it.token0_a) + (row_t >> a.pack_shift);
                         n_vis = min(n_vis, it.gen_base + token + 1 - t * kTileN);
                         masked = true;
                     }
@@ -919,7 +939,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     const int valid = it.main_len - j * kTileN;
                     if (valid < kTileN) { n_vis = valid; masked = true; }
                     if (a.mode != kModePhase2 && t == n - 1) {
-                        n_vis = min(n_vis, (s ? it.row0_b : it.row0_a) + (row_t >> a.pack_shift) - j * kTileN + 1);
+                        n_vis = min(n_vis, (tile ? it.row0_b : it.row0_a) + (row_t >> a.pack_shift) - j * kTileN + 1);
                         masked = true;
                     }
                 }
@@ -927,9 +947,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 // kSingle: buffer and barriers alternate with the CTA's key-tile count
                 const uint32_t gb = kSingle ? (g_tile & 1u) : 0u;
                 const uint32_t tS = tS_own + gb * 128;
-                uint64_t* bar_s = bars + SL::bSFull + s + gb;
-                uint64_t* bar_p = bars + SL::bPFull + s + gb;
-                uint64_t* bar_p2 = bars + SL::bPFull2 + s + gb;
+                uint64_t* bar_s = bars + SL::bSFull + tile + gb;
+                uint64_t* bar_p = bars + (kHalves && s ? SL::bPFull2 : SL::bPFull) + tile + gb;
+                uint64_t* bar_p2 = bars + SL::bPFull2 + tile + gb;
                 ok = __all_sync(0xffffffffu,
                                 ok && mbar_wait(bar_s, kSingle ? ((g_tile >> 1) & 1u) : (s_cnt & 1u), abort_flag, a.status));
                 ++s_cnt;
@@ -1012,17 +1032,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     continue;
                 }
 
-                uint32_t r[kTileN];
+                uint32_t r[kCols];
                 PULSAR_TMEM_LD32_AT(tS + 0, r, 0);
                 PULSAR_TMEM_LD32_AT(tS + 32, r, 32);
-                PULSAR_TMEM_LD32_AT(tS + 64, r, 64);
-                PULSAR_TMEM_LD32_AT(tS + 96, r, 96);
+                if constexpr (!kHalves) {
+                    PULSAR_TMEM_LD32_AT(tS + 64, r, 64);
+                    PULSAR_TMEM_LD32_AT(tS + 96, r, 96);
+                }
                 tmem_wait_ld();
 
                 if (masked) {
 #pragma unroll
-                    for (int c = 0; c < kTileN; ++c)
-                        if (c >= n_vis) r[c] = 0xff800000u;          // -inf
+                    for (int c = 0; c < kCols; ++c)
+                        if (key0 + c >= n_vis) r[c] = 0xff800000u;   // -inf
                 }
                 // After the first key tile the running maximum is nearly always good enough, so the first piece of P is
                 // formed with it at once, and whether it was is seen afterwards: its own sum bounds every one of its
@@ -1033,15 +1055,17 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 float s1 = 0.f, neg_m = -m_used;
                 bool fast = !masked && t > 0 && !tile_max;
                 if (fast) {
-                    s1 = exp_row128<0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
+                    s1 = exp_row<0, kFirst>(r, a.scale_log2, neg_m, tS);
                     float m2 = -INFINITY;
+                    if constexpr (!kHalves) {
 #pragma unroll
-                    for (int c = kFirstKeys; c < kTileN; c += 2) m2 = max3(m2, __uint_as_float(r[c]), __uint_as_float(r[c + 1]));
+                        for (int c = kFirst; c < kCols; c += 2) m2 = max3(m2, __uint_as_float(r[c]), __uint_as_float(r[c + 1]));
+                    }
                     fast = !__any_sync(0xffffffffu, !(s1 <= kPieceSumBound) || m2 * a.scale_log2 > m_used + kRescaleThreshold);
                 }
                 if (!fast) {
                     tmem_wait_st();          // stores to the same columns have no order among themselves
-                    const float m_tile = row_max128(r) * a.scale_log2;
+                    const float m_tile = row_max(r) * a.scale_log2;
                     const float m_new = next_max(m_tile, m_used, l_run, tile_max);
                     if (__any_sync(0xffffffffu, m_new != m_used)) {
                         if (kSingle && t > 0) {
@@ -1069,7 +1093,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                         }
                     }
                     neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
-                    s1 = exp_row128<0, kFirstKeys>(r, a.scale_log2, neg_m, tS);
+                    s1 = exp_row<0, kFirst>(r, a.scale_log2, neg_m, tS);
                 }
                 l_run += s1;
                 // P goes to the MMA issuer in two pieces, so that the first piece of the PV product runs while the
@@ -1078,34 +1102,62 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_p);
-                l_run += exp_row128<kFirstKeys, 128>(r, a.scale_log2, neg_m, tS);
+                if constexpr (!kHalves) {                            // otherwise the rest of the row is the other warpgroup's
+                    l_run += exp_row<kFirst, kCols>(r, a.scale_log2, neg_m, tS);
 
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_p2);
+                    tmem_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_p2);
+                }
             }
             if (!ok) break;
 
             // ---- epilogue: normalise and store this thread's row ----
             if (n > 0) {
+                if (kHalves) {
+                    half_ml[s * kTileM + row] = make_float2(m_used, l_run);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_half);
+                    ok = mbar_wait(bar_half, o_cnt & 1, abort_flag, a.status);
+                }
                 ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_of, o_cnt & 1, abort_flag, a.status));
                 ++o_cnt;
                 if (!ok) break;
                 tc_fence_after();
-                const int in_tile = row_t >> a.pack_shift, token = (s ? it.token0_b : it.token0_a) + in_tile;
+                float w_own = 1.f, w_other = 0.f;
+                if (kHalves) {
+                    const float2 other = half_ml[(s ^ 1) * kTileM + row];
+                    const float m_row = fmaxf(m_used, other.x);
+                    w_own = m_used == -INFINITY ? 0.f : ex2(m_used - m_row);
+                    w_other = other.x == -INFINITY ? 0.f : ex2(other.x - m_row);
+                    l_run = w_own * l_run + w_other * other.y;
+                    m_used = m_row;
+                }
+                const int in_tile = row_t >> a.pack_shift, token = (tile ? it.token0_b : it.token0_a) + in_tile;
                 const int head = it.head0 + (row_t & ((1 << a.pack_shift) - 1));
                 const int part = kQuad ? it.part * 4 + (warp & 3) : it.part;
                 bool store = token < a.n_tokens;
-                if (a.mode != kModePhase2) store = store && (s ? it.row0_b : it.row0_a) + in_tile < it.main_len;
+                if (a.mode != kModePhase2) store = store && (tile ? it.row0_b : it.row0_a) + in_tile < it.main_len;
                 const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
                 const float lse = (l_run > 0.f) ? (m_used + log2f(l_run)) * 0.6931471805599453f : -INFINITY;
                 const size_t orow = static_cast<size_t>(token) * a.Hq + head;
                 // The whole accumulator row goes to registers first (the logits' registers are free by
                 // now), so that the accumulator can be handed back before the row is scaled and stored.
-                uint32_t o[D];
+                constexpr int kOut = kHalves ? D / 2 : D;          // of the row's outputs, this thread's
+                const int out0 = kHalves ? s * kOut : 0;
+                uint32_t o[kOut];
 #pragma unroll
-                for (int c0 = 0; c0 < D; c0 += 32) PULSAR_TMEM_LD32_AT(tO + c0, o, c0);
+                for (int c0 = 0; c0 < kOut; c0 += 32) PULSAR_TMEM_LD32_AT(tO + out0 + c0, o, c0);
+                if (kHalves) {
+                    uint32_t x[kOut];
+#pragma unroll
+                    for (int c0 = 0; c0 < kOut; c0 += 32) PULSAR_TMEM_LD32_AT(tO_other + out0 + c0, x, c0);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < kOut; ++c)
+                        o[c] = __float_as_uint(__uint_as_float(o[c]) * w_own + __uint_as_float(x[c]) * w_other);
+                }
                 tmem_wait_ld();
                 tc_fence_before();
                 __syncwarp();
@@ -1115,26 +1167,26 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
                     // out in two halves and an item's rows took about 5000 cycles; whole 32-byte sectors per store:
                     // Phase 1 at 16K 0.714 -> 0.701 ms, at 64K 6.05 -> 6.02 ms.
                     if (a.part_O != nullptr) {
-                        float* dst = a.part_O + (static_cast<size_t>(part) * a.n_tokens * a.Hq + orow) * D;
+                        float* dst = a.part_O + (static_cast<size_t>(part) * a.n_tokens * a.Hq + orow) * D + out0;
 #pragma unroll
-                        for (int c = 0; c < D; c += 8) {
+                        for (int c = 0; c < kOut; c += 8) {
                             uint32_t v[8];
 #pragma unroll
                             for (int k = 0; k < 8; ++k) v[k] = __float_as_uint(__uint_as_float(o[c + k]) * inv_l);
                             store_32b(dst + c, v, a.out_wide);
                         }
-                        a.part_LSE[static_cast<size_t>(part) * a.n_tokens * a.Hq + orow] = lse;
+                        if (out0 == 0) a.part_LSE[static_cast<size_t>(part) * a.n_tokens * a.Hq + orow] = lse;
                     } else {
-                        uint16_t* dst = a.O + orow * D;
+                        uint16_t* dst = a.O + orow * D + out0;
 #pragma unroll
-                        for (int c = 0; c < D; c += 16) {
+                        for (int c = 0; c < kOut; c += 16) {
                             uint32_t v[8];
 #pragma unroll
                             for (int k = 0; k < 8; ++k)
                                 v[k] = pack_bf16x2(__uint_as_float(o[c + 2 * k]) * inv_l, __uint_as_float(o[c + 2 * k + 1]) * inv_l);
                             store_32b(dst + c, v, a.out_wide);
                         }
-                        if (a.LSE != nullptr) a.LSE[orow] = lse;
+                        if (out0 == 0 && a.LSE != nullptr) a.LSE[orow] = lse;
                     }
                 }
             }
@@ -1263,7 +1315,7 @@ int causal_pack_shift(int32_t Hq, int32_t Hkv, int32_t d) {
 }
 
 // Causal attention with few items takes work items of one query tile instead of two: twice the items, and a key tile costs
-// the chain of one tile (0.88 us with d = 64, 0.91 with d = 128; an item 2.2 and 2.8 us more) instead of two interleaved
+// the chain of one tile (0.79 us with d = 64, 0.84 with d = 128; an item 2.5 and 2.8 us more) instead of two interleaved
 // ones (1.39 and 1.51 us, 3.0 and 3.4 us).  While every tile has an SM of its own that is the shorter time, and with more pairs than
 // SMs the pair is the better unit.  Between the two, tiles that cost alike are walked two after the other and lose
 // (one block of 1024 of 32 heads, d = 64, behind 8192 prefix rows: 130 us against 110), tiles that differ are dealt out
@@ -1279,7 +1331,7 @@ constexpr int kMaxCausalRuns = 512;             // more runs than that are more 
 
 bool causal_single(const CausalRun* runs, int n_runs, int64_t heads, int tile_tokens, int32_t d) {
     const int sms = sm_count();
-    struct { int64_t tile, item; } const cost[2] = {{d == 64 ? 882 : 906, d == 64 ? 2185 : 2761},
+    struct { int64_t tile, item; } const cost[2] = {{d == 64 ? 785 : 840, d == 64 ? 2500 : 2760},
                                                     {d == 64 ? 1392 : 1513, d == 64 ? 2986 : 3390}};     // ns, of one tile and of a pair
     const auto items = [&](int64_t tokens) {
         int64_t n = 0;
