@@ -12,8 +12,8 @@ LIB = os.path.join(HERE, "libpulsar.so")
 NATIVE = os.path.join(HERE, "_native.so")
 NATIVE_SOURCE = os.path.join(CSRC, "binding.cpp")
 NATIVE_KEY = os.path.join(HERE, "build", "_native.key")     # what NATIVE was compiled against
-SOURCES = ["api.cu", "select.cu", "merge.cu", "attn.cu", "rope.cu"]
-HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(os.path.dirname(HERE), "include", "pulsar.h")]
+SOURCES = ["api.cu", "select.cu", "merge.cu", "attn.cu", "decode.cu", "rope.cu"]
+HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "decode.cuh"), os.path.join(os.path.dirname(HERE), "include", "pulsar.h")]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
     "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
@@ -39,7 +39,7 @@ def native_key() -> str:
 
 
 def _native_stale() -> bool:
-    if _stale(NATIVE, [NATIVE_SOURCE, HEADERS[1]]) or not os.path.exists(NATIVE_KEY):
+    if _stale(NATIVE, [NATIVE_SOURCE, HEADERS[-1]]) or not os.path.exists(NATIVE_KEY):
         return True
     with open(NATIVE_KEY) as f:
         return f.read() != native_key()

@@ -24,11 +24,9 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "decode.cuh"
 
 namespace pulsar {
-
-int32_t launch_lse_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t rows, int32_t d,
-                         uint16_t* O, float* LSE, cudaStream_t stream);
 
 namespace {
 
@@ -1712,11 +1710,13 @@ extern "C" size_t pulsar_phase2_workspace_bytes(int32_t nq, int32_t B, int32_t b
     return n_splits == 1 ? 256 : a + b + 256;              // partials and the work counter
 }
 
-extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint16_t* Kb, const uint16_t* Vb,
-                                      int32_t B, int32_t block_size, int32_t Hq, int32_t Hkv, int32_t d,
-                                      float softmax_scale, int32_t n_splits, uint16_t* O, float* LSE, float* part_O,
-                                      float* part_LSE, void* workspace, size_t workspace_bytes,
-                                      int32_t* device_status, void* stream_) {
+namespace {
+// pulsar_phase2_attn up to the merge, which is left to the caller (todo).
+int32_t phase2_launch(const uint16_t* Qq, int32_t nq, const uint16_t* Kb, const uint16_t* Vb, int32_t B, int32_t block_size,
+                      int32_t Hq, int32_t Hkv, int32_t d, float softmax_scale, int32_t n_splits, uint16_t* O, float* LSE,
+                      float* part_O, float* part_LSE, void* workspace, size_t workspace_bytes, int32_t* device_status,
+                      MergeTodo& todo, void* stream_) {
+    todo = {};
     size_t po_bytes, pl_bytes;
     const bool user_parts = part_O != nullptr;
     if ((part_O == nullptr) != (part_LSE == nullptr)) return PULSAR_ERR_INVALID_ARG;
@@ -1740,6 +1740,24 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
 
     const int64_t L = static_cast<int64_t>(B) * block_size;
     const int g = Hq / Hkv;
+    const float scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
+    if (!user_parts && decode_takes(nq, Hq, Hkv, L)) {
+        DecodeCall c{};
+        c.Q = Qq;
+        c.n = nq;
+        c.Hq = Hq;
+        c.Hkv = Hkv;
+        c.d = d;
+        c.K = Kb;
+        c.V = Vb;
+        c.ctx_len = L;
+        c.scale_log2 = scale_log2;
+        c.O = O;
+        c.LSE = LSE;
+        c.workspace = workspace;
+        c.max_parts = need_ws ? static_cast<int64_t>(n_splits) * copies : 0;
+        return launch_decode(c, todo, stream);
+    }
     CUtensorMap tmQ, tmK, tmV;
     if (!make_map_3d(&tmQ, Qq, nq, Hq, d, g, (quad ? 32 : kTileM) / g) ||
         !make_map_2d(&tmK, Kb, L, static_cast<int64_t>(Hkv) * d) ||
@@ -1760,7 +1778,7 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
     a.split_len = static_cast<int>(phase2_split_len(L, n_splits));
     a.kv_len = static_cast<int>(L);
     a.quad = quad ? 1 : 0;
-    a.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
+    a.scale_log2 = scale_log2;
     a.O = O;
     a.LSE = LSE;
     a.part_O = partial_out ? pO : nullptr;
@@ -1781,10 +1799,26 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
     }
     rc = d == 128 ? launch_attn<128>(tmQ, tmK, tmV, tmK, tmV, a, stream)
                   : launch_attn<64>(tmQ, tmK, tmV, tmK, tmV, a, stream);
-    if (rc != PULSAR_OK) return rc;
-    if (partial_out)
-        return launch_lse_merge(pO, pL, n_splits * copies, static_cast<int64_t>(nq) * Hq, d, O, LSE, stream);
-    return PULSAR_OK;
+    if (rc == PULSAR_OK && partial_out) todo = {pO, pL, n_splits * copies};
+    return rc;
+}
+
+int32_t merge_launch(const MergeTodo& todo, int32_t nq, int32_t Hq, int32_t d, uint16_t* O, float* LSE, void* stream) {
+    if (todo.n_parts == 0) return PULSAR_OK;
+    return launch_lse_merge(todo.part_O, todo.part_LSE, todo.n_parts, static_cast<int64_t>(nq) * Hq, d, O, LSE,
+                            static_cast<cudaStream_t>(stream));
+}
+}  // namespace
+
+extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint16_t* Kb, const uint16_t* Vb,
+                                      int32_t B, int32_t block_size, int32_t Hq, int32_t Hkv, int32_t d,
+                                      float softmax_scale, int32_t n_splits, uint16_t* O, float* LSE, float* part_O,
+                                      float* part_LSE, void* workspace, size_t workspace_bytes,
+                                      int32_t* device_status, void* stream) {
+    MergeTodo todo;
+    const int32_t rc = phase2_launch(Qq, nq, Kb, Vb, B, block_size, Hq, Hkv, d, softmax_scale, n_splits, O, LSE, part_O, part_LSE,
+                                     workspace, workspace_bytes, device_status, todo, stream);
+    return rc != PULSAR_OK ? rc : merge_launch(todo, nq, Hq, d, O, LSE, stream);
 }
 
 // =============================================================================================
@@ -1832,6 +1866,31 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
 
     const int64_t L = static_cast<int64_t>(B) * block_size;
     const int g = Hq / Hkv;
+    const float scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
+    if (decode_takes(n_new, Hq, Hkv, L)) {
+        DecodeCall c{};
+        c.Q = Qnew;
+        c.n = n_new;
+        c.Hq = Hq;
+        c.Hkv = Hkv;
+        c.d = d;
+        c.K = Kb;
+        c.V = Vb;
+        c.ctx_len = L;
+        c.Kgen = Kgen;
+        c.Vgen = Vgen;
+        c.Knew = Knew;
+        c.Vnew = Vnew;
+        c.gen_len = gen_len;
+        c.scale_log2 = scale_log2;
+        c.O = O;
+        c.LSE = LSE;
+        c.workspace = workspace;
+        c.max_parts = static_cast<int64_t>(n_splits + 1) * copies;
+        MergeTodo todo;
+        rc = launch_decode(c, todo, stream);
+        return rc != PULSAR_OK ? rc : merge_launch(todo, n_new, Hq, d, O, LSE, stream);
+    }
     const size_t row_bytes = static_cast<size_t>(Hkv) * d * 2;
     CUtensorMap tmQ, tmK, tmV, tmKg, tmVg;
     if (!make_map_3d(&tmQ, Qnew, n_new, Hq, d, g, (quad ? 32 : kTileM) / g) ||
@@ -1860,7 +1919,7 @@ extern "C" int32_t pulsar_phase2_generate_step(const uint16_t* Qnew, const uint1
     a.gen_len = gen_len;
     a.gen_total = gen_len + n_new;
     a.quad = quad ? 1 : 0;
-    a.scale_log2 = (softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf(static_cast<float>(d))) * 1.4426950408889634f;
+    a.scale_log2 = scale_log2;
     a.O = O;
     a.LSE = LSE;
     a.part_O = pO;

@@ -19,6 +19,10 @@ void    count_launch(int n = 1);              // adds to the process-wide kernel
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Merge of an attention launch's partials [n_parts, rows, d] into bf16 (merge.cu).
+int32_t launch_lse_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t rows, int32_t d,
+                         uint16_t* O, float* LSE, cudaStream_t stream);
+
 // Kernel launch, optionally with programmatic stream serialization: a dependent launch may be
 // scheduled while the launch before it on the stream still runs (that launch must call
 // grid_launch_dependents) and waits for it with grid_dependency_wait before it touches its results.
