@@ -390,6 +390,25 @@ int32_t pulsar_phase2_attn(const uint16_t *Qq, int32_t nq,
                            int32_t *device_status, void *stream);
 
 /* ------------------------------------------------------------------------------------------
+ * One layer of one context (Algorithm 1 lines 3-13 on one GPU): pulsar_maxidf_select, pulsar_phase1_attn on the prefix it
+ * selects, and pulsar_phase2_attn of the query over all L retained rows, which are K and V themselves.  Arguments,
+ * requirements, workspaces and results are those of the three calls (Phase 2 with B = 1, block_size = L and no caller
+ * partials; prefix_total = sink + (B - 1) * k * chunk entries of prefix_idx); what does not depend on each other is overlapped
+ * on the device.  A call that is refused may have written the outputs of the parts before the one that refused it.
+ * ------------------------------------------------------------------------------------------ */
+int32_t pulsar_encode_step(const uint32_t *token_ids, int64_t L, int32_t vocab_size,
+                           int32_t block_size, int32_t chunk, int32_t k, int32_t sink,
+                           int32_t *sel_chunks, int32_t *prefix_idx, int32_t *prefix_len,
+                           void *select_workspace, size_t select_workspace_bytes,
+                           const uint16_t *Q, const uint16_t *K, const uint16_t *V,
+                           int32_t Hq, int32_t Hkv, int32_t d, int32_t prefix_total,
+                           float softmax_scale, uint16_t *O, float *LSE,
+                           void *phase1_workspace, size_t phase1_workspace_bytes,
+                           const uint16_t *Qq, int32_t nq, int32_t n_splits, uint16_t *O2, float *LSE2,
+                           void *phase2_workspace, size_t phase2_workspace_bytes,
+                           int32_t *device_status, void *stream);
+
+/* ------------------------------------------------------------------------------------------
  * Phase-2 generation step (Algorithm 1 lines 11-16; Section 3.2).
  *
  * The n_new newest tokens (the whole query on the first step, one generated token afterwards)

@@ -38,7 +38,7 @@ EXPORTS = (
     "pulsar_phase2_choose_splits", "pulsar_phase2_workspace_bytes", "pulsar_phase2_attn",
     "pulsar_phase2_generate_workspace_bytes", "pulsar_phase2_generate_step",
     "pulsar_lse_merge", "pulsar_lse_merge_strided", "pulsar_lse_merge_peers",
-    "pulsar_assemble_positions", "pulsar_rope_apply", "pulsar_rope_apply_qk",
+    "pulsar_assemble_positions", "pulsar_rope_apply", "pulsar_rope_apply_qk", "pulsar_encode_step",
 )
 
 
@@ -288,6 +288,18 @@ def pulsar_phase2_attn(Qq, Kblocks, Vblocks, n_blocks: int, block_size: int, sof
     res = _native_module().phase2_attn(Qq, Kblocks, Vblocks, n_blocks, block_size, softmax_scale, n_splits, want_partials, out,
                                        lse_out, workspace, status, pO, pL)
     return res if want_partials or partials is not None else res[:2]
+
+
+def pulsar_encode_step(token_ids, vocab_size: int, block_size: int, chunk: int, k: int, sink: int, Q, K, V, Qq, sel_out, O, LSE,
+                       O2, LSE2, workspaces, softmax_scale: float = 0.0, n_splits: int = 0, status=None):
+    """One layer of one context in one call: ``pulsar_maxidf_select``, ``pulsar_phase1_attn`` on the prefix it selects, and
+    ``pulsar_phase2_attn`` of ``Qq`` over all of K, V; the same results, with what does not depend on each other
+    overlapped.  Everything is preallocated: ``sel_out`` as ``out`` of the selection, O, LSE, O2, LSE2 the outputs, ``workspaces``
+    the three calls' (selection, Phase 1, Phase 2).  Returns the selection's dict."""
+    sel, prefix_idx, prefix_len = _native_module().encode_step(
+        token_ids, vocab_size, block_size, chunk, k, sink, Q, K, V, Qq, softmax_scale, n_splits, status, *sel_out, O, LSE, O2, LSE2,
+        *workspaces)
+    return dict(sel_chunks=sel, prefix_idx=prefix_idx, prefix_len=prefix_len)
 
 
 def pulsar_phase2_generate_step(Qnew, Knew, Vnew, Kblocks, Vblocks, n_blocks: int, block_size: int, Kgen, Vgen,

@@ -88,6 +88,7 @@ struct AttnArgs {
     float* LSE;            // f32  [tokens, Hq] or null
     float* part_O;         // f32  [parts, tokens, Hq, d] (partial output mode) or null
     float* part_LSE;       // f32  [parts, tokens, Hq]
+    int beside;            // phase 2: see launch_lse_merge
     int out_wide;          // the base of O (or part_O) is 32-byte aligned
     int32_t* status;
 };
@@ -565,7 +566,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
     // The CTAs of this launch may have been placed while the launch before it was still running; everything above
     // (barriers, tensor maps, TMEM) overlaps its end, nothing below may.
-    grid_dependency_wait();
+    if (!a.beside) grid_dependency_wait();
     // The launch that follows (the merge of this launch's partials, or another call's) may be placed as
     // SMs become free; it waits for this grid to finish before it reads anything.
     grid_launch_dependents();
@@ -1196,6 +1197,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
+    if (a.beside) grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1715,7 +1717,7 @@ namespace {
 int32_t phase2_launch(const uint16_t* Qq, int32_t nq, const uint16_t* Kb, const uint16_t* Vb, int32_t B, int32_t block_size,
                       int32_t Hq, int32_t Hkv, int32_t d, float softmax_scale, int32_t n_splits, uint16_t* O, float* LSE,
                       float* part_O, float* part_LSE, void* workspace, size_t workspace_bytes, int32_t* device_status,
-                      MergeTodo& todo, void* stream_) {
+                      bool beside, MergeTodo& todo, void* stream_) {
     todo = {};
     size_t po_bytes, pl_bytes;
     const bool user_parts = part_O != nullptr;
@@ -1756,6 +1758,7 @@ int32_t phase2_launch(const uint16_t* Qq, int32_t nq, const uint16_t* Kb, const 
         c.LSE = LSE;
         c.workspace = workspace;
         c.max_parts = need_ws ? static_cast<int64_t>(n_splits) * copies : 0;
+        c.beside = beside;
         return launch_decode(c, todo, stream);
     }
     CUtensorMap tmQ, tmK, tmV;
@@ -1778,6 +1781,7 @@ int32_t phase2_launch(const uint16_t* Qq, int32_t nq, const uint16_t* Kb, const 
     a.split_len = static_cast<int>(phase2_split_len(L, n_splits));
     a.kv_len = static_cast<int>(L);
     a.quad = quad ? 1 : 0;
+    a.beside = beside ? 1 : 0;
     a.scale_log2 = scale_log2;
     a.O = O;
     a.LSE = LSE;
@@ -1803,10 +1807,10 @@ int32_t phase2_launch(const uint16_t* Qq, int32_t nq, const uint16_t* Kb, const 
     return rc;
 }
 
-int32_t merge_launch(const MergeTodo& todo, int32_t nq, int32_t Hq, int32_t d, uint16_t* O, float* LSE, void* stream) {
+int32_t merge_launch(const MergeTodo& todo, int32_t nq, int32_t Hq, int32_t d, uint16_t* O, float* LSE, void* stream, bool beside = false) {
     if (todo.n_parts == 0) return PULSAR_OK;
     return launch_lse_merge(todo.part_O, todo.part_LSE, todo.n_parts, static_cast<int64_t>(nq) * Hq, d, O, LSE,
-                            static_cast<cudaStream_t>(stream));
+                            static_cast<cudaStream_t>(stream), beside);
 }
 }  // namespace
 
@@ -1817,8 +1821,33 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
                                       int32_t* device_status, void* stream) {
     MergeTodo todo;
     const int32_t rc = phase2_launch(Qq, nq, Kb, Vb, B, block_size, Hq, Hkv, d, softmax_scale, n_splits, O, LSE, part_O, part_LSE,
-                                     workspace, workspace_bytes, device_status, todo, stream);
+                                     workspace, workspace_bytes, device_status, false, todo, stream);
     return rc != PULSAR_OK ? rc : merge_launch(todo, nq, Hq, d, O, LSE, stream);
+}
+
+// =============================================================================================
+// One layer of a context: selection, Phase 1 and the Phase-2 attention of its query
+// =============================================================================================
+// Phase 2 needs nothing of Phase 1 but the keys and values that both read, so its attention is launched beside the
+// selection, which is a chain of latencies on 16 SMs, and its merge beside Phase 1.
+extern "C" int32_t pulsar_encode_step(const uint32_t* token_ids, int64_t L, int32_t vocab_size, int32_t block_size, int32_t chunk,
+                                      int32_t k, int32_t sink, int32_t* sel_chunks, int32_t* prefix_idx, int32_t* prefix_len,
+                                      void* select_workspace, size_t select_workspace_bytes, const uint16_t* Q, const uint16_t* K,
+                                      const uint16_t* V, int32_t Hq, int32_t Hkv, int32_t d, int32_t prefix_total,
+                                      float softmax_scale, uint16_t* O, float* LSE, void* phase1_workspace,
+                                      size_t phase1_workspace_bytes, const uint16_t* Qq, int32_t nq, int32_t n_splits,
+                                      uint16_t* O2, float* LSE2, void* phase2_workspace, size_t phase2_workspace_bytes,
+                                      int32_t* device_status, void* stream) {
+    int32_t rc = pulsar_maxidf_select(token_ids, L, vocab_size, block_size, chunk, k, sink, sel_chunks, prefix_idx, prefix_len, nullptr,
+                                      nullptr, select_workspace, select_workspace_bytes, device_status, stream);
+    if (rc != PULSAR_OK) return rc;
+    MergeTodo todo;
+    rc = phase2_launch(Qq, nq, K, V, 1, static_cast<int32_t>(L), Hq, Hkv, d, softmax_scale, n_splits, O2, LSE2, nullptr, nullptr,
+                       phase2_workspace, phase2_workspace_bytes, device_status, true, todo, stream);
+    if (rc != PULSAR_OK) return rc;
+    rc = pulsar_phase1_attn(Q, K, V, L, Hq, Hkv, d, block_size, prefix_total > 0 ? prefix_idx : nullptr, prefix_len, prefix_total,
+                            softmax_scale, O, LSE, nullptr, nullptr, phase1_workspace, phase1_workspace_bytes, device_status, stream);
+    return rc != PULSAR_OK ? rc : merge_launch(todo, nq, Hq, d, O2, LSE2, stream, true);
 }
 
 // =============================================================================================

@@ -25,7 +25,7 @@ namespace {
     X(pulsar_gather_kv_rows) X(pulsar_phase1_attn_sharded) X(pulsar_causal_varlen_attn) X(pulsar_retain_block_kv)  \
     X(pulsar_phase2_choose_splits) X(pulsar_phase2_workspace_bytes) X(pulsar_phase2_attn)                          \
     X(pulsar_phase2_generate_workspace_bytes) X(pulsar_phase2_generate_step) X(pulsar_lse_merge_strided)           \
-    X(pulsar_rope_apply_qk)
+    X(pulsar_rope_apply_qk) X(pulsar_encode_step)
 
 struct Entries {
 #define X(name) decltype(&::name) name = nullptr;
@@ -418,6 +418,33 @@ PyObject* phase2_generate_step(Args& a) {
     return result({out, lse});
 }
 
+// (token_ids, vocab, block, chunk, k, sink, Q, K, V, Qq, scale, n_splits, status, sel_buf, prefix_idx, prefix_len, O1, LSE1, O2,
+//  LSE2, ws_select, ws_phase1, ws_phase2): the three calls of a step with everything preallocated
+PyObject* encode_step(Args& a) {
+    at::Tensor ids = a.i32s("token_ids");
+    SelectShape z(a, ids.numel());
+    Qkv x(a);
+    Query y;
+    y.Q = a.bf16("Qq", 3);
+    y.K = x.K;
+    y.V = x.V;
+    y.shape();
+    const float scale = static_cast<float>(a.real());
+    const int32_t splits = a.i32();
+    at::Tensor status = a.tensor(), sel = a.i32s("sel_chunks"), pidx = a.i32s("prefix_idx"), plen = a.i32s("prefix_len"), O1 = a.tensor(),
+               LSE1 = a.tensor(), O2 = a.tensor(), LSE2 = a.tensor(), ws_s = a.tensor(), ws_1 = a.tensor(), ws_2 = a.tensor();
+    if (x.rows != z.L) raise(PyExc_ValueError, "one token id per row of Q, K and V");
+    call("pulsar_encode_step", [&, st = stream()] {
+        return g.pulsar_encode_step(ptr<uint32_t>(ids), z.L, z.V, z.block, z.chunk, z.k, z.sink, ptr<int32_t>(sel), ptr<int32_t>(pidx),
+                                    ptr<int32_t>(plen), ptr<void>(ws_s), static_cast<size_t>(ws_s.numel()), in16(x.Q), in16(x.K),
+                                    in16(x.V), x.Hq, x.Hkv, x.d, static_cast<int32_t>(z.prefix()), scale, ptr<uint16_t>(O1),
+                                    ptr<float>(LSE1), ptr<void>(ws_1), static_cast<size_t>(ws_1.numel()), in16(y.Q), y.nq, splits,
+                                    ptr<uint16_t>(O2), ptr<float>(LSE2), ptr<void>(ws_2), static_cast<size_t>(ws_2.numel()),
+                                    ptr<int32_t>(status), st);
+    });
+    return result({head(sel, z.B * z.k).view({z.B, z.k}), head(pidx, z.prefix()), head(plen, z.B)});
+}
+
 // (part_O, part_LSE, n_parts, stride_O, stride_LSE, rows, d, out, lse_out)
 PyObject* lse_merge_strided(Args& a) {
     at::Tensor pO = a.needed(at::kFloat, "part_O"), pL = a.needed(at::kFloat, "part_LSE");
@@ -473,7 +500,7 @@ PyObject* bind(Args& a) {
 #define M(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(entry<name>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {M(bind), M(maxidf_select), M(chunk_select), M(phase1_attn), M(phase1_attn_sharded), M(causal_varlen_attn),
                          M(retain_block_kv), M(pack_summary_kv), M(gather_kv_rows), M(phase2_attn), M(phase2_generate_step),
-                         M(lse_merge_strided), M(rope_apply_qk), {nullptr, nullptr, 0, nullptr}};
+                         M(lse_merge_strided), M(rope_apply_qk), M(encode_step), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

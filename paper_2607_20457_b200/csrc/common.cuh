@@ -20,8 +20,11 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Merge of an attention launch's partials [n_parts, rows, d] into bf16 (merge.cu).
+// beside: the launch before it on the stream is one whose CTAs have all found complete what this one reads and touch none of
+// what it writes (they let their dependents in after their own wait).  The kernel then works beside that launch and waits for
+// it at its end, so that whatever waits for this one still waits for both.
 int32_t launch_lse_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t rows, int32_t d,
-                         uint16_t* O, float* LSE, cudaStream_t stream);
+                         uint16_t* O, float* LSE, cudaStream_t stream, bool beside = false);
 
 // Kernel launch, optionally with programmatic stream serialization: a dependent launch may be
 // scheduled while the launch before it on the stream still runs (that launch must call

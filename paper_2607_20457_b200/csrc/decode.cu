@@ -39,6 +39,7 @@ struct DecodeArgs {
     int Hq, Hkv, g_shift, n_rows;                // n_rows = n * g query rows of a KV head
     int cluster_shift, clusters;                 // log2 of the CTAs per cluster, clusters per KV head
     float scale_log2;
+    int beside;                                  // see launch_lse_merge
     uint16_t* O;
     float* LSE;
     float *part_O, *part_LSE;                    // clusters > 1: [clusters, n, Hq, D] and [clusters, n, Hq]
@@ -122,7 +123,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
     const int C = 1 << a.cluster_shift;
 
     if (C > 1) cluster_arrive();                               // waited for before another CTA's memory is written
-    grid_dependency_wait();
+    if (!a.beside) grid_dependency_wait();
     grid_launch_dependents();
 
     // ---- this CTA's pieces of kKeys keys: the context's first, then the shard's ----
@@ -386,6 +387,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
             if (at_d == 0 && a.LSE != nullptr) a.LSE[row] = lse;
         }
     }
+    if (a.beside) grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -473,6 +475,7 @@ int32_t launch_decode_as(const DecodeCall& c, const DecodePlan& p, MergeTodo& to
     a.cluster_shift = p.shift;
     a.clusters = p.clusters;
     a.scale_log2 = c.scale_log2;
+    a.beside = c.beside ? 1 : 0;
     a.O = c.O;
     a.LSE = c.LSE;
     a.part_rows = static_cast<int64_t>(c.n) * c.Hq;

@@ -18,6 +18,7 @@ struct DecodeCall {
     float* LSE;
     void* workspace;                             // for partials; max_parts of them fit (0: none)
     int64_t max_parts;
+    bool beside;                                 // see launch_lse_merge
 };
 
 // What is left of a Phase-2 call when its attention has been launched: the merge of n_parts partials (0: nothing).

@@ -12,8 +12,8 @@ template <bool kF32>
 __global__ void __launch_bounds__(256)
 lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ part_LSE, int n_parts,
                  int64_t stride_O, int64_t stride_L, int64_t rows, int d, void* __restrict__ O_,
-                 float* __restrict__ LSE) {
-    grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
+                 float* __restrict__ LSE, int beside) {
+    if (!beside) grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
     grid_launch_dependents();
     const int vec_per_row = d >> 2;
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -49,6 +49,7 @@ lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ par
         *reinterpret_cast<uint2*>(static_cast<uint16_t*>(O_) + row * d + v * 4) = packed;
     }
     if (LSE != nullptr && v == 0) LSE[row] = (m > -INFINITY) ? m + logf(denom) : -INFINITY;
+    if (beside) grid_dependency_wait();
 }
 
 // The same merge for rows of 32 * kVec floats (d = 64, 128): a warp loads a part's row as one contiguous run,
@@ -62,9 +63,9 @@ template <bool kF32, int kVec, int kWarps, int kRows>
 __global__ void __launch_bounds__(32 * kWarps * kRows)
 lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict__ part_LSE, int n_parts,
                       int64_t stride_O, int64_t stride_L, int64_t rows, void* __restrict__ O_,
-                      float* __restrict__ LSE) {
+                      float* __restrict__ LSE, int beside) {
     static_assert(kRows == 1 || kWarps == 1, "a CTA has one row, or one warp per row");
-    grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
+    if (!beside) grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
     grid_launch_dependents();
     constexpr int kD = 32 * kVec, kInFlight = 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -168,6 +169,7 @@ lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict_
         else *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(acc[0], acc[1]);
     }
     if (LSE != nullptr && lane == 0) LSE[row] = (m > -INFINITY) ? m + logf(denom) : -INFINITY;
+    if (beside) grid_dependency_wait();
 }
 
 // The merge with every part at its own address: part j is the buffer parts[j], laid out
@@ -249,7 +251,7 @@ int merge_warps(int32_t n_parts, int64_t rows, int32_t d) {
 }
 
 int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t stride_O, int64_t stride_L,
-                     int64_t rows, int32_t d, void* O, bool f32, float* LSE, cudaStream_t stream) {
+                     int64_t rows, int32_t d, void* O, bool f32, float* LSE, cudaStream_t stream, bool beside = false) {
     if (rows == 0) return PULSAR_OK;
     const int warps = (d == 64 || d == 128) ? merge_warps(n_parts, rows, d) : 0;
     if (warps > 0) {
@@ -258,7 +260,7 @@ int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts
         auto kernel = d == 128 ? (f32 ? merge_rows_kernel<true, 4>(warps) : merge_rows_kernel<false, 4>(warps))
                                : (f32 ? merge_rows_kernel<true, 2>(warps) : merge_rows_kernel<false, 2>(warps));
         PULSAR_CUDA_OK(launch_kernel(kernel, dim3(static_cast<unsigned>(blocks)), dim3(warps == 1 ? 256 : 32 * warps), 0, stream,
-                                     true, part_O, part_LSE, n_parts, stride_O, stride_L, rows, O, LSE));
+                                     true, part_O, part_LSE, n_parts, stride_O, stride_L, rows, O, LSE, beside ? 1 : 0));
         count_launch();
         return PULSAR_OK;
     }
@@ -267,7 +269,7 @@ int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts
     if (blocks > 0x7fffffffll) return PULSAR_ERR_SHAPE;
     auto kernel = f32 ? lse_merge_kernel<true> : lse_merge_kernel<false>;
     PULSAR_CUDA_OK(launch_kernel(kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, stream, true, part_O, part_LSE,
-                                 n_parts, stride_O, stride_L, rows, d, O, LSE));
+                                 n_parts, stride_O, stride_L, rows, d, O, LSE, beside ? 1 : 0));
     count_launch();
     return PULSAR_OK;
 }
@@ -275,9 +277,10 @@ int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts
 
 // Placed as the CTAs of the launch before it leave (programmatic stream serialization), waits until that has finished
 // (grid_dependency_wait): no launch gap separates the merge from the attention launch that writes the partials.
+// beside: see common.cuh.
 int32_t launch_lse_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t rows, int32_t d,
-                         uint16_t* O, float* LSE, cudaStream_t stream) {
-    return launch_merge(part_O, part_LSE, n_parts, rows * d, rows, rows, d, O, false, LSE, stream);
+                         uint16_t* O, float* LSE, cudaStream_t stream, bool beside) {
+    return launch_merge(part_O, part_LSE, n_parts, rows * d, rows, rows, d, O, false, LSE, stream, beside);
 }
 
 }  // namespace pulsar

@@ -59,25 +59,27 @@ class ContextEncoder:
     def step_device(self, ids, Q, K, V, Qq, record=None, slot=None):
         """Run selection, Phase 1 and Phase 2 on device tensors; outputs land in ``slot``
         (default: slot 0).  ``record``: optional list of four CUDA events recorded before,
-        between and after the three calls."""
+        between and after the three calls; without it they are one call that overlaps what it can."""
         w = self.w
         slot = self.slots[0] if slot is None else slot
-        if record:
-            record[0].record()
+        if not record and ids.numel() == Q.shape[0] == w.L:
+            sel = binding.pulsar_encode_step(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink, Q, K, V, Qq, slot["sel"],
+                                             slot["O1"], slot["LSE1"], slot["O2"], slot["LSE2"],
+                                             (self.ws_select, self.ws_p1, self.ws_p2), n_splits=self.n_splits, status=self.status)
+            return dict(sel=sel, O1=slot["O1"], LSE1=slot["LSE1"], O2=slot["O2"], LSE2=slot["LSE2"], prefix_idx=sel["prefix_idx"])
+        mark = lambda i: record[i].record() if record else None
+        mark(0)
         sel = binding.pulsar_maxidf_select(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink,
                                            workspace=self.ws_select, status=self.status, out=slot["sel"])
-        if record:
-            record[1].record()
+        mark(1)
         O1, LSE1, K_ret, V_ret = binding.pulsar_phase1_attn(
             Q, K, V, w.block_size, sel["prefix_idx"], sel["prefix_len"], out=slot["O1"], lse_out=slot["LSE1"],
             workspace=self.ws_p1, status=self.status)
-        if record:
-            record[2].record()
+        mark(2)
         O2, LSE2 = binding.pulsar_phase2_attn(Qq, K_ret, V_ret, *self.kv_shape, n_splits=self.n_splits,
                                               out=slot["O2"], lse_out=slot["LSE2"], workspace=self.ws_p2,
                                               status=self.status)
-        if record:
-            record[3].record()
+        mark(3)
         return dict(sel=sel, O1=O1, LSE1=LSE1, O2=O2, LSE2=LSE2, prefix_idx=sel["prefix_idx"])
 
     def capture_step(self, slot_index: int = 0):
