@@ -1,6 +1,7 @@
 // Max-IDF summary selection (Section 3.1, Eq. 2-4; Algorithm 1 lines 3 and 6).
 //
-// Four launches on one stream, no host synchronisation:
+// Up to 16 blocks of ordinary length are one launch, a cluster of a CTA per block (select_cluster_kernel).  Other problems take
+// four launches on one stream, no host synchronisation:
 //   presence_kernel   one CTA per block: a V-bit presence set of the block's token ids, built
 //                     with shared-memory atomicOr and written to the workspace
 //   df_idf_kernel     one thread per vocabulary entry: df(t) = number of blocks whose set holds
@@ -16,6 +17,7 @@
 // topk_score_kernel (rank by score, ties to the lower index).
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include <math_constants.h>
 
@@ -528,6 +530,351 @@ int32_t plan_select(int64_t L, int32_t vocab_size, int32_t block_size, int32_t c
     return PULSAR_OK;
 }
 
+// ---------------------------------------------------------------------------------------------
+// The whole selection in one launch, for sequences of at most 16 blocks: a CTA per block, the CTAs one cluster.
+// The presence sets stay in shared memory and are read there by the CTAs that form the df of a slice of the vocabulary
+// each; the df of the block's tokens, the chunks' ranks and the selected chunks are the CTA's own.  What crosses
+// CTAs are two cluster barriers instead of three launches, and the df table (a byte per entry, in L2).  Bound by a chain of
+// latencies: each thread's loads are issued together (one at a time: 45,011 tokens 10.2 us, 8.0 like this and with a look at
+// the presence bit before the atomic).
+// ---------------------------------------------------------------------------------------------
+constexpr int kClusterThreads = 1024;
+constexpr int kClusterBlocks = 16;              // CTAs of the largest cluster
+constexpr int kClusterTokens = 8192;            // of a block: its ids, and a term per id, are kept in shared memory
+constexpr int kClusterChunks = 1024;            // of a block: a thread each in the selection
+constexpr int kModeLevels = -1;                 // chunks ranked by their least df (pulsar_maxidf_select), without scores
+
+struct ClusterShape {
+    size_t bits, tokens, dfs, ranks, chosen, terms, total;       // offsets in shared memory
+    __host__ __device__ ClusterShape(int words, int block_size, int C, int chunk, int k, bool scores) {
+        const auto up = [](size_t x) { return (x + 15) / 16 * 16; };
+        bits = 0;
+        tokens = up(static_cast<size_t>(words) * 4);
+        dfs = tokens + up(static_cast<size_t>(block_size) * 4);
+        ranks = dfs + up(block_size);
+        chosen = ranks + up(static_cast<size_t>(C) * (scores ? 8 : 4));
+        terms = chosen + up(static_cast<size_t>(k) * 4);
+        // a term per position; chunks an odd number of terms apart, so that the threads that add them up meet in no bank
+        total = terms + (scores ? static_cast<size_t>(C) * (chunk | 1) * 8 : 0);
+    }
+};
+
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr, int rank) {
+    uint32_t v;
+    asm volatile("{\n\t.reg .u32 a;\n\tmapa.shared::cluster.u32 a, %1, %2;\n\tld.shared::cluster.u32 %0, [a];\n\t}"
+                 : "=r"(v) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, int rank, uint32_t v) {
+    asm volatile("{\n\t.reg .u32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.u32 [a], %2;\n\t}"
+                 ::"r"(addr), "r"(rank), "r"(v) : "memory");
+}
+
+// The position of the calling thread's chunk among those taken (one bit a thread, in thread order).
+__device__ __forceinline__ int taken_before(bool take, int* warp_sums) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t mine = __ballot_sync(0xffffffffu, take);
+    if (lane == 0) warp_sums[warp] = __popc(mine);
+    __syncthreads();
+    const int base = __reduce_add_sync(0xffffffffu, lane < warp ? warp_sums[lane] : 0);
+    __syncthreads();
+    return base + __popc(mine & ((1u << lane) - 1));
+}
+
+struct ClusterArgs {
+    const uint32_t* ids;
+    int64_t L;
+    int block_size, chunk, k, sink, vocab_size, words;
+    uint8_t* df_table;                          // [vocab_size rounded up to 32]
+    int32_t *sel_chunks, *prefix_idx, *prefix_len;
+    uint32_t* df_out;
+    float* idf_out;
+    double* score;                              // [blocks, C] or null
+    int32_t* status;
+};
+
+template <int kMode>
+__global__ void __launch_bounds__(kClusterThreads, 1)
+select_cluster_kernel(const __grid_constant__ ClusterArgs a,
+                      const __grid_constant__ std::conditional_t<kMode == kModeLevels, int, ScoreTable<kClusterBlocks>> tab) {
+    constexpr bool kScores = kMode != kModeLevels;
+    extern __shared__ __align__(16) uint8_t smem_c[];
+    __shared__ int s_warp[32], s_hist[32], s_short[kClusterBlocks], s_threshold, s_need;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = blockIdx.x, n_blocks = gridDim.x;
+    const int C = (a.block_size + a.chunk - 1) / a.chunk;
+    const ClusterShape at(a.words, a.block_size, C, a.chunk, a.k, kScores);
+    uint32_t* bits = reinterpret_cast<uint32_t*>(smem_c + at.bits);
+    uint32_t* tok = reinterpret_cast<uint32_t*>(smem_c + at.tokens);
+    uint8_t* dfs = smem_c + at.dfs;
+    int* chosen = reinterpret_cast<int*>(smem_c + at.chosen);
+    const uint32_t V = static_cast<uint32_t>(a.vocab_size);
+    const PrefixGeometry geo = prefix_geometry(b, n_blocks, a.L, a.block_size, a.chunk, a.k, a.sink);
+    const int64_t lo = static_cast<int64_t>(b) * a.block_size;
+    const int len_b = static_cast<int>(min(static_cast<int64_t>(a.block_size), a.L - lo));
+
+    for (int w = tid; w < a.words; w += kClusterThreads) bits[w] = 0u;
+    if (tid < 32) s_hist[tid] = 0;
+    grid_dependency_wait();            // the token ids, and the workspace, may be in use by the launch before this one
+    grid_launch_dependents();
+    __syncthreads();
+    constexpr int kPerThread = kClusterTokens / kClusterThreads;       // all of a thread's loads are under way at once
+    uint32_t mine_t[kPerThread];
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j) mine_t[j] = tid + j * kClusterThreads < len_b ? a.ids[lo + tid + j * kClusterThreads] : 0u;
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j) {
+        const int i = tid + j * kClusterThreads;
+        if (i >= len_b) break;
+        if (kMode == PULSAR_SCORE_BM25 || kMode == PULSAR_SCORE_TYPE_TOKEN) tok[i] = mine_t[j];
+        if (mine_t[j] < V) {
+            // (most tokens of a block repeat, and an atomic on a word that many lanes want is done lane by lane)
+            const uint32_t bit = 1u << (mine_t[j] & 31);
+            if ((*const_cast<volatile uint32_t*>(bits + (mine_t[j] >> 5)) & bit) == 0u) atomicOr(&bits[mine_t[j] >> 5], bit);
+        } else {
+            report(a.status, PULSAR_DEV_BAD_TOKEN);
+        }
+    }
+    cluster_sync();                    // every block's set is complete
+
+    // ---- df of this CTA's slice of the vocabulary: the sets' words added up bit by bit, 32 entries a thread ----
+    const int per_cta = (a.words + n_blocks - 1) / n_blocks, w_end = min(a.words, (b + 1) * per_cta);
+    for (int w = b * per_cta + tid; w < w_end; w += kClusterThreads) {
+        uint32_t x[kClusterBlocks], plane[5] = {0u, 0u, 0u, 0u, 0u};
+        const uint32_t addr = smem_u32(bits + w);
+#pragma unroll
+        for (int j = 0; j < kClusterBlocks; ++j) x[j] = j < n_blocks ? ld_cluster_u32(addr, j) : 0u;
+#pragma unroll
+        for (int j = 0; j < kClusterBlocks; ++j) {
+            uint32_t carry = x[j];
+#pragma unroll
+            for (int p = 0; p < 5; ++p) {
+                const uint32_t next = plane[p] & carry;
+                plane[p] ^= carry;
+                carry = next;
+            }
+        }
+        uint32_t out[8];
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {                          // four entries: bit i of a plane's nibble to byte i
+            out[n] = 0u;
+#pragma unroll
+            for (int p = 0; p < 5; ++p) out[n] |= ((((plane[p] >> (4 * n)) & 15u) * 0x00204081u) & 0x01010101u) << p;
+        }
+        uint4* dst = reinterpret_cast<uint4*>(a.df_table + static_cast<size_t>(w) * 32);
+        dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
+        dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        if (a.df_out != nullptr || a.idf_out != nullptr)
+            for (int i = 0; i < 32 && w * 32 + i < a.vocab_size; ++i) {
+                uint32_t df = 0;
+#pragma unroll
+                for (int p = 0; p < 5; ++p) df |= ((plane[p] >> i) & 1u) << p;
+                if (a.df_out != nullptr) a.df_out[w * 32 + i] = df;
+                if (a.idf_out != nullptr) a.idf_out[w * 32 + i] = logf(static_cast<float>(n_blocks) / static_cast<float>(df > 0 ? df : 1));
+            }
+    }
+    cluster_sync();                    // the table is complete
+    constexpr uint32_t kNoToken = 255;
+    uint32_t mine_df[kPerThread];
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j)
+        mine_df[j] = tid + j * kClusterThreads < len_b && mine_t[j] < V ? a.df_table[mine_t[j]] : kNoToken;
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j)
+        if (tid + j * kClusterThreads < len_b) dfs[tid + j * kClusterThreads] = static_cast<uint8_t>(mine_df[j]);
+    __syncthreads();
+
+    // ---- a rank per chunk slot: its least df, or its score; see chunk_level_kernel and chunk_score_kernel ----
+    const int k = geo.k_b;
+    int* level = reinterpret_cast<int*>(smem_c + at.ranks);
+    double* score = reinterpret_cast<double*>(smem_c + at.ranks);
+    bool take;
+    if constexpr (!kScores) {
+        for (int c = warp; c < C; c += kClusterThreads / 32) {
+            const int len = max(0, min(a.chunk, len_b - c * a.chunk));
+            uint32_t least = static_cast<uint32_t>(len > 0 ? n_blocks + 1 : n_blocks + 2);
+            for (int p = lane; p < len; p += 32) {
+                const uint32_t df = dfs[c * a.chunk + p];
+                if (df != kNoToken) least = min(least, df);
+            }
+            least = __reduce_min_sync(0xffffffffu, least);
+            if (lane == 0) level[c] = static_cast<int>(least);
+        }
+        __syncthreads();
+        for (int c0 = warp * 32; c0 < C; c0 += kClusterThreads) {                              // at most once
+            const int own = c0 + lane < C ? level[c0 + lane] : -1;
+            const uint32_t same = __match_any_sync(0xffffffffu, own);
+            if (own >= 0 && lane == __ffs(same) - 1) atomicAdd(&s_hist[own], __popc(same));
+        }
+        __syncthreads();
+        // threshold level: all chunks below it are taken, s_need more at it (lowest indices first)
+        if (warp == 0) {
+            int cum = s_hist[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int n = __shfl_up_sync(0xffffffffu, cum, o);
+                if (lane >= o) cum += n;
+            }
+            const uint32_t enough = __ballot_sync(0xffffffffu, cum >= k);
+            if (lane == __ffs(enough) - 1) {
+                s_threshold = lane;
+                s_need = k - (cum - s_hist[lane]);
+            }
+        }
+        __syncthreads();
+        const int mine = tid < C ? level[tid] : n_blocks + 3, T = s_threshold;
+        const int rank_T = taken_before(mine == T, s_warp);
+        take = mine < T || (mine == T && rank_T < s_need);
+    } else {
+        double* term = reinterpret_cast<double*>(smem_c + at.terms);
+        const int stride = a.chunk | 1;
+        for (int c = warp; c < C; c += kClusterThreads / 32) {
+            const int len = max(0, min(a.chunk, len_b - c * a.chunk));
+            const uint32_t* ct = tok + c * a.chunk;
+            const uint8_t* cd = dfs + c * a.chunk;
+            double* terms = term + c * stride;
+            if (kMode == PULSAR_SCORE_MAX_IDF) {               // the largest IDF is that of the least df
+                uint32_t least = kNoToken;
+                for (int p = lane; p < len; p += 32) least = min(least, static_cast<uint32_t>(cd[p]));
+                least = __reduce_min_sync(0xffffffffu, least);
+                if (lane == 0) score[c] = least == kNoToken ? -CUDART_INF : tab.by_df[least];
+                continue;
+            }
+            double k1_times_D = 0.0;
+            if (kMode == PULSAR_SCORE_BM25)
+                k1_times_D = __dmul_rn(
+                    tab.k1, __dadd_rn(tab.one_minus_b, __dmul_rn(tab.b, __ddiv_rn(static_cast<double>(len), tab.mean_len))));
+            int distinct = 0;
+            for (int p0 = 0; p0 < len; p0 += 32) {
+                const int p = p0 + lane;
+                const bool in = p < len;
+                bool first = in;
+                int tf = 0;
+                if (kMode != PULSAR_SCORE_TF_IDF) {
+                    const uint32_t t = in ? ct[p] : ~0u;
+                    if (len <= 32) {
+                        // (an id of ~0 meets the lanes past the end, which come after it: its count, unused, is too large)
+                        const uint32_t same = __match_any_sync(0xffffffffu, t);
+                        first = in && lane == __ffs(same) - 1;
+                        tf = __popc(same);
+                    } else {
+                        int before = 0;
+                        for (int q = 0; q < len; ++q) {
+                            const int eq = ct[q] == t ? 1 : 0;
+                            tf += eq;
+                            before += q < p ? eq : 0;
+                        }
+                        first = in && before == 0;
+                    }
+                }
+                if (kMode == PULSAR_SCORE_TYPE_TOKEN) {
+                    distinct += __popc(__ballot_sync(0xffffffffu, first));
+                } else if (in) {
+                    const uint32_t df = cd[p];
+                    double x = 0.0;
+                    if (first && df != kNoToken) {
+                        x = tab.by_df[df];
+                        if (kMode == PULSAR_SCORE_BM25) {
+                            const double tfd = static_cast<double>(tf);
+                            x = __ddiv_rn(__dmul_rn(x, __dmul_rn(tfd, tab.k1_plus_1)), __dadd_rn(tfd, k1_times_D));
+                        }
+                    }
+                    terms[p] = x;
+                }
+            }
+            if (kMode == PULSAR_SCORE_TYPE_TOKEN && lane == 0) score[c] = static_cast<double>(distinct);
+        }
+        __syncthreads();
+        if (kMode != PULSAR_SCORE_MAX_IDF && tid < C) {
+            const int len = max(0, min(a.chunk, len_b - tid * a.chunk));
+            double sum = kMode == PULSAR_SCORE_TYPE_TOKEN ? score[tid] : 0.0;
+            if (kMode != PULSAR_SCORE_TYPE_TOKEN) {            // in the order of the equations
+#pragma unroll 8
+                for (int p = 0; p < len; ++p) sum = __dadd_rn(sum, term[tid * stride + p]);
+            }
+            score[tid] = len == 0 ? -CUDART_INF : kMode == PULSAR_SCORE_BM25 ? sum : __ddiv_rn(sum, static_cast<double>(len));
+        }
+        // How many chunks beat each (a larger score, or the same at a lower index), counted by as many threads as there are to a chunk.
+        int* better = reinterpret_cast<int*>(term);            // [C]; the terms are used up
+        __syncthreads();
+        for (int c = tid; c < C; c += kClusterThreads) better[c] = 0;
+        __syncthreads();
+        const int Cb = (len_b + a.chunk - 1) / a.chunk, span = (C + 31) / 32 * 32, parts = kClusterThreads / span;
+        const int part = tid / span, c = tid - part * span;
+        if (part < parts && c < Cb) {
+            const double mine = score[c];
+            const int end = Cb * (part + 1) / parts, c_warp = c & ~31;
+            int n = 0, o = Cb * part / parts;
+#pragma unroll 4
+            for (; o < min(end, c_warp); ++o) n += score[o] >= mine ? 1 : 0;                       // before every lane's own
+            for (; o < min(end, c_warp + 32); ++o) n += (score[o] > mine || (score[o] == mine && o < c)) ? 1 : 0;
+#pragma unroll 4
+            for (; o < end; ++o) n += score[o] > mine ? 1 : 0;
+            atomicAdd(&better[c], n);
+        }
+        if (a.score != nullptr)
+            for (int i = tid; i < C; i += kClusterThreads) a.score[static_cast<size_t>(b) * C + i] = score[i];
+        __syncthreads();
+        take = tid < Cb && better[tid] < k;
+    }
+    const int pos = taken_before(take, s_warp);
+    if (take && pos < k) {
+        chosen[pos] = tid;
+        a.sel_chunks[static_cast<size_t>(b) * a.k + pos] = tid;
+    }
+    // ---- the prefix list; its entries are shifted by earlier blocks that selected their short last chunk ----
+    int offset = geo.sink_eff + b * a.k * a.chunk;
+    if (geo.tail != a.chunk && a.k > 0 && n_blocks > 1) {
+        const uint32_t is_short = tid == C - 1 && take && len_b == a.block_size ? 1u : 0u;
+        if (tid == C - 1)
+            for (int j = 0; j < n_blocks; ++j) st_cluster_u32(smem_u32(s_short + b), j, is_short);
+        cluster_sync();
+        int n_short = 0;
+        for (int j = 0; j < b; ++j) n_short += s_short[j];
+        offset -= n_short * (a.chunk - geo.tail);
+    }
+    __syncthreads();
+    write_block_prefix(b, n_blocks, a.block_size, a.chunk, a.k, geo, offset, chosen, a.sel_chunks, a.prefix_idx, a.prefix_len);
+}
+
+// Whether a selection of this shape is the cluster's: at most 16 blocks that their CTAs get through in less time than the host
+// takes for three launches more.  us a call in a row of them, one launch / four: levels, blocks of 1024 tokens 6.3 / 12.6, of
+// 4157 7.9 / 12.9, of 5000 8.0 / 12.6, of 8192 about even; BM25, 1024 8.6 / 15.2, 1665 13.7 / 15.4, 4157 15.6 / 15.5 (the
+// divisions of a block's terms are one SM's then), the other scores between the two.
+constexpr int kClusterLevelTokens = 6144, kClusterScoreTokens = 2048;
+bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32_t k, bool scores) {
+    return p.n_blocks <= kClusterBlocks && block_size <= (scores ? kClusterScoreTokens : kClusterLevelTokens) && p.C <= kClusterChunks &&
+           ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 1024 &&
+           static_cast<size_t>(p.words) * 32 <= p.df_bytes;
+}
+
+template <int kMode, typename Table>
+cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const Table& tab, cudaStream_t stream) {
+    const size_t smem = ClusterShape(p.words, args.block_size, p.C, args.chunk, args.k, kMode != kModeLevels).total;
+    auto kernel = select_cluster_kernel<kMode>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess && p.n_blocks > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(p.n_blocks);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(p.n_blocks);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, args, tab);
+}
+
 }  // namespace
 }  // namespace pulsar
 
@@ -557,6 +904,14 @@ extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, in
     if (rc != PULSAR_OK) return rc;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
 
+    if (cluster_takes(p, block_size, chunk, k, false)) {
+        const ClusterArgs args{token_ids, L, block_size, chunk, k, sink, vocab_size, p.words,
+                               static_cast<uint8_t*>(workspace) + p.bitmap_bytes, sel_chunks, prefix_idx, prefix_len, df_out, idf_out,
+                               nullptr, device_status};
+        PULSAR_CUDA_OK(launch_cluster<kModeLevels>(p, args, 0, stream));
+        count_launch();
+        return PULSAR_OK;
+    }
     uint32_t* bitmaps = static_cast<uint32_t*>(workspace);
     uint16_t* df_table = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + p.bitmap_bytes);
     uint16_t* level = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + p.bitmap_bytes + p.df_bytes);
@@ -608,8 +963,7 @@ int32_t plan_score(int64_t L, int32_t vocab_size, int32_t block_size, int32_t ch
 }
 
 template <int kBlocks>
-cudaError_t launch_scores(const SelectPlan& b, int32_t score_mode, const uint32_t* token_ids, const uint16_t* df_table, int64_t L,
-                          int32_t block_size, int32_t chunk, int32_t vocab_size, double* score, cudaStream_t stream) {
+ScoreTable<kBlocks> score_table(const SelectPlan& b, int32_t score_mode, int64_t L, int32_t block_size, int32_t chunk) {
     // The logarithms of Eq. 5 / Eq. 7 for every possible df, in float64 from the host's libm.
     ScoreTable<kBlocks> tab;
     const double N = static_cast<double>(b.n_blocks);
@@ -627,7 +981,13 @@ cudaError_t launch_scores(const SelectPlan& b, int32_t score_mode, const uint32_
     tab.b = bb;
     tab.one_minus_b = 1.0 - bb;
     tab.mean_len = static_cast<double>(L) / static_cast<double>(n_chunks);
+    return tab;
+}
 
+template <int kBlocks>
+cudaError_t launch_scores(const SelectPlan& b, int32_t score_mode, const uint32_t* token_ids, const uint16_t* df_table, int64_t L,
+                          int32_t block_size, int32_t chunk, int32_t vocab_size, double* score, cudaStream_t stream) {
+    const ScoreTable<kBlocks> tab = score_table<kBlocks>(b, score_mode, L, block_size, chunk);
     const int n_chunks_total = b.n_blocks * b.C;
     if (chunk <= kThreadFormChunk && n_chunks_total >= kThreadFormSlots) {
         auto kernel = score_mode == PULSAR_SCORE_MAX_IDF ? chunk_score_thread_kernel<PULSAR_SCORE_MAX_IDF, kBlocks>
@@ -672,6 +1032,18 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const SelectPlan& b = p.base;
 
+    if (cluster_takes(b, block_size, chunk, k, true)) {
+        const ClusterArgs args{token_ids, L, block_size, chunk, k, sink, vocab_size, b.words,
+                               static_cast<uint8_t*>(workspace) + b.bitmap_bytes, sel_chunks, prefix_idx, prefix_len, nullptr, nullptr,
+                               score_out, device_status};
+        const auto tab = score_table<kClusterBlocks>(b, score_mode, L, block_size, chunk);
+        PULSAR_CUDA_OK(score_mode == PULSAR_SCORE_MAX_IDF ? launch_cluster<PULSAR_SCORE_MAX_IDF>(b, args, tab, stream)
+                       : score_mode == PULSAR_SCORE_TF_IDF ? launch_cluster<PULSAR_SCORE_TF_IDF>(b, args, tab, stream)
+                       : score_mode == PULSAR_SCORE_BM25   ? launch_cluster<PULSAR_SCORE_BM25>(b, args, tab, stream)
+                                                           : launch_cluster<PULSAR_SCORE_TYPE_TOKEN>(b, args, tab, stream));
+        count_launch();
+        return PULSAR_OK;
+    }
     uint32_t* bitmaps = static_cast<uint32_t*>(workspace);
     uint16_t* df_table = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + b.bitmap_bytes);
     double* score = score_out ? score_out

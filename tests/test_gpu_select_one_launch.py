@@ -1,0 +1,42 @@
+"""The selection in one launch (a cluster, one CTA per block) at the edges of what it takes, against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import kernel_names, to_dev_ids
+from paper_2607_20457_b200 import binding
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("L,block,chunk,k,sink,vocab,one_launch", [
+    (2048, 2048, 2, 5, 3, 31, True),               # one block, 1024 chunks: a thread each
+    (2049, 2049, 3, 5, 3, 32, None),               # a token more than a block may have under a score
+    (6144, 6144, 8, 5, 3, 33, None),               # as many as it may have without
+    (6145, 6145, 8, 5, 3, 33, False),
+    (2050, 1025, 1, 7, 3, 33, False),              # 1025 chunks
+    (16 * 300 - 7, 300, 7, 4, 11, 128256, True),   # 16 blocks, short last chunks, the largest vocabulary
+    (17 * 64, 64, 8, 2, 5, 100, False),            # 17 blocks
+    (9 * 50 - 49, 50, 3, 17, 50, 1000, True),      # a last block of one token, every chunk selected
+    (1024, 128, 33, 3, 0, 5, True),
+])
+def test_selection_at_the_edges_of_one_launch(L, block, chunk, k, sink, vocab, one_launch):
+    rng = np.random.default_rng(L)
+    ids = np.minimum((rng.random(L) ** 3 * vocab).astype(np.uint32), vocab - 1)
+    ids_d = to_dev_ids(ids, DEV)
+    call = lambda: binding.pulsar_maxidf_select(ids_d, vocab, block, chunk, k, sink, want_df=True, want_idf=True)
+    got, ref = call(), oracle.maxidf_select(ids, vocab, block, chunk, k, sink)
+    for name in ("sel_chunks", "prefix_idx", "prefix_len"):
+        np.testing.assert_array_equal(got[name].cpu().numpy(), ref[name], err_msg=name)
+    np.testing.assert_array_equal(got["df"].cpu().numpy().view(np.uint32), ref["df"])
+    np.testing.assert_allclose(got["idf"].cpu().numpy(), ref["idf"], rtol=0, atol=1e-6)
+    assert (len(kernel_names(call)) == 1) == (one_launch is not False)
+    for mode in binding.SCORE_MODES:
+        got = binding.pulsar_chunk_select(ids_d, vocab, block, chunk, k, sink, mode, want_score=True)
+        ref = oracle.chunk_select(ids, vocab, block, chunk, k, sink, mode)
+        for name in ("sel_chunks", "prefix_idx", "prefix_len"):
+            np.testing.assert_array_equal(got[name].cpu().numpy(), ref[name], err_msg=f"{mode} {name}")
+        names = kernel_names(lambda: binding.pulsar_chunk_select(ids_d, vocab, block, chunk, k, sink, mode))
+        assert (len(names) == 1) == (one_launch is True)
+        assert np.array_equal(got["score"].cpu().numpy(), ref["score"]), mode
