@@ -1303,17 +1303,6 @@ int log2_of(int g) {
     return s;
 }
 
-// log2 of the heads of a KV head that share a query tile of causal attention.  With all g heads of 128/g tokens in a tile,
-// both tiles of a work item end in the same key tile; with 128 tokens of one head the second needs one more, which
-// it walks alone.  Half a key tile per item is saved, but the items that run at the same time then cover g times as
-// many tokens and no longer read the same K/V tiles in step.  With d = 64, where a tile is half as large and the GPU is
-// below its power limit, packing gains 3.5 % (45K ragged 0.916 -> 0.884 ms); with d = 128 it costs 0.7-1 % from 32K on
-// (64K 5.33 -> 5.37 ms, 128K 14.12 -> 14.27 ms; 16K the same).  The group must be a power of two up to 16.
-int causal_pack_shift(int32_t Hq, int32_t Hkv, int32_t d) {
-    const int g = Hq / Hkv;
-    return d == 64 && g <= 16 && (g & (g - 1)) == 0 ? log2_of(g) : 0;
-}
-
 // Causal attention with few items takes work items of one query tile instead of two: twice the items, and a key tile costs
 // the chain of one tile (0.79 us with d = 64, 0.84 with d = 128; an item 2.5 and 2.8 us more) instead of two interleaved
 // ones (1.39 and 1.51 us, 3.0 and 3.4 us).  While every tile has an SM of its own that is the shorter time, and with more pairs than
@@ -1328,11 +1317,16 @@ struct CausalRun {
     int len;
 };
 constexpr int kMaxCausalRuns = 512;             // more runs than that are more pairs than SMs
+struct CausalCost {
+    int64_t tile, item;                         // ns
+};
+CausalCost causal_cost(int per_item, int32_t d) {
+    return per_item == 1 ? CausalCost{d == 64 ? 785 : 840, d == 64 ? 2500 : 2760} : CausalCost{d == 64 ? 1392 : 1513, d == 64 ? 2986 : 3390};
+}
 
 bool causal_single(const CausalRun* runs, int n_runs, int64_t heads, int tile_tokens, int32_t d) {
     const int sms = sm_count();
-    struct { int64_t tile, item; } const cost[2] = {{d == 64 ? 785 : 840, d == 64 ? 2500 : 2760},
-                                                    {d == 64 ? 1392 : 1513, d == 64 ? 2986 : 3390}};     // ns, of one tile and of a pair
+    const CausalCost cost[2] = {causal_cost(1, d), causal_cost(2, d)};
     const auto items = [&](int64_t tokens) {
         int64_t n = 0;
         for (int r = 0; r < n_runs; ++r) n += (runs[r].len + tokens - 1) / tokens * heads;
@@ -1366,6 +1360,34 @@ bool causal_single(const CausalRun* runs, int n_runs, int64_t heads, int tile_to
     return time[0] < time[1];
 }
 
+// log2 of the heads of a KV head that share a query tile of causal attention.  With all g heads of 128/g tokens in a tile,
+// both tiles of a work item end in the same key tile; with 128 tokens of one head the second needs one more, which
+// it walks alone, and a run's last pair of tiles is the emptier the fewer of its 256 rows the run has left.  Against that, the
+// items that run at the same time cover g times as many tokens and no longer read the same K/V tiles in step.  With d = 64, where a
+// tile is half as large and the GPU is below its power limit, packing gains 3.5 % (45K ragged 0.916 -> 0.884 ms); with
+// d = 128 it costs 0.7-1 % from 32K on (64K 5.33 -> 5.37 ms, 128K 14.12 -> 14.27 ms; 16K the same), so there the items have
+// to take kPackGain per cent of their time at most.  Causal attention alone, 32 heads of 8 KV heads, us, apart / together: 14
+// blocks of 186 tokens 28.7 / 22.3, 16 of 300 53.5 / 38.2, 11 of 512 51.0 / 47.8, 13 of 767 93.6 / 89.3, 16 of 1000 (93 % of
+// the time by the rule) 175 / 173, 16 of 1500 (95 %) 313 / 317; 60 of 130, 16 heads of 4, 51.2 / 36.8.  The group must be a power
+// of two up to 16.
+constexpr int kPackGain = 94;
+int causal_pack_shift(const CausalRun* runs, int n_runs, int32_t Hq, int32_t Hkv, int32_t d) {
+    const int g = Hq / Hkv;
+    if (g > 16 || (g & (g - 1)) != 0) return 0;
+    if (d == 64 || g == 1) return log2_of(g);
+    const CausalCost cost = causal_cost(2, d);
+    const auto time = [&](int64_t heads, int tile_tokens) {
+        int64_t t = 0;
+        for (int r = 0; r < n_runs; ++r) {
+            const int64_t n_pref = (runs[r].prefix + kTileN - 1) / kTileN;
+            for (int row = 0; row < runs[r].len; row += 2 * tile_tokens)
+                t += (n_pref + (std::min(row + 2 * tile_tokens, runs[r].len) + kTileN - 1) / kTileN) * cost.tile + cost.item;
+        }
+        return t * heads;
+    };
+    return time(Hkv, kTileM / g) * 100 < time(Hq, kTileM) * kPackGain ? log2_of(g) : 0;
+}
+
 // whole_only: the entry point takes only sequences made of whole blocks.
 int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block_size, int32_t prefix_total,
                     Phase1Plan& p, bool whole_only = false) {
@@ -1380,17 +1402,17 @@ int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block
     p.last_len = static_cast<int>(L - (B - 1) * block_size);
     p.pref_bytes = round_up(p.pref_rows * Hkv * d * 2, 256);
     p.total = 2 * p.pref_bytes + 256;                        // gathered prefix K, V and the work counter
-    p.pack_shift = causal_pack_shift(Hq, Hkv, d);
-    const int64_t heads = p.pack_shift ? Hkv : Hq;
     // How long each block's prefix is stands on the device.  It is taken to grow evenly to prefix_total, as in a whole
     // context and as blocks are dealt to GPUs in turn or in zigzag; a single block is taken to see all of it.  (Several
     // blocks that all see a long prefix, the last GPU of a context cut into runs of blocks, would do 1.1-1.2 times
     // better with pairs; pairs would cost the others up to 1.6 times.)
-    const int tile_tokens = kTileM >> p.pack_shift;
     CausalRun runs[kMaxCausalRuns];
-    if (B <= kMaxCausalRuns)
-        for (int64_t i = 0; i < B; ++i)
-            runs[i] = {B > 1 ? prefix_total * (B - 1 - i) / (B - 1) : prefix_total, i == 0 ? p.last_len : block_size};
+    const int n_runs = static_cast<int>(std::min<int64_t>(B, kMaxCausalRuns));
+    for (int64_t i = 0; i < n_runs; ++i)
+        runs[i] = {B > 1 ? prefix_total * (B - 1 - i) / (B - 1) : prefix_total, i == 0 ? p.last_len : block_size};
+    p.pack_shift = causal_pack_shift(runs, n_runs, Hq, Hkv, d);
+    const int64_t heads = p.pack_shift ? Hkv : Hq;
+    const int tile_tokens = kTileM >> p.pack_shift;
     p.single = B <= kMaxCausalRuns && causal_single(runs, static_cast<int>(B), heads, tile_tokens, d) ? 1 : 0;
     const int64_t tokens = static_cast<int64_t>(p.single ? 1 : 2) * tile_tokens;
     p.items_block = static_cast<int>((block_size + tokens - 1) / tokens);
@@ -2007,10 +2029,10 @@ extern "C" int32_t pulsar_causal_varlen_attn(const uint16_t* Q, const uint16_t* 
     VarlenTable vt{};
     vt.n_seq = n_seq;
     for (int j = 0; j <= n_seq; ++j) vt.start[j] = cu_seqlens_host[j];
-    const int pack_shift = causal_pack_shift(Hq, Hkv, d), heads = pack_shift ? Hkv : Hq;
-    const int tile_tokens = kTileM >> pack_shift;
     CausalRun runs[kMaxVarlenSeqs];
     for (int k = 0; k < n_seq; ++k) runs[k] = {0, vt.start[n_seq - k] - vt.start[n_seq - 1 - k]};
+    const int pack_shift = causal_pack_shift(runs, n_seq, Hq, Hkv, d), heads = pack_shift ? Hkv : Hq;
+    const int tile_tokens = kTileM >> pack_shift;
     const int single = causal_single(runs, n_seq, heads, tile_tokens, d) ? 1 : 0, tokens = (single ? 1 : 2) * tile_tokens;
     int64_t pairs_total = 0;
     for (int k = 0; k < n_seq; ++k) {
