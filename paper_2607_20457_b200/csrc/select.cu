@@ -537,12 +537,14 @@ int32_t plan_select(int64_t L, int32_t vocab_size, int32_t block_size, int32_t c
 // CTAs are two cluster barriers instead of three launches, and the df table (a byte per entry, in L2).  Bound by a chain of
 // latencies: each thread's loads are issued together (one at a time: 45,011 tokens 10.2 us, 8.0 like this and with a look at
 // the presence bit before the atomic).
+// kModeTable ends with the df table.
 // ---------------------------------------------------------------------------------------------
 constexpr int kClusterThreads = 1024;
 constexpr int kClusterBlocks = 16;              // CTAs of the largest cluster
 constexpr int kClusterTokens = 8192;            // of a block: its ids, and a term per id, are kept in shared memory
 constexpr int kClusterChunks = 1024;            // of a block: a thread each in the selection
 constexpr int kModeLevels = -1;                 // chunks ranked by their least df (pulsar_maxidf_select), without scores
+constexpr int kModeTable = -2;                  // the df table alone, 16 bits an entry, for score launches of their own
 
 struct ClusterShape {
     size_t bits, tokens, dfs, ranks, chosen, terms, total;       // offsets in shared memory
@@ -589,7 +591,7 @@ struct ClusterArgs {
     const uint32_t* ids;
     int64_t L;
     int block_size, chunk, k, sink, vocab_size, words;
-    uint8_t* df_table;                          // [vocab_size rounded up to 32]
+    uint8_t* df_table;                          // [vocab_size rounded up to 32], of uint16 with kModeTable
     int32_t *sel_chunks, *prefix_idx, *prefix_len;
     uint32_t* df_out;
     float* idf_out;
@@ -600,8 +602,8 @@ struct ClusterArgs {
 template <int kMode>
 __global__ void __launch_bounds__(kClusterThreads, 1)
 select_cluster_kernel(const __grid_constant__ ClusterArgs a,
-                      const __grid_constant__ std::conditional_t<kMode == kModeLevels, int, ScoreTable<kClusterBlocks>> tab) {
-    constexpr bool kScores = kMode != kModeLevels;
+                      const __grid_constant__ std::conditional_t<kMode < 0, int, ScoreTable<kClusterBlocks>> tab) {
+    constexpr bool kScores = kMode >= 0;
     extern __shared__ __align__(16) uint8_t smem_c[];
     __shared__ int s_warp[32], s_hist[32], s_short[kClusterBlocks], s_threshold, s_need;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -665,9 +667,16 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
 #pragma unroll
             for (int p = 0; p < 5; ++p) out[n] |= ((((plane[p] >> (4 * n)) & 15u) * 0x00204081u) & 0x01010101u) << p;
         }
-        uint4* dst = reinterpret_cast<uint4*>(a.df_table + static_cast<size_t>(w) * 32);
-        dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
-        dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        uint4* dst = reinterpret_cast<uint4*>(a.df_table + static_cast<size_t>(w) * (kMode == kModeTable ? 64 : 32));
+        if (kMode == kModeTable) {
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+                dst[n] = make_uint4(__byte_perm(out[2 * n], 0u, 0x4140), __byte_perm(out[2 * n], 0u, 0x4342),
+                                    __byte_perm(out[2 * n + 1], 0u, 0x4140), __byte_perm(out[2 * n + 1], 0u, 0x4342));
+        } else {
+            dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
+            dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        }
         if (a.df_out != nullptr || a.idf_out != nullptr)
             for (int i = 0; i < 32 && w * 32 + i < a.vocab_size; ++i) {
                 uint32_t df = 0;
@@ -677,7 +686,8 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
                 if (a.idf_out != nullptr) a.idf_out[w * 32 + i] = logf(static_cast<float>(n_blocks) / static_cast<float>(df > 0 ? df : 1));
             }
     }
-    cluster_sync();                    // the table is complete
+    cluster_sync();                    // the table is complete, and no CTA reads another's set any more
+    if constexpr (kMode == kModeTable) return;
     constexpr uint32_t kNoToken = 255;
     uint32_t mine_df[kPerThread];
 #pragma unroll
@@ -845,16 +855,23 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
 // takes for three launches more.  us a call in a row of them, one launch / four: levels, blocks of 1024 tokens 6.3 / 12.6, of
 // 4157 7.9 / 12.9, of 5000 8.0 / 12.6, of 8192 about even; BM25, 1024 8.6 / 15.2, 1665 13.7 / 15.4, 4157 15.6 / 15.5 (the
 // divisions of a block's terms are one SM's then), the other scores between the two.
+// Blocks above that share the df table's launch and have the scores formed by the whole chip, three launches instead of four: BM25
+// over 16 blocks of 8192 15.5 -> 14.4, the type-token ratio over 6 of 4157 15.5 -> 14.2 (on the device 12.3 -> 8.7).
 constexpr int kClusterLevelTokens = 6144, kClusterScoreTokens = 2048;
+bool cluster_table_takes(const SelectPlan& p, int32_t block_size) {
+    return p.n_blocks <= kClusterBlocks && block_size <= kClusterTokens && static_cast<size_t>(p.words) * 64 <= p.df_bytes &&
+           ClusterShape(p.words, block_size, p.C, 1, 0, false).tokens <= kMaxDynSmem - 2048;
+}
 bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32_t k, bool scores) {
     return p.n_blocks <= kClusterBlocks && block_size <= (scores ? kClusterScoreTokens : kClusterLevelTokens) && p.C <= kClusterChunks &&
-           ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 1024 &&
+           ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 2048 &&
            static_cast<size_t>(p.words) * 32 <= p.df_bytes;
 }
 
 template <int kMode, typename Table>
 cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const Table& tab, cudaStream_t stream) {
-    const size_t smem = ClusterShape(p.words, args.block_size, p.C, args.chunk, args.k, kMode != kModeLevels).total;
+    const ClusterShape shape(p.words, args.block_size, p.C, args.chunk, args.k, kMode >= 0);
+    const size_t smem = kMode == kModeTable ? shape.tokens : shape.total;
     auto kernel = select_cluster_kernel<kMode>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e == cudaSuccess && p.n_blocks > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1049,16 +1066,23 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
     double* score = score_out ? score_out
                               : reinterpret_cast<double*>(static_cast<char*>(workspace) + b.bitmap_bytes + b.df_bytes);
 
-    if (b.presence_smem > 48 * 1024)
-        PULSAR_CUDA_OK(cudaFuncSetAttribute(presence_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            static_cast<int>(b.presence_smem)));
-    PULSAR_CUDA_OK(launch_kernel(presence_kernel, dim3(b.n_blocks), dim3(kPresenceThreads), b.presence_smem, stream, true,
-                                 token_ids, L, block_size, vocab_size, b.words, bitmaps, device_status));
-    count_launch();
+    if (cluster_table_takes(b, block_size)) {
+        const ClusterArgs args{token_ids, L, block_size, chunk, k, sink, vocab_size, b.words, reinterpret_cast<uint8_t*>(df_table),
+                               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, device_status};
+        PULSAR_CUDA_OK(launch_cluster<kModeTable>(b, args, 0, stream));
+        count_launch();
+    } else {
+        if (b.presence_smem > 48 * 1024)
+            PULSAR_CUDA_OK(cudaFuncSetAttribute(presence_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                static_cast<int>(b.presence_smem)));
+        PULSAR_CUDA_OK(launch_kernel(presence_kernel, dim3(b.n_blocks), dim3(kPresenceThreads), b.presence_smem, stream, true,
+                                     token_ids, L, block_size, vocab_size, b.words, bitmaps, device_status));
+        count_launch();
+        PULSAR_CUDA_OK(launch_kernel(df_idf_kernel, dim3((vocab_size + 255) / 256), dim3(256), 0, stream, true, bitmaps,
+                                     b.n_blocks, b.words, vocab_size, df_table, nullptr, nullptr));
+        count_launch();
+    }
     // Programmatic dependents of the launch before them, as in pulsar_maxidf_select.
-    PULSAR_CUDA_OK(launch_kernel(df_idf_kernel, dim3((vocab_size + 255) / 256), dim3(256), 0, stream, true, bitmaps,
-                                 b.n_blocks, b.words, vocab_size, df_table, nullptr, nullptr));
-    count_launch();
     PULSAR_CUDA_OK(b.n_blocks <= kFewScoreBlocks
                        ? launch_scores<kFewScoreBlocks>(b, score_mode, token_ids, df_table, L, block_size, chunk, vocab_size, score, stream)
                        : launch_scores<kMaxScoreBlocks>(b, score_mode, token_ids, df_table, L, block_size, chunk, vocab_size, score, stream));
