@@ -609,8 +609,10 @@ def run_extras(binding, w, dev, K_d, V_d, peaks):
             binding.pulsar_phase2_attn(Qd, K_d, V_d, w.n_blocks, w.block_size, n_splits=J, out=O, workspace=ws)
         ms = time_after_flush(call, flush_clean, 12)["median_ms"]
         ms_dirty = time_after_flush(call, flush_dirty, 12)["median_ms"]
-        # four partials per KV part while all query rows of a KV head fit a quarter tile (8 and 1 tokens)
-        nbytes = cm.phase2_hbm_bytes(nq, w.L, w.Hq, w.Hkv, w.d, (4 if nq * (w.Hq // w.Hkv) <= 32 else 1) * J)
+        # four partials per KV part while all query rows of a KV head fit a quarter tile (8 tokens); up to eight rows are merged
+        # on chip but for a few partials per head, which are not counted
+        rows = nq * (w.Hq // w.Hkv)
+        nbytes = cm.phase2_hbm_bytes(nq, w.L, w.Hq, w.Hkv, w.d, (0 if rows <= 8 else 4 if rows <= 32 else 1) * J)
         out[name] = dict(ms=ms, splits=J, gbs=nbytes / (ms * 1e-3) / 1e9,
                          frac_of_measured_hbm=nbytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                          ms_after_write_only_flush=ms_dirty,
@@ -631,12 +633,12 @@ def run_extras(binding, w, dev, K_d, V_d, peaks):
                                             out=Og, workspace=wsg)
     ms = time_after_flush(gen_call, flush_clean, 12)["median_ms"]
     ms_dirty = time_after_flush(gen_call, flush_dirty, 12)["median_ms"]
-    nbytes = cm.phase2_hbm_bytes(1, w.L, w.Hq, w.Hkv, w.d, 4 * (J + 1))
+    nbytes = cm.phase2_hbm_bytes(1, w.L, w.Hq, w.Hkv, w.d)
     out["phase2_generate_step_1tok"] = dict(ms=ms, context_parts=J, shard_rows=65, gbs=nbytes / (ms * 1e-3) / 1e9,
                                             frac_of_measured_hbm=nbytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                                             ms_after_write_only_flush=ms_dirty,
                                             frac_after_write_only_flush=nbytes / (ms_dirty * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                                            launches="attention (appends the new rows) + merge", l2=how)
+                                            launches="attention (stores the new rows) + merge", l2=how)
     del flush_words
     del flush
     w4 = W.CONFIGS["64k"]
