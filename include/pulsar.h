@@ -362,7 +362,9 @@ int32_t pulsar_retain_block_kv(const uint16_t *K, const uint16_t *V, int64_t tot
  *               divides the B*block_size keys, every part has that many keys (n_splits == B
  *               gives the per-block (A_h, l_h) of Algorithm 1 line 12); if not, the parts are
  *               whole 128-key tiles, ceil(tiles / n_splits) each, the last one shorter, and a
- *               count that would leave a part empty is rejected.
+ *               count that would leave a part empty is rejected.  At most eight rows per KV head
+ *               (nq * Hq/Hkv) against 1024 keys or more, without caller partials, are cut as the
+ *               library sees fit; the count is checked all the same.
  *   O           out [nq, Hq, d] bf16        LSE out [nq, Hq] float32 (natural log), or NULL
  *   part_O      out [n_splits, nq, Hq, d] float32 or NULL (requires n_splits > 0)
  *   part_LSE    out [n_splits, nq, Hq]    float32 or NULL (both or neither)
@@ -427,7 +429,8 @@ int32_t pulsar_encode_step(const uint32_t *token_ids, int64_t L, int32_t vocab_s
  *               generated tokens; rows [gen_len, gen_len + n_new) are written by this call;
  *               rows from gen_len + n_new on are never read (they may hold anything, NaN included)
  *   n_splits    0 = library's choice, else the parts the context alone would be cut into (a count that
- *               would leave one of them empty is rejected as in pulsar_phase2_attn)
+ *               would leave one of them empty is rejected as in pulsar_phase2_attn; few rows against a
+ *               long context are cut as the library sees fit, as there)
  *   O           out [n_new, Hq, d] bf16       LSE out [n_new, Hq] float32 or NULL
  *
  * Requirements as for pulsar_phase2_attn, plus gen_len >= 0 and gen_len + n_new <= gen_capacity

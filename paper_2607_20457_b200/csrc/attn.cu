@@ -11,8 +11,8 @@
 //            the block's own rows up to the diagonal tile (causal mask on that tile only).
 //   Phase 2: rows = (128/g tokens) x (the g query heads of one KV head); key tiles = one
 //            contiguous part of the retained KV, no mask; output is the fp32 partial (A_j, l_j)
-//            or, with a single part, the final bf16 result.  With at most 32 such rows (decode)
-//            the rows are replicated into the four lane quarters of the tile and each softmax
+//            or, with a single part, the final bf16 result.  With at most 32 such rows (decode; up to
+//            eight against a long context are decode.cu's) the rows are replicated into the four lane quarters of the tile and each softmax
 //            warp takes a quarter of the keys; the generation shard of Algorithm 1 l.11-16, causal by
 //            token, is one more part or stands in front of the last part's context keys.
 //   Assembled inputs (Algorithm 1 l.8 as the paper runs it): sequences of any lengths packed back

@@ -1,7 +1,7 @@
 // Native half of the Python binding: checks the tensors, allocates what the caller did not pass, and calls the C ABI
 // on the current stream.
 //
-// A call of the library is three to nine short launches; done from Python (attribute look-ups, ctypes conversions
+// A call of the library is one to six short launches; done from Python (attribute look-ups, ctypes conversions
 // of twenty arguments, torch.cuda.current_stream alone 3.2 us) the calls of a decoding step took 24 us on the host for
 // 16 us of device time.  The functions take positional arguments in the order of their Python wrappers
 // (binding.py), which hold the names, the defaults and the documentation.  The library's entry points arrive as

@@ -12,7 +12,7 @@
 //                     lower index, then the block's part of the prefix list (Eq. 4)
 // Ranking uses the integer df only, so the selection is exact.
 //
-// pulsar_chunk_select runs the same first two launches, then chunk_score_kernel (a float64 score
+// pulsar_chunk_select runs the same first two launches (one for up to 16 blocks), then chunk_score_kernel (a float64 score
 // per chunk under TF-IDF, BM25, the type-token ratio or Max-IDF, Appendix C Eq. 6-9) and
 // topk_score_kernel (rank by score, ties to the lower index).
 #include <cmath>
