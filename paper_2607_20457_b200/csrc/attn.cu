@@ -541,7 +541,8 @@ __device__ __forceinline__ float exp_row(const uint32_t (&r)[N], float scale, fl
 // 36.9 -> 36.0); launches that stream from HBM take what they took.
 // kTileMax: see next_max; generation steps whose parts were made longer.  An instance of its own, since the test alone
 // costs Phase 1 0.4 % (16K 658 -> 661 us).
-template <int D, bool kQuad, bool kSingle, bool kTileMax>
+// kBeside: see launch_lse_merge (an instance of its own: the test alone cost calls of 20-40 us 0.1-0.2 us).
+template <int D, bool kQuad, bool kSingle, bool kTileMax, bool kBeside>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
             const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKp,
@@ -599,7 +600,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
     // The CTAs of this launch may have been placed while the launch before it was still running; everything above
     // (barriers, tensor maps, TMEM) overlaps its end, nothing below may.
-    if (!a.beside) grid_dependency_wait();
+    if (!kBeside) grid_dependency_wait();
     // The launch that follows (the merge of this launch's partials, or another call's) may be placed as
     // SMs become free; it waits for this grid to finish before it reads anything.
     grid_launch_dependents();
@@ -1230,7 +1231,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tmem_base, 512);
-    if (a.beside) grid_dependency_wait();
+    if (kBeside) grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1309,13 +1310,15 @@ int32_t launch_attn(const CUtensorMap& q, const CUtensorMap& k, const CUtensorMa
     };
     static const VarlenTable kNoSequences{};
     const VarlenTable& tab = table ? *table : kNoSequences;
-    const auto pick = [&](auto tile_max) -> cudaError_t {
-        constexpr bool kTileMax = decltype(tile_max)::value;
-        return a.quad     ? launch(attn_kernel<D, true, true, kTileMax>, NoTable{})
-               : a.single ? launch(attn_kernel<D, false, true, kTileMax>, tab)
-                          : launch(attn_kernel<D, false, false, kTileMax>, tab);
+    const auto pick = [&](auto tile_max, auto beside) -> cudaError_t {
+        constexpr bool kTileMax = decltype(tile_max)::value, kBeside = decltype(beside)::value;
+        return a.quad     ? launch(attn_kernel<D, true, true, kTileMax, kBeside>, NoTable{})
+               : a.single ? launch(attn_kernel<D, false, true, kTileMax, kBeside>, tab)
+                          : launch(attn_kernel<D, false, false, kTileMax, kBeside>, tab);
     };
-    PULSAR_CUDA_OK(a.tile_max ? pick(std::true_type{}) : pick(std::false_type{}));
+    PULSAR_CUDA_OK(a.beside     ? pick(std::false_type{}, std::true_type{})        // (tile_max is the generation step's)
+                   : a.tile_max ? pick(std::true_type{}, std::false_type{})
+                                : pick(std::false_type{}, std::false_type{}));
     count_launch();
     return PULSAR_OK;
 }

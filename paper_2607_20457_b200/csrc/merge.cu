@@ -12,8 +12,8 @@ template <bool kF32>
 __global__ void __launch_bounds__(256)
 lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ part_LSE, int n_parts,
                  int64_t stride_O, int64_t stride_L, int64_t rows, int d, void* __restrict__ O_,
-                 float* __restrict__ LSE, int beside) {
-    if (!beside) grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
+                 float* __restrict__ LSE) {
+    grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
     grid_launch_dependents();
     const int vec_per_row = d >> 2;
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -49,7 +49,6 @@ lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ par
         *reinterpret_cast<uint2*>(static_cast<uint16_t*>(O_) + row * d + v * 4) = packed;
     }
     if (LSE != nullptr && v == 0) LSE[row] = (m > -INFINITY) ? m + logf(denom) : -INFINITY;
-    if (beside) grid_dependency_wait();
 }
 
 // The same merge for rows of 32 * kVec floats (d = 64, 128): a warp loads a part's row as one contiguous run,
@@ -59,13 +58,14 @@ lse_merge_kernel(const float* __restrict__ part_O, const float* __restrict__ par
 // two such rounds cover all parts.  The order of the sums is fixed, so the result is reproducible.
 // Measured tail from the end of the attention launch to the end of the merge: 384 rows of 19 parts
 // 8.5 us with one thread per four outputs, 3.4 us with this form.
-template <bool kF32, int kVec, int kWarps, int kRows>
+// kBeside: see launch_lse_merge (an instance of its own: the test alone cost 0.2 us of a 20 us query).
+template <bool kF32, int kVec, int kWarps, int kRows, bool kBeside>
 __global__ void __launch_bounds__(32 * kWarps * kRows)
 lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict__ part_LSE, int n_parts,
                       int64_t stride_O, int64_t stride_L, int64_t rows, void* __restrict__ O_,
-                      float* __restrict__ LSE, int beside) {
+                      float* __restrict__ LSE) {
     static_assert(kRows == 1 || kWarps == 1, "a CTA has one row, or one warp per row");
-    if (!beside) grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
+    if (!kBeside) grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
     grid_launch_dependents();
     constexpr int kD = 32 * kVec, kInFlight = 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -169,7 +169,7 @@ lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict_
         else *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(acc[0], acc[1]);
     }
     if (LSE != nullptr && lane == 0) LSE[row] = (m > -INFINITY) ? m + logf(denom) : -INFINITY;
-    if (beside) grid_dependency_wait();
+    if (kBeside) grid_dependency_wait();
 }
 
 // The merge with every part at its own address: part j is the buffer parts[j], laid out
@@ -223,13 +223,13 @@ lse_merge_table_kernel(const __grid_constant__ PartTable parts, int n_parts, int
 }
 
 namespace {
-template <bool kF32, int kVec>
+template <bool kF32, int kVec, bool kBeside>
 auto merge_rows_kernel(int warps) {
-    return warps == 16  ? lse_merge_rows_kernel<kF32, kVec, 16, 1>
-           : warps == 8 ? lse_merge_rows_kernel<kF32, kVec, 8, 1>
-           : warps == 4 ? lse_merge_rows_kernel<kF32, kVec, 4, 1>
-           : warps == 2 ? lse_merge_rows_kernel<kF32, kVec, 2, 1>
-                        : lse_merge_rows_kernel<kF32, kVec, 1, 8>;
+    return warps == 16  ? lse_merge_rows_kernel<kF32, kVec, 16, 1, kBeside>
+           : warps == 8 ? lse_merge_rows_kernel<kF32, kVec, 8, 1, kBeside>
+           : warps == 4 ? lse_merge_rows_kernel<kF32, kVec, 4, 1, kBeside>
+           : warps == 2 ? lse_merge_rows_kernel<kF32, kVec, 2, 1, kBeside>
+                        : lse_merge_rows_kernel<kF32, kVec, 1, 8, kBeside>;
 }
 
 // Warps that share an output row; 0: one thread per four outputs (lse_merge_kernel).  That form reads the l_j before
@@ -252,15 +252,20 @@ int merge_warps(int32_t n_parts, int64_t rows, int32_t d) {
 
 int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t stride_O, int64_t stride_L,
                      int64_t rows, int32_t d, void* O, bool f32, float* LSE, cudaStream_t stream, bool beside = false) {
+    // (beside is honoured where f32 is not asked for; the thread form always waits at its start, which is right as well)
     if (rows == 0) return PULSAR_OK;
     const int warps = (d == 64 || d == 128) ? merge_warps(n_parts, rows, d) : 0;
     if (warps > 0) {
         const int64_t blocks = warps == 1 ? (rows + 7) / 8 : rows;
         if (blocks > 0x7fffffffll) return PULSAR_ERR_SHAPE;
-        auto kernel = d == 128 ? (f32 ? merge_rows_kernel<true, 4>(warps) : merge_rows_kernel<false, 4>(warps))
-                               : (f32 ? merge_rows_kernel<true, 2>(warps) : merge_rows_kernel<false, 2>(warps));
+        auto kernel = d == 128 ? (f32      ? merge_rows_kernel<true, 4, false>(warps)
+                                  : beside ? merge_rows_kernel<false, 4, true>(warps)
+                                           : merge_rows_kernel<false, 4, false>(warps))
+                               : (f32      ? merge_rows_kernel<true, 2, false>(warps)
+                                  : beside ? merge_rows_kernel<false, 2, true>(warps)
+                                           : merge_rows_kernel<false, 2, false>(warps));
         PULSAR_CUDA_OK(launch_kernel(kernel, dim3(static_cast<unsigned>(blocks)), dim3(warps == 1 ? 256 : 32 * warps), 0, stream,
-                                     true, part_O, part_LSE, n_parts, stride_O, stride_L, rows, O, LSE, beside ? 1 : 0));
+                                     true, part_O, part_LSE, n_parts, stride_O, stride_L, rows, O, LSE));
         count_launch();
         return PULSAR_OK;
     }
@@ -269,7 +274,7 @@ int32_t launch_merge(const float* part_O, const float* part_LSE, int32_t n_parts
     if (blocks > 0x7fffffffll) return PULSAR_ERR_SHAPE;
     auto kernel = f32 ? lse_merge_kernel<true> : lse_merge_kernel<false>;
     PULSAR_CUDA_OK(launch_kernel(kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, stream, true, part_O, part_LSE,
-                                 n_parts, stride_O, stride_L, rows, d, O, LSE, beside ? 1 : 0));
+                                 n_parts, stride_O, stride_L, rows, d, O, LSE));
     count_launch();
     return PULSAR_OK;
 }
