@@ -42,7 +42,6 @@ struct DecodeArgs {
     int Hq, Hkv, g_shift, n_rows;                // n_rows = n * g query rows of a KV head
     int cluster_shift, clusters;                 // log2 of the CTAs per cluster, clusters per KV head
     float scale_log2;
-    int beside;                                  // see launch_lse_merge
     uint16_t* O;
     float* LSE;
     float *part_O, *part_LSE;                    // clusters > 1: [clusters, n, Hq, D] and [clusters, n, Hq]
@@ -109,7 +108,8 @@ __device__ __forceinline__ float weight(float m, float M) { return m == -INFINIT
 
 // Two CTAs per SM: while the keys of one are on their way, the other computes, and the next launch's CTAs find room
 // beside the last of this one's.
-template <int D>
+// kBeside: see launch_lse_merge.
+template <int D, bool kBeside>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_kernel(const __grid_constant__ DecodeArgs a) {
     constexpr int kKeys = kUnitBytes / (2 * D);                // keys of a unit: 16 (d = 128), 32 (d = 64)
@@ -126,7 +126,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
     const int C = 1 << a.cluster_shift;
 
     if (C > 1) cluster_arrive();                               // waited for before another CTA's memory is written
-    if (!a.beside) grid_dependency_wait();
+    if (!kBeside) grid_dependency_wait();
     grid_launch_dependents();
 
     // ---- this CTA's pieces of kKeys keys: the context's first, then the shard's ----
@@ -390,7 +390,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
             if (at_d == 0 && a.LSE != nullptr) a.LSE[row] = lse;
         }
     }
-    if (a.beside) grid_dependency_wait();
+    if (kBeside) grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -419,7 +419,7 @@ int active_clusters(int shift) {
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    DecodeKernel kernel = decode_kernel<128>;
+    DecodeKernel kernel = decode_kernel<128, false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess ||
         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
@@ -479,7 +479,6 @@ int32_t launch_decode_as(const DecodeCall& c, const DecodePlan& p, MergeTodo& to
     a.cluster_shift = p.shift;
     a.clusters = p.clusters;
     a.scale_log2 = c.scale_log2;
-    a.beside = c.beside ? 1 : 0;
     a.O = c.O;
     a.LSE = c.LSE;
     a.part_rows = static_cast<int64_t>(c.n) * c.Hq;
@@ -487,7 +486,8 @@ int32_t launch_decode_as(const DecodeCall& c, const DecodePlan& p, MergeTodo& to
         a.part_O = static_cast<float*>(c.workspace);
         a.part_LSE = a.part_O + p.clusters * a.part_rows * c.d;
     }
-    const DecodeKernel kernel = c.d == 128 ? decode_kernel<128> : decode_kernel<64>;
+    const DecodeKernel kernel = c.d == 128 ? (c.beside ? decode_kernel<128, true> : decode_kernel<128, false>)
+                                           : (c.beside ? decode_kernel<64, true> : decode_kernel<64, false>);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(p.clusters << p.shift), static_cast<unsigned>(c.Hkv));
     cfg.blockDim = dim3(kThreads);
