@@ -936,10 +936,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         uint64_t* bar_pv = bars + SL::bOFull + 1;              // kSingle: one completion per PV product
         uint32_t g_tile = 0;                                   // kSingle: key tiles this CTA has walked
         uint64_t* bar_oe = bars + SL::bOEmpty + tile;
-        // kHalves: maximum and sum of each half of a row [2][128], where the second query tile would be, behind a barrier of
-        // their own
-        float2* half_ml = reinterpret_cast<float2*>(sQ + SL::kTileBytes);
+        // kHalves: maximum and sum of each half of a row [2][2][128], where the second query tile would be, behind a barrier of
+        // their own.  Items take the two places in turn: an item of one or two key tiles can end before a warp of the other
+        // warpgroup has read what the item before it left, because S of its key tiles waits for no epilogue.  The
+        // barrier of the item between orders those reads before the next writes to the same place.
+        float2* half_all = reinterpret_cast<float2*>(sQ + SL::kTileBytes);
         uint64_t* bar_half = bars + SL::bOEmpty + 1;
+        static_assert(!kHalves || 2 * 2 * kTileM * sizeof(float2) <= SL::kTileBytes, "the halves' sums take a tile's place");
         uint32_t s_cnt = 0, o_cnt = 0;
         bool ok = true;
 
@@ -1148,6 +1151,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 
             // ---- epilogue: normalise and store this thread's row ----
             if (n > 0) {
+                float2* half_ml = half_all + (o_cnt & 1) * (2 * kTileM);
                 if (kHalves) {
                     half_ml[s * kTileM + row] = make_float2(m_used, l_run);
                     __syncwarp();
