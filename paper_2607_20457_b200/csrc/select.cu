@@ -606,6 +606,7 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
     constexpr bool kScores = kMode >= 0;
     extern __shared__ __align__(16) uint8_t smem_c[];
     __shared__ int s_warp[32], s_hist[32], s_short[kClusterBlocks], s_threshold, s_need;
+    __shared__ float s_idf[kClusterBlocks + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x, n_blocks = gridDim.x;
     const int C = (a.block_size + a.chunk - 1) / a.chunk;
@@ -677,17 +678,30 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
             dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
             dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
         }
-        if (a.df_out != nullptr || a.idf_out != nullptr)
-            for (int i = 0; i < 32 && w * 32 + i < a.vocab_size; ++i) {
-                uint32_t df = 0;
-#pragma unroll
-                for (int p = 0; p < 5; ++p) df |= ((plane[p] >> i) & 1u) << p;
-                if (a.df_out != nullptr) a.df_out[w * 32 + i] = df;
-                if (a.idf_out != nullptr) a.idf_out[w * 32 + i] = logf(static_cast<float>(n_blocks) / static_cast<float>(df > 0 ? df : 1));
-            }
     }
     cluster_sync();                    // the table is complete, and no CTA reads another's set any more
     if constexpr (kMode == kModeTable) return;
+    // The caller's tables, from this CTA's slice of the byte table: neighbouring threads write neighbouring entries, and the
+    // logarithms are one per df.  (A thread that wrote its 32 entries out of the bit planes touched a sector per store: 128,256
+    // entries of one block 207 us a call, 31 like this; of four blocks 54 and 12.)
+    if (a.df_out != nullptr || a.idf_out != nullptr) {
+        if (tid <= n_blocks) s_idf[tid] = logf(static_cast<float>(n_blocks) / static_cast<float>(tid > 0 ? tid : 1));
+        __syncthreads();
+        const int end = min(a.vocab_size, w_end * 32);
+        constexpr int kBatch = 8;
+        for (int i0 = b * per_cta * 32 + tid; i0 < end; i0 += kBatch * kClusterThreads) {
+            uint32_t df[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) df[j] = i0 + j * kClusterThreads < end ? a.df_table[i0 + j * kClusterThreads] : 0u;
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                const int i = i0 + j * kClusterThreads;
+                if (i >= end) break;
+                if (a.df_out != nullptr) a.df_out[i] = df[j];
+                if (a.idf_out != nullptr) a.idf_out[i] = s_idf[df[j]];
+            }
+        }
+    }
     constexpr uint32_t kNoToken = 255;
     uint32_t mine_df[kPerThread];
 #pragma unroll
