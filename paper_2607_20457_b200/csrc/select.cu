@@ -30,6 +30,19 @@ constexpr int kPresenceThreads = 1024;
 constexpr int kTopkThreads = 256;
 constexpr size_t kMaxDynSmem = 227 * 1024;
 
+// Dynamic shared memory above 48 KB has to be allowed, and what is allowed belongs to the kernel on its device, not to the
+// launch: it is always set to all there is beside the kernel's own, because another thread may set it for its call between
+// here and the launch.
+template <typename Kernel>
+cudaError_t allow_smem(Kernel* kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    cudaFuncAttributes own;
+    const cudaError_t e = cudaFuncGetAttributes(&own, kernel);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(kMaxDynSmem - own.sharedSizeBytes));
+}
+
 __global__ void __launch_bounds__(kPresenceThreads)
 presence_kernel(const uint32_t* __restrict__ ids, int64_t L, int block_size, int vocab_size, int words,
                 uint32_t* __restrict__ bitmaps, int32_t* status) {
@@ -887,7 +900,7 @@ cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const T
     const ClusterShape shape(p.words, args.block_size, p.C, args.chunk, args.k, kMode >= 0);
     const size_t smem = kMode == kModeTable ? shape.tokens : shape.total;
     auto kernel = select_cluster_kernel<kMode>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = allow_smem(kernel, smem);
     if (e == cudaSuccess && p.n_blocks > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
@@ -947,13 +960,8 @@ extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, in
     uint16_t* df_table = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + p.bitmap_bytes);
     uint16_t* level = reinterpret_cast<uint16_t*>(static_cast<char*>(workspace) + p.bitmap_bytes + p.df_bytes);
 
-    if (p.presence_smem > 48 * 1024)
-        PULSAR_CUDA_OK(cudaFuncSetAttribute(presence_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            static_cast<int>(p.presence_smem)));
-    if (p.topk_smem > 48 * 1024)
-        PULSAR_CUDA_OK(cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            static_cast<int>(p.topk_smem)));
-
+    PULSAR_CUDA_OK(allow_smem(presence_kernel, p.presence_smem));
+    PULSAR_CUDA_OK(allow_smem(topk_kernel, p.topk_smem));
     PULSAR_CUDA_OK(launch_kernel(presence_kernel, dim3(p.n_blocks), dim3(kPresenceThreads), p.presence_smem, stream, true,
                                  token_ids, L, block_size, vocab_size, p.words, bitmaps, device_status));
     count_launch();
@@ -1086,9 +1094,7 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
         PULSAR_CUDA_OK(launch_cluster<kModeTable>(b, args, 0, stream));
         count_launch();
     } else {
-        if (b.presence_smem > 48 * 1024)
-            PULSAR_CUDA_OK(cudaFuncSetAttribute(presence_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                static_cast<int>(b.presence_smem)));
+        PULSAR_CUDA_OK(allow_smem(presence_kernel, b.presence_smem));
         PULSAR_CUDA_OK(launch_kernel(presence_kernel, dim3(b.n_blocks), dim3(kPresenceThreads), b.presence_smem, stream, true,
                                      token_ids, L, block_size, vocab_size, b.words, bitmaps, device_status));
         count_launch();

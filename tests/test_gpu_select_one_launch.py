@@ -1,6 +1,9 @@
 """The selection in one launch (a cluster, one CTA per block) at the edges of what it takes, against the oracle."""
+import threading
+
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from helpers import kernel_names, to_dev_ids
@@ -43,3 +46,29 @@ def test_selection_at_the_edges_of_one_launch(L, block, chunk, k, sink, vocab, o
         table = L <= 16 * block and block <= 8192                  # the df table in one launch, the scores in theirs
         assert len(names) == (1 if one_launch is True else 3 if table else 4), names
         assert np.array_equal(got["score"].cpu().numpy(), ref["score"]), mode
+
+
+@pytest.mark.parametrize("blocks", [4, 17])                       # one launch, and four
+def test_threads_with_different_shapes(blocks):
+    """The shared memory that a kernel is allowed is the kernel's, not the call's: a small call beside a large one."""
+    shapes = [(blocks * 64, 64, vocab) for vocab in (1200000, 500000, 100)] * 5
+    failed = []
+
+    def work(L, block, vocab):
+        torch.cuda.set_device(0)
+        ids = torch.arange(L, dtype=torch.int32, device=DEV) % min(vocab, 97)
+        ws = binding._workspace(binding.maxidf_select_workspace_bytes(L, vocab, block, 8, 2, 4), DEV)
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(1500):
+                    binding.pulsar_maxidf_select(ids, vocab, block, 8, 2, 4, workspace=ws)
+        except Exception as e:
+            failed.append((vocab, e))
+
+    threads = [threading.Thread(target=work, args=s) for s in shapes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed, failed
