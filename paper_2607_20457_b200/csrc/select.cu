@@ -15,6 +15,7 @@
 // pulsar_chunk_select runs the same first two launches (one for up to 16 blocks), then chunk_score_kernel (a float64 score
 // per chunk under TF-IDF, BM25, the type-token ratio or Max-IDF, Appendix C Eq. 6-9) and
 // topk_score_kernel (rank by score, ties to the lower index).
+#include <atomic>
 #include <cmath>
 #include <mutex>
 #include <type_traits>
@@ -878,6 +879,40 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
     write_block_prefix(b, n_blocks, a.block_size, a.chunk, a.k, geo, offset, chosen, a.sel_chunks, a.prefix_idx, a.prefix_len);
 }
 
+// Whether a cluster of that many CTAs can be resident on the current device, whatever its mode and shared memory (an SM holds one
+// CTA of any).  A process that sees a part of the GPU, or a GPU with smaller clusters of SMs, takes the four launches.
+bool cluster_fits(int ctas) {
+    static std::atomic<signed char> known[64][kClusterBlocks + 1];     // per device; 0: not asked yet, else 1 or -1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    const signed char seen = known[dev][ctas].load(std::memory_order_relaxed);
+    if (seen != 0) return seen > 0;
+    auto kernel = select_cluster_kernel<kModeLevels>;
+    const size_t smem = kMaxDynSmem - 2048;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(ctas);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (allow_smem(kernel, smem) != cudaSuccess ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    known[dev][ctas].store(n > 0 ? 1 : -1, std::memory_order_relaxed);
+    return n > 0;
+}
+
 // Whether a selection of this shape is the cluster's: at most 16 blocks that their CTAs get through in less time than the host
 // takes for three launches more.  us a call in a row of them, one launch / four: levels, blocks of 1024 tokens 6.3 / 12.6, of
 // 4157 7.9 / 12.9, of 5000 8.0 / 12.6, of 8192 about even; BM25, 1024 8.6 / 15.2, 1665 13.7 / 15.4, 4157 15.6 / 15.5 (the
@@ -887,12 +922,12 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
 constexpr int kClusterLevelTokens = 6144, kClusterScoreTokens = 2048;
 bool cluster_table_takes(const SelectPlan& p, int32_t block_size) {
     return p.n_blocks <= kClusterBlocks && block_size <= kClusterTokens && static_cast<size_t>(p.words) * 64 <= p.df_bytes &&
-           ClusterShape(p.words, block_size, p.C, 1, 0, false).tokens <= kMaxDynSmem - 2048;
+           ClusterShape(p.words, block_size, p.C, 1, 0, false).tokens <= kMaxDynSmem - 2048 && cluster_fits(p.n_blocks);
 }
 bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32_t k, bool scores) {
     return p.n_blocks <= kClusterBlocks && block_size <= (scores ? kClusterScoreTokens : kClusterLevelTokens) && p.C <= kClusterChunks &&
            ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 2048 &&
-           static_cast<size_t>(p.words) * 32 <= p.df_bytes;
+           static_cast<size_t>(p.words) * 32 <= p.df_bytes && cluster_fits(p.n_blocks);
 }
 
 template <int kMode, typename Table>
