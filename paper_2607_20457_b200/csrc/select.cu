@@ -545,9 +545,9 @@ int32_t plan_select(int64_t L, int32_t vocab_size, int32_t block_size, int32_t c
 }
 
 // ---------------------------------------------------------------------------------------------
-// The whole selection in one launch, for sequences of at most 16 blocks: a CTA per block, the CTAs one cluster.
-// The presence sets stay in shared memory and are read there by the CTAs that form the df of a slice of the vocabulary
-// each; the df of the block's tokens, the chunks' ranks and the selected chunks are the CTA's own.  What crosses
+// The whole selection in one launch, for sequences of at most 16 blocks: a CTA per block, in a cluster of 16 (8).
+// The presence sets stay in shared memory and are read there by the CTAs, those without a block too, that form the df of a slice
+// of the vocabulary each; the df of the block's tokens, the chunks' ranks and the selected chunks are the CTA's own.  What crosses
 // CTAs are two cluster barriers instead of three launches, and the df table (a byte per entry, in L2).  Bound by a chain of
 // latencies: each thread's loads are issued together (one at a time: 45,011 tokens 10.2 us, 8.0 like this and with a look at
 // the presence bit before the atomic).
@@ -604,7 +604,7 @@ __device__ __forceinline__ int taken_before(bool take, int* warp_sums) {
 struct ClusterArgs {
     const uint32_t* ids;
     int64_t L;
-    int block_size, chunk, k, sink, vocab_size, words;
+    int n_blocks, block_size, chunk, k, sink, vocab_size, words;
     uint8_t* df_table;                          // [vocab_size rounded up to 32], of uint16 with kModeTable
     int32_t *sel_chunks, *prefix_idx, *prefix_len;
     uint32_t* df_out;
@@ -622,7 +622,7 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
     __shared__ int s_warp[32], s_hist[32], s_short[kClusterBlocks], s_threshold, s_need;
     __shared__ float s_idf[kClusterBlocks + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b = blockIdx.x, n_blocks = gridDim.x;
+    const int b = blockIdx.x, n_blocks = a.n_blocks;            // CTAs from n_blocks on have a slice of the vocabulary only
     const int C = (a.block_size + a.chunk - 1) / a.chunk;
     const ClusterShape at(a.words, a.block_size, C, a.chunk, a.k, kScores);
     uint32_t* bits = reinterpret_cast<uint32_t*>(smem_c + at.bits);
@@ -632,9 +632,10 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
     const uint32_t V = static_cast<uint32_t>(a.vocab_size);
     const PrefixGeometry geo = prefix_geometry(b, n_blocks, a.L, a.block_size, a.chunk, a.k, a.sink);
     const int64_t lo = static_cast<int64_t>(b) * a.block_size;
-    const int len_b = static_cast<int>(min(static_cast<int64_t>(a.block_size), a.L - lo));
+    const int len_b = b < n_blocks ? static_cast<int>(min(static_cast<int64_t>(a.block_size), a.L - lo)) : 0;
 
-    for (int w = tid; w < a.words; w += kClusterThreads) bits[w] = 0u;
+    if (b < n_blocks)
+        for (int w = tid; w < a.words; w += kClusterThreads) bits[w] = 0u;
     if (tid < 32) s_hist[tid] = 0;
     grid_dependency_wait();            // the token ids, and the workspace, may be in use by the launch before this one
     grid_launch_dependents();
@@ -659,7 +660,7 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
     cluster_sync();                    // every block's set is complete
 
     // ---- df of this CTA's slice of the vocabulary: the sets' words added up bit by bit, 32 entries a thread ----
-    const int per_cta = (a.words + n_blocks - 1) / n_blocks, w_end = min(a.words, (b + 1) * per_cta);
+    const int n_ctas = gridDim.x, per_cta = (a.words + n_ctas - 1) / n_ctas, w_end = min(a.words, (b + 1) * per_cta);
     for (int w = b * per_cta + tid; w < w_end; w += kClusterThreads) {
         uint32_t x[kClusterBlocks], plane[5] = {0u, 0u, 0u, 0u, 0u};
         const uint32_t addr = smem_u32(bits + w);
@@ -715,6 +716,11 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
                 if (a.idf_out != nullptr) a.idf_out[i] = s_idf[df[j]];
             }
         }
+    }
+    const bool shifted = geo.tail != a.chunk && a.k > 0 && n_blocks > 1;       // a third barrier at the end, the same for all CTAs
+    if (b >= n_blocks) {
+        if (shifted) cluster_sync();
+        return;
     }
     constexpr uint32_t kNoToken = 255;
     uint32_t mine_df[kPerThread];
@@ -866,7 +872,7 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
     }
     // ---- the prefix list; its entries are shifted by earlier blocks that selected their short last chunk ----
     int offset = geo.sink_eff + b * a.k * a.chunk;
-    if (geo.tail != a.chunk && a.k > 0 && n_blocks > 1) {
+    if (shifted) {
         const uint32_t is_short = tid == C - 1 && take && len_b == a.block_size ? 1u : 0u;
         if (tid == C - 1)
             for (int j = 0; j < n_blocks; ++j) st_cluster_u32(smem_u32(s_short + b), j, is_short);
@@ -913,21 +919,36 @@ bool cluster_fits(int ctas) {
     return n > 0;
 }
 
-// Whether a selection of this shape is the cluster's: at most 16 blocks that their CTAs get through in less time than the host
-// takes for three launches more.  us a call in a row of them, one launch / four: levels, blocks of 1024 tokens 6.3 / 12.6, of
-// 4157 7.9 / 12.9, of 5000 8.0 / 12.6, of 8192 about even; BM25, 1024 8.6 / 15.2, 1665 13.7 / 15.4, 4157 15.6 / 15.5 (the
-// divisions of a block's terms are one SM's then), the other scores between the two.
-// Blocks above that share the df table's launch and have the scores formed by the whole chip, three launches instead of four: BM25
-// over 16 blocks of 8192 15.5 -> 14.4, the type-token ratio over 6 of 4157 15.5 -> 14.2 (on the device 12.3 -> 8.7).
-constexpr int kClusterLevelTokens = 6144, kClusterScoreTokens = 2048;
-bool cluster_table_takes(const SelectPlan& p, int32_t block_size) {
-    return p.n_blocks <= kClusterBlocks && block_size <= kClusterTokens && static_cast<size_t>(p.words) * 64 <= p.df_bytes &&
-           ClusterShape(p.words, block_size, p.C, 1, 0, false).tokens <= kMaxDynSmem - 2048 && cluster_fits(p.n_blocks);
+// CTAs of the cluster; 0 where none fits.  Sixteen also for few blocks, since the vocabulary is shared out among all of them: with a
+// CTA per block one block took 13.4 us with 128,256 entries and 71 with a million (the four launches 5.8 and 10.5 on the device), with
+// eight CTAs 5.7 and 13.3, with sixteen 5.4 and 9.5.
+int cluster_ctas(const SelectPlan& p) {
+    if (p.n_blocks <= kClusterBlocks && cluster_fits(kClusterBlocks)) return kClusterBlocks;
+    return p.n_blocks <= 8 && cluster_fits(8) ? 8 : 0;
 }
-bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32_t k, bool scores) {
-    return p.n_blocks <= kClusterBlocks && block_size <= (scores ? kClusterScoreTokens : kClusterLevelTokens) && p.C <= kClusterChunks &&
-           ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 2048 &&
-           static_cast<size_t>(p.words) * 32 <= p.df_bytes && cluster_fits(p.n_blocks);
+
+// Whether a selection of this shape is the cluster's: at most 16 blocks that their CTAs get through in less time than the host
+// takes for three launches more.  us a call in a row of them from Python, one launch / four, with the time on the device in brackets:
+// levels, blocks of 128 to 6144 tokens, up to 500,000 entries 9.6-12.5 (5-12) / 16.8 (5-12); the caller's tables of 128,256 entries as
+// well 13.9 (6.9-9.1) / 21.1 (5.8-8.5), of a million 31 (20) / 21.3 (12).  Scores, 16 blocks, one launch / three (see below): BM25,
+// blocks of 1024 11.4 (8.0) / 17.6 (7.0), of 2048 11.4 (9.6) / 17.8 (7.5); the divisions of a block's terms are one SM's in one launch.
+// Blocks above that share the df table's launch and have the scores formed by the whole chip, three launches instead of
+// four: BM25 over blocks of 8192, 128,256 entries, 1 block 17.1 (9.9) / 19.5 (10.7), 16 blocks 17.3 (13.2) / 19.7 (14.7); with more
+// entries the table costs the few CTAs more than the launch does: 500,000 18.3 (12.8) / 20.2 (12.6), a million 24.3 (17.4) / 19.8 (15.8).
+constexpr int kClusterLevelTokens = 6144, kClusterScoreTokens = 2048;
+constexpr int kClusterDfWords = 4096, kClusterTableWords = 16384;
+bool cluster_table_takes(const SelectPlan& p, int32_t block_size) {
+    return p.n_blocks <= kClusterBlocks && block_size <= kClusterTokens && p.words <= kClusterTableWords &&
+           static_cast<size_t>(p.words) * 64 <= p.df_bytes &&
+           ClusterShape(p.words, block_size, p.C, 1, 0, false).tokens <= kMaxDynSmem - 2048 && cluster_ctas(p) > 0;
+}
+// mode: a score or kModeLevels.  tables: the caller wants df or IDF.
+bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32_t k, int mode, bool tables) {
+    const bool scores = mode != kModeLevels;
+    if (p.n_blocks > kClusterBlocks || block_size > (scores ? kClusterScoreTokens : kClusterLevelTokens) || p.C > kClusterChunks) return false;
+    if (tables && p.words > kClusterDfWords) return false;
+    return ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 2048 &&
+           static_cast<size_t>(p.words) * 32 <= p.df_bytes && cluster_ctas(p) > 0;
 }
 
 template <int kMode, typename Table>
@@ -936,10 +957,11 @@ cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const T
     const size_t smem = kMode == kModeTable ? shape.tokens : shape.total;
     auto kernel = select_cluster_kernel<kMode>;
     cudaError_t e = allow_smem(kernel, smem);
-    if (e == cudaSuccess && p.n_blocks > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    const int ctas = cluster_ctas(p);
+    if (e == cudaSuccess && ctas > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(p.n_blocks);
+    cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(kClusterThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -947,7 +969,7 @@ cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const T
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = static_cast<unsigned>(p.n_blocks);
+    attr[1].val.clusterDim.x = static_cast<unsigned>(ctas);
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
@@ -983,8 +1005,8 @@ extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, in
     if (rc != PULSAR_OK) return rc;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
 
-    if (cluster_takes(p, block_size, chunk, k, false)) {
-        const ClusterArgs args{token_ids, L, block_size, chunk, k, sink, vocab_size, p.words,
+    if (cluster_takes(p, block_size, chunk, k, kModeLevels, df_out != nullptr || idf_out != nullptr)) {
+        const ClusterArgs args{token_ids, L, p.n_blocks, block_size, chunk, k, sink, vocab_size, p.words,
                                static_cast<uint8_t*>(workspace) + p.bitmap_bytes, sel_chunks, prefix_idx, prefix_len, df_out, idf_out,
                                nullptr, device_status};
         PULSAR_CUDA_OK(launch_cluster<kModeLevels>(p, args, 0, stream));
@@ -1106,8 +1128,8 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const SelectPlan& b = p.base;
 
-    if (cluster_takes(b, block_size, chunk, k, true)) {
-        const ClusterArgs args{token_ids, L, block_size, chunk, k, sink, vocab_size, b.words,
+    if (cluster_takes(b, block_size, chunk, k, score_mode, false)) {
+        const ClusterArgs args{token_ids, L, b.n_blocks, block_size, chunk, k, sink, vocab_size, b.words,
                                static_cast<uint8_t*>(workspace) + b.bitmap_bytes, sel_chunks, prefix_idx, prefix_len, nullptr, nullptr,
                                score_out, device_status};
         const auto tab = score_table<kClusterBlocks>(b, score_mode, L, block_size, chunk);
@@ -1124,7 +1146,7 @@ extern "C" int32_t pulsar_chunk_select(const uint32_t* token_ids, int64_t L, int
                               : reinterpret_cast<double*>(static_cast<char*>(workspace) + b.bitmap_bytes + b.df_bytes);
 
     if (cluster_table_takes(b, block_size)) {
-        const ClusterArgs args{token_ids, L, block_size, chunk, k, sink, vocab_size, b.words, reinterpret_cast<uint8_t*>(df_table),
+        const ClusterArgs args{token_ids, L, b.n_blocks, block_size, chunk, k, sink, vocab_size, b.words, reinterpret_cast<uint8_t*>(df_table),
                                nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, device_status};
         PULSAR_CUDA_OK(launch_cluster<kModeTable>(b, args, 0, stream));
         count_launch();

@@ -25,6 +25,9 @@ DEV = "cuda:0"
     (17 * 64, 64, 8, 2, 5, 100, False),            # 17 blocks
     (9 * 50 - 49, 50, 3, 17, 50, 1000, True),      # a last block of one token, every chunk selected
     (1024, 128, 33, 3, 0, 5, True),
+    (700, 700, 9, 4, 3, 131072, True),             # one block: the vocabulary shared out among CTAs without one; the most entries
+    (700, 700, 9, 4, 3, 131073, None),             # of tables for the caller, and one more
+    (3 * 500 - 1, 500, 33, 4, 3, 524289, None),    # more entries than the launch of the df table takes
 ])
 def test_selection_at_the_edges_of_one_launch(L, block, chunk, k, sink, vocab, one_launch):
     rng = np.random.default_rng(L)
@@ -36,15 +39,19 @@ def test_selection_at_the_edges_of_one_launch(L, block, chunk, k, sink, vocab, o
         np.testing.assert_array_equal(got[name].cpu().numpy(), ref[name], err_msg=name)
     np.testing.assert_array_equal(got["df"].cpu().numpy().view(np.uint32), ref["df"])
     np.testing.assert_allclose(got["idf"].cpu().numpy(), ref["idf"], rtol=0, atol=1e-6)
-    assert (len(kernel_names(call)) == 1) == (one_launch is not False)
+    tables = vocab > 131072
+    assert (len(kernel_names(call)) == 1) == (one_launch is not False and not tables)
+    if one_launch is None and tables:                              # without the tables it is one launch again
+        assert len(kernel_names(lambda: binding.pulsar_maxidf_select(ids_d, vocab, block, chunk, k, sink))) == 1
     for mode in binding.SCORE_MODES:
         got = binding.pulsar_chunk_select(ids_d, vocab, block, chunk, k, sink, mode, want_score=True)
         ref = oracle.chunk_select(ids, vocab, block, chunk, k, sink, mode)
         for name in ("sel_chunks", "prefix_idx", "prefix_len"):
             np.testing.assert_array_equal(got[name].cpu().numpy(), ref[name], err_msg=f"{mode} {name}")
         names = kernel_names(lambda: binding.pulsar_chunk_select(ids_d, vocab, block, chunk, k, sink, mode))
-        table = L <= 16 * block and block <= 8192                  # the df table in one launch, the scores in theirs
-        assert len(names) == (1 if one_launch is True else 3 if table else 4), names
+        one = L <= 16 * block and block <= 2048 and block <= 1024 * chunk
+        table = L <= 16 * block and block <= 8192 and vocab <= 16384 * 32        # the df table in one launch, the scores in theirs
+        assert len(names) == (1 if one else 3 if table else 4), names
         assert np.array_equal(got["score"].cpu().numpy(), ref["score"]), mode
 
 
