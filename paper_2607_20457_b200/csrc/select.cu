@@ -931,8 +931,10 @@ int cluster_ctas(const SelectPlan& p) {
 // takes for three launches more.  us a call in a row of them from Python, one launch / four, with the time on the device in brackets:
 // levels, blocks of 128 to 6144 tokens, up to 500,000 entries 9.6-12.5 (5-12) / 16.8 (5-12); the caller's tables of 128,256 entries as
 // well 13.9 (6.9-9.1) / 21.1 (5.8-8.5), of a million 31 (20) / 21.3 (12).  Scores, 16 blocks, one launch / three (see below): BM25,
-// blocks of 1024 11.4 (8.0) / 17.6 (7.0), of 2048 11.4 (9.6) / 17.8 (7.5); the divisions of a block's terms are one SM's in one launch.
-// Blocks above that share the df table's launch and have the scores formed by the whole chip, three launches instead of
+// blocks of 1024 11.4 (8.0) / 17.6 (7.0), of 2048 11.4 (9.6) / 17.8 (7.5); the divisions of a block's terms are one SM's in one launch, as are
+// the comparisons of a long chunk's positions: chunks of 64 in blocks of 2048 13.8 / 17.9, of 100 21.4 / 18.0, in blocks of
+// 1024 16.2 / 17.7, of 512 in blocks of 1024 87 / 93; type-token ratio, chunks of 128 14.3 / 17.5, of 256 29.7 / 23.6.
+// Blocks and chunks above that share the df table's launch and have the scores formed by the whole chip, three launches instead of
 // four: BM25 over blocks of 8192, 128,256 entries, 1 block 17.1 (9.9) / 19.5 (10.7), 16 blocks 17.3 (13.2) / 19.7 (14.7); with more
 // entries the table costs the few CTAs more than the launch does: 500,000 18.3 (12.8) / 20.2 (12.6), a million 24.3 (17.4) / 19.8 (15.8).
 constexpr int kClusterLevelTokens = 6144, kClusterScoreTokens = 2048;
@@ -947,6 +949,8 @@ bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32
     const bool scores = mode != kModeLevels;
     if (p.n_blocks > kClusterBlocks || block_size > (scores ? kClusterScoreTokens : kClusterLevelTokens) || p.C > kClusterChunks) return false;
     if (tables && p.words > kClusterDfWords) return false;
+    if (mode == PULSAR_SCORE_BM25 && chunk > 64 && block_size > 1024) return false;
+    if (mode == PULSAR_SCORE_TYPE_TOKEN && chunk > 128) return false;
     return ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 2048 &&
            static_cast<size_t>(p.words) * 32 <= p.df_bytes && cluster_ctas(p) > 0;
 }

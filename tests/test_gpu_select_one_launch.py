@@ -28,6 +28,8 @@ DEV = "cuda:0"
     (700, 700, 9, 4, 3, 131072, True),             # one block: the vocabulary shared out among CTAs without one; the most entries
     (700, 700, 9, 4, 3, 131073, None),             # of tables for the caller, and one more
     (3 * 500 - 1, 500, 33, 4, 3, 524289, None),    # more entries than the launch of the df table takes
+    (2050, 1025, 65, 4, 3, 100, True),             # long chunks in long blocks: the scores that compare positions are apart
+    (1024, 1024, 129, 2, 3, 100, True),
 ])
 def test_selection_at_the_edges_of_one_launch(L, block, chunk, k, sink, vocab, one_launch):
     rng = np.random.default_rng(L)
@@ -49,7 +51,8 @@ def test_selection_at_the_edges_of_one_launch(L, block, chunk, k, sink, vocab, o
         for name in ("sel_chunks", "prefix_idx", "prefix_len"):
             np.testing.assert_array_equal(got[name].cpu().numpy(), ref[name], err_msg=f"{mode} {name}")
         names = kernel_names(lambda: binding.pulsar_chunk_select(ids_d, vocab, block, chunk, k, sink, mode))
-        one = L <= 16 * block and block <= 2048 and block <= 1024 * chunk
+        apart = mode == "bm25" and chunk > 64 and block > 1024 or mode == "type_token" and chunk > 128
+        one = L <= 16 * block and block <= 2048 and block <= 1024 * chunk and not apart
         table = L <= 16 * block and block <= 8192 and vocab <= 16384 * 32        # the df table in one launch, the scores in theirs
         assert len(names) == (1 if one else 3 if table else 4), names
         assert np.array_equal(got["score"].cpu().numpy(), ref["score"]), mode
