@@ -294,8 +294,9 @@ def pulsar_encode_step(token_ids, vocab_size: int, block_size: int, chunk: int, 
                        O2, LSE2, workspaces, softmax_scale: float = 0.0, n_splits: int = 0, status=None):
     """One layer of one context in one call: ``pulsar_maxidf_select``, ``pulsar_phase1_attn`` on the prefix it selects, and
     ``pulsar_phase2_attn`` of ``Qq`` over all of K, V; the same results, with what does not depend on each other
-    overlapped.  Everything is preallocated: ``sel_out`` as ``out`` of the selection, O, LSE, O2, LSE2 the outputs, ``workspaces``
-    the three calls' (selection, Phase 1, Phase 2).  Returns the selection's dict."""
+    overlapped.  ``Qq`` has the heads and the head size of Q.  Everything is preallocated: ``sel_out`` as ``out`` of the selection, O,
+    LSE, O2, LSE2 the outputs (contiguous CUDA tensors of bf16 and float32; LSE and LSE2 may be None), ``workspaces`` the three calls'
+    (selection, Phase 1, Phase 2; CUDA bytes).  Returns the selection's dict."""
     sel, prefix_idx, prefix_len = _native_module().encode_step(
         token_ids, vocab_size, block_size, chunk, k, sink, Q, K, V, Qq, softmax_scale, n_splits, status, *sel_out, O, LSE, O2, LSE2,
         *workspaces)

@@ -419,28 +419,39 @@ PyObject* phase2_generate_step(Args& a) {
 }
 
 // (token_ids, vocab, block, chunk, k, sink, Q, K, V, Qq, scale, n_splits, status, sel_buf, prefix_idx, prefix_len, O1, LSE1, O2,
-//  LSE2, ws_select, ws_phase1, ws_phase2): the three calls of a step with everything preallocated
+//  LSE2, ws_select, ws_phase1, ws_phase2): the three calls of a step with everything preallocated; LSE1 and LSE2 may be None
 PyObject* encode_step(Args& a) {
     at::Tensor ids = a.i32s("token_ids");
     SelectShape z(a, ids.numel());
     Qkv x(a);
-    Query y;
-    y.Q = a.bf16("Qq", 3);
-    y.K = x.K;
-    y.V = x.V;
-    y.shape();
+    at::Tensor Qq = a.bf16("Qq", 3);
     const float scale = static_cast<float>(a.real());
     const int32_t splits = a.i32();
-    at::Tensor status = a.tensor(), sel = a.i32s("sel_chunks"), pidx = a.i32s("prefix_idx"), plen = a.i32s("prefix_len"), O1 = a.tensor(),
-               LSE1 = a.tensor(), O2 = a.tensor(), LSE2 = a.tensor(), ws_s = a.tensor(), ws_1 = a.tensor(), ws_2 = a.tensor();
+    at::Tensor status = a.tensor();
+    const int64_t nq = Qq.size(0);
     if (x.rows != z.L) raise(PyExc_ValueError, "one token id per row of Q, K and V");
+    if (Qq.size(1) != x.Hq || Qq.size(2) != x.d) raise(PyExc_ValueError, "Qq: expected the heads and the head size of Q");
+    const auto output = [&](at::ScalarType dtype, const char* name, int64_t n) {
+        at::Tensor t = a.needed(dtype, name);
+        if (t.numel() < n) raise(PyExc_ValueError, std::string(name) + ": expected at least " + std::to_string(n) + " entries");
+        return t;
+    };
+    const auto lse = [&](const char* name, int64_t n) {
+        if (a.i < a.n && a.v[a.i] == Py_None) return a.tensor();
+        return output(at::kFloat, name, n);
+    };
+    at::Tensor sel = output(at::kInt, "sel_chunks", z.B * z.k), pidx = output(at::kInt, "prefix_idx", z.prefix()),
+               plen = output(at::kInt, "prefix_len", z.B), O1 = output(at::kBFloat16, "O", x.rows * x.Hq * x.d),
+               LSE1 = lse("LSE", x.rows * x.Hq), O2 = output(at::kBFloat16, "O2", nq * x.Hq * x.d), LSE2 = lse("LSE2", nq * x.Hq),
+               ws_s = output(at::kByte, "selection workspace", 0), ws_1 = output(at::kByte, "Phase-1 workspace", 0),
+               ws_2 = output(at::kByte, "Phase-2 workspace", 0);                       // (their sizes are the library's to check)
     call("pulsar_encode_step", [&, st = stream()] {
         return g.pulsar_encode_step(ptr<uint32_t>(ids), z.L, z.V, z.block, z.chunk, z.k, z.sink, ptr<int32_t>(sel), ptr<int32_t>(pidx),
                                     ptr<int32_t>(plen), ptr<void>(ws_s), static_cast<size_t>(ws_s.numel()), in16(x.Q), in16(x.K),
                                     in16(x.V), x.Hq, x.Hkv, x.d, static_cast<int32_t>(z.prefix()), scale, ptr<uint16_t>(O1),
-                                    ptr<float>(LSE1), ptr<void>(ws_1), static_cast<size_t>(ws_1.numel()), in16(y.Q), y.nq, splits,
-                                    ptr<uint16_t>(O2), ptr<float>(LSE2), ptr<void>(ws_2), static_cast<size_t>(ws_2.numel()),
-                                    ptr<int32_t>(status), st);
+                                    ptr<float>(LSE1), ptr<void>(ws_1), static_cast<size_t>(ws_1.numel()), in16(Qq),
+                                    static_cast<int32_t>(nq), splits, ptr<uint16_t>(O2), ptr<float>(LSE2), ptr<void>(ws_2),
+                                    static_cast<size_t>(ws_2.numel()), ptr<int32_t>(status), st);
     });
     return result({head(sel, z.B * z.k).view({z.B, z.k}), head(pidx, z.prefix()), head(plen, z.B)});
 }

@@ -2,8 +2,8 @@
 
 ``ContextEncoder`` owns device buffers, workspaces and the status word for one
 workload shape, so that a step allocates nothing.  ``step_device`` takes inputs
-already resident on the GPU.  ``step_host`` takes pinned host tensors, copies them
-in, runs the same three C-ABI calls and copies every result back to pinned host
+already resident on the GPU and is one C-ABI call.  ``step_host`` takes pinned host tensors, copies them
+in, runs the same step and copies every result back to pinned host
 memory.  ``run_host_pipelined`` does that for a sequence of steps with two buffer
 sets and three streams, so that one step's copies overlap its neighbours'
 compute (PCIe is full duplex).  ``capture_step`` records a step as a CUDA graph.  All
@@ -59,14 +59,18 @@ class ContextEncoder:
     def step_device(self, ids, Q, K, V, Qq, record=None, slot=None):
         """Run selection, Phase 1 and Phase 2 on device tensors; outputs land in ``slot``
         (default: slot 0).  ``record``: optional list of four CUDA events recorded before,
-        between and after the three calls; without it they are one call that overlaps what it can."""
+        between and after selection, Phase 1 and Phase 2, which are three calls then; without it they are one call that
+        overlaps what it can."""
         w = self.w
         slot = self.slots[0] if slot is None else slot
-        if not record and ids.numel() == Q.shape[0] == w.L:
-            sel = binding.pulsar_encode_step(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink, Q, K, V, Qq, slot["sel"],
-                                             slot["O1"], slot["LSE1"], slot["O2"], slot["LSE2"],
-                                             (self.ws_select, self.ws_p1, self.ws_p2), n_splits=self.n_splits, status=self.status)
-            return dict(sel=sel, O1=slot["O1"], LSE1=slot["LSE1"], O2=slot["O2"], LSE2=slot["LSE2"], prefix_idx=sel["prefix_idx"])
+        if not record and ids.numel() == w.L and slot["LSE1"] is not None and slot["LSE2"] is not None:
+            try:
+                sel = binding.pulsar_encode_step(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink, Q, K, V, Qq, slot["sel"],
+                                                 slot["O1"], slot["LSE1"], slot["O2"], slot["LSE2"],
+                                                 (self.ws_select, self.ws_p1, self.ws_p2), n_splits=self.n_splits, status=self.status)
+                return dict(sel=sel, O1=slot["O1"], LSE1=slot["LSE1"], O2=slot["O2"], LSE2=slot["LSE2"], prefix_idx=sel["prefix_idx"])
+            except (TypeError, ValueError):
+                pass          # not what the one call takes (a query of other heads, outputs left to the calls): nothing was launched
         mark = lambda i: record[i].record() if record else None
         mark(0)
         sel = binding.pulsar_maxidf_select(ids, w.vocab_size, w.block_size, w.chunk, w.k, w.sink,
@@ -83,9 +87,9 @@ class ContextEncoder:
         return dict(sel=sel, O1=O1, LSE1=LSE1, O2=O2, LSE2=LSE2, prefix_idx=sel["prefix_idx"])
 
     def capture_step(self, slot_index: int = 0):
-        """The three calls of a step captured once as a CUDA graph on the slot's own device buffers
+        """A step captured once as a CUDA graph on the slot's own device buffers
         (fill ``slots[i]["ids" | "Q" | "K" | "V" | "Qq"]``, then ``graph.replay()``): one launch from
-        the host instead of nine, which matters when a step is shorter than the host's launch cadence.
+        the host instead of four to nine, which matters when a step is shorter than the host's launch cadence.
         Returns (graph, results); the results are the slot's output tensors."""
         slot = self.slots[slot_index]
         args = (slot["ids"], slot["Q"], slot["K"], slot["V"], slot["Qq"])

@@ -3,6 +3,7 @@ import pytest
 import torch
 
 from helpers import to_dev_ids
+from paper_2607_20457_b200 import binding
 from paper_2607_20457_b200 import workloads as W
 from paper_2607_20457_b200.pipeline import ContextEncoder
 
@@ -34,3 +35,53 @@ def test_one_call_equals_three(shape):
         got = keep(enc.step_device(*args))
         assert all(torch.equal(a, b) for a, b in zip(got, want))
     assert int(enc.status.item()) == 0
+
+
+def _encoder(**shape):
+    w = W.shrink(W.CONFIGS["tiny"], **shape)
+    enc = ContextEncoder(w, DEV)
+    Q, K, V = (t.to(DEV) for t in W.qkv(w))
+    return w, enc, (to_dev_ids(W.token_ids(w), DEV), Q, K, V, W.phase2_query(w).to(DEV))
+
+
+def _one_call(w, enc, args, slot, **other):
+    ids, Q, K, V, Qq = args
+    at = dict(Qq=Qq, O=slot["O1"], LSE=slot["LSE1"], O2=slot["O2"], LSE2=slot["LSE2"], sel=slot["sel"], K=K, V=V,
+              ws=(enc.ws_select, enc.ws_p1, enc.ws_p2), ids=ids) | other
+    return binding.pulsar_encode_step(at["ids"], w.vocab_size, w.block_size, w.chunk, w.k, w.sink, Q, at["K"], at["V"], at["Qq"], at["sel"],
+                                      at["O"], at["LSE"], at["O2"], at["LSE2"], at["ws"], n_splits=enc.n_splits, status=enc.status)
+
+
+def test_query_and_buffers_are_checked():
+    w, enc, args = _encoder(Hq=4, Hkv=2)
+    slot = enc.slots[0]
+    bf = lambda *s: torch.empty(*s, dtype=torch.bfloat16, device=DEV)
+    sel = slot["sel"]
+    bad = [(ValueError, dict(Qq=bf(w.nq, 2, w.d))), (ValueError, dict(Qq=bf(w.nq, w.Hq, 2 * w.d))),      # a query of another shape
+           (ValueError, dict(O=bf(w.L, w.Hq, w.d - 1))), (ValueError, dict(O2=bf(w.nq - 1, w.Hq, w.d))),
+           (ValueError, dict(LSE=slot["LSE1"][1:])), (ValueError, dict(LSE2=slot["LSE2"][1:])),
+           (TypeError, dict(O=None)), (TypeError, dict(O2=slot["O2"].float())), (TypeError, dict(LSE=slot["LSE1"].cpu())),
+           (TypeError, dict(O=bf(w.L, w.Hq, 2 * w.d)[..., ::2])),
+           (ValueError, dict(sel=(sel[0][:w.k], *sel[1:]))), (ValueError, dict(sel=(sel[0], sel[1][:5], sel[2]))),
+           (TypeError, dict(ws=(enc.ws_select, enc.ws_p1, None))), (TypeError, dict(ws=(enc.ws_select, enc.ws_p1.cpu(), enc.ws_p2)))]
+    before = binding.launch_count()
+    for error, other in bad:
+        with pytest.raises(error):
+            _one_call(w, enc, args, slot, **other)
+    assert binding.launch_count() == before
+    want = {k: slot[k].clone() for k in ("O1", "O2")} if _one_call(w, enc, args, slot) else None
+    _one_call(w, enc, args, slot, LSE=None, LSE2=None)                       # which are wanted or not
+    assert all(torch.equal(slot[k], t) for k, t in want.items())
+
+
+def test_what_one_call_does_not_take_goes_through_three():
+    w, enc, args = _encoder(Hq=4, Hkv=2, nq=64)
+    full = {k: t.clone() for k, t in enc.step_device(*args).items() if k != "sel"}
+    left = {k: None for k in ("O1", "LSE1", "O2", "LSE2", "sel")}            # outputs left to the calls to allocate
+    for slot in (left, {**enc.slots[0], "LSE1": None}, {**enc.slots[0], "LSE2": None}):
+        got = enc.step_device(*args, slot=slot)
+        assert all(torch.equal(got[k], t) for k, t in full.items())
+    few = args[4][:, :2].contiguous()                                        # a query of fewer heads than the context's
+    got = enc.step_device(*args[:4], few)
+    O2, _ = binding.pulsar_phase2_attn(few, args[2], args[3], 1, w.L, n_splits=enc.n_splits)
+    assert torch.equal(got["O2"].reshape(-1)[: O2.numel()], O2.reshape(-1))
