@@ -396,7 +396,8 @@ int32_t pulsar_phase2_attn(const uint16_t *Qq, int32_t nq,
  * selects, and pulsar_phase2_attn of the query over all L retained rows, which are K and V themselves.  Arguments,
  * requirements, workspaces and results are those of the three calls (Phase 2 with B = 1, block_size = L and no caller
  * partials; prefix_total = sink + (B - 1) * k * chunk entries of prefix_idx); what does not depend on each other is overlapped
- * on the device.  A call that is refused may have written the outputs of the parts before the one that refused it.
+ * on the device.  For that the workspaces and the outputs have to be apart from each other: where Phase 2's meet memory of the
+ * other two (a workspace given twice), it runs after them, as with three calls.  A call that is refused may have written the outputs of the parts before the one that refused it.
  * ------------------------------------------------------------------------------------------ */
 int32_t pulsar_encode_step(const uint32_t *token_ids, int64_t L, int32_t vocab_size,
                            int32_t block_size, int32_t chunk, int32_t k, int32_t sink,

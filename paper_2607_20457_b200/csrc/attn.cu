@@ -1906,6 +1906,23 @@ extern "C" int32_t pulsar_phase2_attn(const uint16_t* Qq, int32_t nq, const uint
 // Phase 2 needs nothing of Phase 1 but the keys and values that both read, so its attention is launched beside the
 // selection, which is a chain of latencies on 16 SMs, and its merge beside Phase 1 (4096 tokens 32.6 -> 24.6 us with the
 // selection's one launch).  With more work items than SMs, whose counter has to be cleared before it, it follows Phase 1.
+// So it does where it shares memory with the other two, which the three calls may, one after the other.
+namespace {
+struct Span {
+    const void* p;
+    uint64_t bytes;
+};
+bool meet(const Span& a, const Span& b) {
+    const auto begin = [](const Span& s) { return static_cast<uint64_t>(reinterpret_cast<uintptr_t>(s.p)); };
+    const auto end = [&](const Span& s) { return begin(s) + std::min<uint64_t>(s.bytes, UINT64_MAX - begin(s)); };      // (a size may be "all there is")
+    return a.p != nullptr && b.p != nullptr && begin(a) < end(b) && begin(b) < end(a);
+}
+template <int N, int M>
+bool meet(const Span (&a)[N], const Span (&b)[M]) {
+    return std::any_of(a, a + N, [&](const Span& x) { return std::any_of(b, b + M, [&](const Span& y) { return meet(x, y); }); });
+}
+}  // namespace
+
 extern "C" int32_t pulsar_encode_step(const uint32_t* token_ids, int64_t L, int32_t vocab_size, int32_t block_size, int32_t chunk,
                                       int32_t k, int32_t sink, int32_t* sel_chunks, int32_t* prefix_idx, int32_t* prefix_len,
                                       void* select_workspace, size_t select_workspace_bytes, const uint16_t* Q, const uint16_t* K,
@@ -1931,7 +1948,14 @@ extern "C" int32_t pulsar_encode_step(const uint32_t* token_ids, int64_t L, int3
     rc = plan_phase2(nq, 1, static_cast<int32_t>(L), Hq, Hkv, d, parts, unused_a, unused_b);
     if (rc != PULSAR_OK) return rc;
     const int64_t pairs = (static_cast<int64_t>(nq) * (Hq / Hkv) + 2 * kTileM - 1) / (2 * kTileM);
-    const bool beside = pairs * Hkv * parts <= sm_count();
+    const uint64_t n = static_cast<uint64_t>(L), B = (n + block_size - 1) / block_size;
+    const uint64_t entries = std::max<uint64_t>(prefix_total, sink + (B - 1) * k * chunk), row_q = 2ull * Hq * d, row_kv = 2ull * Hkv * d;
+    const Span written2[] = {{O2, nq * row_q}, {LSE2, 4ull * nq * Hq}, {phase2_workspace, phase2_workspace_bytes}};
+    const Span written1[] = {{O, n * row_q}, {LSE, 4 * n * Hq}, {phase1_workspace, phase1_workspace_bytes},
+                             {select_workspace, select_workspace_bytes}, {sel_chunks, 4 * B * k}, {prefix_idx, 4 * entries},
+                             {prefix_len, 4 * B}};
+    const Span read1[] = {{token_ids, 4 * n}, {Q, n * row_q}, {K, n * row_kv}, {V, n * row_kv}}, read2[] = {{Qq, nq * row_q}};
+    const bool beside = pairs * Hkv * parts <= sm_count() && !meet(written2, written1) && !meet(written2, read1) && !meet(written1, read2);
     rc = beside ? phase2(true) : phase1();
     if (rc != PULSAR_OK) return rc;
     rc = beside ? phase1() : phase2(false);

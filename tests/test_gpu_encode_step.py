@@ -2,7 +2,7 @@
 import pytest
 import torch
 
-from helpers import to_dev_ids
+from helpers import kernel_names, to_dev_ids
 from paper_2607_20457_b200 import binding
 from paper_2607_20457_b200 import workloads as W
 from paper_2607_20457_b200.pipeline import ContextEncoder
@@ -85,3 +85,35 @@ def test_what_one_call_does_not_take_goes_through_three():
     got = enc.step_device(*args[:4], few)
     O2, _ = binding.pulsar_phase2_attn(few, args[2], args[3], 1, w.L, n_splits=enc.n_splits)
     assert torch.equal(got["O2"].reshape(-1)[: O2.numel()], O2.reshape(-1))
+
+
+@pytest.mark.parametrize("nq", [1, 48])
+@pytest.mark.parametrize("shared", ["workspaces", "O2 in Q", "LSE2 in the selection's workspace", "Qq in O", "none"])
+def test_shared_memory_puts_phase_2_last(shared, nq):
+    """What three calls in a row may share, one call may: Phase 2 then follows the other two."""
+    w, enc, args = _encoder(nq=nq)
+    ids, Q, K, V, Qq = args
+    slot = enc.slots[0]
+    want = {k: t.clone() for k, t in enc.step_device(*args).items() if k != "sel"}
+    one = torch.empty(max(t.numel() for t in (enc.ws_select, enc.ws_p1, enc.ws_p2)), dtype=torch.uint8, device=DEV)
+    keep = Q.clone()
+    at = dict(workspaces=dict(ws=(one, one, one)), none={})
+    at["O2 in Q"] = dict(O2=Q[3: 3 + nq])                                   # Q is used up when Phase 2 writes
+    at["LSE2 in the selection's workspace"] = dict(LSE2=enc.ws_select[256: 256 + 4 * nq * w.Hq].view(torch.float32).view(nq, w.Hq))
+    at["Qq in O"] = dict(Qq=slot["O1"][:nq])                                # the query is Phase 1's output
+    other = at[shared]
+    for _ in range(3):
+        Q.copy_(keep)
+        _one_call(w, enc, args, slot, **other)
+        O2, LSE2 = other.get("O2", slot["O2"]).clone(), other.get("LSE2", slot["LSE2"]).clone()
+        if shared == "Qq in O":
+            ref = binding.pulsar_phase2_attn(want["O1"][:nq].contiguous(), K, V, 1, w.L, n_splits=enc.n_splits)
+        else:
+            ref = want["O2"], want["LSE2"]
+        assert torch.equal(O2, ref[0]) and torch.equal(LSE2, ref[1])
+        for k in ("O1", "LSE1", "prefix_idx"):
+            assert torch.equal(want[k], slot["sel"][1][: w.prefix_total] if k == "prefix_idx" else slot[k]), k
+    Q.copy_(keep)
+    names = [n for n, _ in kernel_names(lambda: _one_call(w, enc, args, slot, **other))]
+    phase2 = max(i for i, n in enumerate(names) if n in ("attn_kernel", "decode_kernel")) if shared != "none" else names.index("decode_kernel" if nq == 1 else "attn_kernel")
+    assert (phase2 > names.index("gather_prefix_kernel")) == (shared != "none"), names
