@@ -441,22 +441,31 @@ struct DecodePlan {
 };
 
 // One cluster per KV head, as large as fits for all heads at once, merges on chip.  More of them per head share the keys
-// better but leave a merge to a second launch.  A CTA takes 12.5 ns per kilobyte of keys and values, the chip 0.15; to that one
-// cluster adds 5 us and more of them 6.5.  Measured, one / several, us: 6001 keys of 2 heads 7.5 / 7.6, 20,000 13.1 / 8.9,
+// better but leave a merge to a second launch.  Measured, one / several, us: 6001 keys of 2 heads 7.5 / 7.6, 20,000 13.1 / 8.9,
 // 55,734 27.5 / 14.8; 16,384 of 8 heads 16.6 / 16.7, 32,768 27.7 / 27.7, 131,072 86.4 / 83.5; 22,842 of 8 heads, d = 64,
-// 13.0 / 12.7.  Of several, at least five per head: 131,072 keys of 8 heads 83.5 in 8 clusters of 4, 84.4 in 4 of 8.
+// 13.0 / 12.7.  Of several, at least five per head: 131,072 keys of 8 heads 83.5 in 8 clusters of 4, 84.4 in 4 of 8.  Clusters of
+// four from two per head on: of two CTAs they leave the launch with twice the clusters and partials, and 103,998 keys
+// of 16 heads take 129.8 us, in 4 clusters of four 125.4 (the tensor cores' form 123.6), of 24 heads 183.5, 180.1 in two of four (180.8).
+// The times are a fit to calls in a row, whose keys partly stay in L2 (so the rates are above the copy rate): what a call takes
+// besides the data, 5.1 us with one cluster, 6.5 with a second launch; the data at a CTA's rate or at the chip's, 1.2 us
+// later with one cluster, whose CTAs are fewer and end less evenly.  Several have to win by a microsecond, since one needs no
+// second launch where a launch costs more than in a row of calls.  Over 63 shapes (4 to 64 KV heads, 8000 to 103,998 keys) the
+// choice takes 1.00 times the time of the better form in the middle and 1.3 at most, and 1.015 of the tensor cores' at most, 0.87 in the middle.
 DecodePlan plan_decode(const DecodeCall& c) {
     const double bytes = 4.0 * (c.ctx_len + c.gen_len + c.n) * c.Hkv * c.d;
-    const auto per_cta = [&](const DecodePlan& p) { return bytes / (static_cast<double>(p.clusters) * c.Hkv * (1 << p.shift)) / 80e3; };
+    constexpr double kCtaRate = 80e3, kOneRate = 6.6e6, kMoreRate = 6.9e6;       // bytes per us
+    constexpr double kOne = 5.1, kOneTail = 1.2, kMore = 6.5, kMargin = 1.0;     // us
+    const auto per_cta = [&](const DecodePlan& p) { return bytes / (static_cast<double>(p.clusters) * c.Hkv * (1 << p.shift)) / kCtaRate; };
     DecodePlan one{0, 1}, more{0, 1};
     for (int shift = 1; shift <= kMaxClusterShift; ++shift) {
         const int heads_fit = active_clusters(shift) / c.Hkv;
         if (heads_fit >= 1) one.shift = shift;
-        if (heads_fit >= 5) more = {shift, static_cast<int>(std::min<int64_t>(heads_fit, c.max_parts))};
+        if (heads_fit >= (shift == 2 ? 2 : 5)) more = {shift, static_cast<int>(std::min<int64_t>(heads_fit, c.max_parts))};
     }
     if (more.clusters <= 1) return one;
-    const double t_one = 5.1 + std::max(per_cta(one), bytes / 6.6e6 + 1.2), t_more = 6.5 + std::max(per_cta(more), bytes / 6.9e6);
-    return t_more + 1.0 < t_one ? more : one;
+    const double t_one = kOne + std::max(per_cta(one), bytes / kOneRate + kOneTail);
+    const double t_more = kMore + std::max(per_cta(more), bytes / kMoreRate);
+    return t_more + kMargin < t_one ? more : one;
 }
 
 int32_t launch_decode_as(const DecodeCall& c, const DecodePlan& p, MergeTodo& todo, cudaStream_t stream) {

@@ -36,6 +36,7 @@ def draw(seed, *shapes):
     (1030, 3, 1, 200, 200),        # more KV heads than SMs: one CTA each
     (40000, 90, 1, 8, 2),          # long enough for every SM and a merge launch
     (30011, 1000, 4, 2, 1),
+    (60000, 5, 1, 16, 16),         # several clusters of four per KV head, fewer than five
 ])
 def test_generation_step(L, gen_len, n_new, Hq, Hkv, d):
     cap = gen_len + n_new + 5
