@@ -129,6 +129,32 @@ def test_gather_rows_and_bad_index():
     assert int(st.item()) & 0x2 and torch.equal(Ko[2], K[0])
 
 
+@pytest.mark.parametrize("rows,Hkv,d", [(1, 1, 8), (1023, 1, 8), (1025, 1, 8), (341, 3, 8), (342, 3, 8), (9, 16, 128), (700, 5, 24), (4, 1, 9000)])
+def test_row_copies_where_rows_and_ctas_do_not_meet(rows, Hkv, d):
+    """1024 vectors of 8 elements to a CTA: rows of 1 to 1125 of them, the last CTA full, over and short; one bad index."""
+    gen = torch.Generator(device=DEV).manual_seed(rows)
+    K, V = (torch.randn(2 * rows + 8, Hkv, d, generator=gen, device=DEV).bfloat16() for _ in range(2))
+    idx = torch.randint(0, K.shape[0], (rows,), generator=gen, device=DEV, dtype=torch.int32)
+    Ko, Vo = torch.full((2, rows + 1, Hkv, d), 7.0, device=DEV, dtype=torch.bfloat16)
+    st = binding.new_status(DEV)
+    binding.pulsar_gather_kv_rows(K, V, idx, Ko[:rows], Vo[:rows], status=st)
+    assert torch.equal(Ko[:rows], K[idx.long()]) and torch.equal(Vo[:rows], V[idx.long()]) and int(st.item()) == 0
+    assert (Ko[rows:] == 7).all() and (Vo[rows:] == 7).all()
+    idx[rows // 2] = -1
+    binding.pulsar_gather_kv_rows(K, V, idx, Ko[:rows], Vo[:rows], status=st)
+    assert int(st.item()) & 0x2 and torch.equal(Ko[:rows], K[idx.clamp(min=0).long()]) and (Vo[rows:] == 7).all()
+    # packing: two blocks of `rows` tokens in chunks of one, all but one chunk of each selected in descending order, three sink rows
+    n, k, sink = 2, max(rows - 1, 1), min(3, rows)
+    sel = torch.arange(rows - 1, rows - 1 - k, -1, device=DEV, dtype=torch.int32).repeat(4, 1)
+    Ks, Vs = torch.full((2, sink + n * k + 1, Hkv, d), 7.0, device=DEV, dtype=torch.bfloat16)
+    st.zero_()
+    binding.pulsar_pack_summary_kv(K[: n * rows], V[: n * rows], rows, sel, torch.tensor([1, 3], dtype=torch.int32, device=DEV), 4, 1, k,
+                                   sink, Ks, Vs, status=st)
+    src = torch.cat([torch.arange(sink, device=DEV)] + [s * rows + sel[0].long() for s in range(n)])
+    assert torch.equal(Ks[:-1], K[src]) and torch.equal(Vs[:-1], V[src]) and int(st.item()) == 0
+    assert (Ks[-1] == 7).all() and (Vs[-1] == 7).all()
+
+
 @pytest.mark.parametrize("H,nq", [(1, 5), (2, 37), (4, 1), (4, 130)])
 def test_phase2_with_the_exchange_fused_into_the_merge(H, nq):
     """Every rank merges its slice of the rows straight from all ranks' partial buffers (here all on
