@@ -68,6 +68,9 @@ lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict_
     if (!kBeside) grid_dependency_wait();        // launched beside the attention kernel that writes the partials: wait for it
     grid_launch_dependents();
     constexpr int kD = 32 * kVec, kInFlight = 8;
+    // Beside another launch the partials are read from L2, where the launch that wrote them has left them: no wait stands
+    // between an SM's L1, which may hold the last call's, and these loads.
+    const auto load = [](const auto* p) { return kBeside ? __ldcg(p) : *p; };
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t row = static_cast<int64_t>(blockIdx.x) * kRows + (kWarps == 1 ? warp : 0);
     if (row >= rows) return;                                     // kRows > 1 only: no barrier follows
@@ -83,13 +86,13 @@ lse_merge_rows_kernel(const float* __restrict__ part_O, const float* __restrict_
             const int j = j0 + i * kWarps;
             l[i] = -INFINITY;
             if (j < n_parts) {
-                l[i] = part_LSE[static_cast<size_t>(j) * stride_L + row];
+                l[i] = load(part_LSE + static_cast<size_t>(j) * stride_L + row);
                 const float* p = src + static_cast<size_t>(j) * stride_O;
                 if (kVec == 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(p);
+                    const float4 v = load(reinterpret_cast<const float4*>(p));
                     o[i][0] = v.x; o[i][1] = v.y; o[i][kVec - 2] = v.z; o[i][kVec - 1] = v.w;
                 } else {
-                    const float2 v = *reinterpret_cast<const float2*>(p);
+                    const float2 v = load(reinterpret_cast<const float2*>(p));
                     o[i][0] = v.x; o[i][1] = v.y;
                 }
             } else {
