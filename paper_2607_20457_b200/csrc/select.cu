@@ -290,12 +290,65 @@ struct ScoreTable {
     double k1_plus_1, k1, b, one_minus_b, mean_len;   // BM25: D(C) = (1 - b) + b * (|C| / mean chunk length)
 };
 
+// The terms of a chunk's sum under TF-IDF and BM25, formed by a warp side by side, one per position; a position that carries no
+// term holds 0.0, which leaves the sum's bits as they are.  Under BM25 and the type-token ratio each position is compared with all
+// others of the chunk, for a chunk of at most 32 tokens in one warp match.  Returns the number of types (type-token ratio).
+// df_of(p, first): the df of the token at position p, kNoDf where its id lies outside the vocabulary; tok: the ids, read only
+// where positions are compared.
+template <int kMode, uint32_t kNoDf, int kBlocks, typename DfOf>
+__device__ __forceinline__ int chunk_terms(const uint32_t* tok, int len, const ScoreTable<kBlocks>& tab, DfOf df_of, double* term) {
+    const int lane = threadIdx.x & 31;
+    double k1_times_D = 0.0;
+    if (kMode == PULSAR_SCORE_BM25)
+        // D(C) = (1 - b) + b * (|C| / mean chunk length), then k1 * D(C): one rounding per operation
+        k1_times_D =
+            __dmul_rn(tab.k1, __dadd_rn(tab.one_minus_b, __dmul_rn(tab.b, __ddiv_rn(static_cast<double>(len), tab.mean_len))));
+    int distinct = 0;
+    for (int p0 = 0; p0 < len; p0 += 32) {
+        const int p = p0 + lane;
+        const bool in = p < len;
+        bool first = in;
+        int tf = 0;
+        if (kMode != PULSAR_SCORE_TF_IDF) {
+            const uint32_t t = in ? tok[p] : ~0u;
+            if (len <= 32) {
+                // (an id of ~0 meets the lanes past the end, which come after it: its count, unused, is too large)
+                const uint32_t same = __match_any_sync(0xffffffffu, t);
+                first = in && lane == __ffs(same) - 1;
+                tf = __popc(same);
+            } else {
+                int before = 0;
+#pragma unroll 16                                    // 1024 positions 256 us, with the compiler's four at a time 314
+                for (int q = 0; q < len; ++q) {
+                    const int eq = tok[q] == t ? 1 : 0;
+                    tf += eq;
+                    before += q < p ? eq : 0;
+                }
+                first = in && before == 0;
+            }
+        }
+        if (kMode == PULSAR_SCORE_TYPE_TOKEN) {
+            distinct += __popc(__ballot_sync(0xffffffffu, first));
+        } else if (in) {
+            const uint32_t df = df_of(p, first);
+            double x = 0.0;
+            if (first && df != kNoDf) {
+                x = tab.by_df[df];
+                if (kMode == PULSAR_SCORE_BM25) {
+                    const double tfd = static_cast<double>(tf);
+                    x = __ddiv_rn(__dmul_rn(x, __dmul_rn(tfd, tab.k1_plus_1)), __dadd_rn(tfd, k1_times_D));
+                }
+            }
+            term[p] = x;
+        }
+    }
+    return distinct;
+}
+
 // One warp per chunk slot.  Slot c of block b covers the tokens [b*block_size + c*chunk, +chunk)
 // that lie inside the block and the sequence (|C| = len); a slot without a chunk scores -inf.
-// The lanes form the terms of the sum side by side -- for BM25 and the type-token ratio each position is
-// compared with all others of the chunk, for a chunk of at most 32 tokens in one warp match -- and
-// lane 0 adds them up in the order of the equations.  A position that carries no term holds 0.0, which
-// leaves the sum's bits as they are.  Latency-bound: one thread per chunk, walking the chunk's pairs
+// The lanes form the terms (chunk_terms), and lane 0 adds them up in the order of the equations.
+// Latency-bound: one thread per chunk, walking the chunk's pairs
 // of positions serially, took 92 us for 4096 chunks of 32 tokens under BM25 (the whole call 115 us, 16 us with
 // this form and the four launches chained as programmatic dependents).
 constexpr int kScoreWarps = 4;
@@ -331,47 +384,8 @@ chunk_score_kernel(const uint32_t* __restrict__ ids, const uint16_t* __restrict_
         if (lane == 0) score[slot] = best;
         return;
     }
-    double k1_times_D = 0.0;
-    if (kMode == PULSAR_SCORE_BM25)
-        // D(C) = (1 - b) + b * (|C| / mean chunk length), then k1 * D(C): one rounding per operation
-        k1_times_D =
-            __dmul_rn(tab.k1, __dadd_rn(tab.one_minus_b, __dmul_rn(tab.b, __ddiv_rn(static_cast<double>(len), tab.mean_len))));
-    int distinct = 0;
-    for (int p0 = 0; p0 < len; p0 += 32) {
-        const int p = p0 + lane;
-        const bool in = p < len;
-        const uint32_t t = in ? tok[p] : 0u;
-        bool first = in;
-        int tf = 0;
-        if (kMode != PULSAR_SCORE_TF_IDF) {
-            if (len <= 32) {
-                const uint32_t same = __match_any_sync(0xffffffffu, in ? static_cast<uint64_t>(t) : ~0ull);
-                first = in && lane == __ffs(same) - 1;
-                tf = __popc(same);
-            } else {
-                int before = 0;
-                for (int q = 0; q < len; ++q) {
-                    const int eq = tok[q] == t ? 1 : 0;
-                    tf += eq;
-                    before += q < p ? eq : 0;
-                }
-                first = in && before == 0;
-            }
-        }
-        if (kMode == PULSAR_SCORE_TYPE_TOKEN) {
-            distinct += __popc(__ballot_sync(0xffffffffu, first));
-        } else if (in) {
-            double x = 0.0;
-            if (first && t < V) {
-                x = tab.by_df[df_table[t]];
-                if (kMode == PULSAR_SCORE_BM25) {
-                    const double tfd = static_cast<double>(tf);
-                    x = __ddiv_rn(__dmul_rn(x, __dmul_rn(tfd, tab.k1_plus_1)), __dadd_rn(tfd, k1_times_D));
-                }
-            }
-            term[p] = x;
-        }
-    }
+    const int distinct = chunk_terms<kMode, ~0u>(
+        tok, len, tab, [&](int p, bool first) { return first && tok[p] < V ? df_table[tok[p]] : ~0u; }, term);
     __syncwarp();
     // The selection's CTAs, one per block and bound by float64 compares, are placed where there is room.  Let in while this grid
     // still fills the chip they were put several to an SM: 16 blocks of 2048 chunks of 4 tokens under BM25 took 829 us, 190 us
@@ -562,11 +576,12 @@ constexpr int kModeTable = -2;                  // the df table alone, 16 bits a
 
 struct ClusterShape {
     size_t bits, tokens, dfs, ranks, chosen, terms, total;       // offsets in shared memory
-    __host__ __device__ ClusterShape(int words, int block_size, int C, int chunk, int k, bool scores) {
+    __host__ __device__ ClusterShape(int words, int block_size, int C, int chunk, int k, int mode) {
         const auto up = [](size_t x) { return (x + 15) / 16 * 16; };
+        const bool scores = mode >= 0, ids = mode == PULSAR_SCORE_BM25 || mode == PULSAR_SCORE_TYPE_TOKEN;
         bits = 0;
         tokens = up(static_cast<size_t>(words) * 4);
-        dfs = tokens + up(static_cast<size_t>(block_size) * 4);
+        dfs = tokens + (ids ? up(static_cast<size_t>(block_size) * 4) : 0);
         ranks = dfs + up(block_size);
         chosen = ranks + up(static_cast<size_t>(C) * (scores ? 8 : 4));
         terms = chosen + up(static_cast<size_t>(k) * 4);
@@ -624,7 +639,7 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x, n_blocks = a.n_blocks;            // CTAs from n_blocks on have a slice of the vocabulary only
     const int C = (a.block_size + a.chunk - 1) / a.chunk;
-    const ClusterShape at(a.words, a.block_size, C, a.chunk, a.k, kScores);
+    const ClusterShape at(a.words, a.block_size, C, a.chunk, a.k, kMode);
     uint32_t* bits = reinterpret_cast<uint32_t*>(smem_c + at.bits);
     uint32_t* tok = reinterpret_cast<uint32_t*>(smem_c + at.tokens);
     uint8_t* dfs = smem_c + at.dfs;
@@ -788,48 +803,7 @@ select_cluster_kernel(const __grid_constant__ ClusterArgs a,
                 if (lane == 0) score[c] = least == kNoToken ? -CUDART_INF : tab.by_df[least];
                 continue;
             }
-            double k1_times_D = 0.0;
-            if (kMode == PULSAR_SCORE_BM25)
-                k1_times_D = __dmul_rn(
-                    tab.k1, __dadd_rn(tab.one_minus_b, __dmul_rn(tab.b, __ddiv_rn(static_cast<double>(len), tab.mean_len))));
-            int distinct = 0;
-            for (int p0 = 0; p0 < len; p0 += 32) {
-                const int p = p0 + lane;
-                const bool in = p < len;
-                bool first = in;
-                int tf = 0;
-                if (kMode != PULSAR_SCORE_TF_IDF) {
-                    const uint32_t t = in ? ct[p] : ~0u;
-                    if (len <= 32) {
-                        // (an id of ~0 meets the lanes past the end, which come after it: its count, unused, is too large)
-                        const uint32_t same = __match_any_sync(0xffffffffu, t);
-                        first = in && lane == __ffs(same) - 1;
-                        tf = __popc(same);
-                    } else {
-                        int before = 0;
-                        for (int q = 0; q < len; ++q) {
-                            const int eq = ct[q] == t ? 1 : 0;
-                            tf += eq;
-                            before += q < p ? eq : 0;
-                        }
-                        first = in && before == 0;
-                    }
-                }
-                if (kMode == PULSAR_SCORE_TYPE_TOKEN) {
-                    distinct += __popc(__ballot_sync(0xffffffffu, first));
-                } else if (in) {
-                    const uint32_t df = cd[p];
-                    double x = 0.0;
-                    if (first && df != kNoToken) {
-                        x = tab.by_df[df];
-                        if (kMode == PULSAR_SCORE_BM25) {
-                            const double tfd = static_cast<double>(tf);
-                            x = __ddiv_rn(__dmul_rn(x, __dmul_rn(tfd, tab.k1_plus_1)), __dadd_rn(tfd, k1_times_D));
-                        }
-                    }
-                    terms[p] = x;
-                }
-            }
+            const int distinct = chunk_terms<kMode, kNoToken>(ct, len, tab, [&](int p, bool) { return cd[p]; }, terms);
             if (kMode == PULSAR_SCORE_TYPE_TOKEN && lane == 0) score[c] = static_cast<double>(distinct);
         }
         __syncthreads();
@@ -933,7 +907,8 @@ int cluster_ctas(const SelectPlan& p) {
 // well 13.9 (6.9-9.1) / 21.1 (5.8-8.5), of a million 31 (20) / 21.3 (12).  Scores, 16 blocks, one launch / three (see below): BM25,
 // blocks of 1024 11.4 (8.0) / 17.6 (7.0), of 2048 11.4 (9.6) / 17.8 (7.5); the divisions of a block's terms are one SM's in one launch, as are
 // the comparisons of a long chunk's positions: chunks of 64 in blocks of 2048 13.8 / 17.9, of 100 21.4 / 18.0, in blocks of
-// 1024 16.2 / 17.7, of 512 in blocks of 1024 87 / 93; type-token ratio, chunks of 128 14.3 / 17.5, of 256 29.7 / 23.6.
+// 1024 16.2 / 17.7, of 512 in blocks of 1024 87 / 93; type-token ratio, chunks of 128 14.3 / 17.5, of 256 29.7 / 23.6.  (Where the
+// host's launches cost nothing, in a graph, four launches are up to 4 us faster: 1024 chunks of two tokens a block 8.5 against 12.1.)
 // Blocks and chunks above that share the df table's launch and have the scores formed by the whole chip, three launches instead of
 // four: BM25 over blocks of 8192, 128,256 entries, 1 block 17.1 (9.9) / 19.5 (10.7), 16 blocks 17.3 (13.2) / 19.7 (14.7); with more
 // entries the table costs the few CTAs more than the launch does: 500,000 18.3 (12.8) / 20.2 (12.6), a million 24.3 (17.4) / 19.8 (15.8).
@@ -942,7 +917,7 @@ constexpr int kClusterDfWords = 4096, kClusterTableWords = 16384;
 bool cluster_table_takes(const SelectPlan& p, int32_t block_size) {
     return p.n_blocks <= kClusterBlocks && block_size <= kClusterTokens && p.words <= kClusterTableWords &&
            static_cast<size_t>(p.words) * 64 <= p.df_bytes &&
-           ClusterShape(p.words, block_size, p.C, 1, 0, false).tokens <= kMaxDynSmem - 2048 && cluster_ctas(p) > 0;
+           ClusterShape(p.words, block_size, p.C, 1, 0, kModeTable).tokens <= kMaxDynSmem - 2048 && cluster_ctas(p) > 0;
 }
 // mode: a score or kModeLevels.  tables: the caller wants df or IDF.
 bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32_t k, int mode, bool tables) {
@@ -951,13 +926,13 @@ bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32
     if (tables && p.words > kClusterDfWords) return false;
     if (mode == PULSAR_SCORE_BM25 && chunk > 64 && block_size > 1024) return false;
     if (mode == PULSAR_SCORE_TYPE_TOKEN && chunk > 128) return false;
-    return ClusterShape(p.words, block_size, p.C, chunk, k, scores).total <= kMaxDynSmem - 2048 &&
+    return ClusterShape(p.words, block_size, p.C, chunk, k, mode).total <= kMaxDynSmem - 2048 &&
            static_cast<size_t>(p.words) * 32 <= p.df_bytes && cluster_ctas(p) > 0;
 }
 
 template <int kMode, typename Table>
 cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const Table& tab, cudaStream_t stream) {
-    const ClusterShape shape(p.words, args.block_size, p.C, args.chunk, args.k, kMode >= 0);
+    const ClusterShape shape(p.words, args.block_size, p.C, args.chunk, args.k, kMode);
     const size_t smem = kMode == kModeTable ? shape.tokens : shape.total;
     auto kernel = select_cluster_kernel<kMode>;
     cudaError_t e = allow_smem(kernel, smem);
