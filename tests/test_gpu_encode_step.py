@@ -1,4 +1,5 @@
 """The step as one call against its three calls."""
+import numpy as np
 import pytest
 import torch
 
@@ -21,20 +22,51 @@ DEV = "cuda:0"
     dict(L=1300, block_size=1300, nq=64),                       # one block
 ])
 def test_one_call_equals_three(shape):
+    """Two contexts in turn through one encoder: whatever a step leaves in its workspaces and outputs is another context's, or
+    not a number, when the next one reads too early."""
     w = W.shrink(W.CONFIGS["tiny"], **shape)
-    enc = ContextEncoder(w, DEV)
-    Q, K, V = (t.to(DEV) for t in W.qkv(w))
-    args = to_dev_ids(W.token_ids(w), DEV), Q, K, V, W.phase2_query(w).to(DEV)
-    events = [torch.cuda.Event() for _ in range(4)]
-    keep = lambda r: [r[k].clone() for k in ("O1", "LSE1", "O2", "LSE2", "prefix_idx")] + [r["sel"]["prefix_len"].clone(), r["sel"]["sel_chunks"].clone()]
-    want = keep(enc.step_device(*args, record=events))
-    for _ in range(3):                                          # back to back: a step beside the end of the one before
-        for t in enc.slots[0].values():
-            if isinstance(t, torch.Tensor) and t.dtype == torch.float32:
-                t.fill_(7.0)
-        got = keep(enc.step_device(*args))
-        assert all(torch.equal(a, b) for a, b in zip(got, want))
-    assert int(enc.status.item()) == 0
+    enc, three = ContextEncoder(w, DEV, slots=6), ContextEncoder(w, DEV)
+    gen = torch.Generator(device=DEV).manual_seed(w.L + w.nq)
+    inputs, want = [], []
+    for seed in range(2):
+        Q, K, V = (torch.randn(w.L, h, w.d, generator=gen, device=DEV, dtype=torch.bfloat16) for h in (w.Hq, w.Hkv, w.Hkv))
+        Qq = torch.randn(w.nq, w.Hq, w.d, generator=gen, device=DEV, dtype=torch.bfloat16)
+        inputs.append((to_dev_ids(ids_with_rare_chunks(w, seed), DEV), Q, K, V, Qq))
+        for t in (three.ws_select, three.ws_p1, three.ws_p2):
+            t.fill_(0xFF)
+        events = [torch.cuda.Event() for _ in range(4)]
+        want.append([t.clone() for t in outputs(three.step_device(*inputs[-1], record=events))])
+    if w.k and w.n_blocks > 1:                                  # the two select different chunks
+        assert not torch.equal(want[0][4], want[1][4]) and not torch.equal(want[0][6], want[1][6])
+    for poisoned in (False, True):
+        for slot in enc.slots if poisoned else []:
+            for t in (slot["O1"], slot["LSE1"], slot["O2"], slot["LSE2"]):
+                t.fill_(float("nan"))
+            for t in slot["sel"]:
+                t.fill_(-0x01010102)
+        got = []
+        for i, slot in enumerate(enc.slots):                    # back to back: a step beside the end of the one before
+            if poisoned:
+                for t in (enc.ws_select, enc.ws_p1, enc.ws_p2):
+                    t.fill_(0xFF)
+            got.append(outputs(enc.step_device(*inputs[i % 2], slot=slot)))
+        for i, res in enumerate(got):
+            assert all(torch.equal(a, b) for a, b in zip(res, want[i % 2])), (poisoned, i)
+    assert int(enc.status.item()) == 0 and int(three.status.item()) == 0
+
+
+def ids_with_rare_chunks(w, seed):
+    """Ids that every block has, and k chunks of each block with an id of their own."""
+    rng = np.random.default_rng(seed)
+    ids = rng.integers(0, 8, w.L).astype(np.uint32)
+    for b in range(w.n_blocks):
+        for c in rng.choice(w.chunks_per_block, w.k, replace=False):
+            ids[min(b * w.block_size + c * w.chunk, w.L - 1)] = 1000 + b * w.chunks_per_block + c
+    return ids
+
+
+def outputs(r):
+    return [r[k] for k in ("O1", "LSE1", "O2", "LSE2", "prefix_idx")] + [r["sel"]["prefix_len"], r["sel"]["sel_chunks"]]
 
 
 def _encoder(**shape):
