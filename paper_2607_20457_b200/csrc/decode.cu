@@ -147,22 +147,24 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
     const auto load = [&](const uint16_t* ctx, const uint16_t* gen, const uint16_t* fresh, int p, int slot) {
         if (p < p_end) {
             const uint32_t dst = ring + slot * kUnitBytes + copy_row * (D * 2);
-            const bool shard = p >= ctx_pieces;
-            const int row0 = (shard ? p - ctx_pieces : p) * kKeys;
-            const int there = (shard ? a.gen_len : a.ctx_len) - row0, total = shard ? a.gen_total - row0 : there;
-            const uint16_t* src = (shard ? gen : ctx) + row0 * pitch + lane_at;
-            if (there >= kKeys) {
+            if (p < ctx_pieces) {
+                const int row0 = p * kKeys, n = a.ctx_len - row0;
+                const uint16_t* src = ctx + row0 * pitch + lane_at;
 #pragma unroll
                 for (int i = 0; i < kCopies; ++i, src += copy_step) {
                     const int r = i * kRowsPerCopy + copy_row;
-                    cp_async16(dst + i * (kRowsPerCopy * D * 2) + ((copy_vec ^ (r & 7)) << 4), src, 16);
+                    const uint32_t to = dst + i * (kRowsPerCopy * D * 2) + ((copy_vec ^ (r & 7)) << 4);
+                    if (n >= kKeys) cp_async16(to, src, 16);
+                    else cp_async16(to, r < n ? src : ctx, r < n ? 16 : 0);
                 }
-            } else {                                           // the context's end, or new tokens behind the shard's rows
+            } else {
+                const int row0 = (p - ctx_pieces) * kKeys;
 #pragma unroll
-                for (int i = 0; i < kCopies; ++i, src += copy_step) {
-                    const int r = i * kRowsPerCopy + copy_row;
-                    const uint16_t* from = r < there ? src : fresh + (r - there) * pitch + head_at;
-                    cp_async16(dst + i * (kRowsPerCopy * D * 2) + ((copy_vec ^ (r & 7)) << 4), r < total ? from : ctx, r < total ? 16 : 0);
+                for (int i = 0; i < kCopies; ++i) {
+                    const int r = i * kRowsPerCopy + copy_row, row = row0 + r;
+                    const uint32_t to = dst + i * (kRowsPerCopy * D * 2) + ((copy_vec ^ (r & 7)) << 4);
+                    const uint16_t* src = (row < a.gen_len ? gen + row * pitch : fresh + (row - a.gen_len) * pitch) + head_at;
+                    cp_async16(to, row < a.gen_total ? src : ctx, row < a.gen_total ? 16 : 0);
                 }
             }
         }
@@ -225,9 +227,8 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
         }
         // keys that do not exist, or that the token of a row must not see yet
         const bool shard = p >= ctx_pieces;
-        const int row0 = (shard ? p - ctx_pieces : p) * kKeys;
-        const bool whole = row0 + kKeys <= (shard ? a.gen_len : a.ctx_len);    // rows that were there before the call, and all tokens see
-        if (!whole) {
+        if (shard || a.ctx_len - p * kKeys < kKeys) {
+            const int row0 = (shard ? p - ctx_pieces : p) * kKeys;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const int token = (2 * tig + k) >> a.g_shift;
@@ -286,8 +287,11 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
                 ldmatrix4_trans(v_lane + at_v + j * (16 * D * 2) + ((c * 32) ^ v_x), f);
                 mma_bf16(o[c], f, pb[j][0], pb[j][1]);
             }
-        // The new tokens' rows go to the shard from the warp that has just read them (from Knew, so nothing waits for it).
-        if (shard && !whole) {
+        // The new tokens' rows go to the shard from the warp that has just read them (from Knew, so nothing waits for it).  Only the
+        // last pieces have any: walked over every piece of the shard, this took half the time of calls with a long one (two tokens of
+        // 32 heads, 20,000 keys and 1000 generated ones 21.5 us, 16.7 like this).  Reading the shard's whole pieces without
+        // choosing each row's source gave another 0.2-1.8 us to such calls and cost the others 0.1-0.2.
+        if (const int row0 = (p - ctx_pieces) * kKeys; shard && row0 + kKeys > a.gen_len) {
 #pragma unroll 1
             for (int i = 0; i < kCopies; ++i) {
                 const int row = row0 + i * kRowsPerCopy + copy_row;
