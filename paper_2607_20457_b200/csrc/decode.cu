@@ -450,26 +450,30 @@ struct DecodePlan {
 // 13.0 / 12.7.  Of several, at least five per head: 131,072 keys of 8 heads 83.5 in 8 clusters of 4, 84.4 in 4 of 8.  Clusters of
 // four from two per head on: of two CTAs they leave the launch with twice the clusters and partials, and 103,998 keys
 // of 16 heads take 129.8 us, in 4 clusters of four 125.4 (the tensor cores' form 123.6), of 24 heads 183.5, 180.1 in two of four (180.8).
-// The times are a fit to calls in a row, whose keys partly stay in L2 (so the rates are above the copy rate): what a call takes
-// besides the data, 5.1 us with one cluster, 6.5 with a second launch; the data at a CTA's rate or at the chip's, 1.2 us
-// later with one cluster, whose CTAs are fewer and end less evenly.  Several have to win by a microsecond, since one needs no
-// second launch where a launch costs more than in a row of calls.  Over 63 shapes (4 to 64 KV heads, 8000 to 103,998 keys) the
-// choice takes 1.00 times the time of the better form in the middle and 1.3 at most, and 1.015 of the tensor cores' at most, 0.87 in the middle.
+// What a call takes besides the data is 5.1 us with one cluster and 6.5 with a second launch.  The data goes at its CTAs' rate, 85
+// kilobytes per us, 60 where two share an SM -- more CTAs than SMs, and clusters of eight or sixteen even of half as many, since a
+// cluster keeps to few SMs -- or at the chip's: L2 where it holds the keys, else HBM, which CTAs packed that way do not use up.
+// A microsecond goes to the form that needs no second launch, since keys that are not in L2 make the two more alike (40 MB of 16 heads, d = 64,
+// 9.4 and 9.4 us from L2, 10.9 and 12.0 from HBM).  Fitted to calls in a row of 141 shapes (1 to 48 KV heads,
+// 4 to 400 MB of keys): the choice takes 1.00 times the better form's time in the middle, more than 1.1 in three, and 1.012 of the
+// tensor cores' form at most, 0.75 in the middle (20,020 keys of 8 heads 12.9, one cluster 16.2, tensor cores 15.4).
 DecodePlan plan_decode(const DecodeCall& c) {
+    constexpr double kOne = 5.1, kMore = 6.5, kMargin = 1.0;                                       // us
+    constexpr double kAlone = 85e3, kShared = 60e3, kL2 = 12.8e6, kHbm = 6.8e6, kHbmPacked = 6.2e6, kL2Bytes = 126e6;   // bytes (per us)
     const double bytes = 4.0 * (c.ctx_len + c.gen_len + c.n) * c.Hkv * c.d;
-    constexpr double kCtaRate = 80e3, kOneRate = 6.6e6, kMoreRate = 6.9e6;       // bytes per us
-    constexpr double kOne = 5.1, kOneTail = 1.2, kMore = 6.5, kMargin = 1.0;     // us
-    const auto per_cta = [&](const DecodePlan& p) { return bytes / (static_cast<double>(p.clusters) * c.Hkv * (1 << p.shift)) / kCtaRate; };
+    const int sms = sm_count();
+    const auto time = [&](const DecodePlan& p) {
+        const int64_t ctas = static_cast<int64_t>(p.clusters) * c.Hkv << p.shift;
+        const bool packed = p.shift >= 3 && ctas > sms / 2 && ctas <= sms, shared = packed || ctas > sms;
+        return std::max(bytes / (ctas * (shared ? kShared : kAlone)), bytes / (bytes < kL2Bytes ? kL2 : packed ? kHbmPacked : kHbm));
+    };
     DecodePlan one{0, 1}, more{0, 1};
     for (int shift = 1; shift <= kMaxClusterShift; ++shift) {
         const int heads_fit = active_clusters(shift) / c.Hkv;
         if (heads_fit >= 1) one.shift = shift;
         if (heads_fit >= (shift == 2 ? 2 : 5)) more = {shift, static_cast<int>(std::min<int64_t>(heads_fit, c.max_parts))};
     }
-    if (more.clusters <= 1) return one;
-    const double t_one = kOne + std::max(per_cta(one), bytes / kOneRate + kOneTail);
-    const double t_more = kMore + std::max(per_cta(more), bytes / kMoreRate);
-    return t_more + kMargin < t_one ? more : one;
+    return more.clusters > 1 && kMore + time(more) + kMargin < kOne + time(one) ? more : one;
 }
 
 int32_t launch_decode_as(const DecodeCall& c, const DecodePlan& p, MergeTodo& todo, cudaStream_t stream) {
