@@ -1497,8 +1497,10 @@ int32_t plan_phase1(int64_t L, int32_t Hq, int32_t Hkv, int32_t d, int32_t block
 // minimises a simple time model --
 //   rounds(J) * (tiles per part * t_tile + t_item)  +  partial traffic(J) / HBM bandwidth,
 // rounds = ceil(items / CTAs).  More parts fill the last round better and shorten it, but every
-// part writes and re-reads fp32 partials.  Constants are measured on B200 (one pair of query
-// tiles against one 128-key tile: about 2 us; per-item prologue and epilogue: about 6 us).
+// part writes and re-reads fp32 partials.  The constants are those of a pair of query tiles against 128-key tiles that come from
+// HBM (about 2 us a tile; per-item prologue and epilogue about 6 us) and stand for every call: items of one query tile take
+// about 0.8 and 2.8 us from L2 (causal_cost), so against their partials' traffic
+// the model cuts them somewhat finer than these costs would.  Few rows against long contexts are cut by plan_decode, which takes only the room for partials from here.
 int32_t choose_splits(int32_t nq, int64_t L, int32_t Hq, int32_t Hkv, int32_t d) {
     const int g = Hq / Hkv;
     const int64_t row_tiles = (static_cast<int64_t>(nq) * g + kTileM - 1) / kTileM;

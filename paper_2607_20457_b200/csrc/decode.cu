@@ -10,7 +10,7 @@
 // tcgen05 would want 128 rows (4 of them used by a single token of 4 heads) and a round trip through TMEM, four
 // barriers and a second launch for the merge on the way of every key tile.
 // One token, us, that form / this one: 6001 keys of 2 heads 10.0 / 7.5, 22,842 of 8 (d = 64) 16.8 / 13.4, 55,734 of 2
-// 20.6 / 15.2, 131,072 of 8 90.4 / 84.7 (0.98 of the measured copy rate).  A key costs an SM about 8 cycles (shared memory written
+// 20.6 / 15.2, 131,072 of 8 91.8 / 84.4 (0.99 of the measured copy rate).  A key costs an SM about 8 cycles (shared memory written
 // and read once), HBM delivers one in 23 when all SMs read.
 #include <algorithm>
 #include <atomic>

@@ -1,6 +1,6 @@
 // Max-IDF summary selection (Section 3.1, Eq. 2-4; Algorithm 1 lines 3 and 6).
 //
-// Up to 16 blocks of ordinary length are one launch, a cluster of a CTA per block (select_cluster_kernel).  Other problems take
+// Up to 16 blocks of ordinary length are one launch, a cluster with a CTA per block (select_cluster_kernel).  Other problems take
 // four launches on one stream, no host synchronisation:
 //   presence_kernel   one CTA per block: a V-bit presence set of the block's token ids, built
 //                     with shared-memory atomicOr and written to the workspace
@@ -350,7 +350,7 @@ __device__ __forceinline__ int chunk_terms(const uint32_t* tok, int len, const S
 // The lanes form the terms (chunk_terms), and lane 0 adds them up in the order of the equations.
 // Latency-bound: one thread per chunk, walking the chunk's pairs
 // of positions serially, took 92 us for 4096 chunks of 32 tokens under BM25 (the whole call 115 us, 16 us with
-// this form and the four launches chained as programmatic dependents).
+// this form and its launches, three or four, chained as programmatic dependents).
 constexpr int kScoreWarps = 4;
 
 template <int kMode, int kBlocks>
