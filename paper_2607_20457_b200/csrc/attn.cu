@@ -1953,8 +1953,8 @@ extern "C" int32_t pulsar_encode_step(const uint32_t* token_ids, int64_t L, int3
                                       size_t phase1_workspace_bytes, const uint16_t* Qq, int32_t nq, int32_t n_splits,
                                       uint16_t* O2, float* LSE2, void* phase2_workspace, size_t phase2_workspace_bytes,
                                       int32_t* device_status, void* stream) {
-    int32_t rc = pulsar_maxidf_select(token_ids, L, vocab_size, block_size, chunk, k, sink, sel_chunks, prefix_idx, prefix_len, nullptr,
-                                      nullptr, select_workspace, select_workspace_bytes, device_status, stream);
+    int32_t rc = launch_maxidf_select(token_ids, L, vocab_size, block_size, chunk, k, sink, sel_chunks, prefix_idx, prefix_len, nullptr,
+                                      nullptr, select_workspace, select_workspace_bytes, device_status, stream, true);
     if (rc != PULSAR_OK) return rc;
     MergeTodo todo;
     const auto phase1 = [&] {

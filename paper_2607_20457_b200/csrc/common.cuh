@@ -26,6 +26,11 @@ inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 int32_t launch_lse_merge(const float* part_O, const float* part_LSE, int32_t n_parts, int64_t rows, int32_t d,
                          uint16_t* O, float* LSE, cudaStream_t stream, bool beside = false);
 
+// pulsar_maxidf_select (select.cu).  shared: a launch that follows wants SMs meanwhile.
+int32_t launch_maxidf_select(const uint32_t* token_ids, int64_t L, int32_t vocab_size, int32_t block_size, int32_t chunk, int32_t k,
+                             int32_t sink, int32_t* sel_chunks, int32_t* prefix_idx, int32_t* prefix_len, uint32_t* df_out,
+                             float* idf_out, void* workspace, size_t workspace_bytes, int32_t* device_status, void* stream, bool shared);
+
 // Kernel launch, optionally with programmatic stream serialization: a dependent launch may be
 // scheduled while the launch before it on the stream still runs (that launch must call
 // grid_launch_dependents) and waits for it with grid_dependency_wait before it touches its results.

@@ -127,6 +127,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
 
     if (C > 1) cluster_arrive();                               // waited for before another CTA's memory is written
     if (!kBeside) grid_dependency_wait();
+    else __threadfence();                                      // (the query rows are read through L1: nothing it holds of the last step)
     grid_launch_dependents();
 
     // ---- this CTA's pieces of kKeys keys: the context's first, then the shard's ----
@@ -175,17 +176,15 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
     load(a.K, a.Kgen, a.Knew, p_first, 0);
     load(a.V, a.Vgen, a.Vnew, p_first, 1);
 
-    // ---- the query rows (row = token * g + head of the group) as B fragments; beside another launch from L2, as in the merge
-    // (every warp reads them: through L1 131,072 keys take 82.7 us, from L2 85.9) ----
-    const auto load_q = [](const uint32_t* p) { return kBeside ? __ldcg(p) : *p; };
+    // ---- the query rows (row = token * g + head of the group) as B fragments ----
     uint32_t q[D / 16][2];
     {
         const int token = gid >> a.g_shift, head = (kvh << a.g_shift) + (gid & ((1 << a.g_shift) - 1));
         const uint32_t* src = reinterpret_cast<const uint32_t*>(a.Q + (static_cast<int64_t>(token) * a.Hq + head) * D) + tig;
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
-            q[kk][0] = gid < a.n_rows ? load_q(src + kk * 8) : 0u;
-            q[kk][1] = gid < a.n_rows ? load_q(src + kk * 8 + 4) : 0u;
+            q[kk][0] = gid < a.n_rows ? src[kk * 8] : 0u;
+            q[kk][1] = gid < a.n_rows ? src[kk * 8 + 4] : 0u;
         }
     }
     // rows 2 tig and 2 tig + 1; o[c]: outputs 16 c + gid and 16 c + 8 + gid of both

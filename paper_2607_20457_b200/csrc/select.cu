@@ -559,7 +559,7 @@ int32_t plan_select(int64_t L, int32_t vocab_size, int32_t block_size, int32_t c
 }
 
 // ---------------------------------------------------------------------------------------------
-// The whole selection in one launch, for sequences of at most 16 blocks: a CTA per block, in a cluster of 16 (8).
+// The whole selection in one launch, for sequences of at most 16 blocks: a CTA per block, in a cluster of 8 or 16.
 // The presence sets stay in shared memory and are read there by the CTAs, those without a block too, that form the df of a slice
 // of the vocabulary each; the df of the block's tokens, the chunks' ranks and the selected chunks are the CTA's own.  What crosses
 // CTAs are two cluster barriers instead of three launches, and the df table (a byte per entry, in L2).  Bound by a chain of
@@ -893,11 +893,20 @@ bool cluster_fits(int ctas) {
     return n > 0;
 }
 
-// CTAs of the cluster; 0 where none fits.  Sixteen also for few blocks, since the vocabulary is shared out among all of them: with a
+constexpr int kClusterDfWords = 4096, kClusterTableWords = 16384;       // of 32 entries: see the rules below
+// CTAs of the cluster; 0 where none fits.  More than blocks where these are few, since the vocabulary is shared out among all: with a
 // CTA per block one block took 13.4 us with 128,256 entries and 71 with a million (the four launches 5.8 and 10.5 on the device), with
-// eight CTAs 5.7 and 13.3, with sixteen 5.4 and 9.5.
-int cluster_ctas(const SelectPlan& p) {
-    if (p.n_blocks <= kClusterBlocks && cluster_fits(kClusterBlocks)) return kClusterBlocks;
+// eight CTAs 5.7 and 13.3, with sixteen 5.4 and 9.5.  Up to 131,072 entries, unless the caller wants their tables as well (8.3 us
+// with eight, 6.9 with sixteen), eight do: sixteen have to find an SM each in one GPC at the end of the launch before them, and
+// a step of 4062 tokens in seven blocks takes 54.8 us instead of 54.3.
+// shared: another launch wants the SMs meanwhile (pulsar_encode_step).  Then it is a CTA per block as long as each has 1024
+// words of the vocabulary at most: 136 work items of Phase 2 beside the selection of 12 blocks found no SM for four of them beside
+// sixteen CTAs, and the step took 37.5 us instead of 33.8.
+int cluster_ctas(const SelectPlan& p, bool tables, bool shared) {
+    if (p.n_blocks > kClusterBlocks) return 0;
+    if (shared && p.words <= 1024 * p.n_blocks && cluster_fits(p.n_blocks)) return p.n_blocks;
+    const bool eight = p.n_blocks <= 8 && p.words <= kClusterDfWords && !tables;
+    if (!eight && cluster_fits(kClusterBlocks)) return kClusterBlocks;
     return p.n_blocks <= 8 && cluster_fits(8) ? 8 : 0;
 }
 
@@ -913,11 +922,10 @@ int cluster_ctas(const SelectPlan& p) {
 // four: BM25 over blocks of 8192, 128,256 entries, 1 block 17.1 (9.9) / 19.5 (10.7), 16 blocks 17.3 (13.2) / 19.7 (14.7); with more
 // entries the table costs the few CTAs more than the launch does: 500,000 18.3 (12.8) / 20.2 (12.6), a million 24.3 (17.4) / 19.8 (15.8).
 constexpr int kClusterLevelTokens = 6144, kClusterScoreTokens = 2048;
-constexpr int kClusterDfWords = 4096, kClusterTableWords = 16384;
 bool cluster_table_takes(const SelectPlan& p, int32_t block_size) {
     return p.n_blocks <= kClusterBlocks && block_size <= kClusterTokens && p.words <= kClusterTableWords &&
            static_cast<size_t>(p.words) * 64 <= p.df_bytes &&
-           ClusterShape(p.words, block_size, p.C, 1, 0, kModeTable).tokens <= kMaxDynSmem - 2048 && cluster_ctas(p) > 0;
+           ClusterShape(p.words, block_size, p.C, 1, 0, kModeTable).tokens <= kMaxDynSmem - 2048 && cluster_ctas(p, false, false) > 0;
 }
 // mode: a score or kModeLevels.  tables: the caller wants df or IDF.
 bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32_t k, int mode, bool tables) {
@@ -927,16 +935,16 @@ bool cluster_takes(const SelectPlan& p, int32_t block_size, int32_t chunk, int32
     if (mode == PULSAR_SCORE_BM25 && chunk > 64 && block_size > 1024) return false;
     if (mode == PULSAR_SCORE_TYPE_TOKEN && chunk > 128) return false;
     return ClusterShape(p.words, block_size, p.C, chunk, k, mode).total <= kMaxDynSmem - 2048 &&
-           static_cast<size_t>(p.words) * 32 <= p.df_bytes && cluster_ctas(p) > 0;
+           static_cast<size_t>(p.words) * 32 <= p.df_bytes && cluster_ctas(p, tables, false) > 0;
 }
 
 template <int kMode, typename Table>
-cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const Table& tab, cudaStream_t stream) {
+cudaError_t launch_cluster(const SelectPlan& p, const ClusterArgs& args, const Table& tab, cudaStream_t stream, bool shared = false) {
     const ClusterShape shape(p.words, args.block_size, p.C, args.chunk, args.k, kMode);
     const size_t smem = kMode == kModeTable ? shape.tokens : shape.total;
     auto kernel = select_cluster_kernel<kMode>;
     cudaError_t e = allow_smem(kernel, smem);
-    const int ctas = cluster_ctas(p);
+    const int ctas = cluster_ctas(p, args.df_out != nullptr || args.idf_out != nullptr, shared);
     if (e == cudaSuccess && ctas > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
@@ -967,11 +975,10 @@ extern "C" size_t pulsar_maxidf_select_workspace_bytes(int64_t L, int32_t vocab_
     return p.total;
 }
 
-extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, int32_t vocab_size,
-                                        int32_t block_size, int32_t chunk, int32_t k, int32_t sink,
-                                        int32_t* sel_chunks, int32_t* prefix_idx, int32_t* prefix_len,
-                                        uint32_t* df_out, float* idf_out, void* workspace,
-                                        size_t workspace_bytes, int32_t* device_status, void* stream_) {
+int32_t pulsar::launch_maxidf_select(const uint32_t* token_ids, int64_t L, int32_t vocab_size, int32_t block_size, int32_t chunk,
+                                     int32_t k, int32_t sink, int32_t* sel_chunks, int32_t* prefix_idx, int32_t* prefix_len,
+                                     uint32_t* df_out, float* idf_out, void* workspace, size_t workspace_bytes,
+                                     int32_t* device_status, void* stream_, bool shared) {
     SelectPlan p;
     int32_t rc = plan_select(L, vocab_size, block_size, chunk, k, sink, p);
     if (rc != PULSAR_OK) return rc;
@@ -988,7 +995,7 @@ extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, in
         const ClusterArgs args{token_ids, L, p.n_blocks, block_size, chunk, k, sink, vocab_size, p.words,
                                static_cast<uint8_t*>(workspace) + p.bitmap_bytes, sel_chunks, prefix_idx, prefix_len, df_out, idf_out,
                                nullptr, device_status};
-        PULSAR_CUDA_OK(launch_cluster<kModeLevels>(p, args, 0, stream));
+        PULSAR_CUDA_OK(launch_cluster<kModeLevels>(p, args, 0, stream, shared));
         count_launch();
         return PULSAR_OK;
     }
@@ -1014,6 +1021,15 @@ extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, in
                                  p.n_blocks, L, block_size, chunk, k, sink, sel_chunks, prefix_idx, prefix_len));
     count_launch();
     return PULSAR_OK;
+}
+
+extern "C" int32_t pulsar_maxidf_select(const uint32_t* token_ids, int64_t L, int32_t vocab_size,
+                                        int32_t block_size, int32_t chunk, int32_t k, int32_t sink,
+                                        int32_t* sel_chunks, int32_t* prefix_idx, int32_t* prefix_len,
+                                        uint32_t* df_out, float* idf_out, void* workspace,
+                                        size_t workspace_bytes, int32_t* device_status, void* stream) {
+    return launch_maxidf_select(token_ids, L, vocab_size, block_size, chunk, k, sink, sel_chunks, prefix_idx, prefix_len, df_out, idf_out,
+                                workspace, workspace_bytes, device_status, stream, false);
 }
 
 // =============================================================================================
