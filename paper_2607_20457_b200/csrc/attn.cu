@@ -205,18 +205,21 @@ retain_block_kv_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
 // Rows of K and V copied to consecutive ones of Kout and Vout: a thread moves four vectors of each, so that a CTA covers the
 // rows that its vectors come to and waits for the launch before it once for all of them.  (A CTA of 128 threads per row, as dependents
 // of the launch before them: 13,235 rows of 8 x 64 14.6 us, 10.3 as plain launches, 6.4 like this.)
-// row_of(j, first): the source row of row j; first: the calling thread has the row's first vector.
+// row_of(j): the source row of row j, found once for each of the CTA's rows (for every vector, packing few rows 3.5 us instead of 2.9).
 template <typename RowOf>
 __device__ __forceinline__ void copy_rows(const uint4* __restrict__ K, const uint4* __restrict__ V, uint4* __restrict__ Kout,
                                           uint4* __restrict__ Vout, int64_t n_rows, int row_vecs, RowOf row_of) {
-    const int64_t base = blockIdx.x * kCopyVecs, j0 = base / row_vecs, n = n_rows * row_vecs - base;      // vectors from base on
-    const uint32_t r0 = static_cast<uint32_t>(base - j0 * row_vecs);
+    __shared__ int s_src[kCopyVecs + 1];                                     // (a vector per row, and a row begun before)
+    const int64_t base = blockIdx.x * kCopyVecs, j0 = base / row_vecs, left = n_rows * row_vecs - base;
+    const uint32_t r0 = static_cast<uint32_t>(base - j0 * row_vecs), n = static_cast<uint32_t>(min(left, kCopyVecs));    // vectors from base on
+    for (uint32_t j = threadIdx.x; j * row_vecs < r0 + n; j += kCopyThreads) s_src[j] = row_of(j0 + j);
+    __syncthreads();
     uint4 k[kCopyUnroll], v[kCopyUnroll];
 #pragma unroll
     for (int u = 0; u < kCopyUnroll; ++u) {
-        const uint32_t i = threadIdx.x + u * kCopyThreads, j = (r0 + i) / row_vecs, at = r0 + i - j * row_vecs;
+        const uint32_t i = threadIdx.x + u * kCopyThreads, j = (r0 + i) / row_vecs;
         if (i < n) {
-            const int64_t src = static_cast<int64_t>(row_of(j0 + j, at == 0)) * row_vecs + at;
+            const int64_t src = static_cast<int64_t>(s_src[j]) * row_vecs + (r0 + i - j * row_vecs);
             k[u] = K[src];
             v[u] = V[src];
         }
@@ -240,10 +243,10 @@ gather_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, con
                    int32_t* status) {
     grid_dependency_wait();
     grid_launch_dependents();
-    copy_rows(K, V, Kout, Vout, n_idx, row_vecs, [&](int64_t j, bool first) {
+    copy_rows(K, V, Kout, Vout, n_idx, row_vecs, [&](int64_t j) {
         const int src_row = idx[j];
         if (src_row >= 0 && src_row < rows_in) return src_row;
-        if (first) report(status, PULSAR_DEV_BAD_PREFIX);
+        report(status, PULSAR_DEV_BAD_PREFIX);
         return 0;
     });
 }
@@ -258,7 +261,7 @@ pack_summary_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, co
                     int32_t* status) {
     grid_dependency_wait();
     grid_launch_dependents();
-    copy_rows(K, V, Kout, Vout, sink + static_cast<int64_t>(n_local) * k * chunk, row_vecs, [&](int64_t row, bool first) {
+    copy_rows(K, V, Kout, Vout, sink + static_cast<int64_t>(n_local) * k * chunk, row_vecs, [&](int64_t row) {
         const int j = static_cast<int>(row);
         if (j < sink) return j;
         const int t = j - sink, sigma = k * chunk;
@@ -267,11 +270,11 @@ pack_summary_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, co
         const int blk = block_ids[s];
         int ch = 0;
         if (blk < 0 || blk >= n_blocks) {
-            if (first) report(status, PULSAR_DEV_BAD_PREFIX);
+            report(status, PULSAR_DEV_BAD_PREFIX);
         } else {
             ch = sel_chunks[static_cast<size_t>(blk) * k + c];
             if (ch < 0 || (ch + 1) * chunk > block_size) {
-                if (first) report(status, PULSAR_DEV_BAD_PREFIX);
+                report(status, PULSAR_DEV_BAD_PREFIX);
                 ch = 0;
             }
         }
