@@ -452,12 +452,12 @@ struct DecodePlan {
 // What a call takes besides the data is 5.1 us with one cluster and 6.5 with a second launch.  The data goes at its CTAs' rate, 85
 // kilobytes per us, 60 where two share an SM -- more CTAs than SMs, and clusters of eight or sixteen even of half as many, since a
 // cluster keeps to few SMs -- or at the chip's: L2 where it holds the keys, else HBM, which CTAs packed that way do not use up.
-// A microsecond goes to the form that needs no second launch, since keys that are not in L2 make the two more alike (40 MB of 16 heads, d = 64,
-// 9.4 and 9.4 us from L2, 10.9 and 12.0 from HBM).  Fitted to calls in a row of 141 shapes (1 to 48 KV heads,
-// 4 to 400 MB of keys): the choice takes 1.00 times the better form's time in the middle, more than 1.1 in three, and 1.012 of the
-// tensor cores' form at most, 0.75 in the middle (20,020 keys of 8 heads 12.9, one cluster 16.2, tensor cores 15.4).
+// 1.5 us go to the form that needs no second launch: the host takes about one for it, and keys that are not in L2 make the two more
+// alike (40 MB of 16 heads, d = 64, 9.4 and 9.4 us from L2, 10.9 and 12.0 from HBM).  Fitted to calls in a row of 141 shapes
+// (1 to 48 KV heads, 4 to 400 MB of keys): the choice takes 1.00 times the better form's time in the middle, more than 1.1 in five, and
+// 1.012 of the tensor cores' form at most, 0.75 in the middle (20,020 keys of 8 heads 12.9, one cluster 16.2, tensor cores 15.4).
 DecodePlan plan_decode(const DecodeCall& c) {
-    constexpr double kOne = 5.1, kMore = 6.5, kMargin = 1.0;                                       // us
+    constexpr double kOne = 5.1, kMore = 6.5, kMargin = 1.5;                                       // us
     constexpr double kAlone = 85e3, kShared = 60e3, kL2 = 12.8e6, kHbm = 6.8e6, kHbmPacked = 6.2e6, kL2Bytes = 126e6;   // bytes (per us)
     const double bytes = 4.0 * (c.ctx_len + c.gen_len + c.n) * c.Hkv * c.d;
     const int sms = sm_count();
