@@ -458,7 +458,7 @@ struct DecodePlan {
 // 1.012 of the tensor cores' form at most, 0.75 in the middle (20,020 keys of 8 heads 12.9, one cluster 16.2, tensor cores 15.4).
 DecodePlan plan_decode(const DecodeCall& c) {
     constexpr double kOne = 5.1, kMore = 6.5, kMargin = 1.5;                                       // us
-    constexpr double kAlone = 85e3, kShared = 60e3, kL2 = 12.8e6, kHbm = 6.8e6, kHbmPacked = 6.2e6, kL2Bytes = 126e6;   // bytes (per us)
+    constexpr double kAlone = 85e3, kShared = 60e3, kL2 = 12.8e6, kHbm = 6.8e6, kHbmPacked = 5.8e6, kL2Bytes = 126e6;   // bytes (per us)
     const double bytes = 4.0 * (c.ctx_len + c.gen_len + c.n) * c.Hkv * c.d;
     const int sms = sm_count();
     const auto time = [&](const DecodePlan& p) {
